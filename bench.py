@@ -239,14 +239,16 @@ def _peaks():
 
 
 def kernel_source_hash(packed):
-    """sha256[:16] of the all-pairs kernel source a launch shape runs (its .cu file
-    followed by the shared device header), comments and blank lines left out so
+    """sha256[:16] of the all-pairs kernel source a launch shape runs (its .cu file,
+    for the grouped shapes both grouped files, followed by the shared device header), comments and blank lines left out so
     that only code changes count."""
     import hashlib
     csrc = os.path.join(ROOT, "paper_2501_04456_gb300", "csrc")
-    name = "allpairs_grouped.cu" if packed in (2, 3) else "allpairs.cu"
+    files = ["allpairs_grouped.cu", "allpairs_sym.cu"] if packed in (2, 3) else ["allpairs.cu"]
     code = []
-    for f in (name, "npsim_internal.cuh"):
+    for f in files + ["npsim_internal.cuh"]:
+        if not os.path.exists(os.path.join(csrc, f)):
+            continue
         txt = open(os.path.join(csrc, f), encoding="utf-8").read()
         txt = re.sub(r"/\*.*?\*/", "", txt, flags=re.S)  # block comments
         for ln in txt.splitlines():

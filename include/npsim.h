@@ -237,9 +237,10 @@ int npsim_normals(uint64_t seed, int64_t step, int64_t n, double *out);
 /* Launch shape of the all-pairs kernel chosen by the autotuner: threads per
  * CTA, particles i per thread, j-tile length, CTAs launched, the index of the shape in
  * the autotuner's table, and 1 if it is the packed float32x2 Coulomb kernel, 2
- * if it is the packed Coulomb kernel over partners grouped by charge value, 3
- * if it is the packed LJ + Coulomb kernel over partners grouped by type (0: the
- * scalar kernel).  Any pointer may be NULL.  The grouped kernels (2, 3) cut
+ * if it is a packed Coulomb kernel over partners grouped by charge value, 3
+ * if it is a packed LJ + Coulomb kernel over partners grouped by type (0: the
+ * scalar kernel).  Kinds 2 and 3 include the kernels that evaluate each pair
+ * once for both particles.  Any pointer may be NULL.  The grouped kernels (2, 3) cut
  * their work into a number of ranges per CTA that the autotuner also picks and
  * hand the ranges out at run time.  The environment variable
  * NPSIM_AUTOTUNE=1:<index>[:<ranges per CTA>] forces a shape at npsim_create

@@ -31,7 +31,10 @@
 // all-pairs kernels (stream-K), one compensated (hi, lo) float32 partial per
 // (row, range) written to slot row + range.  The ranges are handed out at run
 // time: CTA c starts on range c and then takes the next free range from a
-// device counter.  Two CTAs sharing an SM do not advance at the same rate (the
+// device counter.  These kernels evaluate every ordered pair; those of
+// allpairs_sym.cu, which evaluate each pair once, are faster at every size (1.08
+// to 1.4 times) but keep 6 N^2 / itile bytes of partner sums: one shape of each
+// kernel here serves the sums for which that scratch is too large.  Two CTAs sharing an SM do not advance at the same rate (the
 // warp schedulers favour one), so with a fixed split the favoured CTA finishes
 // early and leaves its SM half occupied; with several ranges per CTA it takes
 // more of them instead.
@@ -207,12 +210,7 @@ struct GEntry {
 
 #define NPSIM_GRP(B, K, J) GEntry{ApConfig{B, K, J, 0}, (const void *)k_coulomb_grp<B, K, J>}
 
-const GEntry kGrp[] = {
-    NPSIM_GRP(512, 2, 512), NPSIM_GRP(256, 2, 512), NPSIM_GRP(256, 4, 256),
-    NPSIM_GRP(256, 2, 256), NPSIM_GRP(128, 4, 256), NPSIM_GRP(512, 1, 512),
-    NPSIM_GRP(1024, 1, 512),
-    NPSIM_GRP(256, 4, 512), NPSIM_GRP(128, 4, 512),
-};
+const GEntry kGrp[] = {NPSIM_GRP(256, 4, 512)};
 
 // CTAs of a dynamic launch (a static StreamK runs one CTA per range)
 int dyn_ctas(const StreamK &sk) { return sk.ctas > 0 ? min(sk.ctas, sk.grid) : sk.grid; }
@@ -227,10 +225,7 @@ cudaError_t launch_g(const StreamK &sk, const float4 *xq, const int *perm, int n
 
 #define NPSIM_LJG(B, K, J) GEntry{ApConfig{B, K, J, 0}, (const void *)k_ljc_grp<B, K, J>}
 
-const GEntry kLjg[] = {
-    NPSIM_LJG(256, 1, 512), NPSIM_LJG(256, 2, 512), NPSIM_LJG(512, 1, 512),
-    NPSIM_LJG(128, 2, 256), NPSIM_LJG(256, 2, 256), NPSIM_LJG(128, 4, 256),
-};
+const GEntry kLjg[] = {NPSIM_LJG(512, 1, 512)};
 
 template <int B, int K, int J>
 cudaError_t launch_l(const StreamK &sk, const float4 *xq, const int *perm, int n_perm,
@@ -262,15 +257,7 @@ cudaError_t launch_allpairs_grouped(int idx, const StreamK &sk, const float4 *xq
                                     unsigned *work, float *slots, cudaStream_t st)
 {
     switch (idx) {
-    case 0: return launch_g<512, 2, 512>(sk, xq, perm, n_perm, qblk, work, slots, st);
-    case 1: return launch_g<256, 2, 512>(sk, xq, perm, n_perm, qblk, work, slots, st);
-    case 2: return launch_g<256, 4, 256>(sk, xq, perm, n_perm, qblk, work, slots, st);
-    case 3: return launch_g<256, 2, 256>(sk, xq, perm, n_perm, qblk, work, slots, st);
-    case 4: return launch_g<128, 4, 256>(sk, xq, perm, n_perm, qblk, work, slots, st);
-    case 5: return launch_g<512, 1, 512>(sk, xq, perm, n_perm, qblk, work, slots, st);
-    case 6: return launch_g<1024, 1, 512>(sk, xq, perm, n_perm, qblk, work, slots, st);
-    case 7: return launch_g<256, 4, 512>(sk, xq, perm, n_perm, qblk, work, slots, st);
-    case 8: return launch_g<128, 4, 512>(sk, xq, perm, n_perm, qblk, work, slots, st);
+    case 0: return launch_g<256, 4, 512>(sk, xq, perm, n_perm, qblk, work, slots, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -294,12 +281,7 @@ cudaError_t launch_allpairs_ljgrp(int idx, const StreamK &sk, const float4 *xq,
                                   unsigned *work, float *slots, cudaStream_t st)
 {
     switch (idx) {
-    case 0: return launch_l<256, 1, 512>(sk, xq, perm, n_perm, tblk, tab, rc2_lim, has_coul, work, slots, st);
-    case 1: return launch_l<256, 2, 512>(sk, xq, perm, n_perm, tblk, tab, rc2_lim, has_coul, work, slots, st);
-    case 2: return launch_l<512, 1, 512>(sk, xq, perm, n_perm, tblk, tab, rc2_lim, has_coul, work, slots, st);
-    case 3: return launch_l<128, 2, 256>(sk, xq, perm, n_perm, tblk, tab, rc2_lim, has_coul, work, slots, st);
-    case 4: return launch_l<256, 2, 256>(sk, xq, perm, n_perm, tblk, tab, rc2_lim, has_coul, work, slots, st);
-    case 5: return launch_l<128, 4, 256>(sk, xq, perm, n_perm, tblk, tab, rc2_lim, has_coul, work, slots, st);
+    case 0: return launch_l<512, 1, 512>(sk, xq, perm, n_perm, tblk, tab, rc2_lim, has_coul, work, slots, st);
     default: return cudaErrorInvalidValue;
     }
 }

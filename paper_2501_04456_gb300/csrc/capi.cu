@@ -148,6 +148,8 @@ void fill_streamk(StreamK &sk, int n, const ApConfig &c, int grid_target)
     sk.W = (long long)sk.n_it * sk.n_jt;
     sk.grid = (int)std::min<long long>(std::max(grid_target, 1), sk.W);
     sk.ctas = 0;
+    sk.tri = 0;
+    sk.len = 0;
 }
 
 // Floats of stream-K partial slots: one slot per (i-tile row, range) pair a
@@ -200,6 +202,7 @@ struct npsim_sim {
     float4 *xq = nullptr;
     int *typ = nullptr;
     float *slots = nullptr;
+    float *F_pair = nullptr;              // [n][8] all-pairs forces (each-pair-once shapes)
     unsigned *ap_work = nullptr;          // range counters of the grouped kernels [2]
     float *F_lj = nullptr;                // [n][8]: (hi x, y, z, lo x | lo y, z, -, -)
     PairTab *tab_full = nullptr, *tab_lj = nullptr, *tab_coul = nullptr;
@@ -279,6 +282,7 @@ struct npsim_sim {
         dfree(xq);
         dfree(typ);
         dfree(slots);
+        dfree(F_pair);
         dfree(ap_work);
         dfree(perm);
         dfree(qblk);
@@ -408,32 +412,90 @@ int ensure_cells(npsim_sim *s, CellGrid &g)
 }
 
 
-// Launch shapes of the all-pairs sum in one index space: [0, A) the
-// identity-order kernels of allpairs.cu (scalar and packed), then [A, A + G) the
-// charge-grouped Coulomb kernels and [A + G, A + G + L) the type-grouped LJ +
-// Coulomb kernels of allpairs_grouped.cu.
-int shape_count() { return ap_num_configs() + grp_num_configs() + ljg_num_configs(); }
+// Launch shapes of the all-pairs sum in one index space: the identity-order
+// kernels of allpairs.cu (scalar and packed), the charge-grouped Coulomb kernels
+// of allpairs_grouped.cu, the Coulomb kernels of allpairs_sym.cu (each pair
+// once), then the LJ + Coulomb kernels of allpairs_grouped.cu and of
+// allpairs_sym.cu.
+enum ShapeFamily { SF_PLAIN, SF_GRP, SF_SYM, SF_LJG, SF_SYMLJ };
 
-bool shape_grouped(int k) { return k >= ap_num_configs(); }
+int family_size(int f)
+{
+    switch (f) {
+    case SF_PLAIN: return ap_num_configs();
+    case SF_GRP: return grp_num_configs();
+    case SF_SYM: return sym_num_configs(false);
+    case SF_LJG: return ljg_num_configs();
+    default: return sym_num_configs(true);
+    }
+}
 
-bool shape_ljg(int k) { return k >= ap_num_configs() + grp_num_configs(); }
+int shape_count()
+{
+    int n = 0;
+    for (int f = SF_PLAIN; f <= SF_SYMLJ; ++f)
+        n += family_size(f);
+    return n;
+}
+
+// Family of shape k; *local receives its index inside the family.
+int shape_family(int k, int *local = nullptr)
+{
+    int f = SF_PLAIN;
+    while (f < SF_SYMLJ && k >= family_size(f))
+        k -= family_size(f++);
+    if (local)
+        *local = k;
+    return f;
+}
+
+bool shape_grouped(int k) { return shape_family(k) != SF_PLAIN; }
+
+// LJ + Coulomb kernels over the grouped order
+bool shape_ljg(int k) { return shape_family(k) >= SF_LJG; }
+
+// kernels that evaluate each pair once
+bool shape_sym(int k)
+{
+    const int f = shape_family(k);
+    return f == SF_SYM || f == SF_SYMLJ;
+}
 
 ApConfig shape_config(int k)
 {
-    if (shape_ljg(k))
-        return ljg_config(k - ap_num_configs() - grp_num_configs());
-    return shape_grouped(k) ? grp_config(k - ap_num_configs()) : ap_config(k);
+    int l = 0;
+    switch (shape_family(k, &l)) {
+    case SF_PLAIN: return ap_config(l);
+    case SF_GRP: return grp_config(l);
+    case SF_LJG: return ljg_config(l);
+    case SF_SYM: return sym_config(false, l);
+    default: return sym_config(true, l);
+    }
 }
+
+// Column partials of the kernels that evaluate each pair once take 6 bytes x
+// N^2 / itile: allowed up to this size (about 1.5 million grouped NPs with the
+// largest row tile); beyond it the one-sided kernels, whose scratch grows with
+// N, remain.
+constexpr size_t kSymMaxBytes = (size_t)8 << 30;
 
 int shape_occupancy(const npsim_sim *s, int k, bool lj)
 {
-    if (shape_grouped(k) && (!s->perm || s->grp_len == 0))
+    int l = 0;
+    const int f = shape_family(k, &l);
+    if (f != SF_PLAIN && (!s->perm || s->grp_len == 0))
         return 0;
-    if (shape_ljg(k))
-        return ljg_occupancy(k - ap_num_configs() - grp_num_configs());
-    if (shape_grouped(k))
-        return lj ? 0 : grp_occupancy(k - ap_num_configs());
-    return ap_occupancy(k, lj);
+    if (f == SF_SYM || f == SF_SYMLJ) {
+        const ApConfig c = shape_config(k);
+        if (sym_col_floats(s->grp_len, c.block * c.ki) * sizeof(float) > kSymMaxBytes)
+            return 0;
+        return f == SF_SYMLJ ? sym_occupancy(true, l) : lj ? 0 : sym_occupancy(false, l);
+    }
+    if (f == SF_LJG)
+        return ljg_occupancy(l);
+    if (f == SF_GRP)
+        return lj ? 0 : grp_occupancy(l);
+    return ap_occupancy(l, lj);
 }
 
 // Stream-K split of shape k on `ctas` CTAs; the grouped kernels cut the
@@ -451,6 +513,12 @@ void shape_streamk(const npsim_sim *s, int k, int ctas, int per_cta, StreamK &sk
     sk.n_it = (s->grp_len + sk.itile - 1) / sk.itile;
     sk.n_jt = s->grp_len / c.jt;
     sk.W = (long long)sk.n_it * sk.n_jt;
+    sk.tri = 0;
+    sk.len = s->grp_len;
+    if (shape_sym(k)) {
+        sk.tri = sk.itile / sk.jtile;
+        sk.W = tri_row_begin(sk, sk.n_it);
+    }
     ctas = std::max(ctas, 1);
     sk.grid = (int)std::min<long long>((long long)ctas * std::max(per_cta, 1), sk.W);
     sk.ctas = std::min(ctas, sk.grid);
@@ -462,19 +530,39 @@ const PairTab *pair_table(const npsim_sim *s, bool lj, bool coul)
     return lj ? (coul ? s->tab_full : s->tab_lj) : s->tab_coul;
 }
 
+size_t shape_slots_floats(const StreamK &sk)
+{
+    return sk.tri ? sym_slots_floats(sk) : slots_floats(sk);
+}
+
 cudaError_t shape_launch(const npsim_sim *s, int k, bool lj, bool coul, const StreamK &sk,
                          float *slots, cudaStream_t st)
 {
-    if (shape_ljg(k))
-        return launch_allpairs_ljgrp(k - ap_num_configs() - grp_num_configs(), sk, s->xq,
-                                     s->perm, s->n_perm, s->tblk, pair_table(s, lj, coul),
-                                     lj ? s->rc2_lim : 0.0f, coul ? s->any_charge : 0,
-                                     s->ap_work, slots, st);
-    if (shape_grouped(k))
-        return launch_allpairs_grouped(k - ap_num_configs(), sk, s->xq, s->perm, s->n_perm,
-                                       s->qblk, s->ap_work, slots, st);
-    return launch_allpairs(k, lj, sk, s->xq, s->typ, s->n, lj ? pair_table(s, lj, coul) : nullptr,
+    int l = 0;
+    const int f = shape_family(k, &l);
+    if (f == SF_SYM || f == SF_SYMLJ)
+        return launch_allpairs_sym(f == SF_SYMLJ, l, sk, s->xq, s->perm, s->tblk,
+                                   pair_table(s, lj, coul), coul ? s->any_charge : 0, s->ap_work,
+                                   slots, st);
+    if (f == SF_LJG)
+        return launch_allpairs_ljgrp(l, sk, s->xq, s->perm, s->n_perm, s->tblk,
+                                     pair_table(s, lj, coul), lj ? s->rc2_lim : 0.0f,
+                                     coul ? s->any_charge : 0, s->ap_work, slots, st);
+    if (f == SF_GRP)
+        return launch_allpairs_grouped(l, sk, s->xq, s->perm, s->n_perm, s->qblk, s->ap_work,
+                                       slots, st);
+    return launch_allpairs(l, lj, sk, s->xq, s->typ, s->n, lj ? pair_table(s, lj, coul) : nullptr,
                            slots, st);
+}
+
+// The sum of shape k's partials that a step pays for beside its all-pairs
+// launch: the reduction into F_pair, or the integrator's read of the slots.
+cudaError_t shape_sum(const npsim_sim *s, int k, const StreamK &sk, const float *slots, float *out,
+                      cudaStream_t st)
+{
+    if (sk.tri)
+        return launch_sym_reduce(sk, slots, s->perm, out, st);
+    return launch_slot_sum(slots, sk, shape_grouped(k) ? s->grp_len : s->n, out, st);
 }
 
 // Queue the pair forces of the current positions and one integrator pass at
@@ -523,6 +611,8 @@ int enqueue_pass(npsim_sim *s, int mode, bool want_lj, bool want_coul, bool ext,
     if (ap) {
         NP_CUDA(mark(KG_ALLPAIRS, 0));
         NP_CUDA(shape_launch(s, s->ap_idx, ap_lj, ap_coul, s->sk, s->slots, st));
+        if (s->sk.tri)
+            NP_CUDA(launch_sym_reduce(s->sk, s->slots, s->perm, s->F_pair, st));
         NP_CUDA(mark(KG_ALLPAIRS, 1));
     }
     IntArgs a{};
@@ -531,11 +621,12 @@ int enqueue_pass(npsim_sim *s, int mode, bool want_lj, bool want_coul, bool ext,
     a.F = Fout;
     a.typ = s->typ;
     a.xq = s->xq;
-    a.slots = ap ? s->slots : nullptr;
+    a.slots = ap && !s->sk.tri ? s->slots : nullptr;
+    a.F_pair = ap && s->sk.tri ? s->F_pair : nullptr;
     a.sk = s->sk;
     a.F_lj = lj_cell ? s->F_lj : nullptr;
     a.ext_on = ext ? 1 : 0;
-    a.field_slots = (ap && !ap_lj && !ljg) ? 1 : 0; // ljg sums C q_a q_b from its table
+    a.field_slots = (a.slots && !ap_lj && !ljg) ? 1 : 0; // ljg sums C q_a q_b from its table
     a.row_pos = grouped ? s->row_pos : nullptr;
     a.spring = s->d_spring;
     a.x_ref = s->cell ? s->nl.x_ref : nullptr;
@@ -718,19 +809,29 @@ int autotune(npsim_sim *s)
     const int n_m = (int)(sizeof(kRangesPerCta) / sizeof(kRangesPerCta[0]));
     int best = 0, best_m = kDefaultRangesPerCta;
     {
-        // scratch big enough for every candidate
-        size_t need = 0;
-        for (int c = 0; c < nc; ++c) {
-            const int occ = shape_occupancy(s, c, lj);
-            if (occ <= 0)
-                continue;
-            StreamK sk;
-            shape_streamk(s, c, occ * s->sms, kRangesPerCta[n_m - 1], sk);
-            need = std::max(need, slots_floats(sk));
-        }
-        const size_t out_floats = 6 * (size_t)std::max(s->n, s->grp_len);
+        // scratch big enough for every candidate; where it does not fit, for the
+        // one-sided ones
+        const size_t out_floats = 8 * (size_t)std::max(s->n, s->grp_len);
         float *tmp = nullptr;
-        NP_CUDA(dalloc(&tmp, need + out_floats));
+        size_t need = 0;
+        for (bool sym : {true, false}) {
+            need = 0;
+            for (int c = 0; c < nc; ++c) {
+                const int occ = shape_occupancy(s, c, lj);
+                if (occ <= 0 || (shape_sym(c) && !sym))
+                    continue;
+                StreamK sk;
+                shape_streamk(s, c, occ * s->sms, kRangesPerCta[n_m - 1], sk);
+                need = std::max(need, shape_slots_floats(sk));
+            }
+            need = (need + 3) & ~(size_t)3; // 16-byte records follow
+            const cudaError_t e = dalloc(&tmp, need + out_floats);
+            if (e == cudaSuccess)
+                break;
+            if (!sym || e != cudaErrorMemoryAllocation)
+                NP_CUDA(e);
+            cudaGetLastError(); // the failed allocation
+        }
         float *sum_out = tmp + need;
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
@@ -748,15 +849,16 @@ int autotune(npsim_sim *s)
                 shape_streamk(s, c, occ * s->sms, m, sk);
                 if (shape_grouped(c) && mi > 0 && sk.grid == sk.ctas)
                     break; // no more ranges than CTAs: the same launch as m = 1
-                const int n_pos = shape_grouped(c) ? s->grp_len : s->n;
+                if (shape_slots_floats(sk) > need)
+                    break; // the scratch did not fit
                 if (shape_launch(s, c, lj, coul, sk, tmp, s->user) != cudaSuccess ||
-                    launch_slot_sum(tmp, sk, n_pos, sum_out, s->user) != cudaSuccess)
+                    shape_sum(s, c, sk, tmp, sum_out, s->user) != cudaSuccess)
                     continue;
                 const int reps = s->n > 100000 ? 2 : 5;
                 cudaEventRecord(e0, s->user);
                 for (int r = 0; r < reps; ++r) {
                     shape_launch(s, c, lj, coul, sk, tmp, s->user);
-                    launch_slot_sum(tmp, sk, n_pos, sum_out, s->user);
+                    shape_sum(s, c, sk, tmp, sum_out, s->user);
                 }
                 cudaEventRecord(e1, s->user);
                 if (cudaEventSynchronize(e1) != cudaSuccess)
@@ -1318,9 +1420,24 @@ int create_impl(const npsim_type_t *types, const npsim_params_t *params, int64_t
         rc = autotune(s);
         if (rc)
             return bail(rc);
-        const int occ = std::max(1, shape_occupancy(s, s->ap_idx, s->ap_lj));
+        int occ = std::max(1, shape_occupancy(s, s->ap_idx, s->ap_lj));
         shape_streamk(s, s->ap_idx, occ * s->sms, s->ap_per_cta, s->sk);
-        BAIL_CUDA(dalloc(&s->slots, slots_floats(s->sk)));
+        ce = dalloc(&s->slots, shape_slots_floats(s->sk));
+        if (ce == cudaSuccess && s->sk.tri)
+            ce = dalloc(&s->F_pair, 8 * (size_t)n);
+        if (ce == cudaErrorMemoryAllocation && s->sk.tri) {
+            // no room for the column partials: a one-sided shape, whose scratch
+            // grows with N only
+            cudaGetLastError();
+            dfree(s->slots);
+            s->ap_idx = 0;
+            while (shape_family(s->ap_idx) != (s->ap_lj ? SF_LJG : SF_GRP))
+                ++s->ap_idx;
+            occ = std::max(1, shape_occupancy(s, s->ap_idx, s->ap_lj));
+            shape_streamk(s, s->ap_idx, occ * s->sms, s->ap_per_cta, s->sk);
+            ce = dalloc(&s->slots, shape_slots_floats(s->sk));
+        }
+        BAIL_CUDA(ce);
     } else {
         s->sk = StreamK{};
         s->sk.itile = 1;
@@ -1585,8 +1702,8 @@ int npsim_allpairs_num_configs(int *count)
 int npsim_launches_per_step(npsim_sim_t s, int *launches)
 {
     NP_REQUIRE(s && launches, "sim and launches are required");
-    // integrator, all-pairs, the gated cell and list builds, the list LJ forces
-    *launches = 1 + (s->ap ? 1 : 0) + (s->cell ? cell_build_launches() + 2 : 0);
+    // integrator, all-pairs (and the sum of its partials), the gated cell and list builds, the list LJ forces
+    *launches = 1 + (s->ap ? (s->sk.tri ? 2 : 1) : 0) + (s->cell ? cell_build_launches() + 2 : 0);
     return NPSIM_OK;
 }
 

@@ -136,6 +136,17 @@ __device__ __forceinline__ void update_particle(const IntArgs &a, const StepPara
                     df_mul(Fh[d], Fl[d], tc.qc);
             }
         }
+        if (a.F_pair && pos >= 0) { // summed already (k_sym_reduce)
+            any = true;
+            const float4 *r = reinterpret_cast<const float4 *>(a.F_pair + 8 * (size_t)i);
+            const float4 r0 = r[0], r1 = r[1];
+            Fh[0] = r0.x;
+            Fh[1] = r0.y;
+            Fh[2] = r0.z;
+            Fl[0] = r0.w;
+            Fl[1] = r1.x;
+            Fl[2] = r1.y;
+        }
         if (a.F_lj) {
             any = true;
             df_add_df(Fh[0], Fl[0], st.flj0.x, st.flj0.w);

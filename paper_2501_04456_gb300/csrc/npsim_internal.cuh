@@ -85,6 +85,9 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float a)
 constexpr float kPairSelfEps = 1e-20f; // added to r^2; the self pair has r_ij = 0 exactly
 constexpr float kPairSelfMin = 1e-12f; // LJ: r^2 below this is the self pair
 constexpr float kPairPad = 1.0e18f;    // padding position: every term with it underflows to 0
+// Smallest |C q_a q_b| in whose units sym_row_segment keeps its sums: below it
+// the division of the LJ depth by it would bring the overflow of s^12 closer.
+constexpr float kSymMinScale = 1e-4f;
 
 // One j-tile of the packed LJ + Coulomb pair sum: KI rows per thread, JP
 // partner pairs staged in shared memory as negated coordinates, s_a = (-x0,
@@ -451,6 +454,328 @@ __device__ __forceinline__ void ljc_row_segment(const float4 *__restrict__ xq,
 }
 
 // ---------------------------------------------------------------------------
+// Each unordered pair once (Newton's third law): the pair force is added to the
+// row's sum and, with the other sign, to the partner's.
+//
+// A warp holds 32 KI rows in registers (KI per lane) and meets 64 partners (32
+// staged entries of two) in 32 steps: at step s lane l takes entry (l + s) mod
+// 32, so the lanes read 32 consecutive entries of shared memory without bank
+// conflicts, and the sum of an entry's partners travels with the entry from
+// lane to lane (three float2 shuffles per step, shared by KI rows).  After 32
+// steps every row has met every partner, each entry's sums are complete over
+// the warp's rows and back in lane (entry).  Per unordered pair 14 packed lanes
+// (3 sub, 3 for r^2, 2 for 1/r^3, 3 + 3 accumulate) where the one-sided sweep
+// spends 2 x 11.  Measured on one full chip of warps (synthetic tiles, 1e10
+// ordered pairs): one-sided 3.43 ms; each pair once 2.53 ms with KI = 4 (96-128
+// registers), 2.29 with KI = 8 (168 registers, 12 warps per SM, steps unrolled
+// eight times), 2.22 with the shuffles left out: the FP32 pipe is the bound
+// (76-79 % of its lanes issue in every one of these forms), and the more rows
+// share a step's shuffles and shared-memory reads the nearer it is.  The sums of
+// two rows or two partners per register pair, folded before the shuffle (three
+// shuffles for six), measured no better (2.38).
+
+// One rotation of an entry's sums: lane l takes lane l + 1's.
+__device__ __forceinline__ void sym_rotate(float2 &g, int src)
+{
+    g.x = __shfl_sync(0xffffffffu, g.x, src);
+    g.y = __shfl_sync(0xffffffffu, g.y, src);
+}
+
+// Coulomb-only: ax += d / r^3 for the rows, g += d / r^3 for the partners (the
+// caller applies the charges and the partners' sign).
+template <int KI>
+__device__ __forceinline__ void coul_sym_sweep(const float4 *__restrict__ s_a,
+                                               const float2 *__restrict__ s_b, int lane,
+                                               const float2 (&xi)[KI], const float2 (&yi)[KI],
+                                               const float2 (&zi)[KI], float2 (&ax)[KI],
+                                               float2 (&ay)[KI], float2 (&az)[KI], float2 &gx,
+                                               float2 &gy, float2 &gz)
+{
+    const float2 eps2 = make_float2(kPairSelfEps, kPairSelfEps);
+    const int src = (lane + 1) & 31;
+#pragma unroll 8
+    for (int s = 0; s < 32; ++s) {
+        const int m = (lane + s) & 31;
+        const float4 a = s_a[m];
+        const float2 nz = s_b[m];
+        const float2 nx = make_float2(a.x, a.y), ny = make_float2(a.z, a.w);
+#pragma unroll
+        for (int k = 0; k < KI; ++k) {
+            const float2 dx = __fadd2_rn(xi[k], nx);
+            const float2 dy = __fadd2_rn(yi[k], ny);
+            const float2 dz = __fadd2_rn(zi[k], nz);
+            float2 r2 = __ffma2_rn(dz, dz, eps2);
+            r2 = __ffma2_rn(dy, dy, r2);
+            r2 = __ffma2_rn(dx, dx, r2);
+            const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+            const float2 f = __fmul2_rn(__fmul2_rn(ri, ri), ri);
+            ax[k] = __ffma2_rn(f, dx, ax[k]);
+            ay[k] = __ffma2_rn(f, dy, ay[k]);
+            az[k] = __ffma2_rn(f, dz, az[k]);
+            gx = __ffma2_rn(f, dx, gx);
+            gy = __ffma2_rn(f, dy, gy);
+            gz = __ffma2_rn(f, dz, gz);
+        }
+        sym_rotate(gx, src);
+        sym_rotate(gy, src);
+        sym_rotate(gz, src);
+    }
+}
+
+// LJ + Coulomb with one set of pair constants (a warp's rows have one type and a
+// tile's partners another): cst = (sigma_ab^2, 24 eps_ab, rc_ab^2, C q_a q_b),
+// as in ljc_tile_sweep without the self pair.
+template <int KI>
+__device__ __forceinline__ void ljc_sym_sweep(const float4 *__restrict__ s_a,
+                                              const float2 *__restrict__ s_b, int lane,
+                                              const float2 (&xi)[KI], const float2 (&yi)[KI],
+                                              const float2 (&zi)[KI], const float4 cst,
+                                              float2 (&ax)[KI], float2 (&ay)[KI],
+                                              float2 (&az)[KI], float2 &gx, float2 &gy, float2 &gz)
+{
+    const float2 eps2 = make_float2(kPairSelfEps, kPairSelfEps);
+    const float2 sig2 = make_float2(cst.x, cst.x);
+    const float2 e48 = make_float2(2.0f * cst.y, 2.0f * cst.y);
+    const float2 em24 = make_float2(-cst.y, -cst.y);
+    const float2 cqq = make_float2(cst.w, cst.w);
+    const int src = (lane + 1) & 31;
+    for (int s = 0; s < 32; ++s) {
+        const int m = (lane + s) & 31;
+        const float4 a = s_a[m];
+        const float2 nz = s_b[m];
+        const float2 nx = make_float2(a.x, a.y), ny = make_float2(a.z, a.w);
+#pragma unroll
+        for (int k = 0; k < KI; ++k) {
+            const float2 dx = __fadd2_rn(xi[k], nx);
+            const float2 dy = __fadd2_rn(yi[k], ny);
+            const float2 dz = __fadd2_rn(zi[k], nz);
+            float2 r2 = __ffma2_rn(dz, dz, eps2);
+            r2 = __ffma2_rn(dy, dy, r2);
+            r2 = __ffma2_rn(dx, dx, r2);
+            const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+            const float2 ri2 = __fmul2_rn(ri, ri);
+            const float2 s2 = __fmul2_rn(sig2, ri2);
+            const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
+            float2 t = __fmul2_rn(s6, __ffma2_rn(e48, s6, em24));
+            t.x = r2.x < cst.z ? t.x : 0.0f;
+            t.y = r2.y < cst.z ? t.y : 0.0f;
+            const float2 f = __fmul2_rn(__ffma2_rn(cqq, ri, t), ri2);
+            ax[k] = __ffma2_rn(f, dx, ax[k]);
+            ay[k] = __ffma2_rn(f, dy, ay[k]);
+            az[k] = __ffma2_rn(f, dz, az[k]);
+            gx = __ffma2_rn(f, dx, gx);
+            gy = __ffma2_rn(f, dy, gy);
+            gz = __ffma2_rn(f, dz, gz);
+        }
+        sym_rotate(gx, src);
+        sym_rotate(gy, src);
+        sym_rotate(gz, src);
+    }
+}
+
+// Shared memory of sym_row_segment: the staged tiles of LjcSmem and the
+// partners' sums of one tile per warp (two buffers: one is summed over the warps
+// while the next tile fills the other).
+template <int BLOCK, int KI, int JT>
+struct SymSmem {
+    LjcSmem<JT> st;
+    float2 g[2][3][BLOCK / 32][JT / 2];
+    float hl[6][KI * BLOCK]; // the rows' compensated sums (hi x, y, z, lo x, y, z)
+};
+
+// Row tile r of the grouped order [gbase, gbase + glen) against its j-tiles
+// jt0 .. jt1 - 1 (all at or beyond the row's own diagonal block, jt >= r ITILE /
+// JT).  In the diagonal block (columns below (r + 1) ITILE) the tile holds both
+// orders of its pairs and is swept one-sided; beyond it each pair is evaluated
+// once for both sides.  Writes
+//  * the rows' sums over these tiles to row_slot [6][ITILE] as compensated (hi,
+//    lo) pairs, one TwoSum per tile, as ljc_row_segment does;
+//  * the partners' sums over the ITILE rows of every two-sided tile to
+//    col[c * col_ld + position - (r + 1) ITILE], c = x, y, z: one float32 per
+//    ITILE rows (a lane adds 32 KI terms, then the warps' sums are added
+//    pairwise), which the reduction adds compensated.
+// A warp's rows are consecutive positions (32 KI divides the groups' 256-block
+// padding), so they have one type.  The sums are kept in units of `scale`, the
+// charge product when it is not small (the Coulomb-only sweep then needs no
+// multiply by it), else 1 with the LJ + Coulomb sweep on every segment.  With LJ
+// false the tables hold no LJ term: no boxes, always the Coulomb sweep.
+template <int BLOCK, int KI, int JT, bool LJ>
+__device__ __forceinline__ void sym_row_segment(const float4 *__restrict__ xq,
+                                                const int *__restrict__ perm,
+                                                const int *__restrict__ tblk, int gbase,
+                                                int glen, const float4 *__restrict__ s_tab,
+                                                int has_coul, int r, int jt0, int jt1,
+                                                SymSmem<BLOCK, KI, JT> &smem,
+                                                float *__restrict__ row_slot,
+                                                float *__restrict__ col, size_t col_ld)
+{
+    constexpr int ITILE = BLOCK * KI;
+    constexpr int JP = JT / 2;
+    constexpr int NSEG = JT / 64;
+    constexpr int NW = BLOCK / 32;
+    constexpr int RT = ITILE / JT;
+    static_assert(JP <= BLOCK && JP % 32 == 0 && ITILE % JT == 0 && 256 % (32 * KI) == 0, "shape");
+    LjcSmem<JT> &sm = smem.st;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int row0 = r * ITILE + warp * (32 * KI); // the warp's first row
+    const bool active = row0 < glen;               // a warp's rows are all in or all out
+    const int trow = (active ? tblk[(gbase + row0) >> 8] : 0) * NPSIM_MAX_TYPES;
+    float2 xi[KI], yi[KI], zi[KI];
+    Box3 wb = box_empty();
+#pragma unroll
+    for (int k = 0; k < KI; ++k) {
+        const int i = active ? perm[gbase + row0 + k * 32 + lane] : -1;
+        float4 q = make_float4(kPairPad, kPairPad, kPairPad, 0.0f);
+        if (i >= 0) {
+            q = xq[i];
+            if (LJ)
+                box_add(wb, q.x, q.y, q.z);
+        }
+        xi[k] = make_float2(q.x, q.x);
+        yi[k] = make_float2(q.y, q.y);
+        zi[k] = make_float2(q.z, q.z);
+#pragma unroll
+        for (int c = 0; c < 6; ++c)
+            smem.hl[c][k * BLOCK + threadIdx.x] = 0.0f;
+    }
+    if (LJ)
+        wb = box_warp_reduce(wb); // the box of this warp's rows
+
+    const bool stager = threadIdx.x < JP;
+    const int m = threadIdx.x;
+    const float4 pad = make_float4(-kPairPad, -kPairPad, -kPairPad, 0.0f);
+    auto stage = [&](int buf, const float4 a, const float4 b, int vmask) {
+        if (LJ) {
+            ljc_stage_entry<JT>(sm, buf, m, a, b, vmask);
+        } else {
+            sm.a[buf][m] = make_float4(-a.x, -b.x, -a.y, -b.y);
+            sm.b[buf][m] = make_float2(-a.z, -b.z);
+        }
+    };
+    int pn0 = -1, pn1 = -1; // partner indices of the tile after the one staged next
+    if (stager) {           // tile jt0 staged synchronously (glen is a multiple of JT)
+        const int k0 = gbase + jt0 * JT + 2 * m;
+        const int j0 = perm[k0], j1 = perm[k0 + 1];
+        if (jt0 + 1 < jt1) {
+            pn0 = perm[k0 + JT];
+            pn1 = perm[k0 + JT + 1];
+        }
+        stage(0, j0 >= 0 ? xq[j0] : pad, j1 >= 0 ? xq[j1] : pad, (j0 >= 0) | ((j1 >= 0) << 1));
+    }
+    __syncthreads();
+
+    for (int jt = jt0; jt < jt1; ++jt) {
+        const int cur = (jt - jt0) & 1;
+        const bool next = jt + 1 < jt1; // uniform over the block
+        int vmask = 0;
+        if (stager && next) { // gather tile jt + 1 while this one is swept
+            vmask = (pn0 >= 0) | ((pn1 >= 0) << 1);
+            if (pn0 >= 0)
+                cp_async16(&sm.raw[2 * m], xq + pn0);
+            else
+                sm.raw[2 * m] = pad;
+            if (pn1 >= 0)
+                cp_async16(&sm.raw[2 * m + 1], xq + pn1);
+            else
+                sm.raw[2 * m + 1] = pad;
+            cp_async_commit();
+            if (jt + 2 < jt1) {
+                const int k2 = gbase + (jt + 2) * JT + 2 * m;
+                pn0 = perm[k2];
+                pn1 = perm[k2 + 1];
+            }
+        }
+
+        float4 cst = s_tab[trow + tblk[(gbase + jt * JT) >> 8]]; // one type per tile
+        // LJ between this warp's rows and a segment only when their boxes come
+        // within the type pair's own cutoff (with a margin for float rounding)
+        const float lj2 = LJ && cst.y != 0.0f ? cst.z * 1.0001f : -1.0f;
+        float scale = cst.w;
+        bool general = false; // LJ + Coulomb sweep on every segment
+        if (LJ) {
+            const bool unit = fabsf(cst.w) < kSymMinScale;
+            general = unit && cst.w != 0.0f && has_coul;
+            scale = unit ? 1.0f : cst.w;
+            cst.y = unit ? cst.y : cst.y / cst.w;
+            cst.w = unit ? cst.w : 1.0f;
+        }
+        float2 ax[KI], ay[KI], az[KI];
+#pragma unroll
+        for (int k = 0; k < KI; ++k)
+            ax[k] = ay[k] = az[k] = make_float2(0.0f, 0.0f);
+        const bool two_sided = jt >= (r + 1) * RT; // uniform over the block
+        if (two_sided) {
+            for (int sg = 0; sg < NSEG; ++sg) { // warp-uniform choice per segment
+                const float4 *sa = sm.a[cur] + 32 * sg;
+                const float2 *sb = sm.b[cur] + 32 * sg;
+                float2 gx = make_float2(0.0f, 0.0f), gy = gx, gz = gx;
+                const bool lj = LJ && active &&
+                                (general || box_gap2(wb, sm.seg[cur][sg]) <= lj2);
+                if (lj)
+                    ljc_sym_sweep<KI>(sa, sb, lane, xi, yi, zi, cst, ax, ay, az, gx, gy, gz);
+                else if (active && (!LJ || (has_coul && cst.w != 0.0f)))
+                    coul_sym_sweep<KI>(sa, sb, lane, xi, yi, zi, ax, ay, az, gx, gy, gz);
+                smem.g[cur][0][warp][32 * sg + lane] = make_float2(-scale * gx.x, -scale * gx.y);
+                smem.g[cur][1][warp][32 * sg + lane] = make_float2(-scale * gy.x, -scale * gy.y);
+                smem.g[cur][2][warp][32 * sg + lane] = make_float2(-scale * gz.x, -scale * gz.y);
+            }
+        } else if (active) {
+            float4 csts[KI];
+#pragma unroll
+            for (int k = 0; k < KI; ++k)
+                csts[k] = cst;
+            for (int sg = 0; sg < NSEG; ++sg) {
+                const float4 *sa = sm.a[cur] + 32 * sg;
+                const float2 *sb = sm.b[cur] + 32 * sg;
+                if (LJ && (general || box_gap2(wb, sm.seg[cur][sg]) <= lj2))
+                    ljc_tile_sweep<KI, true>(sa, sb, 32, xi, yi, zi, csts, ax, ay, az);
+                else if (!LJ || (has_coul && cst.w != 0.0f))
+                    coul_tile_sweep<KI>(sa, sb, 32, xi, yi, zi, ax, ay, az);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < KI; ++k) {
+            const int e = k * BLOCK + threadIdx.x; // this thread's own words
+            two_sum_acc(smem.hl[0][e], smem.hl[3][e], scale * (ax[k].x + ax[k].y));
+            two_sum_acc(smem.hl[1][e], smem.hl[4][e], scale * (ay[k].x + ay[k].y));
+            two_sum_acc(smem.hl[2][e], smem.hl[5][e], scale * (az[k].x + az[k].y));
+        }
+
+        if (stager && next) { // this thread's copies have landed: stage tile jt + 1
+            cp_async_wait_own();
+            stage(cur ^ 1, sm.raw[2 * m], sm.raw[2 * m + 1], vmask);
+        }
+        // tile jt + 1 staged, tile jt's buffer free again, the warps' partner sums
+        // complete (their buffer is filled again after the next tile's barrier)
+        __syncthreads();
+        if (two_sided && threadIdx.x < JP) {
+            float *o = col + (size_t)(jt * JT - (r + 1) * ITILE) + 2 * threadIdx.x;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float2 t[NW];
+#pragma unroll
+                for (int w = 0; w < NW; ++w)
+                    t[w] = smem.g[cur][c][w][threadIdx.x];
+#pragma unroll
+                for (int h = NW / 2; h > 0; h >>= 1)
+#pragma unroll
+                    for (int w = 0; w < h; ++w)
+                        t[w] = __fadd2_rn(t[w], t[w + h]);
+                *reinterpret_cast<float2 *>(o + c * col_ld) = t[0];
+            }
+        }
+    }
+
+#pragma unroll
+    for (int k = 0; k < KI; ++k) {
+        const int idx = warp * (32 * KI) + k * 32 + lane;
+#pragma unroll
+        for (int c = 0; c < 6; ++c)
+            row_slot[c * ITILE + idx] = smem.hl[c][k * BLOCK + threadIdx.x];
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Per-type coefficients used by the integrator (computed on the host in
 // float64 from npsim_type_t and the scenario).
 struct TypeCoef {
@@ -638,7 +963,45 @@ struct StreamK {
     int grid;    // ranges (= CTAs of a static launch)
     int ctas;    // CTAs of a dynamic launch (<= grid; 0 for static launches)
     long long W; // n_it * n_jt
+    // tri > 0: the triangular form of the kernels that evaluate each pair once
+    // (allpairs_sym.cu): row r has the j-tiles tri r .. n_jt - 1 only (tri =
+    // itile / jtile), len = positions covered (a multiple of jtile)
+    int tri;
+    int len;
 };
+
+// First unit of row r of the triangular form (row r has n_jt - tri r units).
+__host__ __device__ __forceinline__ long long tri_row_begin(const StreamK &s, int r)
+{
+    return (long long)r * s.n_jt - (long long)s.tri * r * (r - 1) / 2;
+}
+
+// Row of unit p of the triangular form: the root of the quadratic, then exact.
+__device__ __forceinline__ int tri_row_of(const StreamK &s, long long p)
+{
+    const float b = (float)s.n_jt + 0.5f * (float)s.tri;
+    const float disc = fmaxf(b * b - 2.0f * (float)s.tri * (float)p, 0.0f);
+    int r = min(max((int)((b - sqrtf(disc)) / (float)s.tri), 0), s.n_it - 1);
+    while (r + 1 < s.n_it && tri_row_begin(s, r + 1) <= p)
+        ++r;
+    while (r > 0 && tri_row_begin(s, r) > p)
+        --r;
+    return r;
+}
+
+// Floats before row r's column partials (see sym_row_segment): rows k < r hold
+// 3 planes of len - (k + 1) itile floats each.
+__host__ __device__ __forceinline__ size_t sym_col_offset(int len, int itile, int r)
+{
+    return 3 * ((size_t)r * (size_t)len - (size_t)itile * ((size_t)r * ((size_t)r + 1) / 2));
+}
+
+// Floats of all column partials of a grouped order of `len` positions.
+__host__ __device__ __forceinline__ size_t sym_col_floats(int len, int itile)
+{
+    const int rows = len / itile; // rows k with len - (k + 1) itile > 0 (the last may be 0)
+    return rows > 0 ? sym_col_offset(len, itile, rows) : 0;
+}
 
 __host__ __device__ __forceinline__ long long sk_begin(const StreamK &s, int c)
 {
@@ -654,6 +1017,79 @@ __host__ __device__ __forceinline__ int sk_cta_of(const StreamK &s, long long p)
     while (c > 0 && sk_begin(s, c) > p)
         --c;
     return c;
+}
+
+// ---------------------------------------------------------------------------
+// Sum of a position's partials of the kernels that evaluate each pair once
+// (sym_row_segment): its row's n_rows slots [6][itile] from row_slots on, then
+// the column partials of the row tiles before its own, r' = 0 .. r - 1.  Four
+// threads share a position (64 positions per CTA of 256 threads, so the reads
+// are coalesced and a long column has four times the loads in flight): thread
+// `part` takes every fourth slot, compensated; sym_finish adds the four in a
+// fixed order.
+__device__ __forceinline__ void sym_sum_partials(const float *__restrict__ row_slots, int n_rows,
+                                                 const float *__restrict__ cols, int itile,
+                                                 int len, int r, int p, int part, float (&h)[3],
+                                                 float (&l)[3])
+{
+    const float *rs = row_slots + (p - r * itile);
+    for (int c = part; c < n_rows; c += 4) {
+        const float *q = rs + (size_t)c * 6 * itile;
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            df_add_df(h[d], l[d], __ldcs(q + d * itile), __ldcs(q + (3 + d) * itile));
+    }
+    int k = part;
+    for (; k + 4 < r; k += 8) { // two row tiles' loads before their adds
+        const float *q0 = cols + sym_col_offset(len, itile, k) + (p - (k + 1) * itile);
+        const float *q1 = cols + sym_col_offset(len, itile, k + 4) + (p - (k + 5) * itile);
+        const size_t l0 = (size_t)(len - (k + 1) * itile), l1 = (size_t)(len - (k + 5) * itile);
+        float w[6];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            w[d] = __ldcs(q0 + d * l0);
+            w[3 + d] = __ldcs(q1 + d * l1);
+        }
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            df_add(h[d], l[d], w[d]);
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            df_add(h[d], l[d], w[3 + d]);
+    }
+    for (; k < r; k += 4) {
+        const float *q = cols + sym_col_offset(len, itile, k) + (p - (k + 1) * itile);
+        const size_t ld = (size_t)(len - (k + 1) * itile);
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            df_add(h[d], l[d], __ldcs(q + d * ld));
+    }
+}
+
+// Parts 1 .. 3 added to part 0 in order; the 32-byte record of particle i
+// (hi x, y, z, lo x | lo y, z, 0, 0), none for padding (i < 0).
+__device__ __forceinline__ void sym_finish(float (&s_part)[3][6][64], int part, float (&h)[3],
+                                           float (&l)[3], int i, float *__restrict__ F_pair)
+{
+    const int x = threadIdx.x & 63;
+    if (part > 0) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            s_part[part - 1][d][x] = h[d];
+            s_part[part - 1][3 + d][x] = l[d];
+        }
+    }
+    __syncthreads();
+    if (part == 0 && i >= 0) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                df_add_df(h[d], l[d], s_part[q][d][x], s_part[q][3 + d][x]);
+        float4 *o = reinterpret_cast<float4 *>(F_pair + 8 * (size_t)i);
+        o[0] = make_float4(h[0], h[1], h[2], l[0]);
+        o[1] = make_float4(l[1], l[2], 0.0f, 0.0f);
+    }
 }
 
 // LJ / Coulomb type-pair table entry: (sigma_ab^2, 24 eps_ab, rc_ab^2, C q_a q_b).
@@ -726,6 +1162,20 @@ cudaError_t launch_allpairs_ljgrp(int idx, const StreamK &sk, const float4 *xq,
                                   const int *perm, int n_perm, const int *tblk,
                                   const PairTab *tab, float rc2_lim, int has_coul,
                                   unsigned *work, float *slots, cudaStream_t st);
+// Each pair once (allpairs_sym.cu): the type-grouped order, triangular StreamK,
+// row and column partials in one array (sym_slots_floats floats), summed into
+// one 32-byte record per NP by launch_sym_reduce (F_pair [n][8]: hi x, y, z, lo
+// x, y, z, 0, 0).  Configurations [0, sym_num_configs(false)) sum Coulomb only,
+// those of lj = true LJ + Coulomb as the table says.
+int sym_num_configs(bool lj);
+ApConfig sym_config(bool lj, int idx);
+int sym_occupancy(bool lj, int idx);
+size_t sym_slots_floats(const StreamK &sk);
+cudaError_t launch_allpairs_sym(bool lj, int idx, const StreamK &sk, const float4 *xq,
+                                const int *perm, const int *tblk, const PairTab *tab,
+                                int has_coul, unsigned *work, float *slots, cudaStream_t st);
+cudaError_t launch_sym_reduce(const StreamK &sk, const float *slots, const int *perm,
+                              float *F_pair, cudaStream_t st);
 cudaError_t launch_allpairs(int cfg_idx, bool lj, const StreamK &sk, const float4 *xq,
                             const int *typ, int n, const PairTab *tab, float *slots,
                             cudaStream_t st);
@@ -750,6 +1200,8 @@ struct IntArgs {
     const float *slots;      // stream-K partials [slot][6][itile] (or NULL)
     StreamK sk;
     const float *F_lj;       // cell-list LJ forces [n][8] (hi x, y, z, lo x, y, z, 0, 0) (or NULL)
+    const float *F_pair;     // summed all-pairs forces [n][8] of the kernels that
+                             // evaluate each pair once (or NULL): in place of slots
     const int *row_pos;      // grouped layout: position of particle i in the rows (-1:
                              // no Coulomb partial); NULL: row position = i
     const float4 *x_ref;     // positions at the last neighbour-list build (or NULL)

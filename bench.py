@@ -34,7 +34,9 @@ sys.path.insert(0, ROOT)
 
 METRIC = "pair-interactions/s & particle-steps/s at N=2.5e5; ensemble droplets/s vs plain"
 UNIT = "pair-interactions/s"
-FLOPS_PER_PAIR = 17  # Coulomb pair: 3 sub, 5 for r^2, 2 for r^-3, 1 for q_j, 6 accumulate
+# Flops per ordered Coulomb pair: each unordered pair is evaluated once with 3 sub, 6
+# for r^2 (its guard included), 2 for r^-3 and 6 for each side's sum = 23.
+FLOPS_PER_PAIR = 11.5
 L2_FLUSH_BYTES = 256 << 20
 
 
@@ -283,20 +285,19 @@ def _traffic_from_profile(cfg, full_sum):
 
 # Algorithmic bytes per NP of the ensemble's integrator launch in mode BA: read
 # the position hi words with the charge (16), lo words (12), velocity (12),
-# type (4), droplet index (4) and row position (4); write the position (28) and
-# velocity (12).  Plus the partial slots of the all-pairs launch, read once:
-# 24 bytes per row and work item (6 floats), n_items x itile rows.
-ENS_INT_BYTES_BA = 16 + 12 + 12 + 4 + 4 + 4 + 28 + 12
+# type (4), droplet index (4) and the summed pair force's record (32); write the
+# position (28) and velocity (12).
+ENS_INT_BYTES_BA = 16 + 12 + 12 + 4 + 4 + 32 + 28 + 12
 
 
 def _ensemble_kernels(P, drops, stream, n_tot, pairs, peak_tflops, chunks=4):
     """The ensemble's two launches per step timed apart (CUDA event records in the
     step graph, npsim_ens_profile) over `chunks` graph chunks of a fresh
-    ensemble at the initial state: the all-pairs launch against the measured
-    FP32 rate (17 flops per ordered pair, the Coulomb count; the LJ segments it
-    evaluates near the rows add work that is not credited) and the integrator
-    launch against the measured copy bandwidth (ENS_INT_BYTES_BA per NP plus
-    24 bytes per row of every work item's partial slot)."""
+    ensemble at the initial state: the all-pairs launch with the sum of its
+    partials against the measured FP32 rate (FLOPS_PER_PAIR, the Coulomb count;
+    the LJ segments it evaluates near the rows add work that is not credited) and
+    the integrator launch against the measured copy bandwidth (ENS_INT_BYTES_BA
+    per NP)."""
     with P.Ensemble(drops, stream=stream) as ens:
         n_items, itile = ens.work()
         ens.profile(True)
@@ -309,7 +310,7 @@ def _ensemble_kernels(P, drops, stream, n_tot, pairs, peak_tflops, chunks=4):
             it.append(kt["integrate"])
     ap_ms, int_ms = sum(ap) / len(ap), sum(it) / len(it)
     ach = FLOPS_PER_PAIR * pairs / (ap_ms * 1e-3) / 1e12
-    int_bytes = ENS_INT_BYTES_BA * n_tot + 24 * n_items * itile
+    int_bytes = ENS_INT_BYTES_BA * n_tot
     gbs = int_bytes / (int_ms * 1e-3) / 1e9
     hbm = _hbm_peak()
     return {"allpairs_ms": ap_ms, "integrate_ms": int_ms,
@@ -800,8 +801,8 @@ def run_ours(a):
 
     # roofline of the dominant kernel (all-pairs Coulomb, FP32 CUDA-core ALU):
     # the default path sums the Coulomb term over the charged NPs only (the
-    # neutral NPs' terms are exactly zero), so its algorithmic work is 17 flops
-    # per charged ordered pair; the peak is the FP32 rate measured by the FMA
+    # neutral NPs' terms are exactly zero), so its algorithmic work is
+    # FLOPS_PER_PAIR per charged ordered pair; the peak is the FP32 rate measured by the FMA
     # microbenchmark on this GPU in this run
     peaks = _peaks()
     max_mhz = float(peaks.get("sm_max_mhz") or (clk or {}).get("sm_max_mhz") or 2070.0)

@@ -24,15 +24,8 @@ namespace npsim {
 
 namespace {
 
-template <int BLOCK, int KI>
-constexpr int min_ctas()
-{
-        // 168, 96 (128 with 256 threads or more) or 80 registers per thread
-    return KI >= 8 ? 384 / BLOCK : KI >= 4 ? (BLOCK <= 128 ? 640 : 512) / BLOCK : 768 / BLOCK;
-}
-
 template <int BLOCK, int KI, int JT, bool LJ>
-__global__ void __launch_bounds__(BLOCK, (min_ctas<BLOCK, KI>()))
+__global__ void __launch_bounds__(BLOCK, (sym_min_ctas<BLOCK, KI>()))
 k_pairs_sym(const float4 *__restrict__ xq, const int *__restrict__ perm,
             const int *__restrict__ tblk, const PairTab *__restrict__ tab, int has_coul, StreamK sk, unsigned *__restrict__ work, float *__restrict__ slots)
 {
@@ -89,8 +82,8 @@ k_sym_reduce(StreamK sk, const float *__restrict__ slots, const int *__restrict_
     const int c1 = sk_cta_of(sk, tri_row_begin(sk, r + 1) - 1);
     float h[3] = {0.f, 0.f, 0.f}, l[3] = {0.f, 0.f, 0.f};
     sym_sum_partials(slots + (size_t)(r + c0) * 6 * sk.itile, c1 - c0 + 1,
-                     slots + (size_t)(sk.n_it + sk.grid) * 6 * sk.itile, sk.itile, sk.len, r, p,
-                     part, h, l);
+                     slots + (size_t)(sk.n_it + sk.grid) * 6 * sk.itile, sk.itile, sk.len, r, r,
+                     p, part, h, l);
     sym_finish(s_part, part, h, l, perm[p], F_pair);
 }
 

@@ -2313,21 +2313,23 @@ struct npsim_ens {
     float *F = nullptr, *F_tmp = nullptr; // [6][n_total]
     float4 *xq = nullptr;
     int *typ = nullptr, *drop_of = nullptr;
-    int *perm = nullptr, *tblk = nullptr, *row_pos = nullptr; // type-grouped order
+    int *perm = nullptr, *tblk = nullptr, *dblk = nullptr; // type-grouped order
+    int n_pos = 0;               // its length
     EnsDrop *drops = nullptr;
     PairTab *tabs = nullptr;
-    long long *item0 = nullptr;  // work-item prefix per droplet (n_drops + 1)
+    EnsItem *items = nullptr;    // work items of the all-pairs launch
+    int *row_first = nullptr;    // first slot of every row tile
     unsigned *d_work = nullptr;  // work-item counters of the all-pairs launch
-    float *slots = nullptr;      // one [6][itile] slot per work item
+    float *slots = nullptr;      // one [6][itile] slot per work item, then column partials
+    float *F_pair = nullptr;     // [n_total][8] all-pairs forces
     long long *d_step = nullptr;
     float4 *d_spring = nullptr; // [2][D][NPSIM_MAX_TYPES]
     int *d_flags = nullptr;
     unsigned *d_done = nullptr;
 
     int shape = 0;
-    StreamK sk{};
-    int chunk = 1;          // j-tiles per work item
-    long long n_items = 0;  // work items of one all-pairs launch
+    int ctas = 1;           // CTAs of the all-pairs launch
+    int n_items = 0;        // its work items
     std::map<int, cudaGraphExec_t> graphs;
     int64_t step = 0;
     // kernel timing (npsim_ens_profile): events around the all-pairs launch
@@ -2358,12 +2360,14 @@ struct npsim_ens {
         dfree(drop_of);
         dfree(perm);
         dfree(tblk);
-        dfree(row_pos);
+        dfree(dblk);
         dfree(drops);
         dfree(tabs);
-        dfree(item0);
+        dfree(items);
+        dfree(row_first);
         dfree(d_work);
         dfree(slots);
+        dfree(F_pair);
         dfree(d_step);
         dfree(d_spring);
         dfree(d_flags);
@@ -2376,78 +2380,98 @@ struct npsim_ens {
 namespace {
 
 // Work items per CTA that the chunk size aims at: enough that the last items
-// drawn (the only imbalance of dynamic scheduling) are short, few enough that
-// the per-item slots stay small.
-constexpr int kItemsPerCta = 32;
+// drawn (the only imbalance of dynamic scheduling, longest items first) are
+// short, few enough that the per-item slots stay small.
+constexpr int kItemsPerCta = 12;
 
-// Droplet geometry for launch shape `shape` on grid_target CTAs: row tiles and
-// j-tiles of every droplet, the chunk size (j-tiles per work item) and the
-// work items laid end to end (item0).  Returns the number of items; *chunk_out
-// receives the chunk size.
-long long ens_geometry(npsim_ens *e, int shape, int grid_target, std::vector<long long> &item0,
-                       int *chunk_out)
+// The all-pairs work of an ensemble for one launch shape: work items (longest
+// first, slots numbered in row order), first slot of every row tile, floats of
+// the row slots and column partials.
+struct EnsGeometry {
+    std::vector<EnsItem> items;
+    std::vector<int> row_first;
+    size_t floats = 0;
+    int ctas = 1;
+};
+
+// Geometry for launch shape `shape` on grid_target CTAs; sets the droplets'
+// row0 and col0.
+EnsGeometry ens_geometry(npsim_ens *e, int shape, int grid_target)
 {
     const ApConfig c = ens_config(shape);
     const int itile = c.block * c.ki;
+    const bool sym = ens_sym(shape);
+    const int tri = sym ? itile / c.jt : 0; // first j-tile of row r: tri r
     long long W = 0;
-    for (int d = 0; d < e->D; ++d) {
-        EnsDrop &g = e->h_drops[d];
-        g.n_it = (g.npad + itile - 1) / itile;
-        g.n_jt = g.npad / c.jt; // npad is a multiple of 256, jt divides 256
-        W += (long long)g.n_it * g.n_jt;
+    for (const EnsDrop &g : e->h_drops) { // npad is a multiple of 256, jt divides 256
+        const long long n_it = (g.npad + itile - 1) / itile, n_jt = g.npad / c.jt;
+        W += n_it * n_jt - tri * n_it * (n_it - 1) / 2;
     }
     const long long target = (long long)std::max(grid_target, 1) * kItemsPerCta;
-    const int chunk = (int)std::max<long long>(1, (W + target - 1) / target);
-    long long it = 0;
-    item0.assign(e->D + 1, 0);
+    // items are counted in int: a chunk that keeps them below 2^30
+    const int chunk = (int)std::max<long long>({1, (W + target - 1) / target, W >> 28});
+    EnsGeometry G;
+    long long col = 0;
     for (int d = 0; d < e->D; ++d) {
         EnsDrop &g = e->h_drops[d];
-        g.n_ch = (g.n_jt + chunk - 1) / chunk;
-        g.item0 = it;
-        item0[d] = it;
-        it += (long long)g.n_it * g.n_ch;
+        const int n_it = (g.npad + itile - 1) / itile, n_jt = g.npad / c.jt;
+        g.row0 = (int)G.row_first.size();
+        g.col0 = col;
+        if (sym)
+            col += (long long)sym_col_floats(g.npad, itile);
+        for (int r = 0; r < n_it; ++r) {
+            G.row_first.push_back((int)G.items.size());
+            for (int j = tri * r; j < n_jt; j += chunk)
+                G.items.push_back(EnsItem{d, r, j, std::min(n_jt, j + chunk), (int)G.items.size()});
+        }
     }
-    item0[e->D] = it;
-    if (chunk_out)
-        *chunk_out = chunk;
-    return it;
+    G.row_first.push_back((int)G.items.size());
+    std::stable_sort(G.items.begin(), G.items.end(), [](const EnsItem &a, const EnsItem &b) {
+        return a.jt1 - a.jt0 > b.jt1 - b.jt0;
+    });
+    G.floats = G.items.size() * 6 * (size_t)itile + (size_t)col;
+    G.ctas = (int)std::min<size_t>((size_t)std::max(grid_target, 1), G.items.size());
+    return G;
 }
 
-void ens_streamk(long long n_items, const ApConfig &c, int grid_target, StreamK &sk)
+int ens_upload_geometry(npsim_ens *e, int shape, const EnsGeometry &G)
 {
-    sk.itile = c.block * c.ki;
-    sk.jtile = c.jt;
-    sk.n_it = 0;
-    sk.n_jt = 0;
-    sk.W = n_items;
-    sk.grid = (int)std::min<long long>(std::max(grid_target, 1), n_items);
-    sk.ctas = 0;
-}
-
-int ens_upload_geometry(npsim_ens *e, const std::vector<long long> &item0)
-{
+    dfree(e->items);
+    dfree(e->row_first);
+    NP_CUDA(dalloc(&e->items, G.items.size()));
+    NP_CUDA(dalloc(&e->row_first, G.row_first.size()));
     NP_CUDA(cudaMemcpyAsync(e->drops, e->h_drops.data(), sizeof(EnsDrop) * e->D,
                             cudaMemcpyHostToDevice, e->user));
-    NP_CUDA(cudaMemcpyAsync(e->item0, item0.data(), sizeof(long long) * item0.size(),
+    NP_CUDA(cudaMemcpyAsync(e->items, G.items.data(), sizeof(EnsItem) * G.items.size(),
+                            cudaMemcpyHostToDevice, e->user));
+    NP_CUDA(cudaMemcpyAsync(e->row_first, G.row_first.data(), sizeof(int) * G.row_first.size(),
                             cudaMemcpyHostToDevice, e->user));
     NP_CUDA(cudaStreamSynchronize(e->user));
+    e->shape = shape;
+    e->n_items = (int)G.items.size();
+    e->ctas = G.ctas;
     return NPSIM_OK;
 }
 
 EnsAllpairsArgs ens_ap_args(npsim_ens *e, float *slots)
 {
+    const ApConfig c = ens_config(e->shape);
     EnsAllpairsArgs a{};
     a.xq = e->xq;
     a.perm = e->perm;
     a.tblk = e->tblk;
+    a.dblk = e->dblk;
     a.drops = e->drops;
-    a.item0 = e->item0;
     a.tabs = e->tabs;
-    a.n_drops = e->D;
-    a.chunk = e->chunk;
+    a.items = e->items;
+    a.row_first = e->row_first;
     a.n_items = e->n_items;
+    a.n_pos = e->n_pos;
+    a.itile = c.block * c.ki;
+    a.sym = ens_sym(e->shape) ? 1 : 0;
     a.work = e->d_work;
     a.slots = slots;
+    a.F_pair = e->F_pair;
     return a;
 }
 
@@ -2463,7 +2487,7 @@ int ens_pass(npsim_ens *e, int mode, bool ext, float *Fout, cudaStream_t st,
                     : cudaSuccess;
     };
     NP_CUDA(mark(0, 0));
-    NP_CUDA(launch_ens_allpairs(e->shape, e->sk, ens_ap_args(e, e->slots), st));
+    NP_CUDA(launch_ens_allpairs(e->shape, e->ctas, ens_ap_args(e, e->slots), st));
     NP_CUDA(mark(0, 1));
     EnsIntArgs a{};
     a.x_lo = e->x_lo;
@@ -2472,16 +2496,15 @@ int ens_pass(npsim_ens *e, int mode, bool ext, float *Fout, cudaStream_t st,
     a.typ = e->typ;
     a.xq = e->xq;
     a.drop_of = e->drop_of;
-    a.row_pos = e->row_pos;
     a.drops = e->drops;
-    a.slots = e->slots;
+    a.F_pair = e->F_pair;
     a.spring = e->d_spring;
     a.ext_on = ext ? 1 : 0;
     a.step = e->d_step;
     a.flags = e->d_flags;
     a.done = e->d_done;
     NP_CUDA(mark(1, 0));
-    NP_CUDA(launch_ens_integrate(mode, a, e->n_total, e->D, e->sk, st));
+    NP_CUDA(launch_ens_integrate(mode, a, e->n_total, e->D, st));
     NP_CUDA(mark(1, 1));
     return NPSIM_OK;
 }
@@ -2495,13 +2518,12 @@ int ens_chunk(npsim_ens *e, int k, cudaStream_t st)
     a.typ = e->typ;
     a.xq = e->xq;
     a.drop_of = e->drop_of;
-    a.row_pos = e->row_pos;
     a.drops = e->drops;
     a.spring = e->d_spring;
     a.step = e->d_step;
     a.flags = e->d_flags;
     a.done = e->d_done;
-    NP_CUDA(launch_ens_integrate(MODE_A, a, e->n_total, e->D, e->sk, st));
+    NP_CUDA(launch_ens_integrate(MODE_A, a, e->n_total, e->D, st));
     for (int j = 0; j < k; ++j) {
         int rc = ens_pass(e, j + 1 < k ? MODE_BA : MODE_B, true, e->F, st, j);
         if (rc)
@@ -2543,7 +2565,6 @@ int ens_autotune(npsim_ens *e)
 {
     const int nc = ens_num_configs();
     const char *env = getenv("NPSIM_ENS_SHAPE");
-    std::vector<long long> item0;
     int best = -1;
     if (env) {
         const int idx = atoi(env);
@@ -2567,17 +2588,24 @@ int ens_autotune(npsim_ens *e)
     }
     const bool cached = !pinned && best >= 0;
     if (best < 0) {
-        size_t need = 0;
-        for (int c = 0; c < nc; ++c) {
-            const int occ = ens_occupancy(c);
-            if (occ <= 0)
-                continue;
-            const long long items = ens_geometry(e, c, occ * e->sms, item0, nullptr);
-            const ApConfig cc = ens_config(c);
-            need = std::max(need, (size_t)items * 6 * (size_t)(cc.block * cc.ki));
-        }
+        // scratch big enough for every candidate; where that does not fit, for the
+        // one-sided one alone
         float *tmp = nullptr;
-        NP_CUDA(dalloc(&tmp, need));
+        size_t need = 0;
+        for (bool sym : {true, false}) {
+            need = 0;
+            for (int c = 0; c < nc; ++c) {
+                const int occ = ens_occupancy(c);
+                if (occ > 0 && (sym || !ens_sym(c)))
+                    need = std::max(need, ens_geometry(e, c, occ * e->sms).floats);
+            }
+            const cudaError_t ce = dalloc(&tmp, need);
+            if (ce == cudaSuccess)
+                break;
+            if (!sym || ce != cudaErrorMemoryAllocation)
+                NP_CUDA(ce);
+            cudaGetLastError(); // the failed allocation
+        }
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
@@ -2586,20 +2614,19 @@ int ens_autotune(npsim_ens *e)
             const int occ = ens_occupancy(c);
             if (occ <= 0)
                 continue;
-            e->n_items = ens_geometry(e, c, occ * e->sms, item0, &e->chunk);
-            int rc = ens_upload_geometry(e, item0);
+            const EnsGeometry G = ens_geometry(e, c, occ * e->sms);
+            if (G.floats > need)
+                continue;
+            int rc = ens_upload_geometry(e, c, G);
             if (rc) {
                 cudaFree(tmp);
                 return rc;
             }
-            StreamK sk;
-            ens_streamk(e->n_items, ens_config(c), occ * e->sms, sk);
-            e->shape = c;
-            if (launch_ens_allpairs(c, sk, ens_ap_args(e, tmp), e->user) != cudaSuccess)
+            if (launch_ens_allpairs(c, e->ctas, ens_ap_args(e, tmp), e->user) != cudaSuccess)
                 continue;
             cudaEventRecord(e0, e->user);
             for (int r = 0; r < 2; ++r)
-                launch_ens_allpairs(c, sk, ens_ap_args(e, tmp), e->user);
+                launch_ens_allpairs(c, e->ctas, ens_ap_args(e, tmp), e->user);
             cudaEventRecord(e1, e->user);
             if (cudaEventSynchronize(e1) != cudaSuccess)
                 continue;
@@ -2607,8 +2634,9 @@ int ens_autotune(npsim_ens *e)
             cudaEventElapsedTime(&ms, e0, e1);
             if (getenv("NPSIM_AUTOTUNE_LOG")) {
                 const ApConfig cf = ens_config(c);
-                fprintf(stderr, "npsim ensemble autotune shape %d <%d,%d,%d> grid %d: %.4f ms\n",
-                        c, cf.block, cf.ki, cf.jt, sk.grid, ms / 2);
+                fprintf(stderr,
+                        "npsim ensemble autotune shape %d <%d,%d,%d> grid %d items %d: %.4f ms\n",
+                        c, cf.block, cf.ki, cf.jt, e->ctas, e->n_items, ms / 2);
             }
             if (ms < best_ms) {
                 best_ms = ms;
@@ -2628,15 +2656,18 @@ int ens_autotune(npsim_ens *e)
         std::lock_guard<std::mutex> g(g_tune_mu);
         g_ens_tune_cache[key] = best;
     }
-    e->shape = best;
-    const int grid_target = std::max(1, ens_occupancy(best)) * e->sms;
-    e->n_items = ens_geometry(e, best, grid_target, item0, &e->chunk);
-    ens_streamk(e->n_items, ens_config(best), grid_target, e->sk);
-    int rc = ens_upload_geometry(e, item0);
-    if (rc)
-        return rc;
-    NP_CUDA(dalloc(&e->slots, (size_t)e->n_items * 6 * (size_t)e->sk.itile));
-    return NPSIM_OK;
+    EnsGeometry G = ens_geometry(e, best, std::max(1, ens_occupancy(best)) * e->sms);
+    cudaError_t ce = dalloc(&e->slots, G.floats);
+    if (ce == cudaErrorMemoryAllocation && ens_sym(best)) {
+        // no room for the column partials: the one-sided shape
+        cudaGetLastError();
+        while (ens_sym(best))
+            best = (best + 1) % nc;
+        G = ens_geometry(e, best, std::max(1, ens_occupancy(best)) * e->sms);
+        ce = dalloc(&e->slots, G.floats);
+    }
+    NP_CUDA(ce);
+    return ens_upload_geometry(e, best, G);
 }
 
 } // namespace
@@ -2754,7 +2785,7 @@ int npsim_ens_create(const npsim_droplet_t *drops, int32_t n_drops, void *stream
     }
     // type-grouped order of every droplet: its types in order, each group in
     // Z-order of the initial positions and padded with -1 to a multiple of 256
-    std::vector<int> gperm, gtblk, gpos((size_t)total, -1);
+    std::vector<int> gperm, gtblk, gdblk;
     for (int d = 0; d < n_drops; ++d) {
         EnsDrop &g = e->h_drops[d];
         g.gpos0 = (int)gperm.size();
@@ -2766,17 +2797,18 @@ int npsim_ens_create(const npsim_droplet_t *drops, int32_t n_drops, void *stream
             if (mem.empty())
                 continue;
             morton_sort(mem, drops[d].x0);
-            for (int i : mem) {
-                gpos[(size_t)e->off[d] + i] = (int)gperm.size();
+            for (int i : mem)
                 gperm.push_back(e->off[d] + i);
-            }
             while (gperm.size() % 256)
                 gperm.push_back(-1);
-            while (gtblk.size() < gperm.size() / 256)
+            while (gtblk.size() < gperm.size() / 256) {
                 gtblk.push_back(t);
+                gdblk.push_back(d);
+            }
         }
         g.npad = (int)gperm.size() - g.gpos0;
     }
+    e->n_pos = (int)gperm.size();
 #define EBAIL(call)                                                                     \
     do {                                                                                \
         cudaError_t e_ = (call);                                                        \
@@ -2796,7 +2828,7 @@ int npsim_ens_create(const npsim_droplet_t *drops, int32_t n_drops, void *stream
     EBAIL(dalloc(&e->drop_of, (size_t)total));
     EBAIL(dalloc(&e->drops, (size_t)n_drops));
     EBAIL(dalloc(&e->tabs, (size_t)n_drops));
-    EBAIL(dalloc(&e->item0, (size_t)n_drops + 1));
+    EBAIL(dalloc(&e->F_pair, 8 * (size_t)total));
     EBAIL(dalloc(&e->d_work, 2));
     EBAIL(cudaMemset(e->d_work, 0, 2 * sizeof(unsigned)));
     EBAIL(dalloc(&e->d_step, 1));
@@ -2817,11 +2849,10 @@ int npsim_ens_create(const npsim_droplet_t *drops, int32_t n_drops, void *stream
                      cudaMemcpyHostToDevice));
     EBAIL(dalloc(&e->perm, gperm.size()));
     EBAIL(dalloc(&e->tblk, gtblk.size()));
-    EBAIL(dalloc(&e->row_pos, (size_t)total));
+    EBAIL(dalloc(&e->dblk, gdblk.size()));
     EBAIL(cudaMemcpy(e->perm, gperm.data(), sizeof(int) * gperm.size(), cudaMemcpyHostToDevice));
     EBAIL(cudaMemcpy(e->tblk, gtblk.data(), sizeof(int) * gtblk.size(), cudaMemcpyHostToDevice));
-    EBAIL(cudaMemcpy(e->row_pos, gpos.data(), sizeof(int) * (size_t)total,
-                     cudaMemcpyHostToDevice));
+    EBAIL(cudaMemcpy(e->dblk, gdblk.data(), sizeof(int) * gdblk.size(), cudaMemcpyHostToDevice));
     EBAIL(cudaMemcpy(e->tabs, e->h_tabs.data(), sizeof(PairTab) * (size_t)n_drops,
                      cudaMemcpyHostToDevice));
     for (int i = 0; i < (int)total; ++i) {
@@ -3050,7 +3081,7 @@ int npsim_ens_config(npsim_ens_t e, int *block, int *i_per_thread, int *j_tile, 
     if (j_tile)
         *j_tile = c.jt;
     if (grid)
-        *grid = e->sk.grid;
+        *grid = e->ctas;
     if (index)
         *index = e->shape;
     return NPSIM_OK;
@@ -3061,8 +3092,9 @@ int npsim_ens_work(npsim_ens_t e, int64_t *n_items, int32_t *itile)
     NP_REQUIRE(e, "ensemble is NULL");
     if (n_items)
         *n_items = e->n_items;
+    const ApConfig c = ens_config(e->shape);
     if (itile)
-        *itile = e->sk.itile;
+        *itile = c.block * c.ki;
     return NPSIM_OK;
 }
 

@@ -1,25 +1,29 @@
 // ensemble.cu -- many independent droplets of uneven size advanced together:
-// one all-pairs launch and one integrator launch per step cover every droplet.
+// one all-pairs launch, one sum of its partials and one integrator launch per
+// step cover every droplet.
 //
 // Each droplet d is the system of arXiv 2501.04456 Sec. 2 (its own NP types,
 // charges, LJ table, radius law, seed).  Particles of all droplets are stored
-// back to back (structure of arrays over the concatenation).  The all-pairs
-// work of droplet d is a rectangle of n_it(d) x n_jt(d) (i-tile x j-tile)
-// units; every row tile is cut into work items of at most `chunk` j-tiles,
-// the items of all droplets are numbered end to end, and the CTAs of one
-// launch draw items from a device counter until none are left, so a 512-NP
-// and a 32768-NP droplet share the GPU in proportion to their work within one
-// launch and items rich in LJ segments (which cost more than Coulomb-only
-// ones) are balanced as they run.  An item writes one compensated (hi, lo)
-// float32 partial per row into its own slot; the integrator sums a row's items
-// in item order, so the result does not depend on which CTA ran which item.
+// back to back (structure of arrays over the concatenation).  Inside the
+// ensemble each droplet's particles are listed in a type-grouped order (each
+// type's group padded to 256 positions), so every j-tile holds partners of one
+// type.  The all-pairs work of a droplet is the triangle of its (row tile x
+// j-tile) units at or beyond the diagonal (each pair once, sym_row_segment) or,
+// for the one-sided kernel, the whole square; every row is cut into work items
+// of at most `chunk` j-tiles.  The host lists the items of all droplets once,
+// longest first, and the CTAs of one launch draw them from a device counter
+// until none are left, so a 512-NP and a 32768-NP droplet share the GPU in
+// proportion to their work within one launch and items rich in LJ segments
+// (which cost more than Coulomb-only ones) are balanced as they run.  An item
+// writes one compensated (hi, lo) float32 partial per row into its own slot and
+// its partners' sums to their own places; k_ens_reduce adds them in a fixed
+// order, so the result does not depend on which CTA ran which item.  The
+// reduction runs along the grouped order, in which partials are contiguous, and
+// hands the integrator one 32-byte record per particle (read in particle order;
+// the integrator's own gathers of 24-byte slots by grouped position used to
+// fetch a 32-byte sector per float).
 //
-// Inside the ensemble each droplet's particles are listed in a type-grouped
-// order (each type's group padded to 256 positions), so every j-tile holds
-// partners of one type and the pair body is the packed LJ + Coulomb sweep
-// (ljc_tile_sweep) with the droplet's own type-pair table (sigma_ab^2,
-// 24 eps_ab, rc_ab^2, C q_a q_b) read once per tile;
-// the integrator is the fused BAOAB / overdamped pass of integrate.cu with the
+// The integrator is the fused BAOAB / overdamped pass of integrate.cu with the
 // droplet's own coefficients.  Noise is keyed by the droplet's seed and counted
 // by the particle's index inside its droplet, so a droplet draws the same
 // normals here as in a single-droplet run.
@@ -29,72 +33,107 @@ namespace npsim {
 
 namespace {
 
-// Droplet whose item range contains item u (item0 has n_drops + 1 entries).
-__device__ __forceinline__ int drop_of_item(const long long *__restrict__ item0, int n_drops,
-                                            long long u)
+// Draws the CTA's next item (n_items: none left).  Called by every thread.
+__device__ __forceinline__ int next_item(unsigned *work, int *s_item)
 {
-    int lo = 0, hi = n_drops - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (item0[mid] <= u)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
+    __syncthreads(); // every thread has read *s_item and finished the last item
+    if (threadIdx.x == 0)
+        *s_item = (int)atomicAdd(work, 1u);
+    __syncthreads();
+    return *s_item;
 }
 
-// At least 1024 (one row per thread) or 512 (two rows per thread) threads
-// resident per SM: the register caps this implies (64, 128) hold the sweeps
-// without spills.
-template <int BLOCK, int KI, int JT>
-__global__ void __launch_bounds__(BLOCK, KI == 1 ? 1024 / BLOCK : 512 / BLOCK)
-k_ens_ljc(EnsAllpairsArgs a)
+// The last CTA out resets the counters for the next launch (every CTA has drawn
+// its last item by the time it counts itself out).
+__device__ __forceinline__ void items_done(unsigned *work)
 {
-    constexpr int ITILE = BLOCK * KI;
-    __shared__ LjcSmem<JT> sm;
-    __shared__ float4 s_tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
-    __shared__ long long s_item;
-    int cur = -1;
-
-    for (;;) {
-        __syncthreads(); // every thread has read s_item and finished the last item
-        if (threadIdx.x == 0)
-            s_item = (long long)atomicAdd(a.work, 1u);
-        __syncthreads();
-        const long long item = s_item;
-        if (item >= a.n_items)
-            break;
-        const int d = drop_of_item(a.item0, a.n_drops, item);
-        const EnsDrop &D = a.drops[d];
-        if (d != cur) { // ordered before use by the staging barrier
-            for (int k = threadIdx.x; k < NPSIM_MAX_TYPES * NPSIM_MAX_TYPES; k += BLOCK)
-                s_tab[k] = a.tabs[d].e[k];
-            cur = d;
-        }
-        const int li = (int)(item - D.item0);
-        const int r = li / D.n_ch;
-        const int jt0 = (li - r * D.n_ch) * a.chunk;
-        const int jt1 = min(D.n_jt, jt0 + a.chunk);
-        ljc_row_segment<BLOCK, KI, JT>(a.xq, a.perm, a.tblk, D.gpos0, D.npad, s_tab, D.rc2_lim,
-                                       D.has_coul, r, jt0, jt1, sm,
-                                       a.slots + (size_t)item * 6 * ITILE);
-    }
-    // the last CTA out resets the counters for the next launch (every CTA has
-    // drawn its last item by the time it counts itself out)
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(a.work + 1, 1u) == gridDim.x - 1) {
-            a.work[0] = 0u;
-            a.work[1] = 0u;
+        if (atomicAdd(work + 1, 1u) == gridDim.x - 1) {
+            work[0] = 0u;
+            work[1] = 0u;
             __threadfence();
         }
     }
 }
 
+// One-sided: at least 1024 threads resident per SM, whose register cap (64)
+// holds the sweeps without spills.
+template <int BLOCK, int KI, int JT>
+__global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
+k_ens_ljc(EnsAllpairsArgs a)
+{
+    constexpr int ITILE = BLOCK * KI;
+    __shared__ LjcSmem<JT> sm;
+    __shared__ float4 s_tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    __shared__ int s_item;
+    int cur = -1;
+    for (int it = next_item(a.work, &s_item); it < a.n_items; it = next_item(a.work, &s_item)) {
+        const EnsItem item = a.items[it];
+        const EnsDrop &D = a.drops[item.drop];
+        if (item.drop != cur) { // ordered before use by the staging barrier
+            for (int k = threadIdx.x; k < NPSIM_MAX_TYPES * NPSIM_MAX_TYPES; k += BLOCK)
+                s_tab[k] = a.tabs[item.drop].e[k];
+            cur = item.drop;
+        }
+        ljc_row_segment<BLOCK, KI, JT>(a.xq, a.perm, a.tblk, D.gpos0, D.npad, s_tab, D.rc2_lim,
+                                       D.has_coul, item.row, item.jt0, item.jt1, sm,
+                                       a.slots + (size_t)item.slot * 6 * ITILE);
+    }
+    items_done(a.work);
+}
+
+// Each pair once (see sym_row_segment).
+template <int BLOCK, int KI, int JT>
+__global__ void __launch_bounds__(BLOCK, (sym_min_ctas<BLOCK, KI>()))
+k_ens_sym(EnsAllpairsArgs a)
+{
+    constexpr int ITILE = BLOCK * KI;
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    SymSmem<BLOCK, KI, JT> &sm = *reinterpret_cast<SymSmem<BLOCK, KI, JT> *>(s_dyn);
+    __shared__ float4 s_tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    __shared__ int s_item;
+    int cur = -1;
+    for (int it = next_item(a.work, &s_item); it < a.n_items; it = next_item(a.work, &s_item)) {
+        const EnsItem item = a.items[it];
+        const EnsDrop &D = a.drops[item.drop];
+        if (item.drop != cur) { // ordered before use by the staging barrier
+            for (int k = threadIdx.x; k < NPSIM_MAX_TYPES * NPSIM_MAX_TYPES; k += BLOCK)
+                s_tab[k] = a.tabs[item.drop].e[k];
+            cur = item.drop;
+        }
+        float *col = a.slots + (size_t)a.n_items * 6 * ITILE + (size_t)D.col0 +
+                     sym_col_offset(D.npad, ITILE, item.row);
+        sym_row_segment<BLOCK, KI, JT, true>(a.xq, a.perm, a.tblk, D.gpos0, D.npad, s_tab,
+                                             D.has_coul, item.row, item.jt0, item.jt1, sm,
+                                             a.slots + (size_t)item.slot * 6 * ITILE, col,
+                                             (size_t)(D.npad - (item.row + 1) * ITILE));
+    }
+    items_done(a.work);
+}
+
+// The partials of every grouped position, 64 positions per CTA (they share a
+// droplet and a row tile: both are multiples of 64 long).
+__global__ void __launch_bounds__(256)
+k_ens_reduce(EnsAllpairsArgs a)
+{
+    __shared__ float s_part[3][6][64];
+    const int g0 = blockIdx.x * 64;
+    const EnsDrop &D = a.drops[a.dblk[g0 >> 8]];
+    const int p = g0 - D.gpos0 + (threadIdx.x & 63); // position in the droplet's order
+    const int part = threadIdx.x >> 6;
+    const int r = (g0 - D.gpos0) / a.itile;
+    const int s0 = a.row_first[D.row0 + r], s1 = a.row_first[D.row0 + r + 1];
+    float h[3] = {0.f, 0.f, 0.f}, l[3] = {0.f, 0.f, 0.f};
+    sym_sum_partials(a.slots + (size_t)s0 * 6 * a.itile, s1 - s0,
+                     a.slots + (size_t)a.n_items * 6 * a.itile + (size_t)D.col0, a.itile, D.npad, r,
+                     a.sym ? r : 0, p, part, h, l);
+    sym_finish(s_part, part, h, l, a.perm[D.gpos0 + p], a.F_pair);
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(256)
-k_ens_integrate(EnsIntArgs a, int n_total, int n_drops, StreamK sk)
+k_ens_integrate(EnsIntArgs a, int n_total, int n_drops)
 {
     constexpr bool ASSEMBLE = (MODE != MODE_A);
     constexpr bool DO_A = (MODE == MODE_A || MODE == MODE_BA);
@@ -153,17 +192,15 @@ k_ens_integrate(EnsIntArgs a, int n_total, int n_drops, StreamK sk)
         const TypeCoef tc = D.tc[ti];
         float Fh[3] = {0.f, 0.f, 0.f}, Fl[3] = {0.f, 0.f, 0.f};
         if (ASSEMBLE) {
-            if (a.slots) {
-                const int lpos = a.row_pos[i] - D.gpos0; // row in the droplet's grouped order
-                const int r = lpos / sk.itile;
-                const int idx = lpos - r * sk.itile;
-                const long long it0 = D.item0 + (long long)r * D.n_ch; // the row's items
-                for (int c = 0; c < D.n_ch; ++c) {
-                    const float *slot = a.slots + (size_t)(it0 + c) * 6 * sk.itile + idx;
-#pragma unroll
-                    for (int k = 0; k < 3; ++k)
-                        df_add_df(Fh[k], Fl[k], slot[k * sk.itile], slot[(3 + k) * sk.itile]);
-                }
+            if (a.F_pair) {
+                const float4 *q = reinterpret_cast<const float4 *>(a.F_pair + 8 * (size_t)i);
+                const float4 q0 = q[0], q1 = q[1];
+                Fh[0] = q0.x;
+                Fh[1] = q0.y;
+                Fh[2] = q0.z;
+                Fl[0] = q0.w;
+                Fl[1] = q1.x;
+                Fl[2] = q1.y;
             }
             if (a.ext_on) {
                 float ex, ey, ez;
@@ -190,23 +227,27 @@ k_ens_integrate(EnsIntArgs a, int n_total, int n_drops, StreamK sk)
 struct EEntry {
     ApConfig cfg;
     const void *fn;
+    int smem;
+    bool sym;
 };
 
-#define NPSIM_ENS(B, K, J) EEntry{ApConfig{B, K, J, 0}, (const void *)k_ens_ljc<B, K, J>}
+#define NPSIM_ENS_SYM(B, K, J)                                                              \
+    EEntry                                                                                  \
+    {                                                                                       \
+        ApConfig{B, K, J, 0}, (const void *)k_ens_sym<B, K, J>, (int)sizeof(SymSmem<B, K, J>), \
+            true                                                                            \
+    }
 
-// j-tiles of at most 256 partners: the droplets' type groups are padded to 256
+// j-tiles of at most 256 partners: the droplets' type groups are padded to 256.
+// The last shape is the one-sided kernel, for ensembles whose column partials
+// (6 n^2 / itile bytes per droplet) do not fit; each pair once is faster on all
+// others.
 const EEntry kEns[] = {
-    NPSIM_ENS(128, 2, 256), NPSIM_ENS(256, 1, 256), NPSIM_ENS(256, 2, 256),
-    NPSIM_ENS(1024, 1, 256), NPSIM_ENS(256, 1, 128), NPSIM_ENS(512, 1, 256),
-    NPSIM_ENS(128, 1, 256), NPSIM_ENS(128, 1, 128),
+    NPSIM_ENS_SYM(128, 8, 128), NPSIM_ENS_SYM(64, 8, 128), NPSIM_ENS_SYM(128, 4, 128),
+    NPSIM_ENS_SYM(64, 8, 64),   NPSIM_ENS_SYM(64, 4, 64),  NPSIM_ENS_SYM(128, 2, 128),
+    NPSIM_ENS_SYM(64, 2, 64),
+    EEntry{ApConfig{256, 1, 256, 0}, (const void *)k_ens_ljc<256, 1, 256>, 0, false},
 };
-
-template <int B, int K, int J>
-cudaError_t launch_e(const StreamK &sk, const EnsAllpairsArgs &a, cudaStream_t st)
-{
-    k_ens_ljc<B, K, J><<<sk.grid, B, 0, st>>>(a);
-    return cudaGetLastError();
-}
 
 } // namespace
 
@@ -214,40 +255,48 @@ int ens_num_configs() { return (int)(sizeof(kEns) / sizeof(kEns[0])); }
 
 ApConfig ens_config(int idx) { return kEns[idx].cfg; }
 
+bool ens_sym(int idx) { return kEns[idx].sym; }
+
 int ens_occupancy(int idx)
 {
+    const EEntry &e = kEns[idx];
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kEns[idx].fn, kEns[idx].cfg.block,
-                                                      0) != cudaSuccess)
+    if ((e.smem && cudaFuncSetAttribute(e.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        e.smem) != cudaSuccess) ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, e.fn, e.cfg.block, e.smem) !=
+            cudaSuccess)
         return 0;
     return occ;
 }
 
-cudaError_t launch_ens_allpairs(int idx, const StreamK &sk, const EnsAllpairsArgs &a,
-                                cudaStream_t st)
+cudaError_t launch_ens_allpairs(int idx, int ctas, const EnsAllpairsArgs &a, cudaStream_t st)
 {
-    switch (idx) {
-    case 0: return launch_e<128, 2, 256>(sk, a, st);
-    case 1: return launch_e<256, 1, 256>(sk, a, st);
-    case 2: return launch_e<256, 2, 256>(sk, a, st);
-    case 3: return launch_e<1024, 1, 256>(sk, a, st);
-    case 4: return launch_e<256, 1, 128>(sk, a, st);
-    case 5: return launch_e<512, 1, 256>(sk, a, st);
-    case 6: return launch_e<128, 1, 256>(sk, a, st);
-    case 7: return launch_e<128, 1, 128>(sk, a, st);
-    default: return cudaErrorInvalidValue;
+    const EEntry &e = kEns[idx];
+    if (e.smem) {
+        const cudaError_t rc =
+            cudaFuncSetAttribute(e.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
+        if (rc != cudaSuccess)
+            return rc;
     }
+    EnsAllpairsArgs b = a;
+    void *args[] = {(void *)&b};
+    const cudaError_t rc =
+        cudaLaunchKernel(e.fn, dim3(ctas), dim3(e.cfg.block), args, (size_t)e.smem, st);
+    if (rc != cudaSuccess)
+        return rc;
+    k_ens_reduce<<<a.n_pos / 64, 256, 0, st>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_ens_integrate(int mode, const EnsIntArgs &a, int n_total, int n_drops,
-                                 const StreamK &sk, cudaStream_t st)
+                                 cudaStream_t st)
 {
     const int grid = (n_total + 255) / 256;
     switch (mode) {
-    case MODE_FORCES: k_ens_integrate<MODE_FORCES><<<grid, 256, 0, st>>>(a, n_total, n_drops, sk); break;
-    case MODE_A: k_ens_integrate<MODE_A><<<grid, 256, 0, st>>>(a, n_total, n_drops, sk); break;
-    case MODE_BA: k_ens_integrate<MODE_BA><<<grid, 256, 0, st>>>(a, n_total, n_drops, sk); break;
-    case MODE_B: k_ens_integrate<MODE_B><<<grid, 256, 0, st>>>(a, n_total, n_drops, sk); break;
+    case MODE_FORCES: k_ens_integrate<MODE_FORCES><<<grid, 256, 0, st>>>(a, n_total, n_drops); break;
+    case MODE_A: k_ens_integrate<MODE_A><<<grid, 256, 0, st>>>(a, n_total, n_drops); break;
+    case MODE_BA: k_ens_integrate<MODE_BA><<<grid, 256, 0, st>>>(a, n_total, n_drops); break;
+    case MODE_B: k_ens_integrate<MODE_B><<<grid, 256, 0, st>>>(a, n_total, n_drops); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -576,6 +576,13 @@ __device__ __forceinline__ void ljc_sym_sweep(const float4 *__restrict__ s_a,
 // Shared memory of sym_row_segment: the staged tiles of LjcSmem and the
 // partners' sums of one tile per warp (two buffers: one is summed over the warps
 // while the next tile fills the other).
+template <int BLOCK, int KI>
+constexpr int sym_min_ctas()
+{
+    // 168, 96 (128 with 256 threads or more) or 80 registers per thread
+    return KI >= 8 ? 384 / BLOCK : KI >= 4 ? (BLOCK <= 128 ? 640 : 512) / BLOCK : 768 / BLOCK;
+}
+
 template <int BLOCK, int KI, int JT>
 struct SymSmem {
     LjcSmem<JT> st;
@@ -1022,15 +1029,16 @@ __host__ __device__ __forceinline__ int sk_cta_of(const StreamK &s, long long p)
 // ---------------------------------------------------------------------------
 // Sum of a position's partials of the kernels that evaluate each pair once
 // (sym_row_segment): its row's n_rows slots [6][itile] from row_slots on, then
-// the column partials of the row tiles before its own, r' = 0 .. r - 1.  Four
+// the column partials of the first n_cols row tiles (those before its own, r' =
+// 0 .. r - 1; none in a one-sided sum).  Four
 // threads share a position (64 positions per CTA of 256 threads, so the reads
 // are coalesced and a long column has four times the loads in flight): thread
 // `part` takes every fourth slot, compensated; sym_finish adds the four in a
 // fixed order.
 __device__ __forceinline__ void sym_sum_partials(const float *__restrict__ row_slots, int n_rows,
                                                  const float *__restrict__ cols, int itile,
-                                                 int len, int r, int p, int part, float (&h)[3],
-                                                 float (&l)[3])
+                                                 int len, int r, int n_cols, int p, int part,
+                                                 float (&h)[3], float (&l)[3])
 {
     const float *rs = row_slots + (p - r * itile);
     for (int c = part; c < n_rows; c += 4) {
@@ -1040,7 +1048,7 @@ __device__ __forceinline__ void sym_sum_partials(const float *__restrict__ row_s
             df_add_df(h[d], l[d], __ldcs(q + d * itile), __ldcs(q + (3 + d) * itile));
     }
     int k = part;
-    for (; k + 4 < r; k += 8) { // two row tiles' loads before their adds
+    for (; k + 4 < n_cols; k += 8) { // two row tiles' loads before their adds
         const float *q0 = cols + sym_col_offset(len, itile, k) + (p - (k + 1) * itile);
         const float *q1 = cols + sym_col_offset(len, itile, k + 4) + (p - (k + 5) * itile);
         const size_t l0 = (size_t)(len - (k + 1) * itile), l1 = (size_t)(len - (k + 5) * itile);
@@ -1057,7 +1065,7 @@ __device__ __forceinline__ void sym_sum_partials(const float *__restrict__ row_s
         for (int d = 0; d < 3; ++d)
             df_add(h[d], l[d], w[3 + d]);
     }
-    for (; k < r; k += 4) {
+    for (; k < n_cols; k += 4) {
         const float *q = cols + sym_col_offset(len, itile, k) + (p - (k + 1) * itile);
         const size_t ld = (size_t)(len - (k + 1) * itile);
 #pragma unroll
@@ -1323,34 +1331,43 @@ cudaError_t launch_slot_sum(const float *slots, const StreamK &sk, int n_pos, fl
 
 // Ensemble of droplets (ensemble.cu).  Each droplet's particles are listed in a
 // type-grouped order (groups padded to 256 positions) at positions [gpos0,
-// gpos0 + npad) of the ensemble's grouped order.  Geometry depends on the
-// launch shape: n_it = ceil(npad / itile) row tiles, n_jt = npad / jtile
-// j-tiles, each row tile cut into n_ch = ceil(n_jt / chunk) work items of at
-// most `chunk` consecutive j-tiles; item0 is the prefix sum of n_it * n_ch
-// over the droplets (item = item0 + row * n_ch + chunk index).
+// gpos0 + npad) of the ensemble's grouped order.  The all-pairs work is a list of
+// items (a row tile of a droplet against up to `chunk` of its consecutive
+// j-tiles); the column partials of droplet d (sym_row_segment) start at float
+// col0 of theirs, and its row tiles at row0 of row_first.
 struct EnsDrop {
-    int offset, n, n_it, n_jt, n_ch, rot_mode, wall, integrator;
+    int offset, n, rot_mode, wall, integrator;
     int gpos0, npad;
     float rc2_lim;  // LJ only between tiles within this squared distance (0: no LJ)
     int has_coul;   // 0: tiles out of LJ range add nothing
-    long long item0;
+    int row0;
+    long long col0;
     uint64_t seed;
     double dt, R0, k_evap, g, omega2;
     TypeCoef tc[NPSIM_MAX_TYPES];
+};
+
+struct EnsItem {
+    int drop, row, jt0, jt1; // row tile of the droplet, its j-tiles jt0 .. jt1 - 1
+    int slot;                // where the rows' sums go
 };
 
 struct EnsAllpairsArgs {
     const float4 *xq;
     const int *perm;        // grouped position -> particle (-1: padding)
     const int *tblk;        // type of each 256-position block
+    const int *dblk;        // droplet of each 256-position block
     const EnsDrop *drops;
-    const long long *item0; // n_drops + 1 entries
     const PairTab *tabs;    // one table per droplet
-    int n_drops;
-    int chunk;              // j-tiles per work item
-    long long n_items;
+    const EnsItem *items;   // longest first
+    const int *row_first;   // first slot of every row tile, slots in row order; one past the end
+    int n_items;
+    int n_pos;              // grouped length
+    int itile;
+    int sym;                // kernels that evaluate each pair once (column partials)
     unsigned *work;         // [0] next item, [1] CTAs done (both 0 between launches)
-    float *slots;           // one [6][itile] slot per work item
+    float *slots;           // one [6][itile] slot per work item, then the column partials
+    float *F_pair;          // [n_total][8] (hi x, y, z, lo x, y, z, 0, 0): the summed forces
 };
 
 struct EnsIntArgs {
@@ -1358,9 +1375,8 @@ struct EnsIntArgs {
     const int *typ;
     float4 *xq;
     const int *drop_of;
-    const int *row_pos;      // grouped position of particle i
     const EnsDrop *drops;
-    const float *slots;
+    const float *F_pair;     // all-pairs forces [n_total][8], as in IntArgs (or NULL)
     float4 *spring;          // [2][n_drops][NPSIM_MAX_TYPES], as in IntArgs
     int ext_on;
     int pad_;
@@ -1372,10 +1388,12 @@ struct EnsIntArgs {
 int ens_num_configs();
 ApConfig ens_config(int idx);
 int ens_occupancy(int idx);
-cudaError_t launch_ens_allpairs(int idx, const StreamK &sk, const EnsAllpairsArgs &a,
-                                cudaStream_t st);
+bool ens_sym(int idx); // evaluates each pair once
+// The all-pairs launch on `ctas` CTAs and the reduction of its partials into
+// a.F_pair.
+cudaError_t launch_ens_allpairs(int idx, int ctas, const EnsAllpairsArgs &a, cudaStream_t st);
 cudaError_t launch_ens_integrate(int mode, const EnsIntArgs &a, int n_total, int n_drops,
-                                 const StreamK &sk, cudaStream_t st);
+                                 cudaStream_t st);
 
 // BF16 tensor-core MLP kernels (mlp.cu).
 enum : int {

@@ -102,9 +102,9 @@ struct SEntry {
 // Best launch + reduction by grouped length (ms; one-sided kernel's best in
 // brackets).  Coulomb: 100352 <128,8,128> 2.34 [3.27], 24576 0.168 [0.219],
 // 8704 <64,8,128> 0.035 [0.039], 2560 <64,2,64> 0.015 [0.020].  LJ + Coulomb:
-// 60416 <64,8,128> 1.06 [1.45], 30208 0.321 [0.409], 16384 <128,2,128> 0.122
-// [0.147], 4096 0.025 [0.027], 1024 <64,2,64> 0.019 [0.025]: long rows want many
-// rows per thread, short ones many small units.
+// 60416 <64,8,128> 0.99 [1.39], 30208 0.295 [0.381], 16384 0.112 [0.134], 4096
+// <128,2,128> 0.025 [0.027], 1024 <64,2,64> 0.019 [0.025]: long rows want many rows
+// per thread, short ones many small units.
 const SEntry kSym[] = {
     NPSIM_SYM(128, 8, 128, false), NPSIM_SYM(64, 8, 128, false), NPSIM_SYM(128, 4, 128, false),
     NPSIM_SYM(64, 4, 64, false),   NPSIM_SYM(64, 2, 64, false),

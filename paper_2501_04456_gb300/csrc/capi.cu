@@ -50,6 +50,7 @@ int set_err(int code, const char *fmt, ...)
 
 constexpr int kChunk = 16;      // steps per captured graph
 constexpr double kKf = 1.593;   // fractal prefactor, Sec. 3.1
+constexpr size_t kBoxTableKeys = (size_t)8 << 20; // box-counting tables of one launch: 64 MiB
 
 template <class T> cudaError_t dalloc(T **p, size_t count)
 {
@@ -78,35 +79,29 @@ void free_cells(CellBufs &b)
 }
 
 // Scratch of the statistics of Sec. 3 (allocated on first use, grown as needed):
-// float64 positions, the cell list of the pair histogram, the histograms, the
-// per-CTA partial sums and the box-counting hash table.
+// float64 positions, the cell list of the pair histogram, the results and the
+// box-counting hash tables.
 struct StatsWork {
     double *x = nullptr; // [3][n] float64 positions (hi + lo), when the owner has none
     int x_cap = 0;
     CellGrid grid{};
     CellBufs cb{};
     int cells_cap = 0, cells_n = 0; // cells and NPs the cell buffers hold
-    unsigned long long *hist = nullptr, *rhist = nullptr;
-    int hist_cap = 0, rhist_cap = 0;
-    double *part = nullptr; // 3 doubles per CTA of 256 threads
-    int part_cap = 0;
+    // results of one call, read back in as few copies as its steps allow: 8-byte
+    // words, 6 per CTA of 256 threads (reductions), the histograms, N_surf, boxes
+    unsigned long long *res = nullptr;
+    size_t res_cap = 0;
     double *vec = nullptr;  // centre of mass [3], box origin [3]
     unsigned long long *table = nullptr;
-    unsigned long long table_size = 0;
-    int *count = nullptr;
-    unsigned long long *surf = nullptr; // N_surf counter
+    size_t table_cap = 0;   // keys
 };
 void free_stats(StatsWork &w)
 {
     dfree(w.x);
     free_cells(w.cb);
-    dfree(w.hist);
-    dfree(w.rhist);
-    dfree(w.part);
+    dfree(w.res);
     dfree(w.vec);
     dfree(w.table);
-    dfree(w.count);
-    dfree(w.surf);
     w = StatsWork{};
 }
 
@@ -1832,20 +1827,6 @@ int npsim_kernel_times(npsim_sim_t s, double *ms, int *samples)
 
 namespace {
 
-// One reduction of launch_block_reduce over n positions, its per-CTA partials
-// copied to the host (CTA order).
-int block_partials(StatsWork &w, int mode, const double *x, int n, const double *c,
-                   std::vector<double> &part, cudaStream_t st)
-{
-    const int nblk = (n + 255) / 256;
-    part.resize(3 * (size_t)nblk);
-    NP_CUDA(launch_block_reduce(mode, x, n, c, w.part, st));
-    NP_CUDA(cudaMemcpyAsync(part.data(), w.part, sizeof(double) * part.size(),
-                            cudaMemcpyDeviceToHost, st));
-    NP_CUDA(cudaStreamSynchronize(st));
-    return NPSIM_OK;
-}
-
 // The statistics of Sec. 3 of one droplet of n NPs whose float64 positions
 // ([3][n]) are x, float32 hi words xq and types typ (all device), at droplet
 // radius R: the RDF (Sec. 3.2), the radial concentration C_NPs, N_surf, the
@@ -1862,38 +1843,48 @@ int stats_core(StatsWork &w, const double *x, const float4 *xq, const int *typ, 
     const double pi = 3.14159265358979323846;
 
     const int nblk = (n + 255) / 256;
-    if (!w.vec) {
+    const bool rdf = cfg->n_bins > 0 && rdf_counts, radial = cfg->radial_bins > 0 && radial_counts;
+    if (!w.vec)
         NP_CUDA(dalloc(&w.vec, 8));
-        NP_CUDA(dalloc(&w.count, 1));
-        NP_CUDA(dalloc(&w.surf, 1));
+    // words of the results: [3 nblk] and [3 nblk] of a reduction, RDF bins,
+    // radial bins, N_surf, box counts
+    const size_t o_hist = 6 * (size_t)nblk, o_rhist = o_hist + (rdf ? cfg->n_bins : 0),
+                 o_surf = o_rhist + (radial ? cfg->radial_bins : 0), o_box = o_surf + 1,
+                 n_res = o_box + NPSIM_MAX_SCALES;
+    if (n_res > w.res_cap) {
+        dfree(w.res);
+        w.res_cap = 0;
+        NP_CUDA(dalloc(&w.res, n_res));
+        w.res_cap = n_res;
     }
-    if (nblk > w.part_cap) {
-        dfree(w.part);
-        NP_CUDA(dalloc(&w.part, 3 * (size_t)nblk));
-        w.part_cap = nblk;
-    }
-    std::vector<double> part;
+    std::vector<unsigned long long> res(n_res);
+    double *d_part = reinterpret_cast<double *>(w.res);
+    const double *part = reinterpret_cast<const double *>(res.data());
+    // words [0, count) of the results to the host, after everything queued so far
+    auto fetch = [&](size_t first, size_t count) -> cudaError_t {
+        cudaError_t e = cudaMemcpyAsync(res.data() + first, w.res + first,
+                                        sizeof(unsigned long long) * count,
+                                        cudaMemcpyDeviceToHost, st);
+        return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+    };
     // extent of the cloud: minimum corner (box-counting origin), largest |x_d|
-    int rc = block_partials(w, 2, x, n, nullptr, part, st);
-    if (rc)
-        return rc;
+    NP_CUDA(launch_block_reduce(2, x, n, nullptr, d_part, st));
+    NP_CUDA(launch_block_reduce(3, x, n, nullptr, d_part + 3 * (size_t)nblk, st));
+    NP_CUDA(fetch(0, 6 * (size_t)nblk));
     double o[3] = {INFINITY, INFINITY, INFINITY};
+    double L = R;
     for (int b = 0; b < nblk; ++b)
-        for (int d = 0; d < 3; ++d)
-            o[d] = std::min(o[d], part[3 * b + d]);
+        for (int d = 0; d < 3; ++d) {
+            o[d] = std::min(o[d], part[3 * (size_t)b + d]);
+            L = std::max(L, part[3 * (size_t)(nblk + b) + d]);
+        }
 
-    if (cfg->n_bins > 0 && rdf_counts) {
-        rc = block_partials(w, 3, x, n, nullptr, part, st);
-        if (rc)
-            return rc;
-        // cell grid with edge >= r_max over the cloud (positions are needed in
-        // float32 only to choose candidates)
-        double L = R;
-        for (int b = 0; b < nblk; ++b)
-            for (int d = 0; d < 3; ++d)
-                L = std::max(L, part[3 * b + d]);
+    int rc = NPSIM_OK;
+    if (rdf) {
+        // cell grid over the cloud (positions are needed in float32 only to choose
+        // candidates and for the bins that float32 settles)
         L += cfg->r_max + 1.0;
-        CellGrid g = make_grid(L, cfg->r_max * (1.0 + 1e-4) + 1e-3,
+        CellGrid g = make_grid(L, pair_hist_cell_edge(cfg->r_max, L),
                                std::max<long long>(4 * (long long)n + 4096, 1 << 16));
         if (g.n_cells > w.cells_cap || n > w.cells_n) {
             // grow to hold both this droplet and the largest one seen so far
@@ -1909,78 +1900,55 @@ int stats_core(StatsWork &w, const double *x, const float4 *xq, const int *typ, 
             w.cells_n = na;
         }
         w.grid = g;
-        if (cfg->n_bins > w.hist_cap) {
-            dfree(w.hist);
-            NP_CUDA(dalloc(&w.hist, cfg->n_bins));
-            w.hist_cap = cfg->n_bins;
-        }
         NP_CUDA(launch_cell_build(g, xq, typ, n, w.cb, nullptr, st));
-        NP_CUDA(launch_pair_hist(x, n, cfg->r_max, cfg->n_bins, g, w.cb, w.hist, st));
-        std::vector<unsigned long long> h(cfg->n_bins);
-        NP_CUDA(cudaMemcpyAsync(h.data(), w.hist, sizeof(unsigned long long) * h.size(),
-                                cudaMemcpyDeviceToHost, st));
-        NP_CUDA(cudaStreamSynchronize(st));
+        NP_CUDA(launch_pair_hist(x, n, cfg->r_max, cfg->n_bins, g, w.cb, w.res + o_hist, st));
+    }
+    if (radial)
+        NP_CUDA(launch_radial_hist(x, n, R, cfg->radial_bins, w.res + o_rhist, st));
+    // N_surf: NPs in the band (-r_i, r_i) about the surface
+    SurfHalf hs{};
+    for (int t = 0; t < T; ++t)
+        hs.h[t] = 0.5 * types[t].sigma;
+    NP_CUDA(launch_surface_count(x, typ, n, R, hs, w.res + o_surf, st));
+    NP_CUDA(launch_block_reduce(0, x, n, nullptr, d_part, st));
+    NP_CUDA(fetch(0, o_surf + 1));
+    out->n_surf = (int64_t)res[o_surf];
+    const double V = 4.0 / 3.0 * pi * R * R * R;
+    if (rdf) {
         const double dr = cfg->r_max / (double)cfg->n_bins;
-        const double V = 4.0 / 3.0 * pi * R * R * R;
         for (int b = 0; b < cfg->n_bins; ++b) {
-            rdf_counts[b] = (int64_t)h[b];
+            rdf_counts[b] = (int64_t)res[o_hist + b];
             if (rdf_g) {
                 const double r0 = b * dr, r1 = (b + 1) * dr;
                 const double dV = 4.0 / 3.0 * pi * (r1 * r1 * r1 - r0 * r0 * r0);
-                rdf_g[b] = ((double)h[b] / (double)n) / ((double)(n - 1) * dV / V);
+                rdf_g[b] = ((double)rdf_counts[b] / (double)n) / ((double)(n - 1) * dV / V);
             }
         }
     }
-    if (cfg->radial_bins > 0 && radial_counts) {
-        if (cfg->radial_bins > w.rhist_cap) {
-            dfree(w.rhist);
-            NP_CUDA(dalloc(&w.rhist, cfg->radial_bins));
-            w.rhist_cap = cfg->radial_bins;
-        }
-        NP_CUDA(launch_radial_hist(x, n, R, cfg->radial_bins, w.rhist, st));
-        std::vector<unsigned long long> h(cfg->radial_bins);
-        NP_CUDA(cudaMemcpyAsync(h.data(), w.rhist, sizeof(unsigned long long) * h.size(),
-                                cudaMemcpyDeviceToHost, st));
-        NP_CUDA(cudaStreamSynchronize(st));
+    if (radial) {
         const double dr = R / (double)cfg->radial_bins;
-        const double V = 4.0 / 3.0 * pi * R * R * R;
         for (int b = 0; b < cfg->radial_bins; ++b) {
-            radial_counts[b] = (int64_t)h[b];
+            radial_counts[b] = (int64_t)res[o_rhist + b];
             if (radial_c) {
                 const double r0 = b * dr, r1 = (b + 1) * dr;
                 const double dV = 4.0 / 3.0 * pi * (r1 * r1 * r1 - r0 * r0 * r0);
-                radial_c[b] = ((double)h[b] / (double)n) / (dV / V);
+                radial_c[b] = ((double)radial_counts[b] / (double)n) / (dV / V);
             }
         }
     }
-    // N_surf: NPs in the band (-r_i, r_i) about the surface
-    {
-        SurfHalf hs{};
-        for (int t = 0; t < T; ++t)
-            hs.h[t] = 0.5 * types[t].sigma;
-        unsigned long long cnt = 0;
-        NP_CUDA(launch_surface_count(x, typ, n, R, hs, w.surf, st));
-        NP_CUDA(cudaMemcpyAsync(&cnt, w.surf, sizeof(cnt), cudaMemcpyDeviceToHost, st));
-        NP_CUDA(cudaStreamSynchronize(st));
-        out->n_surf = (int64_t)cnt;
-    }
     // centre of mass and radius of gyration (Eqs. r0, Rg), fractal equation (Eq. N)
-    rc = block_partials(w, 0, x, n, nullptr, part, st);
-    if (rc)
-        return rc;
     double c[3] = {0, 0, 0};
     for (int b = 0; b < nblk; ++b)
         for (int d = 0; d < 3; ++d)
-            c[d] += part[3 * b + d];
+            c[d] += part[3 * (size_t)b + d];
     for (int d = 0; d < 3; ++d)
         c[d] /= (double)n;
     NP_CUDA(cudaMemcpyAsync(w.vec, c, sizeof(c), cudaMemcpyHostToDevice, st));
-    rc = block_partials(w, 1, x, n, w.vec, part, st);
-    if (rc)
-        return rc;
+    NP_CUDA(launch_block_reduce(1, x, n, w.vec, d_part, st));
+    NP_CUDA(fetch(0, 3 * (size_t)nblk));
     double ss = 0.0;
     for (int b = 0; b < nblk; ++b)
-        ss += part[3 * b];
+        ss += part[3 * (size_t)b];
     const double Rg = std::sqrt(ss / (double)n);
     out->Rg = Rg;
     out->Df_rg = std::log((double)n / kKf) / std::log(2.0 * Rg / d_mean);
@@ -1989,26 +1957,31 @@ int stats_core(StatsWork &w, const double *x, const float4 *xq, const int *typ, 
 
     out->Df_box = NAN;
     if (cfg->boxcount) {
-        unsigned long long tsz = 1;
-        while (tsz < 2ull * (unsigned long long)n)
+        size_t tsz = 1;
+        while (tsz < 2 * (size_t)n)
             tsz <<= 1;
-        if (tsz > w.table_size) {
-            dfree(w.table);
-            NP_CUDA(dalloc(&w.table, tsz));
-            w.table_size = tsz;
-        }
-        NP_CUDA(cudaMemcpyAsync(w.vec + 3, o, sizeof(o), cudaMemcpyHostToDevice, st));
         int ns = 0;
         while (ns < cfg->max_scales && d_mean * std::ldexp(1.0, ns) <= 2.0 * Rg)
             ++ns;
-        for (int k = 0; k < ns; ++k) {
-            const double eps = d_mean * std::ldexp(1.0, k);
-            NP_CUDA(launch_boxcount(x, n, w.vec + 3, eps, w.table, tsz, w.count, d_flags, st));
-            int cnt = 0;
-            NP_CUDA(cudaMemcpyAsync(&cnt, w.count, sizeof(int), cudaMemcpyDeviceToHost, st));
-            NP_CUDA(cudaStreamSynchronize(st));
-            out->nbox[k] = cnt;
+        // one table per scale, as many scales per launch as fit kBoxTableKeys (one
+        // at least)
+        const int group = (int)std::max<size_t>(1, std::min<size_t>(ns, kBoxTableKeys / tsz));
+        if (group * tsz > w.table_cap) {
+            dfree(w.table);
+            w.table_cap = 0;
+            NP_CUDA(dalloc(&w.table, group * tsz));
+            w.table_cap = group * tsz;
         }
+        NP_CUDA(cudaMemcpyAsync(w.vec + 3, o, sizeof(o), cudaMemcpyHostToDevice, st));
+        if (ns > 0) {
+            NP_CUDA(cudaMemsetAsync(w.res + o_box, 0, sizeof(unsigned long long) * ns, st));
+            for (int k = 0; k < ns; k += group)
+                NP_CUDA(launch_boxcount(x, n, w.vec + 3, d_mean, k, std::min(group, ns - k),
+                                        w.table, tsz, w.res + o_box, d_flags, st));
+            NP_CUDA(fetch(o_box, ns));
+        }
+        for (int k = 0; k < ns; ++k)
+            out->nbox[k] = (int64_t)res[o_box + k];
         out->n_scales = ns;
         if (ns - 1 >= 2) {
             // least squares of ln N_box on ln eps over scales k >= 1

@@ -1502,6 +1502,7 @@ int cell_build_launches();
 int cell_scan_tiles(int n_cells);
 
 // Stats (stats.cu)
+double pair_hist_cell_edge(double r_max, double L); // cell edge of the histogram's grid
 cudaError_t launch_pair_hist(const double *x, int n, double r_max, int n_bins,
                              const CellGrid &g, const CellBufs &b,
                              unsigned long long *hist, cudaStream_t st);
@@ -1522,9 +1523,12 @@ cudaError_t launch_surface_count(const double *x, const int *typ, int n, double 
                                  const SurfHalf &hs, unsigned long long *count, cudaStream_t st);
 cudaError_t launch_block_reduce(int mode, const double *x, int n, const double *c,
                                 double *part, cudaStream_t st);
-cudaError_t launch_boxcount(const double *x, int n, const double *origin, double eps,
-                            unsigned long long *table, unsigned long long table_size,
-                            int *count, int *flags, cudaStream_t st);
+// Boxes of edge eps0 2^k with a particle, k = k0 .. k0 + n_scales - 1, added to
+// counts[k]; tables: n_scales of table_size keys (a power of two >= 2n).
+cudaError_t launch_boxcount(const double *x, int n, const double *origin, double eps0, int k0,
+                            int n_scales, unsigned long long *tables,
+                            unsigned long long table_size, unsigned long long *counts, int *flags,
+                            cudaStream_t st);
 // Split float64 positions (SoA) into the integrator's hi (mirror) / lo words,
 // and back (x = hi + lo in float64, for statistics).
 cudaError_t launch_mirror(const double *x, const int *typ, const float *charge_by_type,

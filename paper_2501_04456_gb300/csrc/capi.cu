@@ -218,6 +218,7 @@ struct npsim_sim {
     size_t cells_alloc = 0;  // sort keys the cell buffers hold
     NbrList nl{};          // Verlet list over the cells (cell-list LJ)
     int *d_gate = nullptr; // 1: rebuild the cell and neighbour lists at the next pass
+    unsigned *list_bar = nullptr; // counters of the list build's grid barrier [3]
 
     bool ap = false, ap_lj = false;
     int ap_idx = 0;
@@ -292,6 +293,7 @@ struct npsim_sim {
         dfree(d_flags);
         dfree(d_done);
         dfree(d_gate);
+        dfree(list_bar);
         dfree(nl.nbr);
         dfree(nl.nnbr);
         dfree(nl.x_ref);
@@ -334,8 +336,8 @@ void set_extents(CellGrid &g, const double *rl)
     }
 }
 
-// Buffers of a cell list of n NPs over the g.tb * g.n_cells sort keys.  pos starts
-// at 0 so that every slot it names is in range before the first build.
+// Buffers of a cell list of n NPs over the g.tb * g.n_cells sort keys.  pos, sorted
+// and key start at 0 so that what they name is in range before the first build.
 int alloc_cells(CellGrid &g, CellBufs &b, int n)
 {
     const size_t m = (size_t)std::max(g.tb, 1) * (size_t)g.n_cells;
@@ -346,7 +348,8 @@ int alloc_cells(CellGrid &g, CellBufs &b, int n)
     NP_CUDA(dalloc(&b.arrived, n));
     NP_CUDA(dalloc(&b.sorted, n));
     NP_CUDA(dalloc(&b.pos, n));
-    NP_CUDA(cudaMemset(b.pos, 0, sizeof(int) * (size_t)(n > 0 ? n : 1)));
+    for (int *q : {b.pos, b.sorted, b.key})
+        NP_CUDA(cudaMemset(q, 0, sizeof(int) * (size_t)(n > 0 ? n : 1)));
     // one record past the NPs: a position far from every NP (type 0), the
     // partner that pads each neighbour list to whole blocks of four
     NP_CUDA(dalloc(&b.sxq, (size_t)n + 1));
@@ -590,12 +593,11 @@ int enqueue_pass(npsim_sim *s, int mode, bool want_lj, bool want_coul, bool ext,
                     : cudaSuccess;
     };
     if (lj_cell) {
-        // the build kernels run (past their gate check) only after an NP has
-        // moved more than half the skin since the last build
+        // builds (past its gate check) only after an NP has moved more than half the
+        // skin since the last build
         NP_CUDA(mark(KG_CELL_BUILD, 0));
-        NP_CUDA(launch_cell_build(s->grid, s->xq, s->typ, s->n, s->cb, s->d_gate, st));
-        NP_CUDA(launch_nbr_build(s->grid, s->cb, s->n, s->tab_full, s->d_rcc2, kSkin, s->nl,
-                                 s->d_flags, s->d_gate, st));
+        NP_CUDA(launch_list_build(s->grid, s->cb, s->xq, s->typ, s->n, s->tab_full, s->d_rcc2,
+                                  kSkin, s->nl, s->d_flags, s->d_gate, s->list_bar, st));
         NP_CUDA(mark(KG_CELL_BUILD, 1));
         NP_CUDA(mark(KG_CELL_LJ, 0));
         NP_CUDA(launch_lj_nbr(s->grid, s->cb, s->xq, s->typ, s->n,
@@ -727,6 +729,7 @@ int grow_neighbour_list(npsim_sim *s)
     if (e != cudaSuccess)
         return set_err(NPSIM_ERR_OOM, "neighbour list of %d x %d entries: %s", cap, s->n,
                        cudaGetErrorString(e));
+    NP_CUDA(cudaMemsetAsync(nb, 0, sizeof(unsigned) * (size_t)cap * s->n, s->user));
     dfree(s->nl.nbr);
     s->nl.nbr = nb;
     s->nl.cap = cap;
@@ -754,8 +757,15 @@ int read_flags(npsim_sim *s)
         NP_CUDA(cudaMemsetAsync(s->d_flags, 0, sizeof(int), s->user));
         if (h & FLAG_NONFINITE)
             return set_err(NPSIM_ERR_NONFINITE, "a position became non-finite");
-        if (h & FLAG_TIMEOUT)
+        if (h & FLAG_TIMEOUT) {
+            if (s->list_bar) { // the barrier it left, and the lists it did not finish
+                NP_CUDA(cudaMemsetAsync(s->list_bar, 0, 3 * sizeof(unsigned), s->user));
+                int rc = set_gate(s, 1);
+                if (rc)
+                    return rc;
+            }
             return set_err(NPSIM_ERR_TIMEOUT, "a bounded device wait expired");
+        }
         if (h & FLAG_ESCAPED)
             return set_err(NPSIM_ERR_ESCAPED,
                            "an NP was farther than 2 max(R0, R(t)) from the droplet centre");
@@ -1425,6 +1435,10 @@ int create_impl(const npsim_type_t *types, const npsim_params_t *params, int64_t
         BAIL_CUDA(dalloc(&s->nl.builds, 1));
         BAIL_CUDA(cudaMemset(s->nl.builds, 0, sizeof(unsigned long long)));
         BAIL_CUDA(dalloc(&s->d_gate, 1));
+        BAIL_CUDA(dalloc(&s->list_bar, 3));
+        BAIL_CUDA(cudaMemset(s->list_bar, 0, 3 * sizeof(unsigned)));
+        BAIL_CUDA(cudaMemset(s->nl.nnbr, 0, sizeof(int) * (size_t)n));
+        BAIL_CUDA(cudaMemset(s->nl.nbr, 0, sizeof(unsigned) * (size_t)s->nl.cap * n));
     }
     s->ap_lj = params->lj_mode == 1;
     s->ap = params->coulomb == 1 || s->ap_lj;
@@ -1727,8 +1741,9 @@ int npsim_allpairs_num_configs(int *count)
 int npsim_launches_per_step(npsim_sim_t s, int *launches)
 {
     NP_REQUIRE(s && launches, "sim and launches are required");
-    // integrator, all-pairs (and the sum of its partials), the gated cell and list builds, the list LJ forces
-    *launches = 1 + (s->ap ? (s->sk.tri ? 2 : 1) : 0) + (s->cell ? cell_build_launches() + 2 : 0);
+    // integrator, all-pairs (and the sum of its partials), the gated list build, the
+    // list LJ forces
+    *launches = 1 + (s->ap ? (s->sk.tri ? 2 : 1) : 0) + (s->cell ? 2 : 0);
     return NPSIM_OK;
 }
 
@@ -1900,7 +1915,7 @@ int stats_core(StatsWork &w, const double *x, const float4 *xq, const int *typ, 
             w.cells_n = na;
         }
         w.grid = g;
-        NP_CUDA(launch_cell_build(g, xq, typ, n, w.cb, nullptr, st));
+        NP_CUDA(launch_cell_build(g, xq, typ, n, w.cb, st));
         NP_CUDA(launch_pair_hist(x, n, cfg->r_max, cfg->n_bins, g, w.cb, w.res + o_hist, st));
     }
     if (radial)
@@ -2086,6 +2101,7 @@ int restore_lists(npsim_sim *s, const CkptHeader &h, const float4 *x_ref_host)
     if (h.nbr_cap != s->nl.cap) {
         dfree(s->nl.nbr);
         NP_CUDA(dalloc(&s->nl.nbr, (size_t)h.nbr_cap * s->n));
+        NP_CUDA(cudaMemset(s->nl.nbr, 0, sizeof(unsigned) * (size_t)h.nbr_cap * s->n));
         s->nl.cap = h.nbr_cap;
     }
     for (auto &e : s->graphs)
@@ -2093,10 +2109,8 @@ int restore_lists(npsim_sim *s, const CkptHeader &h, const float4 *x_ref_host)
     s->graphs.clear();
     NP_CUDA(cudaMemcpy(s->nl.x_ref, x_ref_host, sizeof(float4) * (size_t)s->n,
                        cudaMemcpyHostToDevice));
-    NP_CUDA(launch_cell_build(s->grid, s->nl.x_ref, s->typ, s->n, s->cb, nullptr, s->user));
-    NP_CUDA(launch_nbr_build(s->grid, s->cb, s->n, s->tab_full, s->d_rcc2, kSkin, s->nl,
-                             s->d_flags,
-                             nullptr, s->user));
+    NP_CUDA(launch_list_build(s->grid, s->cb, s->nl.x_ref, s->typ, s->n, s->tab_full, s->d_rcc2,
+                              kSkin, s->nl, s->d_flags, nullptr, s->list_bar, s->user));
     // the list kernel reads the current positions from the cell-ordered records
     NP_CUDA(launch_cell_refresh(s->cb, s->xq, s->typ, s->n, s->user));
     NP_CUDA(cudaStreamSynchronize(s->user));

@@ -1,7 +1,7 @@
 // celllist.cu -- cell binning (step (i) of the loop in arXiv 2501.04456 Sec. 2.2:
 // NPs are sorted into spatial cells so that near neighbours are found quickly)
-// and the truncated, unshifted Lennard-Jones force over the 27 neighbouring
-// cells (step (ii)):
+// and the truncated, unshifted Lennard-Jones force over the neighbouring cells
+// (step (ii)):
 //   F_i = sum_{j != i, r < rc_ij} 24 eps_ij (2 (s_ij/r)^12 - (s_ij/r)^6) r_ij / r^2.
 //
 // Binning is a counting sort: hash (sort key of each NP, its arrival rank from
@@ -13,8 +13,8 @@
 // lists the key is type * n_cells + cell: the cell order lists the NPs of one
 // type cell by cell, then the next type, so that consecutive threads of the
 // list kernels hold NPs of one type (lists of similar length, read coalesced)
-// in nearby cells (their partners lie in the same few cells).  A gather writes
-// the NP records (position, type in the fourth word) in cell order so the
+// in nearby cells (their partners lie in the same few cells).  The NP records
+// (position, type in the fourth word) are written in cell order too, so the
 // kernels read neighbours from contiguous memory; with a neighbour list the
 // integrator keeps these records current, so the per-step list kernel reads
 // every position in cell order and never gathers by particle index.
@@ -23,7 +23,7 @@
 // edge is the largest cutoff plus a skin, a build lists for every NP the
 // partners within its pair cutoff plus the skin and records the positions it
 // saw; the integrator raises a gate when some NP has moved more than half the
-// skin since then, and only then do the (gated) build kernels run again.  A
+// skin since then, and only then does the next build kernel do its work.  A
 // pair within its cutoff now was within cutoff + skin at the build, so the
 // list (or, for an NP whose list overflowed, the cells of the build) holds
 // every pair that can interact: the forces are those of a rebuild every step.  The
@@ -43,24 +43,21 @@ __device__ __forceinline__ int cell_coord(float x, const CellGrid &g)
     return min(max(c, 0), g.dim - 1);
 }
 
-// Build kernels return at once when a gate is given and reads 0 (no rebuild).
-__device__ __forceinline__ bool gate_closed(const int *gate) { return gate && *gate == 0; }
+// The phases of the counting sort, grid-stride over the launch that runs them: as
+// kernels of their own (statistics) or one after the other between the grid
+// barriers of k_list_build.  Arrays that a phase writes and a later one reads are
+// plain pointers: a phase of the same kernel must not take them through the
+// read-only path.
 
-__global__ void k_cell_zero(int *__restrict__ count, int m, const int *__restrict__ gate)
+__device__ __forceinline__ void cell_zero(int *count, int m)
 {
-    if (gate_closed(gate))
-        return;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < m; c += gridDim.x * blockDim.x)
         count[c] = 0;
 }
 
-__global__ void k_cell_hash(CellGrid g, const float4 *__restrict__ xq,
-                            const int *__restrict__ typ, int n, int *__restrict__ key,
-                            int *__restrict__ rank, int *__restrict__ count,
-                            const int *__restrict__ gate)
+__device__ __forceinline__ void cell_hash(const CellGrid &g, const float4 *xq, const int *typ,
+                                          int n, int *key, int *rank, int *count)
 {
-    if (gate_closed(gate))
-        return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float4 p = xq[i];
         int c = (cell_coord(p.z, g) * g.dim + cell_coord(p.y, g)) * g.dim + cell_coord(p.x, g);
@@ -114,13 +111,9 @@ __device__ __forceinline__ int cta_exclusive_scan(int v, int *s_warp, int *total
     return r;
 }
 
-__global__ void __launch_bounds__(kScanThreads)
-k_scan_tiles(const int *__restrict__ count, int *__restrict__ start, int *__restrict__ tile_sum,
-             int m, const int *__restrict__ gate)
+__device__ __forceinline__ void scan_tiles(const int *count, int *start, int *tile_sum, int m,
+                                           int *s_warp)
 {
-    __shared__ int s_warp[kScanThreads / 32 + 1];
-    if (gate_closed(gate)) // uniform over the block
-        return;
     const int n_tiles = (m + kScanTile - 1) / kScanTile;
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
         const int base = t * kScanTile + threadIdx.x * kScanItems;
@@ -145,13 +138,9 @@ k_scan_tiles(const int *__restrict__ count, int *__restrict__ start, int *__rest
 }
 
 // One CTA: exclusive scan of the tile totals in place; start[m] = grand total.
-__global__ void __launch_bounds__(kScanThreads)
-k_scan_totals(int *__restrict__ tile_sum, int n_tiles, int *__restrict__ start, int m,
-              const int *__restrict__ gate)
+__device__ __forceinline__ void scan_totals(int *tile_sum, int n_tiles, int *start, int m,
+                                            int *s_warp)
 {
-    __shared__ int s_warp[kScanThreads / 32 + 1];
-    if (gate_closed(gate))
-        return;
     int carry = 0;
     for (int b0 = 0; b0 < n_tiles; b0 += kScanTile) {
         const int base = b0 + threadIdx.x * kScanItems;
@@ -176,12 +165,8 @@ k_scan_totals(int *__restrict__ tile_sum, int n_tiles, int *__restrict__ start, 
         start[m] = carry;
 }
 
-__global__ void __launch_bounds__(kScanThreads)
-k_scan_add(int *__restrict__ start, const int *__restrict__ tile_sum, int m,
-           const int *__restrict__ gate)
+__device__ __forceinline__ void scan_add(int *start, const int *tile_sum, int m)
 {
-    if (gate_closed(gate))
-        return;
     const int n_tiles = (m + kScanTile - 1) / kScanTile;
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
         const int off = tile_sum[t];
@@ -195,25 +180,21 @@ k_scan_add(int *__restrict__ start, const int *__restrict__ tile_sum, int m,
     }
 }
 
-__global__ void k_cell_scatter(const int *__restrict__ key, const int *__restrict__ rank,
-                               const int *__restrict__ start, int *__restrict__ arrived,
-                               int n, const int *__restrict__ gate)
+__device__ __forceinline__ void cell_scatter(const int *key, const int *rank, const int *start,
+                                             int *arrived, int n)
 {
-    if (gate_closed(gate))
-        return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         arrived[start[key[i]] + rank[i]] = i;
 }
 
 // Members of every cell in index order: the NP at arrival slot q goes to its
 // cell's start plus the number of members with a smaller index (O(m) per NP for
-// a cell of m members, all NPs in parallel).
-__global__ void k_cell_order(const int *__restrict__ arrived, const int *__restrict__ key,
-                             const int *__restrict__ start, int *__restrict__ sorted,
-                             int *__restrict__ pos, int n, const int *__restrict__ gate)
+// a cell of m members, all NPs in parallel), with its record (x, y, z, type as
+// int bits).
+__device__ __forceinline__ void cell_order(const int *arrived, const int *key, const int *start,
+                                           const float4 *xq, const int *typ, int *sorted, int *pos,
+                                           float4 *sxq, int n)
 {
-    if (gate_closed(gate))
-        return;
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
         const int i = arrived[q];
         const int c = key[i];
@@ -221,18 +202,57 @@ __global__ void k_cell_order(const int *__restrict__ arrived, const int *__restr
         int rank = 0;
         for (int k = b; k < e; ++k)
             rank += arrived[k] < i;
+        const float4 x = xq[i];
         sorted[b + rank] = i;
         pos[i] = b + rank;
+        sxq[b + rank] = make_float4(x.x, x.y, x.z, __int_as_float(typ[i]));
     }
 }
 
-// Cell-ordered records: (x, y, z, type as int bits).
-__global__ void k_cell_gather(const int *__restrict__ sorted, const float4 *__restrict__ xq,
-                              const int *__restrict__ typ, float4 *__restrict__ sxq, int n,
-                              const int *__restrict__ gate)
+__global__ void k_cell_zero(int *count, int m) { cell_zero(count, m); }
+
+__global__ void k_cell_hash(CellGrid g, const float4 *xq, const int *typ, int n, int *key,
+                            int *rank, int *count)
 {
-    if (gate_closed(gate))
-        return;
+    cell_hash(g, xq, typ, n, key, rank, count);
+}
+
+__global__ void __launch_bounds__(kScanThreads)
+k_scan_tiles(const int *count, int *start, int *tile_sum, int m)
+{
+    __shared__ int s_warp[kScanThreads / 32 + 1];
+    scan_tiles(count, start, tile_sum, m, s_warp);
+}
+
+__global__ void __launch_bounds__(kScanThreads)
+k_scan_totals(int *tile_sum, int n_tiles, int *start, int m)
+{
+    __shared__ int s_warp[kScanThreads / 32 + 1];
+    scan_totals(tile_sum, n_tiles, start, m, s_warp);
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_add(int *start, const int *tile_sum, int m)
+{
+    scan_add(start, tile_sum, m);
+}
+
+__global__ void k_cell_scatter(const int *key, const int *rank, const int *start, int *arrived,
+                               int n)
+{
+    cell_scatter(key, rank, start, arrived, n);
+}
+
+__global__ void k_cell_order(const int *arrived, const int *key, const int *start,
+                             const float4 *xq, const int *typ, int *sorted, int *pos, float4 *sxq,
+                             int n)
+{
+    cell_order(arrived, key, start, xq, typ, sorted, pos, sxq, n);
+}
+
+// Cell-ordered records of other positions in the order of the last build.
+__global__ void k_cell_gather(const int *__restrict__ sorted, const float4 *__restrict__ xq,
+                              const int *__restrict__ typ, float4 *__restrict__ sxq, int n)
+{
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
         const int i = sorted[p];
         const float4 q = xq[i];
@@ -272,90 +292,199 @@ __device__ __forceinline__ void load_tables(const PairTab *__restrict__ tab,
     __syncthreads();
 }
 
-// Neighbour lists (gated): for the NP at cell-order slot p (threads in the cell
-// order, so that a warp scans the same cells), the partners within
-// (rc_ab + skin) in the 27 cells, type block by type block in scan order, as
-// their cell-order slots (the partner's type is the fourth word of its
-// record), in blocks of four at nbr[nbr_index(k, p, n)] for k < cap;
-// nnbr[p] = the full count (an NP with more than cap partners is summed from
-// the cells instead).  Lists are written by slot
-// so that the per-step force kernel, which runs in the same order, reads them
-// coalesced.  Records the positions of this build in x_ref (by particle).
-__global__ void __launch_bounds__(128, 8)
-k_nbr_build(const __grid_constant__ CellGrid g, const int *__restrict__ start, const int *__restrict__ sorted,
-            const float4 *__restrict__ sxq, int n, const PairTab *__restrict__ tab,
-            const float *__restrict__ rcc2, float skin,
-            int cap, unsigned *__restrict__ nbr, int *__restrict__ nnbr,
-            float4 *__restrict__ x_ref,
-            unsigned long long *__restrict__ builds, int *__restrict__ flags,
-            const int *__restrict__ gate)
+// Arguments of the list build: the cell grid and buffers, the positions it reads,
+// the lists it writes and its grid barrier.
+struct ListBuildArgs {
+    CellGrid g;
+    CellBufs b;
+    const float4 *xq;
+    const int *typ;
+    int n, cap;
+    const PairTab *tab;
+    const float *rcc2;
+    float skin;
+    unsigned *nbr;
+    int *nnbr;
+    float4 *x_ref;
+    unsigned long long *builds;
+    int *flags;
+    const int *gate;
+    unsigned *bar; // [0] CTAs arrived, [1] CTAs done, [2] slots drawn: 0 between launches
+};
+
+// The neighbour list of the NP at cell-order slot p: the partners within (rc_ab +
+// skin) in the cells its list radii reach, type block by type block in scan
+// order, as their cell-order slots (the partner's type is the fourth word of its
+// record), in blocks of four at nbr[nbr_index(k, p, n)] for k < cap; nnbr[p] =
+// the full count (an NP with more than cap partners is summed from the cells
+// instead).  Lists are written by slot so that the per-step force kernel, which
+// runs in the same order, reads them coalesced.  Records the position of this
+// build in x_ref (by particle).
+__device__ __forceinline__ void nbr_slot(const ListBuildArgs &A, int p, unsigned *__restrict__ nbr,
+                                         const float *s_rl2, const float *s_rmax)
 {
-    if (gate_closed(gate))
-        return;
-    if (builds && blockIdx.x == 0 && threadIdx.x == 0)
-        ++*builds;
-    __shared__ float4 s_tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
-    __shared__ float s_rl2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
-    __shared__ float s_rmax[NPSIM_MAX_TYPES];
-    load_tables(tab, rcc2, skin, s_tab, s_rl2, s_rmax);
+    const CellGrid &g = A.g;
+    const int *start = A.b.start;
+    const float4 *sxq = A.b.sxq;
+    const int n = A.n, cap = A.cap;
     const int tb = g.tb > 1 ? g.tb : 1;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-        const float4 pi = sxq[p];
-        const int i = sorted[p];
-        const int ti = __float_as_int(pi.w);
-        const int row = ti * NPSIM_MAX_TYPES;
-        const float rmax = s_rmax[ti];
-        const int cx = cell_coord(pi.x, g), cy = cell_coord(pi.y, g), cz = cell_coord(pi.z, g);
-        int cnt = 0;
-        for (int t = 0; t < tb; ++t) {
-            if (tb > 1 && s_rl2[row + t] == 0.0f)
-                continue; // no term acts between these types
-            const int kofs = t * g.n_cells;
-            // the cells this type pair's list radius can reach (with tb == 1, the
-            // widest stencil of the row type); with type blocks every candidate
-            // of block t has type t, so its squared list radius is fixed
-            int w = g.ext[row + t];
-            if (tb == 1)
-                for (int b = 1; b < NPSIM_MAX_TYPES; ++b)
-                    w = max(w, (int)g.ext[row + b]);
-            const float rl2_t = tb > 1 ? s_rl2[row + t] : rmax;
-            for (int dz = -w; dz <= w; ++dz) {
-                const int z = cz + dz;
-                if (z < 0 || z >= g.dim)
+    const float4 pi = sxq[p];
+    const int i = A.b.sorted[p];
+    const int ti = __float_as_int(pi.w);
+    const int row = ti * NPSIM_MAX_TYPES;
+    const float rmax = s_rmax[ti];
+    const int cx = cell_coord(pi.x, g), cy = cell_coord(pi.y, g), cz = cell_coord(pi.z, g);
+    int cnt = 0;
+    for (int t = 0; t < tb; ++t) {
+        if (tb > 1 && s_rl2[row + t] == 0.0f)
+            continue; // no term acts between these types
+        const int kofs = t * g.n_cells;
+        // the cells this type pair's list radius can reach (with tb == 1, the
+        // widest stencil of the row type); with type blocks every candidate
+        // of block t has type t, so its squared list radius is fixed
+        int w = g.ext[row + t];
+        if (tb == 1)
+            for (int b = 1; b < NPSIM_MAX_TYPES; ++b)
+                w = max(w, (int)g.ext[row + b]);
+        const float rl2_t = tb > 1 ? s_rl2[row + t] : rmax;
+        for (int dz = -w; dz <= w; ++dz) {
+            const int z = cz + dz;
+            if (z < 0 || z >= g.dim)
+                continue;
+            for (int dy = -w; dy <= w; ++dy) {
+                const int y = cy + dy;
+                if (y < 0 || y >= g.dim)
                     continue;
-                for (int dy = -w; dy <= w; ++dy) {
-                    const int y = cy + dy;
-                    if (y < 0 || y >= g.dim)
+                const int base = kofs + (z * g.dim + y) * g.dim;
+                const int b = start[base + max(cx - w, 0)];
+                const int e = start[base + min(cx + w, g.dim - 1) + 1];
+                for (int q = b; q < e; ++q) {
+                    const float4 pj = sxq[q];
+                    const float dx = pi.x - pj.x, dy2 = pi.y - pj.y, dz2 = pi.z - pj.z;
+                    const float r2 = fmaf(dx, dx, fmaf(dy2, dy2, dz2 * dz2));
+                    if (r2 >= rl2_t || q == p)
                         continue;
-                    const int base = kofs + (z * g.dim + y) * g.dim;
-                    const int b = start[base + max(cx - w, 0)];
-                    const int e = start[base + min(cx + w, g.dim - 1) + 1];
-                    for (int q = b; q < e; ++q) {
-                        const float4 pj = sxq[q];
-                        const float dx = pi.x - pj.x, dy2 = pi.y - pj.y, dz2 = pi.z - pj.z;
-                        const float r2 = fmaf(dx, dx, fmaf(dy2, dy2, dz2 * dz2));
-                        if (r2 >= rl2_t || q == p)
-                            continue;
-                        const int tj = __float_as_int(pj.w);
-                        if (tb > 1 || r2 < s_rl2[row + tj]) {
-                            if (cnt < cap)
-                                nbr[nbr_index(cnt, p, n)] = (unsigned)q;
-                            ++cnt;
-                        }
+                    const int tj = __float_as_int(pj.w);
+                    if (tb > 1 || r2 < s_rl2[row + tj]) {
+                        if (cnt < cap)
+                            nbr[nbr_index(cnt, p, n)] = (unsigned)q;
+                        ++cnt;
                     }
                 }
             }
         }
-        // pad the last block with the far record (whole blocks of four
-        // partners); an empty list gets one block of it, so that the first
-        // block, which the force kernel reads before the count, always names
-        // valid records
-        for (int k = cnt; k < cap && (k < 4 || (k & 3)); ++k)
-            nbr[nbr_index(k, p, n)] = (unsigned)n;
-        nnbr[p] = cnt;
-        if (cnt > cap)
-            atomicOr(flags, FLAG_NBR_OVERFLOW);
-        x_ref[i] = make_float4(pi.x, pi.y, pi.z, 0.0f);
+    }
+    // pad the last block with the far record (whole blocks of four
+    // partners); an empty list gets one block of it, so that the first
+    // block, which the force kernel reads before the count, always names
+    // valid records
+    for (int k = cnt; k < cap && (k < 4 || (k & 3)); ++k)
+        nbr[nbr_index(k, p, n)] = (unsigned)n;
+    A.nnbr[p] = cnt;
+    if (cnt > cap)
+        atomicOr(A.flags, FLAG_NBR_OVERFLOW);
+    A.x_ref[i] = make_float4(pi.x, pi.y, pi.z, 0.0f);
+}
+
+// Barrier over the CTAs of a cooperative launch (all resident): phase = barriers
+// passed so far, the same in every thread.  A wait is bounded (seconds); one that
+// gives up sets FLAG_TIMEOUT and returns false in every thread of its CTA, which
+// then leaves the kernel (the host clears the counters when it reads the flag).
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, int *flags, int *s_ok)
+{
+    __syncthreads();
+    ++phase;
+    if (threadIdx.x == 0) {
+        const unsigned target = phase * gridDim.x;
+        __threadfence();
+        atomicAdd(bar, 1u);
+        int ok = 0;
+        for (int it = 0; it < (1 << 22) && !ok; ++it) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            ok = v >= target;
+            if (!ok && it > 64)
+                __nanosleep(100);
+        }
+        if (!ok)
+            atomicOr(flags, FLAG_TIMEOUT);
+        __threadfence();
+        *s_ok = ok;
+    }
+    __syncthreads();
+    return *s_ok != 0;
+}
+
+// The whole list build in one cooperative launch: counting sort of the NPs into
+// cells, then the lists.  Every step launches it, and unless the integrator has
+// raised the gate (some NP has moved more than half the skin) it returns at once:
+// as nine gated kernels (zero, hash, three scan passes, scatter, order, gather,
+// lists) the closed gate cost nine launches a step, 13 us of the 16 us of a
+// 1000-NP step and 16 of the 33 us of a 250000-NP step of the truncated model.
+// When it does build, the phases are separated by grid barriers.  Warps draw
+// batches of 32 slots for the lists from the last slot back: the cell order lists
+// the types one after another, so the largest NPs, whose lists are the longest,
+// go first.
+__global__ void __launch_bounds__(kScanThreads, 4)
+k_list_build(const __grid_constant__ ListBuildArgs A)
+{
+    __shared__ int s_warp[kScanThreads / 32 + 1];
+    __shared__ int s_ok;
+    __shared__ float4 s_tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    __shared__ float s_rl2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    __shared__ float s_rmax[NPSIM_MAX_TYPES];
+    if (A.gate && *A.gate == 0) // nobody writes it while this kernel runs
+        return;
+    const CellBufs &B = A.b;
+    const int m = (A.g.tb > 1 ? A.g.tb : 1) * A.g.n_cells; // sort keys
+    unsigned phase = 0;
+    auto barrier = [&]() { return grid_barrier(A.bar, phase, A.flags, &s_ok); };
+
+    if (A.builds && blockIdx.x == 0 && threadIdx.x == 0)
+        ++*A.builds;
+    cell_zero(B.count, m);
+    if (!barrier())
+        return;
+    cell_hash(A.g, A.xq, A.typ, A.n, B.key, B.rank, B.count);
+    if (!barrier())
+        return;
+    scan_tiles(B.count, B.start, B.tile_sum, m, s_warp);
+    if (!barrier())
+        return;
+    if (blockIdx.x == 0)
+        scan_totals(B.tile_sum, (m + kScanTile - 1) / kScanTile, B.start, m, s_warp);
+    if (!barrier())
+        return;
+    scan_add(B.start, B.tile_sum, m);
+    if (!barrier())
+        return;
+    cell_scatter(B.key, B.rank, B.start, B.arrived, A.n);
+    if (!barrier())
+        return;
+    cell_order(B.arrived, B.key, B.start, A.xq, A.typ, B.sorted, B.pos, B.sxq, A.n);
+    load_tables(A.tab, A.rcc2, A.skin, s_tab, s_rl2, s_rmax);
+    if (!barrier())
+        return;
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        unsigned first = 0;
+        if (lane == 0)
+            first = atomicAdd(A.bar + 2, 32u);
+        const int left = A.n - (int)__shfl_sync(0xffffffffu, first, 0); // slots not drawn yet
+        if (left <= 0)
+            break;
+        const int p = left - 1 - lane;
+        if (p >= 0)
+            nbr_slot(A, p, A.nbr, s_rl2, s_rmax);
+    }
+    // the last CTA out resets the counters for the next launch
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(A.bar + 1, 1u) == gridDim.x - 1) {
+            A.bar[0] = A.bar[1] = A.bar[2] = 0u;
+            __threadfence();
+        }
     }
 }
 
@@ -557,9 +686,6 @@ k_lj_nbr(const __grid_constant__ CellGrid g, const int *__restrict__ start, cons
 
 } // namespace
 
-// kernels per build: zero, hash, three scan passes, scatter, order, gather
-int cell_build_launches() { return 8; }
-
 int cell_scan_tiles(int n_cells) { return (n_cells + kScanTile - 1) / kScanTile; }
 
 namespace {
@@ -572,45 +698,76 @@ int grid_for(int n, int block)
 } // namespace
 
 cudaError_t launch_cell_build(const CellGrid &g, const float4 *xq, const int *typ, int n,
-                              CellBufs &b, const int *gate, cudaStream_t st)
+                              CellBufs &b, cudaStream_t st)
 {
-    // grid-stride kernels on at most kMaxGrid CTAs: when the gate is closed a
-    // launch costs little more than its CTAs' start
     const int B = 256;
     const int m = (g.tb > 1 ? g.tb : 1) * g.n_cells; // sort keys
     const int gn = grid_for(n, B), gc = grid_for(m, B);
-    k_cell_zero<<<gc, B, 0, st>>>(b.count, m, gate);
-    k_cell_hash<<<gn, B, 0, st>>>(g, xq, typ, n, b.key, b.rank, b.count, gate);
+    k_cell_zero<<<gc, B, 0, st>>>(b.count, m);
+    k_cell_hash<<<gn, B, 0, st>>>(g, xq, typ, n, b.key, b.rank, b.count);
     const int nt = cell_scan_tiles(m);
     const int gt = nt < kMaxGrid ? nt : kMaxGrid;
-    k_scan_tiles<<<gt, kScanThreads, 0, st>>>(b.count, b.start, b.tile_sum, m, gate);
-    k_scan_totals<<<1, kScanThreads, 0, st>>>(b.tile_sum, nt, b.start, m, gate);
-    k_scan_add<<<gt, kScanThreads, 0, st>>>(b.start, b.tile_sum, m, gate);
-    k_cell_scatter<<<gn, B, 0, st>>>(b.key, b.rank, b.start, b.arrived, n, gate);
-    k_cell_order<<<gn, B, 0, st>>>(b.arrived, b.key, b.start, b.sorted, b.pos, n, gate);
-    k_cell_gather<<<gn, B, 0, st>>>(b.sorted, xq, typ, b.sxq, n, gate);
+    k_scan_tiles<<<gt, kScanThreads, 0, st>>>(b.count, b.start, b.tile_sum, m);
+    k_scan_totals<<<1, kScanThreads, 0, st>>>(b.tile_sum, nt, b.start, m);
+    k_scan_add<<<gt, kScanThreads, 0, st>>>(b.start, b.tile_sum, m);
+    k_cell_scatter<<<gn, B, 0, st>>>(b.key, b.rank, b.start, b.arrived, n);
+    k_cell_order<<<gn, B, 0, st>>>(b.arrived, b.key, b.start, xq, typ, b.sorted, b.pos, b.sxq, n);
     return cudaGetLastError();
 }
 
 cudaError_t launch_cell_refresh(const CellBufs &b, const float4 *xq, const int *typ, int n,
                                 cudaStream_t st)
 {
-    k_cell_gather<<<grid_for(n, 256), 256, 0, st>>>(b.sorted, xq, typ, b.sxq, n, nullptr);
+    k_cell_gather<<<grid_for(n, 256), 256, 0, st>>>(b.sorted, xq, typ, b.sxq, n);
     return cudaGetLastError();
 }
 
-cudaError_t launch_nbr_build(const CellGrid &g, const CellBufs &b, int n, const PairTab *tab,
-                             const float *rcc2, float skin, const NbrList &l, int *flags,
-                             const int *gate, cudaStream_t st)
+cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4 *xq,
+                              const int *typ, int n, const PairTab *tab, const float *rcc2,
+                              float skin, const NbrList &l, int *flags, const int *gate,
+                              unsigned *bar, cudaStream_t st)
 {
-    // heavy per-NP work (every candidate of 27 cells): up to four CTAs of
-    // kMaxGrid, so that a compact droplet's build still has one NP per thread
-    const int B = 128;
-    const int gb = (n + B - 1) / B < 4 * kMaxGrid ? (n + B - 1) / B : 4 * kMaxGrid;
-    k_nbr_build<<<gb > 0 ? gb : 1, B, 0, st>>>(g, b.start, b.sorted, b.sxq, n, tab, rcc2, skin,
-                                               l.cap, l.nbr, l.nnbr, l.x_ref, l.builds, flags,
-                                               gate);
-    return cudaGetLastError();
+    ListBuildArgs A{};
+    A.g = g;
+    A.b = b;
+    A.xq = xq;
+    A.typ = typ;
+    A.n = n;
+    A.cap = l.cap;
+    A.tab = tab;
+    A.rcc2 = rcc2;
+    A.skin = skin;
+    A.nbr = l.nbr;
+    A.nnbr = l.nnbr;
+    A.x_ref = l.x_ref;
+    A.builds = l.builds;
+    A.flags = flags;
+    A.gate = gate;
+    A.bar = bar;
+    // CTAs the device holds at once
+    int dev = 0, sms = 0, occ = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_list_build, kScanThreads, 0);
+    if (e != cudaSuccess)
+        return e;
+    // a thread per NP and four keys per thread, at least a warp per 32 NPs on SMs of
+    // their own while there are few
+    const int m = (g.tb > 1 ? g.tb : 1) * g.n_cells;
+    int grid = max((n + 63) / 64, cell_scan_tiles(m));
+    grid = max(1, min(grid, occ * sms));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kScanThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeCooperative;
+    at.val.cooperative = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_list_build, A);
 }
 
 cudaError_t launch_lj_nbr(const CellGrid &g, const CellBufs &b, const float4 *xq,

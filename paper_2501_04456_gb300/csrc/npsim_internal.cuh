@@ -1465,9 +1465,9 @@ struct CellBufs {
                  // sxq[n] is a record far from every NP (type 0) that pads the
                  // neighbour lists
 };
-// Build the cell list of positions xq (gate: NULL = always, else only when *gate != 0).
+// Build the cell list of positions xq.
 cudaError_t launch_cell_build(const CellGrid &g, const float4 *xq, const int *typ, int n,
-                              CellBufs &b, const int *gate, cudaStream_t st);
+                              CellBufs &b, cudaStream_t st);
 // Rewrite the cell-ordered records from positions xq in the order of the last build.
 cudaError_t launch_cell_refresh(const CellBufs &b, const float4 *xq, const int *typ, int n,
                                 cudaStream_t st);
@@ -1492,13 +1492,16 @@ struct NbrList {
 // rcc2 (or NULL): squared cutoffs of the truncated Coulomb term per type pair
 // (8 x 8); with it the lists cover both cutoffs and the list force kernel adds
 // C q_a q_b r_ij / r^3 within the Coulomb cutoff to the LJ term.
-cudaError_t launch_nbr_build(const CellGrid &g, const CellBufs &b, int n, const PairTab *tab,
-                             const float *rcc2, float skin, const NbrList &l, int *flags,
-                             const int *gate, cudaStream_t st);
+// Cell list and neighbour lists of positions xq in one cooperative launch (gate:
+// NULL = always, else only when *gate != 0).  bar: three counters, zero between
+// launches (cleared by the host after FLAG_TIMEOUT).
+cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4 *xq,
+                              const int *typ, int n, const PairTab *tab, const float *rcc2,
+                              float skin, const NbrList &l, int *flags, const int *gate,
+                              unsigned *bar, cudaStream_t st);
 cudaError_t launch_lj_nbr(const CellGrid &g, const CellBufs &b, const float4 *xq,
                           const int *typ, int n, const PairTab *tab, const float *rcc2,
                           const NbrList &l, float *F_lj, int *gate, cudaStream_t st);
-int cell_build_launches();
 int cell_scan_tiles(int n_cells);
 
 // Stats (stats.cu)

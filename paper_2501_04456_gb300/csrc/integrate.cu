@@ -76,6 +76,15 @@ __device__ __forceinline__ void sum_row_slots(const float *__restrict__ slots,
             df_add_df(Fh[d], Fl[d], __ldcs(slot + d * sk.itile), __ldcs(slot + (3 + d) * sk.itile));
 }
 
+// Force terms a launch assembles, fixed at compile time: as run-time choices inside
+// one kernel they cost the free integrator registers and branches (4 M NPs: 71.5 us
+// a step with two of them, 78.4 with three, 63.4 without).
+enum : int {
+    SRC_LIST = 1,  // the list force record F_lj
+    SRC_PAIR = 2,  // the summed all-pairs record F_pair
+    SRC_SLOTS = 4, // the stream-K partial slots
+};
+
 // The state one particle's update reads: type, position (hi + lo), velocity
 // and the list force record.
 struct PartState {
@@ -86,10 +95,9 @@ struct PartState {
     float4 flj0, flj1;
 };
 
-template <int MODE>
+template <int MODE, int SRC>
 __device__ __forceinline__ void load_state(const IntArgs &a, int n, int i, PartState &s)
 {
-    constexpr bool ASSEMBLE = (MODE != MODE_A);
     s.ti = a.typ[i];
     s.xh = a.xq[i];
     s.lx = a.x_lo[i];
@@ -102,7 +110,7 @@ __device__ __forceinline__ void load_state(const IntArgs &a, int n, int i, PartS
     } else {
         s.v[0] = s.v[1] = s.v[2] = 0.f;
     }
-    if (ASSEMBLE && a.F_lj) {
+    if (SRC & SRC_LIST) {
         const float4 *r = reinterpret_cast<const float4 *>(a.F_lj + 8 * (size_t)i);
         s.flj0 = r[0]; // (hx, hy, hz, lx)
         s.flj1 = r[1]; // (ly, lz, -, -)
@@ -113,7 +121,7 @@ __device__ __forceinline__ void load_state(const IntArgs &a, int n, int i, PartS
 
 // Assemble particle i's force (partials, list forces, external forces) and
 // apply the mode's part of the step.
-template <int MODE>
+template <int MODE, int SRC>
 __device__ __forceinline__ void update_particle(const IntArgs &a, const StepParams &p,
                                                 const TypeCoef *s_tc, const float4 *spring,
                                                 float R0f, long long step, int i,
@@ -126,8 +134,8 @@ __device__ __forceinline__ void update_particle(const IntArgs &a, const StepPara
     float Fh[3] = {0.f, 0.f, 0.f}, Fl[3] = {0.f, 0.f, 0.f};
     if (ASSEMBLE) {
         bool any = false; // some force term is in (Fh, Fl) already
-        const int pos = a.row_pos ? a.row_pos[i] : i;
-        if (a.slots && pos >= 0) {
+        const int pos = (SRC & (SRC_PAIR | SRC_SLOTS)) && a.row_pos ? a.row_pos[i] : i;
+        if ((SRC & SRC_SLOTS) && pos >= 0) {
             any = true;
             sum_row_slots(a.slots, a.sk, pos, Fh, Fl);
             if (a.field_slots) { // the Coulomb-only kernels return sum_j q_j r_ij / r^3
@@ -136,7 +144,7 @@ __device__ __forceinline__ void update_particle(const IntArgs &a, const StepPara
                     df_mul(Fh[d], Fl[d], tc.qc);
             }
         }
-        if (a.F_pair && pos >= 0) { // summed already (k_sym_reduce)
+        if ((SRC & SRC_PAIR) && pos >= 0) { // summed already (k_sym_reduce)
             any = true;
             const float4 *r = reinterpret_cast<const float4 *>(a.F_pair + 8 * (size_t)i);
             const float4 r0 = r[0], r1 = r[1];
@@ -147,7 +155,7 @@ __device__ __forceinline__ void update_particle(const IntArgs &a, const StepPara
             Fl[1] = r1.x;
             Fl[2] = r1.y;
         }
-        if (a.F_lj) {
+        if (SRC & SRC_LIST) {
             any = true;
             df_add_df(Fh[0], Fl[0], st.flj0.x, st.flj0.w);
             df_add_df(Fh[1], Fl[1], st.flj0.y, st.flj1.x);
@@ -220,8 +228,10 @@ __device__ __forceinline__ void integrate_commit(const IntArgs &a, long long ste
 // particles: each thread has the next particle's state in flight while it
 // updates the current one, and reads the step counter and the per-type
 // coefficients once for all of its particles.  (One particle per thread, one
-// CTA per 256, measured 1.4 % slower on 8.4 M free NPs.)
-template <int MODE>
+// CTA per 256, measured 1.4 % slower on 8.4 M free NPs.)  Free NPs, 4 M of them:
+// 63.4 us a launch, 5.3 TB/s; with five CTAs per SM (48 registers) 65.0, with six
+// (40, spilling) 80.
+template <int MODE, int SRC>
 __global__ void __launch_bounds__(256, 4)
 k_integrate(IntArgs a, StepParams p)
 {
@@ -232,7 +242,7 @@ k_integrate(IntArgs a, StepParams p)
     const long long step = *a.step + a.step_ofs;
     PartState st{};
     if (i < n)
-        load_state<MODE>(a, n, i, st);
+        load_state<MODE, SRC>(a, n, i, st);
     integrate_prologue<MODE>(a, p, s_tc, step);
     const float4 *spring = a.spring + (step & 1) * NPSIM_MAX_TYPES;
     const float R0f = (float)p.R0; // bound of the escape check
@@ -240,8 +250,8 @@ k_integrate(IntArgs a, StepParams p)
         const int inext = i + stride;
         PartState nx{};
         if (inext < n)
-            load_state<MODE>(a, n, inext, nx);
-        update_particle<MODE>(a, p, s_tc, spring, R0f, step, i, st);
+            load_state<MODE, SRC>(a, n, inext, nx);
+        update_particle<MODE, SRC>(a, p, s_tc, spring, R0f, step, i, st);
         st = nx;
         i = inext;
     }
@@ -366,11 +376,12 @@ cudaError_t launch_slot_sum(const float *slots, const StreamK &sk, int n_pos, fl
     return cudaGetLastError();
 }
 
-cudaError_t launch_integrate(int mode, const IntArgs &a, const StepParams &p,
-                             cudaStream_t st)
+namespace {
+template <int MODE, int SRC>
+cudaError_t launch_int(const IntArgs &a, const StepParams &p, cudaStream_t st)
 {
     const int block = 256;
-    // resident CTAs per device (every mode has the same register bound)
+    // resident CTAs per device
     constexpr int kMaxDev = 64;
     static int resident[kMaxDev] = {};
     int dev = 0;
@@ -382,7 +393,8 @@ cudaError_t launch_integrate(int mode, const IntArgs &a, const StepParams &p,
         int sms = 0, occ = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_integrate<MODE_BA>, block, 0);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_integrate<MODE, SRC>, block,
+                                                              0);
         if (e != cudaSuccess)
             return e;
         gmax = sms * (occ > 0 ? occ : 1);
@@ -394,14 +406,34 @@ cudaError_t launch_integrate(int mode, const IntArgs &a, const StepParams &p,
         grid = gmax;
     if (grid < 1)
         grid = 1;
+    k_integrate<MODE, SRC><<<grid, block, 0, st>>>(a, p);
+    return cudaGetLastError();
+}
+
+template <int MODE>
+cudaError_t launch_src(const IntArgs &a, const StepParams &p, cudaStream_t st)
+{
+    switch ((a.F_lj ? SRC_LIST : 0) | (a.F_pair ? SRC_PAIR : 0) | (a.slots ? SRC_SLOTS : 0)) {
+    case 0: return launch_int<MODE, 0>(a, p, st);
+    case SRC_LIST: return launch_int<MODE, SRC_LIST>(a, p, st);
+    case SRC_PAIR: return launch_int<MODE, SRC_PAIR>(a, p, st);
+    case SRC_PAIR | SRC_LIST: return launch_int<MODE, SRC_PAIR | SRC_LIST>(a, p, st);
+    case SRC_SLOTS: return launch_int<MODE, SRC_SLOTS>(a, p, st);
+    case SRC_SLOTS | SRC_LIST: return launch_int<MODE, SRC_SLOTS | SRC_LIST>(a, p, st);
+    default: return cudaErrorInvalidValue; // a sum gives slots or records, not both
+    }
+}
+} // namespace
+
+cudaError_t launch_integrate(int mode, const IntArgs &a, const StepParams &p, cudaStream_t st)
+{
     switch (mode) {
-    case MODE_FORCES: k_integrate<MODE_FORCES><<<grid, block, 0, st>>>(a, p); break;
-    case MODE_A: k_integrate<MODE_A><<<grid, block, 0, st>>>(a, p); break;
-    case MODE_BA: k_integrate<MODE_BA><<<grid, block, 0, st>>>(a, p); break;
-    case MODE_B: k_integrate<MODE_B><<<grid, block, 0, st>>>(a, p); break;
+    case MODE_FORCES: return launch_src<MODE_FORCES>(a, p, st);
+    case MODE_A: return launch_int<MODE_A, 0>(a, p, st); // from the stored force
+    case MODE_BA: return launch_src<MODE_BA>(a, p, st);
+    case MODE_B: return launch_src<MODE_B>(a, p, st);
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 } // namespace npsim

@@ -151,9 +151,9 @@ __device__ __forceinline__ void mma_commit(uint32_t bar)
 
 constexpr int kGemmThreads = 256;
 
-__global__ void __launch_bounds__(kGemmThreads, 1)
-k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-            GemmArgs g, int stages)
+// Tile (bm, bn) of product z.
+__device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensorMap *tmB,
+                                          const GemmArgs &g, int stages, int bm, int bn, int z)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], done;
@@ -161,8 +161,9 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     __shared__ int s_abort, s_issued;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * kTileM;
-    const int n0 = blockIdx.y * g.n_tile;
+    const int m0 = bm * kTileM;
+    const int n0 = bn * g.n_tile;
+    const int ya = z * g.za + m0, yb = z * g.zb + n0; // operand rows
     const int nt = min(g.n_tile, g.N - n0); // multiple of 16 (N and n_tile are)
     const int nchunks = (g.K + kChunkK - 1) / kChunkK;
     const uint32_t base = smem_addr(smem);
@@ -210,8 +211,8 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 const uint32_t fb = smem_addr(&full[s]);
                 mbar_expect_tx(fb, (uint32_t)((kTileM + g.n_tile) * kc * 2));
                 for (int kg = 0; kg < kc / 8; ++kg) {
-                    tma_load_2d(sa + (uint32_t)(kg * kTileM * 16), &tmA, k0 + kg * 8, m0, fb);
-                    tma_load_2d(sb + (uint32_t)(kg * g.n_tile * 16), &tmB, k0 + kg * 8, n0, fb);
+                    tma_load_2d(sa + (uint32_t)(kg * kTileM * 16), tmA, k0 + kg * 8, ya, fb);
+                    tma_load_2d(sb + (uint32_t)(kg * g.n_tile * 16), tmB, k0 + kg * 8, yb, fb);
                 }
             }
             s_issued = c;
@@ -289,31 +290,42 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         // one warp per output row, lanes along the columns (coalesced)
         const int rows = min(kTileM, g.M - m0);
         constexpr int kWarps = kGemmThreads / 32;
+        const float *bias = g.bias ? g.bias + (size_t)z * g.zbias + n0 : nullptr;
         for (int rr = warp; rr < rows; rr += kWarps) {
-            const size_t ro = (size_t)(m0 + rr) * g.ldc + n0;
-            const float *Sr = S + rr * pitch;
+            const size_t ro = (size_t)z * g.zc + (size_t)(m0 + rr) * g.ldc + n0;
+            float *Sr = S + rr * pitch;
             for (int cc = lane; cc < nt; cc += 32) {
                 const size_t o = ro + cc;
                 float v = Sr[cc];
                 if (g.mode == GEMM_F32) {
-                    if (g.bias)
-                        v += g.bias[n0 + cc];
+                    if (bias)
+                        v += bias[cc];
                     g.Cf[o] = v;
                 } else if (g.mode == GEMM_ACT) {
-                    if (g.bias)
-                        v += g.bias[n0 + cc];
+                    if (bias)
+                        v += bias[cc];
                     if (g.Z)
                         g.Z[o] = v;
                     const float act = g.act ? silu(v) : v;
                     g.Cb[o] = __float2bfloat16_rn(act);
                     if (g.Cf)
                         g.Cf[o] = act;
+                    Sr[cc] = act;
                 } else { // GEMM_DACT: gradient through the SiLU of the previous layer
                     const float d = v * dsilu(g.Z[o]);
                     g.Cb[o] = __float2bfloat16_rn(d);
                     if (g.Cf)
                         g.Cf[o] = d;
+                    Sr[cc] = d;
                 }
+            }
+        }
+        if (g.CbT) { // the transposed copy: one warp per column, lanes along the rows
+            __syncthreads();
+            for (int cc = warp; cc < nt; cc += kWarps) {
+                __nv_bfloat16 *o = g.CbT + (size_t)z * g.zt + (size_t)(n0 + cc) * g.ldt + m0;
+                for (int rr = lane; rr < rows; rr += 32)
+                    o[rr] = __float2bfloat16_rn(S[rr * pitch + cc]);
             }
         }
     }
@@ -322,6 +334,26 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(g.tmem_cols));
+}
+
+// Products g0 (tiles 0 .. nb0 - 1 of blockIdx.x) and g1 (the rest) for the
+// networks blockIdx.y.  The training passes are chains of small products (a few
+// tiles each): what they cost is the launches, so all networks share one, and the
+// weight gradient of a layer runs beside the gradient handed to the layer below.
+__global__ void __launch_bounds__(kGemmThreads, 1)
+k_gemm_bf16(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUtensorMap tB0,
+            const __grid_constant__ CUtensorMap tA1, const __grid_constant__ CUtensorMap tB1,
+            const __grid_constant__ GemmArgs g0, const __grid_constant__ GemmArgs g1, int stages0,
+            int stages1, int nb0)
+{
+    const int x = blockIdx.x;
+    if (x < nb0) {
+        const int mb = (g0.M + kTileM - 1) / kTileM;
+        gemm_tile(&tA0, &tB0, g0, stages0, x % mb, x / mb, blockIdx.y);
+    } else {
+        const int mb = (g1.M + kTileM - 1) / kTileM;
+        gemm_tile(&tA1, &tB1, g1, stages1, (x - nb0) % mb, (x - nb0) / mb, blockIdx.y);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -353,7 +385,8 @@ struct MlpMaps {
 
 struct MlpDev {
     int NL, in_p, H, out_p, bp, tmem_cols, abuf_bytes, stage_bytes;
-    const float *bias[kMaxMlpLayers + 1]; // per layer, n_nets * N stacked
+    const float *bias[kMaxMlpLayers + 1]; // per layer, network k at k bias_stride
+    int bias_stride;
     float *y;                              // [n_nets][bp][out_p]
     int *flags;
 };
@@ -492,7 +525,7 @@ k_mlp_infer(const __grid_constant__ MlpMaps maps, MlpDev d)
             // left the previous layer, so the other parity's buffer is free
             float *bias = s_bias[l & 1];
             if (tid - 64 < N)
-                bias[tid - 64] = d.bias[l][(size_t)net * N + (tid - 64)];
+                bias[tid - 64] = d.bias[l][(size_t)net * d.bias_stride + (tid - 64)];
             mbar_arrive(smem_addr(&bias_ready));
             if (!mbar_wait_bounded(smem_addr(&bias_ready), (uint32_t)(l & 1)) ||
                 !mbar_wait_bounded(smem_addr(&acc_full), (uint32_t)(l & 1))) {
@@ -592,92 +625,117 @@ __global__ void k_transpose_bf16(const __nv_bfloat16 *__restrict__ in, int R, in
 }
 
 // Mean-squared error over rows < m_valid and the first n_valid columns of a
-// padded M x ldy output: dL/dy = 2 w_c (y - t) / (m_valid * n_valid) (FP32 and
-// BF16); loss accumulated (sum of w_c (y - t)^2 / (m_valid n_valid)).
+// padded M x ldy output: dL/dy = 2 w_c (y - t) / (m_valid * n_valid) (FP32, BF16
+// and its transpose); loss accumulated (sum of w_c (y - t)^2 / (m_valid n_valid)).
+// Network blockIdx.y.
 __global__ void k_mse_grad(const float *__restrict__ y, const float *__restrict__ t,
                            const float *__restrict__ w, int M, int m_valid, int n_valid,
                            int ldy, float *__restrict__ gf, __nv_bfloat16 *__restrict__ gb,
-                           float *__restrict__ loss)
+                           __nv_bfloat16 *__restrict__ gbT, float *__restrict__ loss)
 {
+    const size_t z = (size_t)blockIdx.y * M * ldy;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     const int r = idx / ldy, c = idx - r * ldy;
     float g = 0.f, l = 0.f;
     if (r < M) {
         if (r < m_valid && c < n_valid) {
-            const float e = y[idx] - t[(size_t)r * ldy + c];
+            const float e = y[z + idx] - t[z + (size_t)r * ldy + c];
             const float wc = w ? w[c] : 1.f;
             const float s = 1.0f / ((float)m_valid * (float)n_valid);
             g = 2.f * wc * e * s;
             l = wc * e * e * s;
         }
-        gf[idx] = g;
-        gb[idx] = __float2bfloat16_rn(g);
+        gf[z + idx] = g;
+        gb[z + idx] = __float2bfloat16_rn(g);
+        gbT[z + (size_t)c * M + r] = __float2bfloat16_rn(g);
     }
     // warp reduction of the loss, one atomic per warp
     for (int o = 16; o > 0; o >>= 1)
         l += __shfl_down_sync(0xffffffffu, l, o);
     if ((threadIdx.x & 31) == 0 && l != 0.f)
-        atomicAdd(loss, l);
+        atomicAdd(loss + blockIdx.y, l);
 }
 
-// Column sums of an M x N FP32 matrix (bias gradients), one thread per column,
-// rows in fixed order (deterministic).
-__global__ void k_colsum(const float *__restrict__ G, int M, int N, int ld, float *__restrict__ out)
+// Column sums of M x out_p FP32 matrices (bias gradients of layer blockIdx.y,
+// network blockIdx.z), one thread per column, rows in fixed order (deterministic);
+// sixteen rows are read before they are added, so that the chain of adds, not one
+// load's latency per few rows, sets the time.
+__global__ void __launch_bounds__(32)
+k_colsum(ColsumArgs a, const __grid_constant__ NetDims d, float *__restrict__ grads)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int l = blockIdx.y, N = d.out_p[l];
+    const int c = blockIdx.x * 32 + threadIdx.x;
     if (c >= N)
         return;
+    const float *G = a.G[l] + (size_t)blockIdx.z * a.M * N + c;
     float s = 0.f;
-    for (int r = 0; r < M; ++r)
-        s += G[(size_t)r * ld + c];
-    out[c] = s;
+    int r = 0;
+    for (; r + 16 <= a.M; r += 16) {
+        float w[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            w[k] = G[(size_t)(r + k) * N];
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            s += w[k];
+    }
+    for (; r < a.M; ++r)
+        s += G[(size_t)r * N];
+    grads[(size_t)blockIdx.z * d.n_params + d.off[l] + d.out_p[l] * d.in_p[l] + c] = s;
+}
+
+// Writes parameter e of network k (value w) to the BF16 copies its layer keeps.
+__device__ __forceinline__ void put_weight(const NetDims &d, int k, int e, float w)
+{
+    int l = 0;
+    while (l + 1 < d.n_layers && e >= d.off[l + 1])
+        ++l;
+    const int rows = d.out_p[l], cols = d.in_p[l], j = e - d.off[l];
+    if (j >= rows * cols)
+        return; // a bias
+    const __nv_bfloat16 b = __float2bfloat16_rn(w);
+    const size_t base = (size_t)k * rows * cols;
+    d.Wb[l][base + j] = b;
+    const int r = j / cols, c = j - r * cols;
+    d.Wt[l][base + (size_t)c * rows + r] = b;
 }
 
 // AdamW (I. Loshchilov, F. Hutter, "Decoupled weight decay regularization"):
 // m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2; w -= lr (m_hat / (sqrt(v_hat) + eps) + wd w),
-// with m_hat = m / (1 - b1^t), v_hat = v / (1 - b2^t).  Writes the BF16 copy of w,
-// and (if wt) its transpose for back-propagation.  mask (optional) keeps padded
-// entries at zero.
+// with m_hat = m / (1 - b1^t), v_hat = v / (1 - b2^t).  Writes the BF16 copy of w
+// and its transpose for back-propagation.  The mask keeps padded entries at zero;
+// biases do not decay.  Network k0 + blockIdx.y.
 __global__ void k_adamw(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
-                        float *__restrict__ v, int rows, int cols, AdamArgs a,
-                        __nv_bfloat16 *__restrict__ wb, __nv_bfloat16 *__restrict__ wt,
-                        const unsigned char *__restrict__ mask)
+                        float *__restrict__ v, const unsigned char *__restrict__ mask,
+                        const __grid_constant__ NetDims d, int k0, AdamArgs a)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * cols)
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= d.n_params)
         return;
+    const int k = k0 + blockIdx.y;
+    const size_t idx = (size_t)k * d.n_params + e;
     float wi = w[idx];
-    if (!mask || mask[idx]) {
+    const unsigned char mk = mask[e];
+    if (mk & 1) {
+        const float wd = mk & 2 ? a.wd : 0.f;
         const float gi = g[idx];
         const float mi = a.b1 * m[idx] + (1.f - a.b1) * gi;
         const float vi = a.b2 * v[idx] + (1.f - a.b2) * gi * gi;
         m[idx] = mi;
         v[idx] = vi;
         const float mh = mi / a.bc1, vh = vi / a.bc2;
-        wi -= a.lr * (mh / (sqrtf(vh) + a.eps) + a.wd * wi);
+        wi -= a.lr * (mh / (sqrtf(vh) + a.eps) + wd * wi);
         w[idx] = wi;
     }
-    if (wb) {
-        const __nv_bfloat16 b = __float2bfloat16_rn(wi);
-        wb[idx] = b;
-        if (wt) {
-            const int r = idx / cols, c = idx - r * cols;
-            wt[(size_t)c * rows + r] = b;
-        }
-    }
+    put_weight(d, k, e, wi);
 }
 
-// BF16 copy of an FP32 weight matrix (rows x cols) and its transpose.
-__global__ void k_weights_bf16(const float *__restrict__ w, int rows, int cols,
-                               __nv_bfloat16 *__restrict__ wb, __nv_bfloat16 *__restrict__ wt)
+// BF16 copies of the flat parameters of network k.
+__global__ void k_weights_bf16(const float *__restrict__ w, const __grid_constant__ NetDims d, int k)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * cols)
-        return;
-    const __nv_bfloat16 b = __float2bfloat16_rn(w[idx]);
-    wb[idx] = b;
-    const int r = idx / cols, c = idx - r * cols;
-    wt[(size_t)c * rows + r] = b;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < d.n_params)
+        put_weight(d, k, e, w[(size_t)k * d.n_params + e]);
 }
 
 __global__ void k_f32_to_bf16(const float *__restrict__ x, int n, __nv_bfloat16 *__restrict__ y)
@@ -731,11 +789,37 @@ bool encode_operand(CUtensorMap *m, const __nv_bfloat16 *ptr, int rows, int K, i
 
 int gemm_smem_bytes(int n_tile) { return dyn_smem_bytes(n_tile, kMaxStages); }
 
-cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t st)
+namespace {
+bool gemm_ok(const GemmArgs &g)
 {
-    if (g.M <= 0 || g.N <= 0 || g.K <= 0 || (g.N % 16) || (g.K % 16) || (g.n_tile % 16) ||
-        g.n_tile < 16 || g.n_tile > kMaxTileN || (g.lda % 8) || (g.ldb % 8) || g.lda < g.K ||
-        g.ldb < g.K || ((uintptr_t)g.A % 16) || ((uintptr_t)g.B % 16))
+    return !(g.M <= 0 || g.N <= 0 || g.K <= 0 || (g.N % 16) || (g.K % 16) || (g.n_tile % 16) ||
+             g.n_tile < 16 || g.n_tile > kMaxTileN || (g.lda % 8) || (g.ldb % 8) || g.lda < g.K ||
+             g.ldb < g.K || ((uintptr_t)g.A % 16) || ((uintptr_t)g.B % 16) || g.nz < 1);
+}
+
+int gemm_stages(const GemmArgs &g)
+{
+    const int nchunks = (g.K + kChunkK - 1) / kChunkK;
+    int stages = kStageBudget / stage_bytes(g.n_tile);
+    stages = stages < kMaxStages ? stages : kMaxStages;
+    return stages < nchunks ? stages : nchunks;
+}
+
+int gemm_tiles(const GemmArgs &g)
+{
+    return ((g.M + kTileM - 1) / kTileM) * ((g.N + g.n_tile - 1) / g.n_tile);
+}
+
+bool gemm_maps(const GemmArgs &g, CUtensorMap *ta, CUtensorMap *tb)
+{
+    return encode_operand(ta, g.A, (g.nz - 1) * g.za + g.M, g.K, g.lda, kTileM) &&
+           encode_operand(tb, g.B, (g.nz - 1) * g.zb + g.N, g.K, g.ldb, g.n_tile);
+}
+} // namespace
+
+cudaError_t launch_gemm(const GemmArgs &g0, const GemmArgs *g1, cudaStream_t st)
+{
+    if (!gemm_ok(g0) || (g1 && (!gemm_ok(*g1) || g1->nz != g0.nz)))
         return cudaErrorInvalidValue;
     static bool attr_done = false;
     if (!attr_done) {
@@ -745,16 +829,16 @@ cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t st)
             return e;
         attr_done = true;
     }
-    CUtensorMap ta, tb;
-    if (!encode_operand(&ta, g.A, g.M, g.K, g.lda, kTileM) ||
-        !encode_operand(&tb, g.B, g.N, g.K, g.ldb, g.n_tile))
+    CUtensorMap ta0, tb0, ta1{}, tb1{};
+    if (!gemm_maps(g0, &ta0, &tb0) || (g1 && !gemm_maps(*g1, &ta1, &tb1)))
         return cudaErrorInvalidValue;
-    const int nchunks = (g.K + kChunkK - 1) / kChunkK;
-    int stages = kStageBudget / stage_bytes(g.n_tile);
-    stages = stages < kMaxStages ? stages : kMaxStages;
-    stages = stages < nchunks ? stages : nchunks;
-    dim3 grid((g.M + kTileM - 1) / kTileM, (g.N + g.n_tile - 1) / g.n_tile);
-    k_gemm_bf16<<<grid, kGemmThreads, dyn_smem_bytes(g.n_tile, stages), st>>>(ta, tb, g, stages);
+    const int s0 = gemm_stages(g0), s1 = g1 ? gemm_stages(*g1) : 0;
+    const int nb0 = gemm_tiles(g0), nb1 = g1 ? gemm_tiles(*g1) : 0;
+    int smem = dyn_smem_bytes(g0.n_tile, s0);
+    if (g1 && dyn_smem_bytes(g1->n_tile, s1) > smem)
+        smem = dyn_smem_bytes(g1->n_tile, s1);
+    k_gemm_bf16<<<dim3(nb0 + nb1, g0.nz), kGemmThreads, smem, st>>>(
+        ta0, tb0, ta1, tb1, g0, g1 ? *g1 : g0, s0, s1, nb0);
     return cudaGetLastError();
 }
 
@@ -794,6 +878,7 @@ cudaError_t launch_mlp_infer(const MlpInferArgs &a, cudaStream_t st)
             !encode_operand(&maps.w[l], a.W[l], a.n_nets * N, K, K, N))
             return cudaErrorInvalidValue;
         d.bias[l] = a.b[l];
+        d.bias_stride = a.b_stride;
     }
     const int smem = d.abuf_bytes + kInferStages * d.stage_bytes;
     static bool attr_done = false;
@@ -819,37 +904,35 @@ cudaError_t launch_transpose_bf16(const void *in, int R, int C, int ldi, void *o
 }
 
 cudaError_t launch_mse_grad(const float *y, const float *t, const float *w, int M, int m_valid,
-                            int n_valid, int ldy, float *gf, void *gb, float *loss,
-                            cudaStream_t st)
+                            int n_valid, int ldy, int nz, float *gf, void *gb, void *gbT,
+                            float *loss, cudaStream_t st)
 {
     const int n = M * ldy;
-    k_mse_grad<<<(n + 255) / 256, 256, 0, st>>>(y, t, w, M, m_valid, n_valid, ldy, gf,
-                                                (__nv_bfloat16 *)gb, loss);
+    k_mse_grad<<<dim3((n + 255) / 256, nz), 256, 0, st>>>(y, t, w, M, m_valid, n_valid, ldy, gf,
+                                                          (__nv_bfloat16 *)gb,
+                                                          (__nv_bfloat16 *)gbT, loss);
     return cudaGetLastError();
 }
 
-cudaError_t launch_colsum(const float *G, int M, int N, int ld, float *out, cudaStream_t st)
+cudaError_t launch_colsum(const ColsumArgs &c, const NetDims &d, float *grads, cudaStream_t st)
 {
-    k_colsum<<<(N + 127) / 128, 128, 0, st>>>(G, M, N, ld, out);
+    int w = 0;
+    for (int l = 0; l < d.n_layers; ++l)
+        w = d.out_p[l] > w ? d.out_p[l] : w;
+    k_colsum<<<dim3((w + 31) / 32, d.n_layers, c.nz), 32, 0, st>>>(c, d, grads);
     return cudaGetLastError();
 }
 
-cudaError_t launch_adamw(float *w, const float *g, float *m, float *v, int rows, int cols,
-                         const AdamArgs &a, void *wb, void *wt, const unsigned char *mask,
-                         cudaStream_t st)
+cudaError_t launch_adamw(float *w, const float *g, float *m, float *v, const unsigned char *mask,
+                         const NetDims &d, int k0, int nz, const AdamArgs &a, cudaStream_t st)
 {
-    const int n = rows * cols;
-    k_adamw<<<(n + 255) / 256, 256, 0, st>>>(w, g, m, v, rows, cols, a, (__nv_bfloat16 *)wb,
-                                             (__nv_bfloat16 *)wt, mask);
+    k_adamw<<<dim3((d.n_params + 255) / 256, nz), 256, 0, st>>>(w, g, m, v, mask, d, k0, a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_weights_bf16(const float *w, int rows, int cols, void *wb, void *wt,
-                                cudaStream_t st)
+cudaError_t launch_weights_bf16(const float *w, const NetDims &d, int k, cudaStream_t st)
 {
-    const int n = rows * cols;
-    k_weights_bf16<<<(n + 255) / 256, 256, 0, st>>>(w, rows, cols, (__nv_bfloat16 *)wb,
-                                                    (__nv_bfloat16 *)wt);
+    k_weights_bf16<<<(d.n_params + 255) / 256, 256, 0, st>>>(w, d, k);
     return cudaGetLastError();
 }
 

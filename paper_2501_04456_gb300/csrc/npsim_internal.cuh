@@ -1413,16 +1413,33 @@ struct GemmArgs {
     float *Cf;              // FP32 output (M x N, ldc) or NULL
     __nv_bfloat16 *Cb;      // BF16 output or NULL
     float *Z;               // pre-activation (GEMM_ACT writes, GEMM_DACT reads), ldc
+    __nv_bfloat16 *CbT;     // transposed copy of Cb (N x M, ldt) or NULL
+    int ldt;
     int *flags;             // FLAG_TIMEOUT on a bounded wait that expired
     long long wait_cycles;  // bound of the main loop's waits in SM cycles (0: 2^32)
+    // nz products of one shape (networks), product z's operands z za / z zb rows
+    // further, its outputs z zc (Cf, Cb, Z), z zt (CbT), z zbias elements further
+    int nz, za, zb;
+    size_t zc, zt, zbias;
 };
 
 struct AdamArgs {
     float lr, b1, b2, eps, wd, bc1, bc2; // bc = 1 - beta^t
 };
 
+// The parameters of one network as a flat vector: layer l's weights (out_p x in_p)
+// at off[l], its biases right behind; Wb / Wt: the BF16 copy and its transpose of
+// all networks, network k at k out_p in_p.
+constexpr int kMaxLayers = 9; // 8 hidden and the output layer
+struct NetDims {
+    int n_layers, n_params;
+    int off[kMaxLayers], out_p[kMaxLayers], in_p[kMaxLayers];
+    __nv_bfloat16 *Wb[kMaxLayers], *Wt[kMaxLayers];
+};
+
 int gemm_smem_bytes(int n_tile);
-cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t st);
+// One product (g1 NULL), or two independent ones of the same nz in one launch.
+cudaError_t launch_gemm(const GemmArgs &g0, const GemmArgs *g1, cudaStream_t st);
 
 // Fused inference of a whole MLP (mlp.cu): every layer of every network in one
 // launch, activations kept in shared memory, one CTA per (128 rows, network).
@@ -1432,7 +1449,8 @@ constexpr int kMaxMlpLayers = 6; // hidden layers the fused kernel takes
 struct MlpInferArgs {
     const __nv_bfloat16 *X;                    // bp x in_p
     const __nv_bfloat16 *W[kMaxMlpLayers + 1]; // layer l: n_nets * N_l x K_l
-    const float *b[kMaxMlpLayers + 1];         // layer l: n_nets * N_l
+    const float *b[kMaxMlpLayers + 1];         // layer l of network 0; network k at k b_stride
+    int b_stride;
     int NL, in_p, H, out_p, bp, n_nets;
     float *y;
     int *flags;
@@ -1441,16 +1459,25 @@ bool mlp_infer_supported(int NL, int in_p, int H, int out_p);
 cudaError_t launch_mlp_infer(const MlpInferArgs &a, cudaStream_t st);
 cudaError_t launch_transpose_bf16(const void *in, int R, int C, int ldi, void *out, int ldo,
                                   cudaStream_t st);
+// Mean-squared error and its gradient for nz networks, y and gf / gb / gbT (the
+// transposed BF16 gradient, ldy x M) of network z M ldy elements further, loss[z].
 cudaError_t launch_mse_grad(const float *y, const float *t, const float *w, int M, int m_valid,
-                            int n_valid, int ldy, float *gf, void *gb, float *loss,
-                            cudaStream_t st);
-cudaError_t launch_colsum(const float *G, int M, int N, int ld, float *out, cudaStream_t st);
-cudaError_t launch_adamw(float *w, const float *g, float *m, float *v, int rows, int cols,
-                         const AdamArgs &a, void *wb, void *wt, const unsigned char *mask,
-                         cudaStream_t st);
+                            int n_valid, int ldy, int nz, float *gf, void *gb, void *gbT,
+                            float *loss, cudaStream_t st);
+// Bias gradients of every layer: column sums over the M rows of G[l] (width
+// out_p[l], network z M out_p[l] further) into the flat gradients.
+struct ColsumArgs {
+    const float *G[kMaxLayers];
+    int M, nz;
+};
+cudaError_t launch_colsum(const ColsumArgs &c, const NetDims &d, float *grads, cudaStream_t st);
+// AdamW on the flat parameters of nz networks from network k0 on; mask bit 0: a
+// parameter (padding keeps 0), bit 1: decays.
+cudaError_t launch_adamw(float *w, const float *g, float *m, float *v, const unsigned char *mask,
+                         const NetDims &d, int k0, int nz, const AdamArgs &a, cudaStream_t st);
+// BF16 copies of the flat parameters of network k.
+cudaError_t launch_weights_bf16(const float *w, const NetDims &d, int k, cudaStream_t st);
 cudaError_t launch_f32_to_bf16(const float *x, int n, void *y, cudaStream_t st);
-cudaError_t launch_weights_bf16(const float *w, int rows, int cols, void *wb, void *wt,
-                                cudaStream_t st);
 
 // Cell list (celllist.cu).  The sort key of NP i is its cell (tb == 1) or
 // type * n_cells + cell (tb = the number of types): the cell order lists all NPs

@@ -37,15 +37,6 @@ int pow2_at_least(int x)
     return p;
 }
 
-struct Layer {
-    int out = 0, in = 0, out_p = 0, in_p = 0;
-    float *W = nullptr, *b = nullptr;          // FP32 master weights
-    __nv_bfloat16 *Wb = nullptr, *Wt = nullptr; // BF16 copy and its transpose
-    float *mW = nullptr, *vW = nullptr, *mb = nullptr, *vb = nullptr;
-    float *gW = nullptr, *gb = nullptr;
-    unsigned char *mask = nullptr, *bmask = nullptr;
-};
-
 template <class T> cudaError_t dmalloc(T **p, size_t n)
 {
     *p = nullptr;
@@ -63,79 +54,61 @@ template <class T> void dfree2(T *&p)
 
 struct npsim_surr {
     int n_in = 0, n_in_p = 0, H = 0, NL = 0, n_out = 0, n_out_p = 0, n_nets = 0;
-    int bcap = 0; // batch capacity (multiple of 128)
-    std::vector<std::vector<Layer>> nets;
-    // per layer, the BF16 weights and FP32 biases of all networks in one block
-    // (network k at rows k out_p): Layer::Wb and Layer::b point into these
-    std::vector<__nv_bfloat16 *> Wb_stack;
-    std::vector<float *> b_stack;
+    // parameters of all networks as flat vectors [n_nets][n_params] (the layout of
+    // npsim_surr_get_params): FP32 master weights, gradients, AdamW moments; BF16
+    // copies and transposes per layer, all networks in one block (D.Wb, D.Wt)
+    NetDims D{};
+    float *W = nullptr, *G = nullptr, *mom = nullptr, *var = nullptr;
+    unsigned char *mask = nullptr; // [n_params] bit 0: a parameter (not padding), bit 1: decays
     std::vector<float> xm, xs, ym, ys; // normalisation
     cudaStream_t st = nullptr;
-    // activations and gradients for one batch
-    std::vector<__nv_bfloat16 *> a; // NL + 1 (a[0] = input)
-    std::vector<float *> z;         // NL pre-activations
-    float *y = nullptr, *yt = nullptr, *dyf = nullptr;
-    __nv_bfloat16 *dyb = nullptr;
-    __nv_bfloat16 *dz[2] = {nullptr, nullptr};
-    float *dzf[2] = {nullptr, nullptr};
-    __nv_bfloat16 *tA = nullptr, *tB = nullptr; // transposes
-    float *loss = nullptr, *outw = nullptr;
-    float *xin = nullptr;          // normalised FP32 inputs of a batch (staging)
+    // prediction of a batch of up to bcap rows
+    int bcap = 0;
+    float *xin = nullptr;          // normalised FP32 inputs (staging)
+    __nv_bfloat16 *xb = nullptr;   // the same in BF16
     float *y_all = nullptr;        // outputs of every network [n_nets][bcap][n_out_p]
     float *ystat = nullptr;        // ensemble mean and spread [2][bcap][n_out]
+    // activations and gradients of the layer-by-layer passes, networks stacked:
+    // network k of a pass at rows k bp; rcap rows in all.  T: transposed copies
+    // ([width][bp] per network), the operands of the weight gradients
+    size_t rcap = 0, tcap = 0;
+    std::vector<__nv_bfloat16 *> a, aT; // NL + 1 (a[0] = input)
+    std::vector<float *> z;             // NL pre-activations
+    float *y = nullptr, *yt = nullptr, *dyf = nullptr;
+    __nv_bfloat16 *dyb = nullptr, *dyT = nullptr;
+    __nv_bfloat16 *dz[2] = {nullptr, nullptr}, *dzT[2] = {nullptr, nullptr};
+    std::vector<float *> dzf;           // NL (the column sums read them at the end)
+    float *loss = nullptr;              // [n_nets]
+    float *outw = nullptr;
     float *d_ym = nullptr, *d_ys = nullptr; // output de-normalisation (n_out)
     int *flags = nullptr;
     long long adam_t = 0;
-    // dataset on the device
+    // dataset on the device, its staging and the shuffled orders (kept between calls)
+    size_t ds_cap = 0;
     __nv_bfloat16 *dsx = nullptr;
-    float *dsy = nullptr;
-    int ds_n = 0;
+    float *dsy = nullptr, *ds_tmp = nullptr;
+    int *d_idx = nullptr;
 
     ~npsim_surr()
     {
-        for (auto &net : nets)
-            for (auto &L : net) {
-                L.b = nullptr; // inside b_stack / Wb_stack
-                L.Wb = nullptr;
-                dfree2(L.W);
-                dfree2(L.Wt);
-                dfree2(L.mW);
-                dfree2(L.vW);
-                dfree2(L.mb);
-                dfree2(L.vb);
-                dfree2(L.gW);
-                dfree2(L.gb);
-                dfree2(L.mask);
-                dfree2(L.bmask);
-            }
-        for (auto *p : a)
-            dfree2(p);
-        for (auto *p : z)
-            dfree2(p);
-        dfree2(y);
-        dfree2(yt);
-        dfree2(dyf);
-        dfree2(dyb);
-        for (int k = 0; k < 2; ++k) {
-            dfree2(dz[k]);
-            dfree2(dzf[k]);
+        for (int l = 0; l < kMaxLayers; ++l) {
+            dfree2(D.Wb[l]);
+            dfree2(D.Wt[l]);
         }
-        dfree2(tA);
-        dfree2(tB);
-        dfree2(loss);
-        dfree2(outw);
-        dfree2(xin);
-        dfree2(y_all);
-        dfree2(ystat);
-        dfree2(d_ym);
-        dfree2(d_ys);
+        for (float **p : {&W, &G, &mom, &var, &xin, &y_all, &ystat, &y, &yt, &dyf, &loss, &outw,
+                          &d_ym, &d_ys, &dsy, &ds_tmp})
+            dfree2(*p);
+        for (__nv_bfloat16 **p : {&xb, &dyb, &dyT, &dz[0], &dz[1], &dzT[0], &dzT[1], &dsx})
+            dfree2(*p);
+        for (auto *v : {&a, &aT})
+            for (auto *&p : *v)
+                dfree2(p);
+        for (auto *v : {&z, &dzf})
+            for (auto *&p : *v)
+                dfree2(p);
+        dfree2(mask);
+        dfree2(d_idx);
         dfree2(flags);
-        dfree2(dsx);
-        dfree2(dsy);
-        for (auto *p : Wb_stack)
-            dfree2(p);
-        for (auto *p : b_stack)
-            dfree2(p);
         if (st)
             cudaStreamDestroy(st);
     }
@@ -153,15 +126,18 @@ namespace {
                                 __FILE__, __LINE__);                                    \
     } while (0)
 
+// Rows (networks x minibatch) of a training pass.
+constexpr int kTrainRows = 65536;
+
 int n_tile_for(int N) { return (N % 64 == 0) ? 64 : N; }
 
 // Bound of the GEMM kernel's main-loop waits set by npsim_test_wait_cycles
 // (0: the kernel's default).
 std::atomic<long long> g_wait_cycles{0};
 
-cudaError_t gemm(npsim_surr *s, int mode, const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B,
-                 int ldb, int M, int N, int K, const float *bias, float *Cf, __nv_bfloat16 *Cb,
-                 int ldc, float *Z, int act)
+// A product of nk networks (operand rows za / zb, outputs zc elements apart).
+GemmArgs gemm(npsim_surr *s, int mode, const __nv_bfloat16 *A, int lda, int za,
+              const __nv_bfloat16 *B, int ldb, int zb, int M, int N, int K, int ldc, size_t zc, int nk)
 {
     GemmArgs g{};
     g.A = A;
@@ -175,115 +151,162 @@ cudaError_t gemm(npsim_surr *s, int mode, const __nv_bfloat16 *A, int lda, const
     g.n_tile = n_tile_for(N);
     g.tmem_cols = pow2_at_least(g.n_tile);
     g.mode = mode;
-    g.act = act;
-    g.bias = bias;
-    g.Cf = Cf;
-    g.Cb = Cb;
-    g.Z = Z;
     g.flags = s->flags;
     g.wait_cycles = g_wait_cycles.load();
-    return launch_gemm(g, s->st);
+    g.nz = nk;
+    g.za = za;
+    g.zb = zb;
+    g.zc = zc;
+    return g;
 }
 
-int alloc_batch(npsim_surr *s, int bcap)
+// Buffers of a prediction of bp rows.
+int alloc_batch(npsim_surr *s, int bp)
 {
-    if (bcap <= s->bcap)
+    if (bp <= s->bcap)
         return NPSIM_OK;
-    for (auto *&p : s->a)
-        dfree2(p);
-    for (auto *&p : s->z)
-        dfree2(p);
-    dfree2(s->y);
-    dfree2(s->yt);
-    dfree2(s->dyf);
-    dfree2(s->dyb);
-    for (int k = 0; k < 2; ++k) {
-        dfree2(s->dz[k]);
-        dfree2(s->dzf[k]);
-    }
-    dfree2(s->tA);
-    dfree2(s->tB);
+    s->bcap = 0;
     dfree2(s->xin);
+    dfree2(s->xb);
     dfree2(s->y_all);
     dfree2(s->ystat);
-    s->a.assign(s->NL + 1, nullptr);
-    s->z.assign(s->NL, nullptr);
-    SR_CUDA(dmalloc(&s->a[0], (size_t)bcap * s->n_in_p));
-    for (int l = 1; l <= s->NL; ++l)
-        SR_CUDA(dmalloc(&s->a[l], (size_t)bcap * s->H));
-    for (int l = 0; l < s->NL; ++l)
-        SR_CUDA(dmalloc(&s->z[l], (size_t)bcap * s->H));
-    SR_CUDA(dmalloc(&s->y, (size_t)bcap * s->n_out_p));
-    SR_CUDA(dmalloc(&s->yt, (size_t)bcap * s->n_out_p));
-    SR_CUDA(dmalloc(&s->dyf, (size_t)bcap * s->n_out_p));
-    SR_CUDA(dmalloc(&s->dyb, (size_t)bcap * s->n_out_p));
-    for (int k = 0; k < 2; ++k) {
-        SR_CUDA(dmalloc(&s->dz[k], (size_t)bcap * s->H));
-        SR_CUDA(dmalloc(&s->dzf[k], (size_t)bcap * s->H));
-    }
-    const int wmax = std::max(s->H, s->n_out_p);
-    SR_CUDA(dmalloc(&s->tA, (size_t)bcap * wmax));
-    SR_CUDA(dmalloc(&s->tB, (size_t)bcap * wmax));
-    SR_CUDA(dmalloc(&s->xin, (size_t)bcap * s->n_in_p));
-    SR_CUDA(dmalloc(&s->y_all, (size_t)s->n_nets * bcap * s->n_out_p));
-    SR_CUDA(dmalloc(&s->ystat, (size_t)2 * bcap * s->n_out));
-    s->bcap = bcap;
+    SR_CUDA(dmalloc(&s->xin, (size_t)bp * s->n_in_p));
+    SR_CUDA(dmalloc(&s->xb, (size_t)bp * s->n_in_p));
+    SR_CUDA(dmalloc(&s->y_all, (size_t)s->n_nets * bp * s->n_out_p));
+    SR_CUDA(dmalloc(&s->ystat, (size_t)2 * bp * s->n_out));
+    s->bcap = bp;
     return NPSIM_OK;
 }
 
-// Forward pass of network k on the batch in a[0] (bp rows, a multiple of 128):
-// hidden layers write z (FP32) and a (BF16); the output layer writes y_out
-// (FP32; s->y when NULL).
-int forward(npsim_surr *s, int k, int bp, float *y_out = nullptr)
+// Buffers of a layer-by-layer pass of `rows` rows (networks x batch), and with
+// `train` those of the backward pass.
+int alloc_rows(npsim_surr *s, size_t rows, bool train)
 {
-    auto &net = s->nets[k];
-    for (int l = 0; l < s->NL; ++l) {
-        Layer &L = net[l];
-        SR_CUDA(gemm(s, GEMM_ACT, s->a[l], L.in_p, L.Wb, L.in_p, bp, L.out_p, L.in_p, L.b,
-                     nullptr, s->a[l + 1], L.out_p, s->z[l], 1));
+    if (rows > s->rcap) {
+        s->rcap = 0;
+        s->a.resize(s->NL + 1, nullptr);
+        s->z.resize(s->NL, nullptr);
+        for (auto *&p : s->a)
+            dfree2(p);
+        for (auto *&p : s->z)
+            dfree2(p);
+        dfree2(s->y);
+        SR_CUDA(dmalloc(&s->a[0], rows * s->n_in_p));
+        for (int l = 0; l < s->NL; ++l) {
+            SR_CUDA(dmalloc(&s->a[l + 1], rows * s->H));
+            SR_CUDA(dmalloc(&s->z[l], rows * s->H));
+        }
+        SR_CUDA(dmalloc(&s->y, rows * s->n_out_p));
+        s->rcap = rows;
     }
-    Layer &O = net[s->NL];
-    SR_CUDA(gemm(s, GEMM_F32, s->a[s->NL], O.in_p, O.Wb, O.in_p, bp, O.out_p, O.in_p, O.b,
-                 y_out ? y_out : s->y, nullptr, O.out_p, nullptr, 0));
+    if (train && rows > s->tcap) {
+        s->tcap = 0;
+        s->aT.resize(s->NL + 1, nullptr);
+        s->dzf.resize(s->NL, nullptr);
+        for (auto *&p : s->aT)
+            dfree2(p);
+        for (auto *&p : s->dzf)
+            dfree2(p);
+        for (float **p : {&s->yt, &s->dyf})
+            dfree2(*p);
+        for (__nv_bfloat16 **p : {&s->dyb, &s->dyT, &s->dz[0], &s->dz[1], &s->dzT[0], &s->dzT[1]})
+            dfree2(*p);
+        SR_CUDA(dmalloc(&s->aT[0], rows * s->n_in_p));
+        for (int l = 0; l < s->NL; ++l) {
+            SR_CUDA(dmalloc(&s->aT[l + 1], rows * s->H));
+            SR_CUDA(dmalloc(&s->dzf[l], rows * s->H));
+        }
+        SR_CUDA(dmalloc(&s->yt, rows * s->n_out_p));
+        SR_CUDA(dmalloc(&s->dyf, rows * s->n_out_p));
+        SR_CUDA(dmalloc(&s->dyb, rows * s->n_out_p));
+        SR_CUDA(dmalloc(&s->dyT, rows * s->n_out_p));
+        for (int k = 0; k < 2; ++k) {
+            SR_CUDA(dmalloc(&s->dz[k], rows * s->H));
+            SR_CUDA(dmalloc(&s->dzT[k], rows * s->H));
+        }
+        s->tcap = rows;
+    }
     return NPSIM_OK;
 }
 
-// Back-propagation of the mean-squared error on rows < m_valid of the batch:
-// weight gradients gW = dZ^T A_prev (via transposes), bias gradients = column
-// sums of dZ, dZ_prev = (dZ W) * SiLU'(Z_prev).
-int backward(npsim_surr *s, int k, int bp, int m_valid)
+// Forward pass of networks k0 .. k0 + nk - 1 on bp rows each (a multiple of 128),
+// the inputs at x (network k's xz rows further): hidden layers write z (FP32) and a
+// (BF16; with `train` its transpose too), the output layer writes y_out (FP32).
+int forward(npsim_surr *s, int k0, int nk, int bp, const __nv_bfloat16 *x, int xz, float *y_out,
+            bool train)
 {
-    auto &net = s->nets[k];
-    SR_CUDA(cudaMemsetAsync(s->loss, 0, sizeof(float), s->st));
-    SR_CUDA(launch_mse_grad(s->y, s->yt, s->outw, bp, m_valid, s->n_out, s->n_out_p, s->dyf,
-                            s->dyb, s->loss, s->st));
-    // current gradient wrt the pre-activation of layer l: (bf16, fp32, width)
-    const __nv_bfloat16 *g_b = s->dyb;
-    const float *g_f = s->dyf;
-    int g_w = s->n_out_p;
+    const NetDims &D = s->D;
+    for (int l = 0; l <= s->NL; ++l) {
+        const int N = D.out_p[l], K = D.in_p[l];
+        const bool out = l == s->NL;
+        GemmArgs g = gemm(s, out ? GEMM_F32 : GEMM_ACT, l == 0 ? x : s->a[l], K, l == 0 ? xz : bp,
+                          D.Wb[l] + (size_t)k0 * N * K, K, N, bp, N, K, N, (size_t)bp * N, nk);
+        g.bias = s->W + (size_t)k0 * D.n_params + D.off[l] + N * K;
+        g.zbias = (size_t)D.n_params;
+        if (out) {
+            g.Cf = y_out;
+        } else {
+            g.act = 1;
+            g.Z = s->z[l];
+            g.Cb = s->a[l + 1];
+            if (train) {
+                g.CbT = s->aT[l + 1];
+                g.ldt = bp;
+                g.zt = (size_t)bp * N;
+            }
+        }
+        SR_CUDA(launch_gemm(g, nullptr, s->st));
+    }
+    return NPSIM_OK;
+}
+
+// Back-propagation of the mean-squared error on rows < m_valid of the batch for
+// networks k0 .. k0 + nk - 1: weight gradients gW = dZ^T A_prev (from the
+// transposed copies the producing kernels wrote), dZ_prev = (dZ W) * SiLU'(Z_prev)
+// beside it in the same launch, bias gradients = column sums of every dZ at the
+// end.  loss[0 .. nk) must be zero.
+int backward(npsim_surr *s, int k0, int nk, int bp, int m_valid)
+{
+    const NetDims &D = s->D;
+    SR_CUDA(launch_mse_grad(s->y, s->yt, s->outw, bp, m_valid, s->n_out, s->n_out_p, nk, s->dyf,
+                            s->dyb, s->dyT, s->loss, s->st));
+    // current gradient wrt the pre-activation of layer l, and its transpose
+    const __nv_bfloat16 *d = s->dyb, *dT = s->dyT;
+    ColsumArgs cs{};
+    cs.M = bp;
+    cs.nz = nk;
+    cs.G[s->NL] = s->dyf;
     int ping = 0;
     for (int l = s->NL; l >= 0; --l) {
-        Layer &L = net[l];
-        // gW = dZ^T (out_p x bp) * A_prev^T^T: A = dZ^T (out_p x bp), B = A_prev^T (in_p x bp)
-        SR_CUDA(launch_transpose_bf16(g_b, bp, g_w, g_w, s->tA, bp, s->st));
-        SR_CUDA(launch_transpose_bf16(s->a[l], bp, L.in_p, L.in_p, s->tB, bp, s->st));
-        SR_CUDA(gemm(s, GEMM_F32, s->tA, bp, s->tB, bp, L.out_p, L.in_p, bp, nullptr, L.gW,
-                     nullptr, L.in_p, nullptr, 0));
-        SR_CUDA(launch_colsum(g_f, bp, L.out_p, g_w, L.gb, s->st));
-        if (l > 0) {
-            // dZ_prev = (dZ W) * SiLU'(Z_prev): A = dZ (bp x out_p), B = W^T (in_p x out_p)
-            SR_CUDA(gemm(s, GEMM_DACT, g_b, g_w, L.Wt, L.out_p, bp, L.in_p, L.out_p, nullptr,
-                         s->dzf[ping], s->dz[ping], L.in_p, s->z[l - 1], 0));
-            g_b = s->dz[ping];
-            g_f = s->dzf[ping];
-            g_w = L.in_p;
-            ping ^= 1;
+        const int N = D.out_p[l], K = D.in_p[l];
+        // gW (N x K) = dZ^T (N x bp) * (A_prev^T (K x bp))^T
+        GemmArgs gw = gemm(s, GEMM_F32, dT, bp, N, s->aT[l], bp, K, N, K, bp, K,
+                           (size_t)D.n_params, nk);
+        gw.Cf = s->G + (size_t)k0 * D.n_params + D.off[l];
+        if (l == 0) {
+            SR_CUDA(launch_gemm(gw, nullptr, s->st));
+            break;
         }
+        // dZ_prev (bp x K) = dZ (bp x N) * (W^T (K x N))^T
+        GemmArgs gx = gemm(s, GEMM_DACT, d, N, bp, D.Wt[l] + (size_t)k0 * N * K, N, K, bp, K, N, K,
+                           (size_t)bp * K, nk);
+        gx.Z = s->z[l - 1];
+        gx.Cf = s->dzf[l - 1];
+        gx.Cb = s->dz[ping];
+        gx.CbT = s->dzT[ping];
+        gx.ldt = bp;
+        gx.zt = (size_t)bp * K;
+        SR_CUDA(launch_gemm(gx, &gw, s->st));
+        cs.G[l - 1] = s->dzf[l - 1];
+        d = s->dz[ping];
+        dT = s->dzT[ping];
+        ping ^= 1;
     }
+    SR_CUDA(launch_colsum(cs, D, s->G + (size_t)k0 * D.n_params, s->st));
     return NPSIM_OK;
 }
 
-int adamw_step(npsim_surr *s, int k, float lr, float wd)
+int adamw_step(npsim_surr *s, int k0, int nk, float lr, float wd)
 {
     AdamArgs a{};
     a.lr = lr;
@@ -294,17 +317,11 @@ int adamw_step(npsim_surr *s, int k, float lr, float wd)
     const double t = (double)s->adam_t;
     a.bc1 = (float)(1.0 - std::pow(0.9, t));
     a.bc2 = (float)(1.0 - std::pow(0.999, t));
-    for (auto &L : s->nets[k]) {
-        SR_CUDA(launch_adamw(L.W, L.gW, L.mW, L.vW, L.out_p, L.in_p, a, L.Wb, L.Wt, L.mask, s->st));
-        AdamArgs ab = a;
-        ab.wd = 0.f; // no decay on biases
-        SR_CUDA(launch_adamw(L.b, L.gb, L.mb, L.vb, 1, L.out_p, ab, nullptr, nullptr, L.bmask,
-                             s->st));
-    }
+    SR_CUDA(launch_adamw(s->W, s->G, s->mom, s->var, s->mask, s->D, k0, nk, a, s->st));
     return NPSIM_OK;
 }
 
-// Upload (normalised, padded, BF16) inputs of `rows` samples into a[0] and the
+// Upload (normalised, padded, BF16) inputs of `rows` samples into xb and the
 // (normalised, padded) targets into yt; rows beyond are zero.
 int upload_batch(npsim_surr *s, const float *X, const float *Y, int rows, int bp)
 {
@@ -314,7 +331,7 @@ int upload_batch(npsim_surr *s, const float *X, const float *Y, int rows, int bp
             xf[(size_t)r * s->n_in_p + c] = (X[(size_t)r * s->n_in + c] - s->xm[c]) / s->xs[c];
     SR_CUDA(cudaMemcpyAsync(s->xin, xf.data(), sizeof(float) * xf.size(), cudaMemcpyHostToDevice,
                             s->st));
-    SR_CUDA(launch_f32_to_bf16(s->xin, (int)xf.size(), s->a[0], s->st));
+    SR_CUDA(launch_f32_to_bf16(s->xin, (int)xf.size(), s->xb, s->st));
     if (Y) {
         std::vector<float> yf((size_t)bp * s->n_out_p, 0.f);
         for (int r = 0; r < rows; ++r)
@@ -340,17 +357,28 @@ int check_flags(npsim_surr *s)
     return NPSIM_OK;
 }
 
+// One minibatch of every network of a group: rows idx[0 .. rows) of network
+// blockIdx.y (its indices idx_ld further) into x, its transpose and y; rows beyond
+// are zero.  Clears the networks' losses.
 __global__ void k_gather_rows(const __nv_bfloat16 *__restrict__ sx, const float *__restrict__ sy,
-                              const int *__restrict__ idx, int rows, int bp, int nx, int ny,
-                              __nv_bfloat16 *__restrict__ x, float *__restrict__ y)
+                              const int *__restrict__ idx, int idx_ld, int rows, int bp, int nx,
+                              int ny, __nv_bfloat16 *__restrict__ x,
+                              __nv_bfloat16 *__restrict__ xT, float *__restrict__ y,
+                              float *__restrict__ loss)
 {
-    const int r = blockIdx.x;
+    const int r = blockIdx.x, k = blockIdx.y;
+    const size_t row = (size_t)k * bp + r;
     const bool ok = r < rows;
-    const int src = ok ? idx[r] : 0;
-    for (int c = threadIdx.x; c < nx; c += blockDim.x)
-        x[(size_t)r * nx + c] = ok ? sx[(size_t)src * nx + c] : __float2bfloat16_rn(0.f);
+    const int src = ok ? idx[(size_t)k * idx_ld + r] : 0;
+    if (r == 0 && threadIdx.x == 0)
+        loss[k] = 0.f;
+    for (int c = threadIdx.x; c < nx; c += blockDim.x) {
+        const __nv_bfloat16 v = ok ? sx[(size_t)src * nx + c] : __float2bfloat16_rn(0.f);
+        x[row * nx + c] = v;
+        xT[((size_t)k * nx + c) * bp + r] = v;
+    }
     for (int c = threadIdx.x; c < ny; c += blockDim.x)
-        y[(size_t)r * ny + c] = ok ? sy[(size_t)src * ny + c] : 0.f;
+        y[row * ny + c] = ok ? sy[(size_t)src * ny + c] : 0.f;
 }
 
 // Mean and spread (population standard deviation) over the networks of the
@@ -411,78 +439,53 @@ int npsim_surr_create(int32_t n_in, int32_t n_hidden, int32_t n_layers, int32_t 
     s->ys.assign(n_out, 1.f);
     if (cudaStreamCreateWithFlags(&s->st, cudaStreamNonBlocking) != cudaSuccess)
         return bail(report_error(NPSIM_ERR_CUDA, "stream create failed"));
-    std::mt19937_64 rng(seed);
-    s->Wb_stack.assign(n_layers + 1, nullptr);
-    s->b_stack.assign(n_layers + 1, nullptr);
+    NetDims &D = s->D;
+    D.n_layers = n_layers + 1;
+    std::vector<unsigned char> mask;
     for (int l = 0; l <= n_layers; ++l) {
-        const size_t in_p = l == 0 ? s->n_in_p : n_hidden;
-        const size_t out_p = l == n_layers ? s->n_out_p : n_hidden;
-        if (dmalloc(&s->Wb_stack[l], (size_t)n_nets * out_p * in_p) != cudaSuccess ||
-            dmalloc(&s->b_stack[l], (size_t)n_nets * out_p) != cudaSuccess)
+        const int in = l == 0 ? n_in : n_hidden, out = l == n_layers ? n_out : n_hidden;
+        D.in_p[l] = l == 0 ? s->n_in_p : n_hidden;
+        D.out_p[l] = l == n_layers ? s->n_out_p : n_hidden;
+        D.off[l] = (int)mask.size();
+        for (int r = 0; r < D.out_p[l]; ++r)
+            for (int c = 0; c < D.in_p[l]; ++c)
+                mask.push_back(r < out && c < in ? 3 : 0);
+        for (int r = 0; r < D.out_p[l]; ++r)
+            mask.push_back(r < out ? 1 : 0);
+        const size_t nw = (size_t)n_nets * D.out_p[l] * D.in_p[l];
+        if (dmalloc(&D.Wb[l], nw) != cudaSuccess || dmalloc(&D.Wt[l], nw) != cudaSuccess)
             return bail(report_error(NPSIM_ERR_OOM, "surrogate weights"));
     }
-    s->nets.resize(n_nets);
-    for (int k = 0; k < n_nets; ++k) {
-        s->nets[k].resize(n_layers + 1);
+    D.n_params = (int)mask.size();
+    const size_t np = (size_t)n_nets * D.n_params;
+    if (dmalloc(&s->W, np) != cudaSuccess || dmalloc(&s->G, np) != cudaSuccess ||
+        dmalloc(&s->mom, np) != cudaSuccess || dmalloc(&s->var, np) != cudaSuccess ||
+        dmalloc(&s->mask, mask.size()) != cudaSuccess)
+        return bail(report_error(NPSIM_ERR_OOM, "surrogate weights"));
+    // He-uniform initialisation on the valid block, zero padding and biases
+    std::mt19937_64 rng(seed);
+    std::vector<float> w(np, 0.f);
+    for (int k = 0; k < n_nets; ++k)
         for (int l = 0; l <= n_layers; ++l) {
-            Layer &L = s->nets[k][l];
-            L.in = l == 0 ? n_in : n_hidden;
-            L.in_p = l == 0 ? s->n_in_p : n_hidden;
-            L.out = l == n_layers ? n_out : n_hidden;
-            L.out_p = l == n_layers ? s->n_out_p : n_hidden;
-            const size_t nw = (size_t)L.out_p * L.in_p;
-            // He-uniform initialisation on the valid block, zero padding
-            std::vector<float> w(nw, 0.f), b(L.out_p, 0.f);
-            std::vector<unsigned char> m(nw, 0), bm(L.out_p, 0);
-            const float lim = std::sqrt(6.0f / (float)L.in);
+            const int in = l == 0 ? n_in : n_hidden, out = l == n_layers ? n_out : n_hidden;
+            const float lim = std::sqrt(6.0f / (float)in);
             std::uniform_real_distribution<float> U(-lim, lim);
-            for (int r = 0; r < L.out; ++r) {
-                bm[r] = 1;
-                for (int c = 0; c < L.in; ++c) {
-                    w[(size_t)r * L.in_p + c] = U(rng);
-                    m[(size_t)r * L.in_p + c] = 1;
-                }
-            }
-            int rc = 0;
-#define SRB(call)                                                                        \
-    do {                                                                                 \
-        cudaError_t e_ = (call);                                                         \
-        if (e_ != cudaSuccess)                                                           \
-            rc = report_error(NPSIM_ERR_CUDA, "%s failed: %s", #call, cudaGetErrorString(e_)); \
-    } while (0)
-            SRB(dmalloc(&L.W, nw));
-            L.b = s->b_stack[l] + (size_t)k * L.out_p;
-            L.Wb = s->Wb_stack[l] + (size_t)k * nw;
-            SRB(dmalloc(&L.Wt, nw));
-            SRB(dmalloc(&L.mW, nw));
-            SRB(dmalloc(&L.vW, nw));
-            SRB(dmalloc(&L.mb, L.out_p));
-            SRB(dmalloc(&L.vb, L.out_p));
-            SRB(dmalloc(&L.gW, nw));
-            SRB(dmalloc(&L.gb, L.out_p));
-            SRB(dmalloc(&L.mask, nw));
-            SRB(dmalloc(&L.bmask, L.out_p));
-            if (rc)
-                return bail(rc);
-            SRB(cudaMemcpy(L.W, w.data(), sizeof(float) * nw, cudaMemcpyHostToDevice));
-            SRB(cudaMemcpy(L.b, b.data(), sizeof(float) * L.out_p, cudaMemcpyHostToDevice));
-            SRB(cudaMemcpy(L.mask, m.data(), nw, cudaMemcpyHostToDevice));
-            SRB(cudaMemcpy(L.bmask, bm.data(), L.out_p, cudaMemcpyHostToDevice));
-            SRB(cudaMemset(L.mW, 0, sizeof(float) * nw));
-            SRB(cudaMemset(L.vW, 0, sizeof(float) * nw));
-            SRB(cudaMemset(L.mb, 0, sizeof(float) * L.out_p));
-            SRB(cudaMemset(L.vb, 0, sizeof(float) * L.out_p));
-            if (rc)
-                return bail(rc);
-            SRB(cudaMemset(L.gW, 0, sizeof(float) * nw));
-            SRB(cudaMemset(L.gb, 0, sizeof(float) * L.out_p));
-            SRB(launch_weights_bf16(L.W, L.out_p, L.in_p, L.Wb, L.Wt, s->st));
-#undef SRB
-            if (rc)
-                return bail(rc);
+            float *wl = w.data() + (size_t)k * D.n_params + D.off[l];
+            for (int r = 0; r < out; ++r)
+                for (int c = 0; c < in; ++c)
+                    wl[(size_t)r * D.in_p[l] + c] = U(rng);
         }
-    }
-    if (dmalloc(&s->loss, 1) != cudaSuccess || dmalloc(&s->flags, 1) != cudaSuccess ||
+    cudaError_t ce = cudaMemcpy(s->W, w.data(), sizeof(float) * np, cudaMemcpyHostToDevice);
+    for (float *q : {s->G, s->mom, s->var})
+        if (ce == cudaSuccess)
+            ce = cudaMemset(q, 0, sizeof(float) * np);
+    if (ce == cudaSuccess)
+        ce = cudaMemcpy(s->mask, mask.data(), mask.size(), cudaMemcpyHostToDevice);
+    for (int k = 0; k < n_nets && ce == cudaSuccess; ++k)
+        ce = launch_weights_bf16(s->W, D, k, s->st);
+    if (ce != cudaSuccess)
+        return bail(report_error(NPSIM_ERR_CUDA, "surrogate weights: %s", cudaGetErrorString(ce)));
+    if (dmalloc(&s->loss, (size_t)n_nets) != cudaSuccess || dmalloc(&s->flags, 1) != cudaSuccess ||
         dmalloc(&s->outw, (size_t)s->n_out_p) != cudaSuccess ||
         dmalloc(&s->d_ym, (size_t)n_out) != cudaSuccess ||
         dmalloc(&s->d_ys, (size_t)n_out) != cudaSuccess)
@@ -540,10 +543,7 @@ int npsim_surr_param_count(npsim_surr_t s, int64_t *count)
 {
     if (!s || !count)
         return report_error(NPSIM_ERR_INVALID_ARG, "surrogate and count are required");
-    int64_t n = 0;
-    for (auto &L : s->nets[0])
-        n += (int64_t)L.out_p * L.in_p + L.out_p;
-    *count = n;
+    *count = s->D.n_params;
     return NPSIM_OK;
 }
 
@@ -552,21 +552,11 @@ int npsim_surr_get_params(npsim_surr_t s, int32_t net, float *flat, float *grads
     if (!s || net < 0 || net >= s->n_nets)
         return report_error(NPSIM_ERR_INVALID_ARG, "bad surrogate or net index");
     SR_CUDA(cudaStreamSynchronize(s->st));
-    size_t off = 0;
-    for (auto &L : s->nets[net]) {
-        const size_t nw = (size_t)L.out_p * L.in_p;
-        if (flat) {
-            SR_CUDA(cudaMemcpy(flat + off, L.W, sizeof(float) * nw, cudaMemcpyDeviceToHost));
-            SR_CUDA(cudaMemcpy(flat + off + nw, L.b, sizeof(float) * L.out_p,
-                               cudaMemcpyDeviceToHost));
-        }
-        if (grads) {
-            SR_CUDA(cudaMemcpy(grads + off, L.gW, sizeof(float) * nw, cudaMemcpyDeviceToHost));
-            SR_CUDA(cudaMemcpy(grads + off + nw, L.gb, sizeof(float) * L.out_p,
-                               cudaMemcpyDeviceToHost));
-        }
-        off += nw + L.out_p;
-    }
+    const size_t np = (size_t)s->D.n_params, off = (size_t)net * np;
+    if (flat)
+        SR_CUDA(cudaMemcpy(flat, s->W + off, sizeof(float) * np, cudaMemcpyDeviceToHost));
+    if (grads)
+        SR_CUDA(cudaMemcpy(grads, s->G + off, sizeof(float) * np, cudaMemcpyDeviceToHost));
     return NPSIM_OK;
 }
 
@@ -574,14 +564,9 @@ int npsim_surr_set_params(npsim_surr_t s, int32_t net, const float *flat)
 {
     if (!s || !flat || net < 0 || net >= s->n_nets)
         return report_error(NPSIM_ERR_INVALID_ARG, "bad surrogate, net index or params");
-    size_t off = 0;
-    for (auto &L : s->nets[net]) {
-        const size_t nw = (size_t)L.out_p * L.in_p;
-        SR_CUDA(cudaMemcpy(L.W, flat + off, sizeof(float) * nw, cudaMemcpyHostToDevice));
-        SR_CUDA(cudaMemcpy(L.b, flat + off + nw, sizeof(float) * L.out_p, cudaMemcpyHostToDevice));
-        SR_CUDA(launch_weights_bf16(L.W, L.out_p, L.in_p, L.Wb, L.Wt, s->st));
-        off += nw + L.out_p;
-    }
+    const size_t np = (size_t)s->D.n_params;
+    SR_CUDA(cudaMemcpy(s->W + (size_t)net * np, flat, sizeof(float) * np, cudaMemcpyHostToDevice));
+    SR_CUDA(launch_weights_bf16(s->W, s->D, net, s->st));
     SR_CUDA(cudaStreamSynchronize(s->st));
     return NPSIM_OK;
 }
@@ -593,15 +578,17 @@ int npsim_surr_grads(npsim_surr_t s, int32_t net, const float *X, const float *Y
         return report_error(NPSIM_ERR_INVALID_ARG, "bad surrogate, net, inputs or batch");
     const int bp = (B + 127) / 128 * 128;
     int rc = alloc_batch(s, bp);
+    if (!rc)
+        rc = alloc_rows(s, (size_t)bp, true);
+    if (!rc)
+        rc = upload_batch(s, X, Y, B, bp);
     if (rc)
         return rc;
-    rc = upload_batch(s, X, Y, B, bp);
-    if (rc)
-        return rc;
-    rc = forward(s, net, bp);
-    if (rc)
-        return rc;
-    rc = backward(s, net, bp, B);
+    SR_CUDA(launch_transpose_bf16(s->xb, bp, s->n_in_p, s->n_in_p, s->aT[0], bp, s->st));
+    SR_CUDA(cudaMemsetAsync(s->loss, 0, sizeof(float), s->st));
+    rc = forward(s, net, 1, bp, s->xb, 0, s->y, true);
+    if (!rc)
+        rc = backward(s, net, 1, bp, B);
     if (rc)
         return rc;
     rc = check_flags(s);
@@ -627,12 +614,25 @@ int npsim_surr_train(npsim_surr_t s, const float *X, const float *Y, int32_t n_s
     if (!s || !X || !Y || n_samples < 1 || epochs < 0 || batch < 1 || batch > 8192)
         return report_error(NPSIM_ERR_INVALID_ARG, "bad training arguments");
     const int bp = (batch + 127) / 128 * 128;
-    int rc = alloc_batch(s, bp);
+    // networks trained side by side: all of them, while their minibatches stay
+    // below kTrainRows rows (their activations and gradients are kept together)
+    const int group = std::max(1, std::min(s->n_nets, kTrainRows / bp));
+    int rc = alloc_rows(s, (size_t)group * bp, true);
     if (rc)
         return rc;
     // dataset on the device, normalised and padded
-    dfree2(s->dsx);
-    dfree2(s->dsy);
+    if ((size_t)n_samples > s->ds_cap) {
+        s->ds_cap = 0;
+        dfree2(s->dsx);
+        dfree2(s->dsy);
+        dfree2(s->ds_tmp);
+        dfree2(s->d_idx);
+        SR_CUDA(dmalloc(&s->dsx, (size_t)n_samples * s->n_in_p));
+        SR_CUDA(dmalloc(&s->ds_tmp, (size_t)n_samples * s->n_in_p));
+        SR_CUDA(dmalloc(&s->dsy, (size_t)n_samples * s->n_out_p));
+        SR_CUDA(dmalloc(&s->d_idx, (size_t)n_samples * s->n_nets));
+        s->ds_cap = (size_t)n_samples;
+    }
     {
         std::vector<float> xf((size_t)n_samples * s->n_in_p, 0.f);
         std::vector<float> yf((size_t)n_samples * s->n_out_p, 0.f);
@@ -642,64 +642,67 @@ int npsim_surr_train(npsim_surr_t s, const float *X, const float *Y, int32_t n_s
             for (int c = 0; c < s->n_out; ++c)
                 yf[(size_t)r * s->n_out_p + c] = (Y[(size_t)r * s->n_out + c] - s->ym[c]) / s->ys[c];
         }
-        float *tmp = nullptr;
-        SR_CUDA(dmalloc(&tmp, xf.size()));
-        SR_CUDA(dmalloc(&s->dsx, xf.size()));
-        SR_CUDA(dmalloc(&s->dsy, yf.size()));
-        SR_CUDA(cudaMemcpy(tmp, xf.data(), sizeof(float) * xf.size(), cudaMemcpyHostToDevice));
-        SR_CUDA(launch_f32_to_bf16(tmp, (int)xf.size(), s->dsx, s->st));
-        SR_CUDA(cudaMemcpy(s->dsy, yf.data(), sizeof(float) * yf.size(), cudaMemcpyHostToDevice));
-        SR_CUDA(cudaStreamSynchronize(s->st));
-        cudaFree(tmp);
-        s->ds_n = n_samples;
+        SR_CUDA(cudaMemcpyAsync(s->ds_tmp, xf.data(), sizeof(float) * xf.size(),
+                                cudaMemcpyHostToDevice, s->st));
+        SR_CUDA(launch_f32_to_bf16(s->ds_tmp, (int)xf.size(), s->dsx, s->st));
+        SR_CUDA(cudaMemcpyAsync(s->dsy, yf.data(), sizeof(float) * yf.size(),
+                                cudaMemcpyHostToDevice, s->st));
+        SR_CUDA(cudaStreamSynchronize(s->st)); // xf and yf live in this block
     }
-    int *d_idx = nullptr;
-    SR_CUDA(dmalloc(&d_idx, (size_t)n_samples));
-    std::vector<std::vector<int>> order(s->n_nets, std::vector<int>(n_samples));
+    // every network's shuffled order of an epoch, drawn network by network; the next
+    // epoch's is drawn while this one runs
+    std::vector<int> order[2];
+    order[0].resize((size_t)s->n_nets * n_samples);
+    order[1].resize(epochs > 1 ? order[0].size() : 0);
     std::mt19937_64 rng(shuffle_seed);
-    float last = 0.f;
-    const int nb = (n_samples + batch - 1) / batch;
-    for (int ep = 0; ep < epochs; ++ep) {
+    auto shuffle = [&](std::vector<int> &ord) {
         for (int k = 0; k < s->n_nets; ++k) {
+            int *o = ord.data() + (size_t)k * n_samples;
             for (int i = 0; i < n_samples; ++i)
-                order[k][i] = i;
-            std::shuffle(order[k].begin(), order[k].end(), rng);
+                o[i] = i;
+            std::shuffle(o, o + n_samples, rng);
         }
-        for (int b = 0; b < nb; ++b) {
+    };
+    int *d_idx = s->d_idx;
+    const int nb = (n_samples + batch - 1) / batch;
+    float last = 0.f;
+    cudaError_t e = cudaSuccess;
+    if (epochs > 0)
+        shuffle(order[0]);
+    for (int ep = 0; ep < epochs && !rc && e == cudaSuccess; ++ep) {
+        e = cudaMemcpyAsync(d_idx, order[ep & 1].data(), sizeof(int) * order[0].size(),
+                            cudaMemcpyHostToDevice, s->st);
+        int kl = 0; // first network of the group that ran last
+        for (int b = 0; b < nb && !rc && e == cudaSuccess; ++b) {
             const int r0 = b * batch, rows = std::min(batch, n_samples - r0);
             ++s->adam_t;
-            for (int k = 0; k < s->n_nets; ++k) {
-                cudaError_t e = cudaMemcpyAsync(d_idx, order[k].data() + r0, sizeof(int) * rows,
-                                                cudaMemcpyHostToDevice, s->st);
-                if (e != cudaSuccess) {
-                    cudaFree(d_idx);
-                    return report_error(NPSIM_ERR_CUDA, "index upload: %s", cudaGetErrorString(e));
-                }
-                k_gather_rows<<<bp, 128, 0, s->st>>>(s->dsx, s->dsy, d_idx, rows, bp, s->n_in_p,
-                                                     s->n_out_p, s->a[0], s->yt);
-                rc = forward(s, k, bp);
-                if (!rc)
-                    rc = backward(s, k, bp, rows);
-                if (!rc)
-                    rc = adamw_step(s, k, lr, wd);
-                if (rc) {
-                    cudaFree(d_idx);
-                    return rc;
-                }
-            }
-            if (b + 1 == nb) {
-                cudaStreamSynchronize(s->st);
-                cudaMemcpy(&last, s->loss, sizeof(float), cudaMemcpyDeviceToHost);
+            for (int k0 = 0; k0 < s->n_nets && !rc && e == cudaSuccess; k0 += group) {
+                const int nk = std::min(group, s->n_nets - k0);
+                kl = k0;
+                k_gather_rows<<<dim3(bp, nk), 96, 0, s->st>>>(
+                    s->dsx, s->dsy, d_idx + (size_t)k0 * n_samples + r0, n_samples, rows, bp,
+                    s->n_in_p, s->n_out_p, s->a[0], s->aT[0], s->yt, s->loss);
+                e = cudaGetLastError();
+                if (e == cudaSuccess)
+                    rc = forward(s, k0, nk, bp, s->a[0], bp, s->y, true);
+                if (!rc && e == cudaSuccess)
+                    rc = backward(s, k0, nk, bp, rows);
+                if (!rc && e == cudaSuccess)
+                    rc = adamw_step(s, k0, nk, lr, wd);
             }
         }
-        rc = check_flags(s);
-        if (rc) {
-            cudaFree(d_idx);
-            return rc;
-        }
+        if (!rc && e == cudaSuccess && ep + 1 < epochs)
+            shuffle(order[(ep + 1) & 1]);
+        if (!rc && e == cudaSuccess)
+            rc = check_flags(s); // waits for the epoch
+        if (!rc && e == cudaSuccess && ep + 1 == epochs)
+            e = cudaMemcpy(&last, s->loss + (s->n_nets - 1 - kl), sizeof(float),
+                           cudaMemcpyDeviceToHost);
     }
-    cudaFree(d_idx);
-    SR_CUDA(cudaStreamSynchronize(s->st));
+    if (rc)
+        return rc;
+    if (e != cudaSuccess)
+        return report_error(NPSIM_ERR_CUDA, "training: %s", cudaGetErrorString(e));
     if (final_loss)
         *final_loss = last;
     return NPSIM_OK;
@@ -722,11 +725,12 @@ int npsim_surr_predict(npsim_surr_t s, const float *X, int32_t B, float *Y_mean,
     if (!layered && mlp_infer_supported(s->NL, s->n_in_p, s->H, s->n_out_p)) {
         // every layer of every network in one launch
         MlpInferArgs f{};
-        f.X = s->a[0];
+        f.X = s->xb;
         for (int l = 0; l <= s->NL; ++l) {
-            f.W[l] = s->Wb_stack[l];
-            f.b[l] = s->b_stack[l];
+            f.W[l] = s->D.Wb[l];
+            f.b[l] = s->W + s->D.off[l] + s->D.out_p[l] * s->D.in_p[l];
         }
+        f.b_stride = s->D.n_params;
         f.NL = s->NL;
         f.in_p = s->n_in_p;
         f.H = s->H;
@@ -737,11 +741,11 @@ int npsim_surr_predict(npsim_surr_t s, const float *X, int32_t B, float *Y_mean,
         f.flags = s->flags;
         SR_CUDA(launch_mlp_infer(f, s->st));
     } else {
-        for (int k = 0; k < s->n_nets; ++k) {
-            rc = forward(s, k, bp, s->y_all + (size_t)k * bp * s->n_out_p);
-            if (rc)
-                return rc;
-        }
+        rc = alloc_rows(s, (size_t)bp, false);
+        for (int k = 0; k < s->n_nets && !rc; ++k)
+            rc = forward(s, k, 1, bp, s->xb, 0, s->y_all + (size_t)k * bp * s->n_out_p, false);
+        if (rc)
+            return rc;
     }
     float *d_mean = s->ystat, *d_spread = s->ystat + (size_t)B * s->n_out;
     const int ne = B * s->n_out;
@@ -798,7 +802,8 @@ int npsim_gemm_bf16(const uint16_t *A, const uint16_t *B, int32_t M, int32_t N, 
     g.Cf = dC;
     g.flags = dflag;
     g.wait_cycles = g_wait_cycles.load();
-    cudaError_t e = launch_gemm(g, 0);
+    g.nz = 1;
+    cudaError_t e = launch_gemm(g, nullptr, 0);
     if (e == cudaSuccess)
         e = cudaDeviceSynchronize();
     int flag = 0;

@@ -218,7 +218,8 @@ struct npsim_sim {
     size_t cells_alloc = 0;  // sort keys the cell buffers hold
     NbrList nl{};          // Verlet list over the cells (cell-list LJ)
     int *d_gate = nullptr; // 1: rebuild the cell and neighbour lists at the next pass
-    unsigned *list_bar = nullptr; // counters of the list build's grid barrier [3]
+    unsigned *list_bar = nullptr; // counters of the list kernels' grid barrier [3], gates [3]
+    float4 *sxq2 = nullptr;       // the other cell-ordered records of fused steps (lazy)
 
     bool ap = false, ap_lj = false;
     int ap_idx = 0;
@@ -294,6 +295,7 @@ struct npsim_sim {
         dfree(d_done);
         dfree(d_gate);
         dfree(list_bar);
+        dfree(sxq2);
         dfree(nl.nbr);
         dfree(nl.nnbr);
         dfree(nl.x_ref);
@@ -352,6 +354,7 @@ int alloc_cells(CellGrid &g, CellBufs &b, int n)
         NP_CUDA(cudaMemset(q, 0, sizeof(int) * (size_t)(n > 0 ? n : 1)));
     // one record past the NPs: a position far from every NP (type 0), the
     // partner that pads each neighbour list to whole blocks of four
+    NP_CUDA(cudaMemset(b.count, 0, sizeof(int) * m)); // the list build leaves them zero
     NP_CUDA(dalloc(&b.sxq, (size_t)n + 1));
     const float4 far = make_float4(kPairPad, kPairPad, kPairPad, 0.0f);
     NP_CUDA(cudaMemcpy(b.sxq + n, &far, sizeof(far), cudaMemcpyHostToDevice));
@@ -759,7 +762,8 @@ int read_flags(npsim_sim *s)
             return set_err(NPSIM_ERR_NONFINITE, "a position became non-finite");
         if (h & FLAG_TIMEOUT) {
             if (s->list_bar) { // the barrier it left, and the lists it did not finish
-                NP_CUDA(cudaMemsetAsync(s->list_bar, 0, 3 * sizeof(unsigned), s->user));
+                NP_CUDA(cudaMemsetAsync(s->list_bar, 0, 6 * sizeof(unsigned), s->user));
+                NP_CUDA(cudaMemsetAsync(s->cb.count, 0, sizeof(int) * s->cells_alloc, s->user));
                 int rc = set_gate(s, 1);
                 if (rc)
                     return rc;
@@ -1435,8 +1439,8 @@ int create_impl(const npsim_type_t *types, const npsim_params_t *params, int64_t
         BAIL_CUDA(dalloc(&s->nl.builds, 1));
         BAIL_CUDA(cudaMemset(s->nl.builds, 0, sizeof(unsigned long long)));
         BAIL_CUDA(dalloc(&s->d_gate, 1));
-        BAIL_CUDA(dalloc(&s->list_bar, 3));
-        BAIL_CUDA(cudaMemset(s->list_bar, 0, 3 * sizeof(unsigned)));
+        BAIL_CUDA(dalloc(&s->list_bar, 6));
+        BAIL_CUDA(cudaMemset(s->list_bar, 0, 6 * sizeof(unsigned)));
         BAIL_CUDA(cudaMemset(s->nl.nnbr, 0, sizeof(int) * (size_t)n));
         BAIL_CUDA(cudaMemset(s->nl.nbr, 0, sizeof(unsigned) * (size_t)s->nl.cap * n));
     }
@@ -1555,6 +1559,38 @@ int regrid_if_needed(npsim_sim *s)
     return set_gate(s, 1);
 }
 
+// Small droplets whose pair forces all come from the lists take many steps per
+// launch (not while the kernels are timed apart).
+bool fused_steps(const npsim_sim *s)
+{
+    return s->cell && !s->ap && s->n <= kMaxFusedNps && !s->profiling;
+}
+
+int enqueue_fused(npsim_sim *s, int k)
+{
+    if (!s->sxq2) {
+        NP_CUDA(dalloc(&s->sxq2, (size_t)s->n + 1));
+        const float4 far = make_float4(kPairPad, kPairPad, kPairPad, 0.0f);
+        NP_CUDA(cudaMemcpyAsync(s->sxq2 + s->n, &far, sizeof(far), cudaMemcpyHostToDevice, s->user));
+        NP_CUDA(cudaStreamSynchronize(s->user)); // far lives on this stack frame
+    }
+    IntArgs a{};
+    a.x_lo = s->x_lo;
+    a.v = s->v;
+    a.F = s->F;
+    a.typ = s->typ;
+    a.xq = s->xq;
+    a.spring = s->d_spring;
+    a.x_ref = s->nl.x_ref;
+    a.nbr_gate = s->d_gate;
+    a.half_skin2 = kHalfSkin2;
+    a.step = s->d_step;
+    a.flags = s->d_flags;
+    NP_CUDA(launch_list_steps(s->grid, s->cb, s->n, s->tab_full, s->d_rcc2, kSkin, s->nl,
+                              s->list_bar, a, s->sp, s->sxq2, s->F_lj, k, s->user));
+    return NPSIM_OK;
+}
+
 int enqueue_steps(npsim_sim *s, int64_t n_steps)
 {
     int64_t rem = n_steps;
@@ -1562,6 +1598,17 @@ int enqueue_steps(npsim_sim *s, int64_t n_steps)
         int rc0 = regrid_if_needed(s);
         if (rc0)
             return rc0;
+        if (fused_steps(s)) {
+            int k = (int)std::min<int64_t>(rem, kMaxFusedSteps);
+            if (follows_droplet(s)) // stop at the next multiple of kRegridPeriod
+                k = (int)std::min<int64_t>(k, kRegridPeriod - s->step % kRegridPeriod);
+            int rc = enqueue_fused(s, k);
+            if (rc)
+                return rc;
+            rem -= k;
+            s->step += k;
+            continue;
+        }
         int k = (int)std::min<int64_t>(rem, kChunk);
         if (follows_droplet(s)) // stop at the next multiple of kRegridPeriod
             k = (int)std::min<int64_t>(k, kRegridPeriod - s->step % kRegridPeriod);
@@ -1742,8 +1789,8 @@ int npsim_launches_per_step(npsim_sim_t s, int *launches)
 {
     NP_REQUIRE(s && launches, "sim and launches are required");
     // integrator, all-pairs (and the sum of its partials), the gated list build, the
-    // list LJ forces
-    *launches = 1 + (s->ap ? (s->sk.tri ? 2 : 1) : 0) + (s->cell ? 2 : 0);
+    // list LJ forces; one launch where it takes many steps
+    *launches = s->cell && !s->ap && s->n <= kMaxFusedNps ? 1 : 1 + (s->ap ? (s->sk.tri ? 2 : 1) : 0) + (s->cell ? 2 : 0);
     return NPSIM_OK;
 }
 

@@ -111,8 +111,9 @@ __device__ __forceinline__ int cta_exclusive_scan(int v, int *s_warp, int *total
     return r;
 }
 
-__device__ __forceinline__ void scan_tiles(const int *count, int *start, int *tile_sum, int m,
-                                           int *s_warp)
+// With `local` the tile-local scans are left in count as well.
+__device__ __forceinline__ void scan_tiles(int *count, int *start, int *tile_sum, int m,
+                                           int *s_warp, bool local)
 {
     const int n_tiles = (m + kScanTile - 1) / kScanTile;
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
@@ -128,8 +129,11 @@ __device__ __forceinline__ void scan_tiles(const int *count, int *start, int *ti
         int run = cta_exclusive_scan(s, s_warp, &total);
 #pragma unroll
         for (int k = 0; k < kScanItems; ++k) {
-            if (base + k < m)
+            if (base + k < m) {
                 start[base + k] = run;
+                if (local)
+                    count[base + k] = run;
+            }
             run += a[k];
         }
         if (threadIdx.x == 0)
@@ -218,10 +222,10 @@ __global__ void k_cell_hash(CellGrid g, const float4 *xq, const int *typ, int n,
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_tiles(const int *count, int *start, int *tile_sum, int m)
+k_scan_tiles(int *count, int *start, int *tile_sum, int m)
 {
     __shared__ int s_warp[kScanThreads / 32 + 1];
-    scan_tiles(count, start, tile_sum, m, s_warp);
+    scan_tiles(count, start, tile_sum, m, s_warp, false);
 }
 
 __global__ void __launch_bounds__(kScanThreads)
@@ -320,12 +324,12 @@ struct ListBuildArgs {
 // instead).  Lists are written by slot so that the per-step force kernel, which
 // runs in the same order, reads them coalesced.  Records the position of this
 // build in x_ref (by particle).
-__device__ __forceinline__ void nbr_slot(const ListBuildArgs &A, int p, unsigned *__restrict__ nbr,
-                                         const float *s_rl2, const float *s_rmax)
+__device__ __forceinline__ void nbr_slot(const ListBuildArgs &A, const float4 *sxq, int p,
+                                         unsigned *__restrict__ nbr, const float *s_rl2,
+                                         const float *s_rmax)
 {
     const CellGrid &g = A.g;
     const int *start = A.b.start;
-    const float4 *sxq = A.b.sxq;
     const int n = A.n, cap = A.cap;
     const int tb = g.tb > 1 ? g.tb : 1;
     const float4 pi = sxq[p];
@@ -415,77 +419,132 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, int
     return *s_ok != 0;
 }
 
-// The whole list build in one cooperative launch: counting sort of the NPs into
-// cells, then the lists.  Every step launches it, and unless the integrator has
-// raised the gate (some NP has moved more than half the skin) it returns at once:
-// as nine gated kernels (zero, hash, three scan passes, scatter, order, gather,
-// lists) the closed gate cost nine launches a step, 13 us of the 16 us of a
-// 1000-NP step and 16 of the 33 us of a 250000-NP step of the truncated model.
-// When it does build, the phases are separated by grid barriers.  Warps draw
-// batches of 32 slots for the lists from the last slot back: the cell order lists
-// the types one after another, so the largest NPs, whose lists are the longest,
-// go first.
-__global__ void __launch_bounds__(kScanThreads, 4)
-k_list_build(const __grid_constant__ ListBuildArgs A)
-{
-    __shared__ int s_warp[kScanThreads / 32 + 1];
-    __shared__ int s_ok;
-    __shared__ float4 s_tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
-    __shared__ float s_rl2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
-    __shared__ float s_rmax[NPSIM_MAX_TYPES];
-    if (A.gate && *A.gate == 0) // nobody writes it while this kernel runs
-        return;
-    const CellBufs &B = A.b;
-    const int m = (A.g.tb > 1 ? A.g.tb : 1) * A.g.n_cells; // sort keys
-    unsigned phase = 0;
-    auto barrier = [&]() { return grid_barrier(A.bar, phase, A.flags, &s_ok); };
+// Shared memory of the list build.
+struct ListBuildSmem {
+    int warp[kScanThreads / 32 + 1];
+    int ok;
+    int off[kScanTile]; // prefix of the scan tiles' totals (when they are few enough)
+    float4 tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    float rl2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    float rmax[NPSIM_MAX_TYPES];
+};
 
-    if (A.builds && blockIdx.x == 0 && threadIdx.x == 0)
-        ++*A.builds;
+// The phases of a build by every CTA of a cooperative launch, between grid barriers
+// (false: one gave up), the records going to sxq.  The counts are zero on entry and
+// left zero.  With up to
+// kScanTile scan tiles (a million sort keys) every CTA scans their totals itself,
+// and the offsets are added while the NPs are scattered: four barriers; beyond,
+// one CTA scans the totals: six.
+__device__ __forceinline__ bool list_build(const ListBuildArgs &A, float4 *sxq, ListBuildSmem &S,
+                                           unsigned &phase)
+{
+    const CellBufs &B = A.b;
+    const int n = A.n;
+    const int m = (A.g.tb > 1 ? A.g.tb : 1) * A.g.n_cells; // sort keys
+    const int n_tiles = (m + kScanTile - 1) / kScanTile;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    auto barrier = [&]() { return grid_barrier(A.bar, phase, A.flags, &S.ok); };
+
+    if (tid == 0) {
+        if (A.builds)
+            ++*A.builds;
+        A.bar[2] = 0u; // slots drawn
+    }
+    cell_hash(A.g, A.xq, A.typ, n, B.key, B.rank, B.count);
+    if (!barrier())
+        return false;
+    const bool few = n_tiles <= kScanTile;
+    scan_tiles(B.count, B.start, B.tile_sum, m, S.warp, few);
+    if (!barrier())
+        return false;
+    if (few) {
+        int a[kScanItems], sum = 0, total;
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            const int t = threadIdx.x * kScanItems + k;
+            a[k] = t < n_tiles ? B.tile_sum[t] : 0;
+            sum += a[k];
+        }
+        int run = cta_exclusive_scan(sum, S.warp, &total);
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            S.off[threadIdx.x * kScanItems + k] = run;
+            run += a[k];
+        }
+        __syncthreads();
+        for (int c = tid; c < m; c += stride)
+            B.start[c] = B.count[c] + S.off[c / kScanTile];
+        if (tid == 0)
+            B.start[m] = total;
+        for (int i = tid; i < n; i += stride) {
+            const int c = B.key[i];
+            B.arrived[B.count[c] + S.off[c / kScanTile] + B.rank[i]] = i;
+        }
+    } else {
+        if (blockIdx.x == 0)
+            scan_totals(B.tile_sum, n_tiles, B.start, m, S.warp);
+        if (!barrier())
+            return false;
+        scan_add(B.start, B.tile_sum, m);
+        if (!barrier())
+            return false;
+        cell_scatter(B.key, B.rank, B.start, B.arrived, n);
+    }
+    if (!barrier())
+        return false;
+    cell_order(B.arrived, B.key, B.start, A.xq, A.typ, B.sorted, B.pos, sxq, n);
     cell_zero(B.count, m);
     if (!barrier())
-        return;
-    cell_hash(A.g, A.xq, A.typ, A.n, B.key, B.rank, B.count);
-    if (!barrier())
-        return;
-    scan_tiles(B.count, B.start, B.tile_sum, m, s_warp);
-    if (!barrier())
-        return;
-    if (blockIdx.x == 0)
-        scan_totals(B.tile_sum, (m + kScanTile - 1) / kScanTile, B.start, m, s_warp);
-    if (!barrier())
-        return;
-    scan_add(B.start, B.tile_sum, m);
-    if (!barrier())
-        return;
-    cell_scatter(B.key, B.rank, B.start, B.arrived, A.n);
-    if (!barrier())
-        return;
-    cell_order(B.arrived, B.key, B.start, A.xq, A.typ, B.sorted, B.pos, B.sxq, A.n);
-    load_tables(A.tab, A.rcc2, A.skin, s_tab, s_rl2, s_rmax);
-    if (!barrier())
-        return;
+        return false;
+    // warps draw batches of 32 slots for the lists from the last slot back: the cell
+    // order lists the types one after another, so the largest NPs, whose lists are
+    // the longest, go first
     const int lane = threadIdx.x & 31;
     for (;;) {
         unsigned first = 0;
         if (lane == 0)
             first = atomicAdd(A.bar + 2, 32u);
-        const int left = A.n - (int)__shfl_sync(0xffffffffu, first, 0); // slots not drawn yet
+        const int left = n - (int)__shfl_sync(0xffffffffu, first, 0); // slots not drawn yet
         if (left <= 0)
             break;
         const int p = left - 1 - lane;
         if (p >= 0)
-            nbr_slot(A, p, A.nbr, s_rl2, s_rmax);
+            nbr_slot(A, sxq, p, A.nbr, S.rl2, S.rmax);
     }
-    // the last CTA out resets the counters for the next launch
+    return true;
+}
+
+// The last CTA out resets the barrier's counters for the next launch; true in its
+// first thread.
+__device__ __forceinline__ bool barrier_done(unsigned *bar)
+{
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(A.bar + 1, 1u) == gridDim.x - 1) {
-            A.bar[0] = A.bar[1] = A.bar[2] = 0u;
-            __threadfence();
-        }
-    }
+    if (threadIdx.x != 0)
+        return false;
+    __threadfence();
+    if (atomicAdd(bar + 1, 1u) != gridDim.x - 1)
+        return false;
+    bar[0] = bar[1] = 0u;
+    __threadfence();
+    return true;
+}
+
+// The list build in one cooperative launch: counting sort of the NPs into cells,
+// then the lists.  Every step launches it, and unless the integrator has raised the
+// gate (some NP has moved more than half the skin) it returns at once: as nine gated
+// kernels (zero, hash, three scan passes, scatter, order, gather, lists) the closed
+// gate cost nine launches a step, 16 of the 33 us of a 250000-NP step of the
+// truncated model; this way 8.
+__global__ void __launch_bounds__(kScanThreads, 4)
+k_list_build(const __grid_constant__ ListBuildArgs A)
+{
+    __shared__ ListBuildSmem S;
+    if (A.gate && *A.gate == 0) // nobody writes it while this kernel runs
+        return;
+    unsigned phase = 0;
+    load_tables(A.tab, A.rcc2, A.skin, S.tab, S.rl2, S.rmax);
+    if (list_build(A, A.b.sxq, S, phase))
+        barrier_done(A.bar);
 }
 
 // The forces of the NP at slot p whose list overflowed: every NP of the cells of
@@ -558,19 +617,17 @@ __device__ __noinline__ void cell_slot_forces(int p, const CellGrid g, const int
 // slots, and for the partners from the nearby cells -- and the 32-byte force
 // record goes to the NP's index i = sorted[p], where the integrator reads it.
 // An NP whose list overflowed sums over the cells of that build instead (a
-// superset of its list).  Writes one (hi x, y, z, lo x, y, z, 0, 0) record.
+// superset of its list).  Returns the (hi x, y, z, lo x | lo y, z, 0, 0) record in
+// o0, o1.
 template <bool COUL>
-__device__ __forceinline__ void slot_forces(int p, const CellGrid &g, const int *__restrict__ start,
-                                            const int *__restrict__ sorted,
-                                            const int *__restrict__ key,
-                                            const float4 *__restrict__ sxq, int n, int cap,
-                                            const unsigned *__restrict__ nbr,
-                                            const int *__restrict__ nnbr,
-                                            float *__restrict__ F_lj, const float4 *s_tab,
-                                            const float *s_rcc2)
+__device__ __forceinline__ void slot_forces(int p, int i, const CellGrid &g, const int *start,
+                                            const int *sorted, const int *key,
+                                            const float4 *sxq, int n, int cap,
+                                            const unsigned *nbr, const int *nnbr, float *F_lj,
+                                            const float4 *s_tab, const float *s_rcc2, float4 &o0,
+                                            float4 &o1)
 {
     const float4 pi = sxq[p];
-    const int i = sorted[p];
     const int ti = __float_as_int(pi.w);
     const int row = ti * NPSIM_MAX_TYPES;
     float hx = 0.f, hy = 0.f, hz = 0.f, lx = 0.f, ly = 0.f, lz = 0.f;
@@ -618,6 +675,9 @@ __device__ __forceinline__ void slot_forces(int p, const CellGrid &g, const int 
     const int cnt = nnbr[p];
     if (cnt > cap) {
         cell_slot_forces<COUL>(p, g, start, sorted, key, sxq, F_lj, s_tab, s_rcc2);
+        const float4 *o = reinterpret_cast<const float4 *>(F_lj + 8 * (size_t)i);
+        o0 = o[0];
+        o1 = o[1];
         return;
     }
     {
@@ -650,10 +710,8 @@ __device__ __forceinline__ void slot_forces(int p, const CellGrid &g, const int 
             nxt = nn;
         }
     }
-    // one 32-byte record per NP, a whole DRAM sector: (hi x, y, z, lo x), (lo y, z)
-    float4 *o = reinterpret_cast<float4 *>(F_lj + 8 * (size_t)i);
-    o[0] = make_float4(hx, hy, hz, lx);
-    o[1] = make_float4(ly, lz, 0.0f, 0.0f);
+    o0 = make_float4(hx, hy, hz, lx);
+    o1 = make_float4(ly, lz, 0.0f, 0.0f);
 }
 
 // List forces, one thread per cell-order slot (slot_forces), and closes the
@@ -680,8 +738,151 @@ k_lj_nbr(const __grid_constant__ CellGrid g, const int *__restrict__ start, cons
     if (gate && blockIdx.x == 0 && threadIdx.x == 0)
         *gate = 0; // every build kernel of this step has run; the integrator may reopen it
     const int p = (int)(gridDim.x - 1 - blockIdx.x) * (int)blockDim.x + (int)threadIdx.x;
-    if (p < n)
-        slot_forces<COUL>(p, g, start, sorted, key, sxq, n, cap, nbr, nnbr, F_lj, s_tab, s_rcc2);
+    if (p < n) {
+        const int i = sorted[p];
+        float4 o0, o1;
+        slot_forces<COUL>(p, i, g, start, sorted, key, sxq, n, cap, nbr, nnbr, F_lj, s_tab, s_rcc2,
+                          o0, o1);
+        // one 32-byte record per NP, a whole DRAM sector
+        float4 *o = reinterpret_cast<float4 *>(F_lj + 8 * (size_t)i);
+        o[0] = o0;
+        o[1] = o1;
+    }
+}
+
+// Up to kMaxFusedSteps steps of a droplet whose pair forces all come from the lists,
+// in one cooperative launch.  A step of a small droplet is three short kernels
+// (gated build, list forces, integrator), 9.2 us at 1000 NPs, of which their work is
+// perhaps two; here a step is one pass over the NPs and one grid barrier:
+//   A part of the first step; then per step: [barrier; build if the gate is open];
+//   list forces, external forces, B and the next step's A part of each NP by the
+//   thread that holds its slot; after the last step's B the counters move on.
+// Arithmetic and order are those of the separate kernels (the same functions), so a
+// run that mixes both is bit-identical.  While some threads still read their
+// partners' records of the current positions others already write new ones, so the
+// cell-ordered records alternate between two arrays; the last step's pass, which
+// moves nothing, leaves them in the first.  The state is read by particle index in
+// cell order (scattered): with the state in L2 that costs less than the launches,
+// beyond kMaxFusedNps it does not.
+struct FusedStepArgs {
+    ListBuildArgs L;
+    IntArgs I;          // xq, x_lo, v, F, typ, spring, step, flags, half_skin2, x_ref
+    float4 *sxq2;       // the other cell-ordered records (n + 1, the last one far)
+    float *F_lj;        // scratch of the overflow path
+    const int *gate;    // set on entry: build in the first pass
+    // Gates inside the launch, zero between launches: pass j reads word j mod 3,
+    // raises word (j + 1) mod 3 and clears word (j + 2) mod 3, so no word is written
+    // in a pass in which a CTA may still read it.
+    unsigned *gates;
+    int steps;
+};
+
+// One particle's external force added to its list force and its update, as
+// update_particle of the integrator does.
+template <int MODE>
+__device__ __forceinline__ void fused_update(const FusedStepArgs &a, const StepParams &p,
+                                             const TypeCoef *s_tc, float R0f, long long step, int i,
+                                             float4 o0, float4 o1, float4 *sxq, int *raise)
+{
+    const IntArgs &I = a.I;
+    const int n = p.n;
+    const int ti = I.typ[i];
+    const TypeCoef &tc = s_tc[ti];
+    const float4 xh = I.xq[i];
+    const float lx = I.x_lo[i], ly = I.x_lo[n + i], lz = I.x_lo[2 * n + i];
+    const float v[3] = {I.v[i], I.v[n + i], I.v[2 * n + i]};
+    float Fh[3] = {0.f, 0.f, 0.f}, Fl[3] = {0.f, 0.f, 0.f};
+    if (MODE != MODE_A) {
+        df_add_df(Fh[0], Fl[0], o0.x, o0.w);
+        df_add_df(Fh[1], Fl[1], o0.y, o1.x);
+        df_add_df(Fh[2], Fl[2], o0.z, o1.y);
+        float ex, ey, ez;
+        external_force(xh, lx, ly, lz, tc.kw, tc.mg, tc.mw2,
+                       I.spring[(step & 1) * NPSIM_MAX_TYPES + ti], p.wall, p.rot_mode, ex, ey, ez,
+                       R0f, I.flags);
+        df_add(Fh[0], Fl[0], ex);
+        df_add(Fh[1], Fl[1], ey);
+        df_add(Fh[2], Fl[2], ez);
+    } else {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            Fh[d] = I.F[d * n + i];
+            Fl[d] = I.F[(3 + d) * n + i];
+        }
+    }
+    advance_particle<MODE>(i, n, (uint32_t)i, tc, p.integrator, 0.5f * (float)p.dt, p.seed, step, xh,
+                           lx, ly, lz, Fh, Fl, v, I.x_lo, I.v, I.F, I.xq, I.flags, I.x_ref, raise,
+                           I.half_skin2, sxq, a.L.b.pos, ti);
+}
+
+template <bool COUL>
+__global__ void __launch_bounds__(kScanThreads, 2)
+k_list_steps(const __grid_constant__ FusedStepArgs a, const __grid_constant__ StepParams p)
+{
+    __shared__ ListBuildSmem S;
+    __shared__ float4 s_tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    __shared__ float s_rl2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    __shared__ float s_rcc2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    __shared__ float s_rmax[NPSIM_MAX_TYPES];
+    __shared__ TypeCoef s_tc[NPSIM_MAX_TYPES];
+    const ListBuildArgs &L = a.L;
+    const int n = p.n;
+    load_tables(L.tab, L.rcc2, L.skin, S.tab, S.rl2, S.rmax);
+    load_tables(L.tab, COUL ? L.rcc2 : nullptr, 0.0f, s_tab, s_rl2, s_rmax, s_rcc2);
+    if (threadIdx.x < NPSIM_MAX_TYPES)
+        s_tc[threadIdx.x] = p.tc[threadIdx.x];
+    __syncthreads();
+    const long long step0 = *a.I.step;
+    const float R0f = (float)p.R0;
+    unsigned phase = 0;
+    // spring radii of step s + 1, by the first CTA in a pass that takes the A part of s
+    auto next_spring = [&](long long s) {
+        if (blockIdx.x == 0 && threadIdx.x < p.n_types)
+            a.I.spring[((s + 1) & 1) * NPSIM_MAX_TYPES + threadIdx.x] =
+                spring_entry(p.R0, p.k_evap, p.dt, s + 1, p.tc[threadIdx.x].half_sigma);
+    };
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    next_spring(step0);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        fused_update<MODE_A>(a, p, s_tc, R0f, step0, i, none, none, L.b.sxq,
+                             reinterpret_cast<int *>(a.gates) + 1);
+    // slots spread over the CTAs a warp at a time
+    const int first = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+    for (int j = 1; j <= a.steps; ++j) {
+        if (!grid_barrier(L.bar, phase, L.flags, &S.ok))
+            return;
+        float4 *cur = (j & 1) ? L.b.sxq : a.sxq2, *nxt = (j & 1) ? a.sxq2 : L.b.sxq;
+        volatile unsigned *w = a.gates;
+        if (w[j % 3] != 0u || (j == 1 && *(volatile int *)a.gate != 0)) {
+            if (!list_build(L, cur, S, phase) || !grid_barrier(L.bar, phase, L.flags, &S.ok))
+                return;
+        }
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            w[(j + 2) % 3] = 0u;
+        int *raise = reinterpret_cast<int *>(a.gates) + (j + 1) % 3;
+        const bool last = j == a.steps;
+        if (!last)
+            next_spring(step0 + j);
+        for (int q = first; q < n; q += gridDim.x * blockDim.x) {
+            const int i = L.b.sorted[q];
+            float4 o0, o1;
+            slot_forces<COUL>(q, i, L.g, L.b.start, L.b.sorted, L.b.key, cur, n, L.cap, L.nbr, L.nnbr,
+                              a.F_lj, s_tab, s_rcc2, o0, o1);
+            if (!last) {
+                fused_update<MODE_BA>(a, p, s_tc, R0f, step0 + j, i, o0, o1, nxt, raise);
+            } else {
+                if (cur != L.b.sxq)
+                    L.b.sxq[q] = cur[q];
+                fused_update<MODE_B>(a, p, s_tc, R0f, step0 + j, i, o0, o1, nullptr, raise);
+            }
+        }
+    }
+    if (barrier_done(L.bar)) { // every thread is past its use of the step and the gates
+        *a.I.step = step0 + a.steps;
+        for (int k = 0; k < 3; ++k)
+            a.gates[k] = 0u;
+        *a.I.nbr_gate = 0; // the last pass has built what the one before it asked for
+    }
 }
 
 } // namespace
@@ -690,6 +891,7 @@ int cell_scan_tiles(int n_cells) { return (n_cells + kScanTile - 1) / kScanTile;
 
 namespace {
 constexpr int kMaxGrid = 1216; // 8 CTAs on each of 152 SMs
+constexpr int kOneCtaPerSm = 152;
 int grid_for(int n, int block)
 {
     const int g = (n + block - 1) / block;
@@ -722,10 +924,11 @@ cudaError_t launch_cell_refresh(const CellBufs &b, const float4 *xq, const int *
     return cudaGetLastError();
 }
 
-cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4 *xq,
+namespace {
+ListBuildArgs list_build_args(const CellGrid &g, const CellBufs &b, const float4 *xq,
                               const int *typ, int n, const PairTab *tab, const float *rcc2,
                               float skin, const NbrList &l, int *flags, const int *gate,
-                              unsigned *bar, cudaStream_t st)
+                              unsigned *bar)
 {
     ListBuildArgs A{};
     A.g = g;
@@ -744,22 +947,24 @@ cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4
     A.flags = flags;
     A.gate = gate;
     A.bar = bar;
-    // CTAs the device holds at once
+    return A;
+}
+
+// A cooperative launch of `want` CTAs of kScanThreads, or as many as the device
+// holds at once.
+template <class... P>
+cudaError_t launch_coop(void (*fn)(P...), int want, cudaStream_t st, const P &...args)
+{
     int dev = 0, sms = 0, occ = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_list_build, kScanThreads, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kScanThreads, 0);
     if (e != cudaSuccess)
         return e;
-    // a thread per NP and four keys per thread, at least a warp per 32 NPs on SMs of
-    // their own while there are few
-    const int m = (g.tb > 1 ? g.tb : 1) * g.n_cells;
-    int grid = max((n + 63) / 64, cell_scan_tiles(m));
-    grid = max(1, min(grid, occ * sms));
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = dim3(max(1, min(want, occ * sms)));
     cfg.blockDim = dim3(kScanThreads);
     cfg.stream = st;
     cudaLaunchAttribute at{};
@@ -767,7 +972,41 @@ cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4
     at.val.cooperative = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_list_build, A);
+    return cudaLaunchKernelEx(&cfg, fn, args...);
+}
+} // namespace
+
+cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4 *xq,
+                              const int *typ, int n, const PairTab *tab, const float *rcc2,
+                              float skin, const NbrList &l, int *flags, const int *gate,
+                              unsigned *bar, cudaStream_t st)
+{
+    const ListBuildArgs A =
+        list_build_args(g, b, xq, typ, n, tab, rcc2, skin, l, flags, gate, bar);
+    // a thread per four NPs or keys
+    const int m = (g.tb > 1 ? g.tb : 1) * g.n_cells;
+    return launch_coop<ListBuildArgs>(k_list_build, max((n + 63) / 64, cell_scan_tiles(m)), st, A);
+}
+
+cudaError_t launch_list_steps(const CellGrid &g, const CellBufs &b, int n, const PairTab *tab,
+                              const float *rcc2, float skin, const NbrList &l, unsigned *bar,
+                              const IntArgs &I, const StepParams &p, float4 *sxq2, float *F_lj,
+                              int steps, cudaStream_t st)
+{
+    FusedStepArgs a{};
+    a.L = list_build_args(g, b, I.xq, I.typ, n, tab, rcc2, skin, l, I.flags, I.nbr_gate, bar);
+    a.I = I;
+    a.sxq2 = sxq2;
+    a.F_lj = F_lj;
+    a.gate = I.nbr_gate;
+    a.gates = bar + 3;
+    a.steps = steps;
+    // a warp's 32 slots per CTA while that leaves SMs free (the other warps help the
+    // builds), then one CTA per SM, two when their threads do not reach n
+    const int warps = (n + 31) / 32;
+    const int want = n <= kOneCtaPerSm * kScanThreads ? min(warps, kOneCtaPerSm) : 2 * kOneCtaPerSm;
+    return rcc2 ? launch_coop<FusedStepArgs, StepParams>(k_list_steps<true>, want, st, a, p)
+                : launch_coop<FusedStepArgs, StepParams>(k_list_steps<false>, want, st, a, p);
 }
 
 cudaError_t launch_lj_nbr(const CellGrid &g, const CellBufs &b, const float4 *xq,

@@ -1526,6 +1526,17 @@ cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4
                               const int *typ, int n, const PairTab *tab, const float *rcc2,
                               float skin, const NbrList &l, int *flags, const int *gate,
                               unsigned *bar, cudaStream_t st);
+// `steps` steps (at most kMaxFusedSteps) from the device step counter on, of a
+// simulation of n <= kMaxFusedNps whose pair forces all come from the lists, in one
+// cooperative launch; I as for the integrator, bar: three words for the barrier and
+// three for the gates, sxq2 a second array of cell-ordered
+// records like b.sxq (its record n far from every NP), F_lj [n][8] scratch.
+constexpr int kMaxFusedSteps = 256;
+constexpr int kMaxFusedNps = 65536;
+cudaError_t launch_list_steps(const CellGrid &g, const CellBufs &b, int n, const PairTab *tab,
+                              const float *rcc2, float skin, const NbrList &l, unsigned *bar,
+                              const IntArgs &I, const StepParams &p, float4 *sxq2, float *F_lj,
+                              int steps, cudaStream_t st);
 cudaError_t launch_lj_nbr(const CellGrid &g, const CellBufs &b, const float4 *xq,
                           const int *typ, int n, const PairTab *tab, const float *rcc2,
                           const NbrList &l, float *F_lj, int *gate, cudaStream_t st);

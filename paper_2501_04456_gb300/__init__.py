@@ -263,7 +263,7 @@ def npsim_get_state(h, n, out=None):
     optional (x, v, F) arrays to fill, e.g. views of page-locked host memory,
     which the device copies reach faster than pageable memory."""
     if out is None:
-        x, v, F = np.empty((n, 3)), np.empty((n, 3)), np.empty((n, 3))
+        x, v, F = np.empty((3, n, 3))  # back to back: one device copy
     else:
         x, v, F = out
         for a in (x, v, F):
@@ -570,9 +570,7 @@ def npsim_ens_step(h, n_steps):
 
 
 def npsim_ens_get_state(h, d, n):
-    x = np.empty((n, 3))
-    v = np.empty((n, 3))
-    F = np.empty((n, 3))
+    x, v, F = np.empty((3, n, 3))  # back to back: one device copy
     st = C.c_int64()
     _check(lib().npsim_ens_get_state(h, int(d), _p(x, C.c_double), _p(v, C.c_double),
                                      _p(F, C.c_double), C.byref(st)))
@@ -764,8 +762,7 @@ class Surrogate:
     def predict(self, X):
         X = _f32(X, (-1, self.n_in))
         B = X.shape[0]
-        m = np.zeros((B, self.n_out), np.float32)
-        sp = np.zeros((B, self.n_out), np.float32)
+        m, sp = np.empty((2, B, self.n_out), np.float32)  # back to back: one device copy
         _check(lib().npsim_surr_predict(self.h, _p(X, C.c_float), B, _p(m, C.c_float),
                                         _p(sp, C.c_float)))
         return m, sp

@@ -289,10 +289,11 @@ __global__ void k_positions_f64(const float4 *__restrict__ xq, const float *__re
 }
 
 // Host-facing copy of the state: AoS float64 n x 3 of the position (hi + lo),
-// the velocity and the force (hi + lo); any output may be NULL.
+// the velocity and the force (hi + lo); any output may be NULL.  x_lo, v and F are
+// rows of [.][ld] arrays.
 __global__ void k_state_aos(const float4 *__restrict__ xq, const float *__restrict__ x_lo,
                             const float *__restrict__ v, const float *__restrict__ F, int n,
-                            double *__restrict__ xo, double *__restrict__ vo,
+                            size_t ld, double *__restrict__ xo, double *__restrict__ vo,
                             double *__restrict__ Fo)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -301,18 +302,18 @@ __global__ void k_state_aos(const float4 *__restrict__ xq, const float *__restri
     if (xo) {
         const float4 h = xq[i];
         xo[3 * (size_t)i + 0] = (double)h.x + (double)x_lo[i];
-        xo[3 * (size_t)i + 1] = (double)h.y + (double)x_lo[n + i];
-        xo[3 * (size_t)i + 2] = (double)h.z + (double)x_lo[2 * n + i];
+        xo[3 * (size_t)i + 1] = (double)h.y + (double)x_lo[ld + i];
+        xo[3 * (size_t)i + 2] = (double)h.z + (double)x_lo[2 * ld + i];
     }
     if (vo) {
 #pragma unroll
         for (int d = 0; d < 3; ++d)
-            vo[3 * (size_t)i + d] = (double)v[d * n + i];
+            vo[3 * (size_t)i + d] = (double)v[d * ld + i];
     }
     if (Fo) {
 #pragma unroll
         for (int d = 0; d < 3; ++d)
-            Fo[3 * (size_t)i + d] = (double)F[d * n + i] + (double)F[(3 + d) * n + i];
+            Fo[3 * (size_t)i + d] = (double)F[d * ld + i] + (double)F[(3 + d) * ld + i];
     }
 }
 
@@ -337,9 +338,10 @@ __global__ void k_slot_sum(const float *__restrict__ slots, StreamK sk, int n_po
 } // namespace
 
 cudaError_t launch_state_aos(const float4 *xq, const float *x_lo, const float *v, const float *F,
-                             int n, double *xo, double *vo, double *Fo, cudaStream_t st)
+                             int n, size_t ld, double *xo, double *vo, double *Fo,
+                             cudaStream_t st)
 {
-    k_state_aos<<<(n + 255) / 256, 256, 0, st>>>(xq, x_lo, v, F, n, xo, vo, Fo);
+    k_state_aos<<<(n + 255) / 256, 256, 0, st>>>(xq, x_lo, v, F, n, ld, xo, vo, Fo);
     return cudaGetLastError();
 }
 

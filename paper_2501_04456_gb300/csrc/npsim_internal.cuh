@@ -1581,9 +1581,11 @@ cudaError_t launch_positions_f64(const float4 *xq, const float *x_lo, int n, dou
 cudaError_t launch_positions_f64_ld(const float4 *xq, const float *x_lo, int n, int ld,
                                     double *x, cudaStream_t st);
 // The state as host-facing AoS float64 (n x 3 each; NULL outputs are skipped):
-// position hi + lo, velocity, force hi + lo (F: [6][n] hi/lo SoA).
+// position hi + lo, velocity, force hi + lo.  x_lo, v and F are rows of [3][ld],
+// [3][ld] and [6][ld] arrays (ld = n, or one droplet's part of an ensemble's).
 cudaError_t launch_state_aos(const float4 *xq, const float *x_lo, const float *v, const float *F,
-                             int n, double *xo, double *vo, double *Fo, cudaStream_t st);
+                             int n, size_t ld, double *xo, double *vo, double *Fo,
+                             cudaStream_t st);
 
 // Test hooks (capi.cu)
 cudaError_t launch_philox(uint64_t seed, const uint32_t ctr[4], long long n_blocks,

@@ -64,8 +64,8 @@ struct npsim_surr {
     cudaStream_t st = nullptr;
     // prediction of a batch of up to bcap rows
     int bcap = 0;
-    float *xin = nullptr;          // normalised FP32 inputs (staging)
-    __nv_bfloat16 *xb = nullptr;   // the same in BF16
+    float *xin = nullptr;          // raw FP32 inputs (staging)
+    __nv_bfloat16 *xb = nullptr;   // normalised, padded, BF16
     float *y_all = nullptr;        // outputs of every network [n_nets][bcap][n_out_p]
     float *ystat = nullptr;        // ensemble mean and spread [2][bcap][n_out]
     // activations and gradients of the layer-by-layer passes, networks stacked:
@@ -80,8 +80,10 @@ struct npsim_surr {
     std::vector<float *> dzf;           // NL (the column sums read them at the end)
     float *loss = nullptr;              // [n_nets]
     float *outw = nullptr;
-    float *d_ym = nullptr, *d_ys = nullptr; // output de-normalisation (n_out)
+    float *d_ym = nullptr, *d_ys = nullptr; // output normalisation (n_out)
+    float *d_xm = nullptr, *d_xs = nullptr; // input normalisation (n_in)
     int *flags = nullptr;
+    int *h_flags = nullptr; // page-locked copy of the flags
     long long adam_t = 0;
     // dataset on the device, its staging and the shuffled orders (kept between calls)
     size_t ds_cap = 0;
@@ -96,7 +98,7 @@ struct npsim_surr {
             dfree2(D.Wt[l]);
         }
         for (float **p : {&W, &G, &mom, &var, &xin, &y_all, &ystat, &y, &yt, &dyf, &loss, &outw,
-                          &d_ym, &d_ys, &dsy, &ds_tmp})
+                          &d_ym, &d_ys, &d_xm, &d_xs, &dsy, &ds_tmp})
             dfree2(*p);
         for (__nv_bfloat16 **p : {&xb, &dyb, &dyT, &dz[0], &dz[1], &dzT[0], &dzT[1], &dsx})
             dfree2(*p);
@@ -109,6 +111,8 @@ struct npsim_surr {
         dfree2(mask);
         dfree2(d_idx);
         dfree2(flags);
+        if (h_flags)
+            cudaFreeHost(h_flags);
         if (st)
             cudaStreamDestroy(st);
     }
@@ -321,40 +325,58 @@ int adamw_step(npsim_surr *s, int k0, int nk, float lr, float wd)
     return NPSIM_OK;
 }
 
-// Upload (normalised, padded, BF16) inputs of `rows` samples into xb and the
-// (normalised, padded) targets into yt; rows beyond are zero.
-int upload_batch(npsim_surr *s, const float *X, const float *Y, int rows, int bp)
+// (v - mean) / std of rows x n raw values, padded with zeros to rows_p x n_p, as
+// BF16 (ob) or FP32 (of).
+__global__ void k_normalise(const float *__restrict__ v, int rows, int n, int rows_p, int n_p,
+                            const float *__restrict__ mean, const float *__restrict__ std,
+                            __nv_bfloat16 *__restrict__ ob, float *__restrict__ of)
 {
-    std::vector<float> xf((size_t)bp * s->n_in_p, 0.f);
-    for (int r = 0; r < rows; ++r)
-        for (int c = 0; c < s->n_in; ++c)
-            xf[(size_t)r * s->n_in_p + c] = (X[(size_t)r * s->n_in + c] - s->xm[c]) / s->xs[c];
-    SR_CUDA(cudaMemcpyAsync(s->xin, xf.data(), sizeof(float) * xf.size(), cudaMemcpyHostToDevice,
-                            s->st));
-    SR_CUDA(launch_f32_to_bf16(s->xin, (int)xf.size(), s->xb, s->st));
-    if (Y) {
-        std::vector<float> yf((size_t)bp * s->n_out_p, 0.f);
-        for (int r = 0; r < rows; ++r)
-            for (int c = 0; c < s->n_out; ++c)
-                yf[(size_t)r * s->n_out_p + c] =
-                    (Y[(size_t)r * s->n_out + c] - s->ym[c]) / s->ys[c];
-        SR_CUDA(cudaMemcpyAsync(s->yt, yf.data(), sizeof(float) * yf.size(),
-                                cudaMemcpyHostToDevice, s->st));
-        SR_CUDA(cudaStreamSynchronize(s->st));
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (size_t)rows_p * n_p)
+        return;
+    const int r = (int)(e / n_p), c = (int)(e - (size_t)r * n_p);
+    const float q =
+        r < rows && c < n ? __fdiv_rn(__fsub_rn(v[(size_t)r * n + c], mean[c]), std[c]) : 0.f;
+    if (ob)
+        ob[e] = __float2bfloat16_rn(q);
+    else
+        of[e] = q;
+}
+
+// Raw host rows to the device (staged in raw) and normalised there.
+int upload_rows(npsim_surr *s, const float *v, int rows, int n, int rows_p, int n_p, float *raw,
+                const float *mean, const float *std, __nv_bfloat16 *ob, float *of)
+{
+    SR_CUDA(cudaMemcpyAsync(raw, v, sizeof(float) * (size_t)rows * n, cudaMemcpyHostToDevice, s->st));
+    const size_t e = (size_t)rows_p * n_p;
+    k_normalise<<<(unsigned)((e + 255) / 256), 256, 0, s->st>>>(raw, rows, n, rows_p, n_p, mean, std,
+                                                                ob, of);
+    SR_CUDA(cudaGetLastError());
+    return NPSIM_OK;
+}
+
+// The error flags behind everything queued so far: copied with the call's last
+// copies, looked at after the stream has been waited for.
+cudaError_t fetch_flags(npsim_surr *s)
+{
+    return cudaMemcpyAsync(s->h_flags, s->flags, sizeof(int), cudaMemcpyDeviceToHost, s->st);
+}
+
+int flags_status(npsim_surr *s)
+{
+    const int h = *s->h_flags;
+    if (h) {
+        SR_CUDA(cudaMemsetAsync(s->flags, 0, sizeof(int), s->st));
+        return report_error(NPSIM_ERR_TIMEOUT, "a tensor-core wait expired (flags 0x%x)", h);
     }
     return NPSIM_OK;
 }
 
 int check_flags(npsim_surr *s)
 {
-    int h = 0;
-    SR_CUDA(cudaMemcpyAsync(&h, s->flags, sizeof(int), cudaMemcpyDeviceToHost, s->st));
+    SR_CUDA(fetch_flags(s));
     SR_CUDA(cudaStreamSynchronize(s->st));
-    if (h) {
-        SR_CUDA(cudaMemsetAsync(s->flags, 0, sizeof(int), s->st));
-        return report_error(NPSIM_ERR_TIMEOUT, "a tensor-core wait expired (flags 0x%x)", h);
-    }
-    return NPSIM_OK;
+    return flags_status(s);
 }
 
 // One minibatch of every network of a group: rows idx[0 .. rows) of network
@@ -488,10 +510,15 @@ int npsim_surr_create(int32_t n_in, int32_t n_hidden, int32_t n_layers, int32_t 
     if (dmalloc(&s->loss, (size_t)n_nets) != cudaSuccess || dmalloc(&s->flags, 1) != cudaSuccess ||
         dmalloc(&s->outw, (size_t)s->n_out_p) != cudaSuccess ||
         dmalloc(&s->d_ym, (size_t)n_out) != cudaSuccess ||
-        dmalloc(&s->d_ys, (size_t)n_out) != cudaSuccess)
+        dmalloc(&s->d_ys, (size_t)n_out) != cudaSuccess ||
+        dmalloc(&s->d_xm, (size_t)n_in) != cudaSuccess ||
+        dmalloc(&s->d_xs, (size_t)n_in) != cudaSuccess ||
+        cudaHostAlloc((void **)&s->h_flags, sizeof(int), cudaHostAllocDefault) != cudaSuccess)
         return bail(report_error(NPSIM_ERR_OOM, "surrogate scratch"));
     cudaMemcpy(s->d_ym, s->ym.data(), sizeof(float) * n_out, cudaMemcpyHostToDevice);
     cudaMemcpy(s->d_ys, s->ys.data(), sizeof(float) * n_out, cudaMemcpyHostToDevice);
+    cudaMemcpy(s->d_xm, s->xm.data(), sizeof(float) * n_in, cudaMemcpyHostToDevice);
+    cudaMemcpy(s->d_xs, s->xs.data(), sizeof(float) * n_in, cudaMemcpyHostToDevice);
     std::vector<float> ow(s->n_out_p, 0.f);
     for (int c = 0; c < n_out; ++c)
         ow[c] = 1.f;
@@ -534,6 +561,10 @@ int npsim_surr_set_norm(npsim_surr_t s, const float *x_mean, const float *x_std,
     SR_CUDA(cudaMemcpyAsync(s->d_ym, s->ym.data(), sizeof(float) * s->n_out,
                             cudaMemcpyHostToDevice, s->st));
     SR_CUDA(cudaMemcpyAsync(s->d_ys, s->ys.data(), sizeof(float) * s->n_out,
+                            cudaMemcpyHostToDevice, s->st));
+    SR_CUDA(cudaMemcpyAsync(s->d_xm, s->xm.data(), sizeof(float) * s->n_in,
+                            cudaMemcpyHostToDevice, s->st));
+    SR_CUDA(cudaMemcpyAsync(s->d_xs, s->xs.data(), sizeof(float) * s->n_in,
                             cudaMemcpyHostToDevice, s->st));
     SR_CUDA(cudaStreamSynchronize(s->st));
     return NPSIM_OK;
@@ -581,7 +612,9 @@ int npsim_surr_grads(npsim_surr_t s, int32_t net, const float *X, const float *Y
     if (!rc)
         rc = alloc_rows(s, (size_t)bp, true);
     if (!rc)
-        rc = upload_batch(s, X, Y, B, bp);
+        rc = upload_rows(s, X, B, s->n_in, bp, s->n_in_p, s->xin, s->d_xm, s->d_xs, s->xb, nullptr);
+    if (!rc) // the targets' raw rows pass through the gradient buffer
+        rc = upload_rows(s, Y, B, s->n_out, bp, s->n_out_p, s->dyf, s->d_ym, s->d_ys, nullptr, s->yt);
     if (rc)
         return rc;
     SR_CUDA(launch_transpose_bf16(s->xb, bp, s->n_in_p, s->n_in_p, s->aT[0], bp, s->st));
@@ -628,27 +661,18 @@ int npsim_surr_train(npsim_surr_t s, const float *X, const float *Y, int32_t n_s
         dfree2(s->ds_tmp);
         dfree2(s->d_idx);
         SR_CUDA(dmalloc(&s->dsx, (size_t)n_samples * s->n_in_p));
-        SR_CUDA(dmalloc(&s->ds_tmp, (size_t)n_samples * s->n_in_p));
+        SR_CUDA(dmalloc(&s->ds_tmp, (size_t)n_samples * std::max(s->n_in, s->n_out)));
         SR_CUDA(dmalloc(&s->dsy, (size_t)n_samples * s->n_out_p));
         SR_CUDA(dmalloc(&s->d_idx, (size_t)n_samples * s->n_nets));
         s->ds_cap = (size_t)n_samples;
     }
-    {
-        std::vector<float> xf((size_t)n_samples * s->n_in_p, 0.f);
-        std::vector<float> yf((size_t)n_samples * s->n_out_p, 0.f);
-        for (int r = 0; r < n_samples; ++r) {
-            for (int c = 0; c < s->n_in; ++c)
-                xf[(size_t)r * s->n_in_p + c] = (X[(size_t)r * s->n_in + c] - s->xm[c]) / s->xs[c];
-            for (int c = 0; c < s->n_out; ++c)
-                yf[(size_t)r * s->n_out_p + c] = (Y[(size_t)r * s->n_out + c] - s->ym[c]) / s->ys[c];
-        }
-        SR_CUDA(cudaMemcpyAsync(s->ds_tmp, xf.data(), sizeof(float) * xf.size(),
-                                cudaMemcpyHostToDevice, s->st));
-        SR_CUDA(launch_f32_to_bf16(s->ds_tmp, (int)xf.size(), s->dsx, s->st));
-        SR_CUDA(cudaMemcpyAsync(s->dsy, yf.data(), sizeof(float) * yf.size(),
-                                cudaMemcpyHostToDevice, s->st));
-        SR_CUDA(cudaStreamSynchronize(s->st)); // xf and yf live in this block
-    }
+    rc = upload_rows(s, X, n_samples, s->n_in, n_samples, s->n_in_p, s->ds_tmp, s->d_xm, s->d_xs,
+                     s->dsx, nullptr);
+    if (!rc)
+        rc = upload_rows(s, Y, n_samples, s->n_out, n_samples, s->n_out_p, s->ds_tmp, s->d_ym,
+                         s->d_ys, nullptr, s->dsy);
+    if (rc)
+        return rc;
     // every network's shuffled order of an epoch, drawn network by network; the next
     // epoch's is drawn while this one runs
     std::vector<int> order[2];
@@ -701,6 +725,8 @@ int npsim_surr_train(npsim_surr_t s, const float *X, const float *Y, int32_t n_s
     }
     if (rc)
         return rc;
+    if (e == cudaSuccess && epochs == 0)
+        e = cudaStreamSynchronize(s->st); // X and Y are the caller's again
     if (e != cudaSuccess)
         return report_error(NPSIM_ERR_CUDA, "training: %s", cudaGetErrorString(e));
     if (final_loss)
@@ -717,7 +743,7 @@ int npsim_surr_predict(npsim_surr_t s, const float *X, int32_t B, float *Y_mean,
     int rc = alloc_batch(s, bp);
     if (rc)
         return rc;
-    rc = upload_batch(s, X, nullptr, B, bp);
+    rc = upload_rows(s, X, B, s->n_in, bp, s->n_in_p, s->xin, s->d_xm, s->d_xs, s->xb, nullptr);
     if (rc)
         return rc;
     // NPSIM_SURR_LAYERED selects the layer-by-layer GEMM path (same arithmetic)
@@ -753,12 +779,18 @@ int npsim_surr_predict(npsim_surr_t s, const float *X, int32_t B, float *Y_mean,
                                                      s->n_out, s->d_ym, s->d_ys, d_mean,
                                                      d_spread);
     SR_CUDA(cudaGetLastError());
-    SR_CUDA(cudaMemcpyAsync(Y_mean, d_mean, sizeof(float) * ne, cudaMemcpyDeviceToHost, s->st));
-    if (Y_spread)
-        SR_CUDA(cudaMemcpyAsync(Y_spread, d_spread, sizeof(float) * ne, cudaMemcpyDeviceToHost,
-                                s->st));
+    SR_CUDA(fetch_flags(s));
+    if (Y_spread == Y_mean + ne) { // back to back on the host too: one copy
+        SR_CUDA(cudaMemcpyAsync(Y_mean, d_mean, sizeof(float) * 2 * (size_t)ne,
+                                cudaMemcpyDeviceToHost, s->st));
+    } else {
+        SR_CUDA(cudaMemcpyAsync(Y_mean, d_mean, sizeof(float) * ne, cudaMemcpyDeviceToHost, s->st));
+        if (Y_spread)
+            SR_CUDA(cudaMemcpyAsync(Y_spread, d_spread, sizeof(float) * ne, cudaMemcpyDeviceToHost,
+                                    s->st));
+    }
     SR_CUDA(cudaStreamSynchronize(s->st));
-    return check_flags(s);
+    return flags_status(s);
 }
 
 int npsim_test_wait_cycles(int64_t cycles)

@@ -1577,6 +1577,25 @@ bool fused_steps(const npsim_sim *s)
     return s->cell && !s->ap && s->n <= kMaxFusedNps && !s->profiling;
 }
 
+// No pair force at all: every NP's steps are its own.
+bool free_steps(const npsim_sim *s) { return !s->cell && !s->ap && !s->profiling; }
+
+int enqueue_free(npsim_sim *s, int k)
+{
+    IntArgs a{};
+    a.x_lo = s->x_lo;
+    a.v = s->v;
+    a.F = s->F;
+    a.typ = s->typ;
+    a.xq = s->xq;
+    a.spring = s->d_spring;
+    a.step = s->d_step;
+    a.flags = s->d_flags;
+    a.done = s->d_done;
+    NP_CUDA(launch_free_steps(a, s->sp, k, s->user));
+    return NPSIM_OK;
+}
+
 int enqueue_fused(npsim_sim *s, int k)
 {
     if (!s->sxq2) {
@@ -1609,6 +1628,15 @@ int enqueue_steps(npsim_sim *s, int64_t n_steps)
         int rc0 = regrid_if_needed(s);
         if (rc0)
             return rc0;
+        if (free_steps(s)) {
+            const int k = (int)std::min<int64_t>(rem, kMaxFreeSteps);
+            int rc = enqueue_free(s, k);
+            if (rc)
+                return rc;
+            rem -= k;
+            s->step += k;
+            continue;
+        }
         if (fused_steps(s)) {
             int k = (int)std::min<int64_t>(rem, kMaxFusedSteps);
             if (follows_droplet(s)) // stop at the next multiple of kRegridPeriod

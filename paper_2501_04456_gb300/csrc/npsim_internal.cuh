@@ -1232,6 +1232,54 @@ struct IntArgs {
     unsigned *done;          // CTAs counted in by the committing launch (zero between)
 };
 
+// Velocity and position of one particle through the closing half kick B and / or
+// the B-A-O-A part of the next step (or the overdamped update, or step (vi) as
+// printed), from the force f; noise of particle noise_idx at `step`.
+template <bool DO_B, bool DO_A>
+__device__ __forceinline__ void kick_drift(const TypeCoef &tc, int integrator, float hdt,
+                                           uint64_t seed, uint32_t noise_idx, long long step,
+                                           const float (&f)[3], float (&v)[3], float (&xhi)[3],
+                                           float (&xlo)[3])
+{
+    const bool baoab = integrator == 0;
+    if (DO_B && baoab) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            v[d] = __fmaf_rn(tc.hdt_m, f[d], v[d]);
+    }
+    if (DO_A) {
+        float nz[3];
+        normals3(seed, noise_idx, step, 0u, nz[0], nz[1], nz[2]);
+        if (baoab) {
+            // the two A half steps around the O step add dt/2 (v' + v'') to the
+            // position (the O step does not depend on x): one compensated add
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                v[d] = __fmaf_rn(tc.hdt_m, f[d], v[d]);               // B
+                const float va = v[d];                                // A (first half)
+                v[d] = __fmaf_rn(tc.c1f, v[d],
+                                 __fmaf_rn(tc.c1lo, v[d], __fmul_rn(tc.sd_of, nz[d]))); // O
+                df_add(xhi[d], xlo[d], __fmul_rn(hdt, __fadd_rn(va, v[d]))); // A + A
+            }
+        } else if (integrator == 1) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                df_add(xhi[d], xlo[d], __fmaf_rn(f[d], tc.dt_mob, __fmul_rn(tc.sd_bdf, nz[d])));
+        } else { // step (vi) as printed: drag and force, a kick of fixed size, drift
+            const float nn = sqrtf(__fmaf_rn(nz[0], nz[0], __fmaf_rn(nz[1], nz[1],
+                                                                     __fmul_rn(nz[2], nz[2]))));
+            const float a = nn > 0.0f ? __fdiv_rn(tc.kick, nn) : 0.0f; // kick / |n|
+            const float dt = 2.0f * hdt;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                v[d] = __fmaf_rn(tc.dt_m, f[d], __fmaf_rn(-tc.gdt, v[d], v[d]));
+                v[d] = __fmaf_rn(a, nz[d], v[d]);
+                df_add(xhi[d], xlo[d], __fmul_rn(dt, v[d]));
+            }
+        }
+    }
+}
+
 // One particle's update after its force (Fh + Fl) has been assembled: store F
 // (MODE_FORCES, MODE_B), the closing half kick B (MODE_BA, MODE_B) and the
 // B-A-O-A part of the next step, or the overdamped update (MODE_A, MODE_BA).
@@ -1264,43 +1312,9 @@ __device__ __forceinline__ void advance_particle(int i, int n, uint32_t noise_id
     const float f[3] = {__fadd_rn(Fh[0], Fl[0]), __fadd_rn(Fh[1], Fl[1]),
                         __fadd_rn(Fh[2], Fl[2])};
     float v[3] = {v0[0], v0[1], v0[2]}; // v_ at i, read by the caller
-    const bool baoab = integrator == 0;
-    if (DO_B && baoab) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d)
-            v[d] = __fmaf_rn(tc.hdt_m, f[d], v[d]);
-    }
+    float xhi[3] = {xh.x, xh.y, xh.z}, xlo[3] = {lx, ly, lz};
+    kick_drift<DO_B, DO_A>(tc, integrator, hdt, seed, noise_idx, step, f, v, xhi, xlo);
     if (DO_A) {
-        float nz[3];
-        normals3(seed, noise_idx, step, 0u, nz[0], nz[1], nz[2]);
-        float xhi[3] = {xh.x, xh.y, xh.z}, xlo[3] = {lx, ly, lz};
-        if (baoab) {
-            // the two A half steps around the O step add dt/2 (v' + v'') to the
-            // position (the O step does not depend on x): one compensated add
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                v[d] = __fmaf_rn(tc.hdt_m, f[d], v[d]);               // B
-                const float va = v[d];                                // A (first half)
-                v[d] = __fmaf_rn(tc.c1f, v[d],
-                                 __fmaf_rn(tc.c1lo, v[d], __fmul_rn(tc.sd_of, nz[d]))); // O
-                df_add(xhi[d], xlo[d], __fmul_rn(hdt, __fadd_rn(va, v[d]))); // A + A
-            }
-        } else if (integrator == 1) {
-#pragma unroll
-            for (int d = 0; d < 3; ++d)
-                df_add(xhi[d], xlo[d], __fmaf_rn(f[d], tc.dt_mob, __fmul_rn(tc.sd_bdf, nz[d])));
-        } else { // step (vi) as printed: drag and force, a kick of fixed size, drift
-            const float nn = sqrtf(__fmaf_rn(nz[0], nz[0], __fmaf_rn(nz[1], nz[1],
-                                                                     __fmul_rn(nz[2], nz[2]))));
-            const float a = nn > 0.0f ? __fdiv_rn(tc.kick, nn) : 0.0f; // kick / |n|
-            const float dt = 2.0f * hdt;
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                v[d] = __fmaf_rn(tc.dt_m, f[d], __fmaf_rn(-tc.gdt, v[d], v[d]));
-                v[d] = __fmaf_rn(a, nz[d], v[d]);
-                df_add(xhi[d], xlo[d], __fmul_rn(dt, v[d]));
-            }
-        }
         xq[i] = make_float4(xhi[0], xhi[1], xhi[2], xh.w);
         if (sxq) // the neighbour-list kernel's cell-ordered copy
             sxq[cell_pos[i]] = make_float4(xhi[0], xhi[1], xhi[2], __int_as_float(ti));
@@ -1321,6 +1335,10 @@ __device__ __forceinline__ void advance_particle(int i, int n, uint32_t noise_id
     v_[2 * n + i] = v[2];
 }
 
+// `steps` steps (at most kMaxFreeSteps) of a simulation without pair forces, from the
+// device step counter on, in one launch.
+constexpr int kMaxFreeSteps = 64;
+cudaError_t launch_free_steps(const IntArgs &a, const StepParams &p, int steps, cudaStream_t st);
 cudaError_t launch_integrate(int mode, const IntArgs &a, const StepParams &p,
                              cudaStream_t st);
 // The integrator's sum of the all-pairs partial slots alone, for positions

@@ -1,6 +1,7 @@
-"""Many steps per launch for small droplets on neighbour lists: the same bits as the
-separate kernels (the path taken while the kernels are timed apart), across list
-builds, list growth and a regrid, for every integrator and both list force terms."""
+"""Many steps per launch, for small droplets on neighbour lists and for NPs without
+pair forces: the same bits as the separate kernels (the path taken while the kernels
+are timed apart), across list builds, list growth and a regrid, for every integrator
+and both list force terms."""
 import numpy as np
 import pytest
 
@@ -42,6 +43,33 @@ def test_same_bits_as_separate_kernels(P, name, n):
                 assert np.array_equal(got, ref), (k,)
             assert np.array_equal(a.forces(1), b.forces(1)), (k,)
         assert a.nbr_info()[2] == b.nbr_info()[2]  # as many list builds
+
+
+@pytest.mark.parametrize("n", [1, 257, 5000])
+@pytest.mark.parametrize("integrator", [0, 1, 2])
+@pytest.mark.parametrize("wall", [0, 1, 2])
+def test_free_steps_same_bits(P, n, integrator, wall):
+    """Without pair forces; steps around the 64 of one launch, up to and past the
+    time at which the droplet has gone (R(t) = 0)."""
+    sc = small(wl.config3(), n)
+    sc = with_(sc, coulomb=False, lj_mode=0, integrator=integrator, g=0.3, omega=0.2, rot_mode=1,
+               v_kick=0.02, wall=wall > 0, wall_band=wall == 2)
+    sc = with_(sc, k_evap=sc.R0 ** 2 / (200 * sc.dt))
+    types, x, v = wl.initial_state(sc)
+    with P.Sim(sc, x, v, types) as a, P.Sim(sc, x, v, types) as b:
+        b.profile(True)
+        for k in (1, 63, 64, 65, 130):
+            codes = []
+            for s in (a, b):
+                try:
+                    s.step(k)
+                    codes.append(0)
+                except P.NpsimError as e:  # an NP left behind by the interface
+                    codes.append(e.code)
+            assert codes[0] == codes[1]
+            for got, ref in zip(a.state(), b.state()):
+                assert np.array_equal(got, ref), (k,)
+            assert np.array_equal(a.forces(0), b.forces(0)), (k,)
 
 
 def test_across_a_regrid_and_recorded_frames(P):

@@ -2532,8 +2532,10 @@ EnsGeometry ens_geometry(npsim_ens *e, int shape, int grid_target)
         }
     }
     G.row_first.push_back((int)G.items.size());
-    std::stable_sort(G.items.begin(), G.items.end(), [](const EnsItem &a, const EnsItem &b) {
-        return a.jt1 - a.jt0 > b.jt1 - b.jt0;
+    // longest first, those nearest the diagonal (rich in LJ) before others
+    std::stable_sort(G.items.begin(), G.items.end(), [tri](const EnsItem &a, const EnsItem &b) {
+        const int la = a.jt1 - a.jt0, lb = b.jt1 - b.jt0;
+        return la != lb ? la > lb : a.jt0 - tri * a.row < b.jt0 - tri * b.row;
     });
     G.floats = G.items.size() * 6 * (size_t)itile + (size_t)col;
     G.ctas = (int)std::min<size_t>((size_t)std::max(grid_target, 1), G.items.size());

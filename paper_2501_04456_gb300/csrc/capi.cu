@@ -219,6 +219,7 @@ struct npsim_sim {
     NbrList nl{};          // Verlet list over the cells (cell-list LJ)
     int *d_gate = nullptr; // 1: rebuild the cell and neighbour lists at the next pass
     unsigned *list_bar = nullptr; // counters of the list kernels' grid barrier [3], gates [3]
+    int fused_cap = 0;            // largest n that takes fused steps
     float4 *sxq2 = nullptr;       // the other cell-ordered records of fused steps (lazy)
 
     bool ap = false, ap_lj = false;
@@ -1450,6 +1451,7 @@ int create_impl(const npsim_type_t *types, const npsim_params_t *params, int64_t
         BAIL_CUDA(dalloc(&s->nl.builds, 1));
         BAIL_CUDA(cudaMemset(s->nl.builds, 0, sizeof(unsigned long long)));
         BAIL_CUDA(dalloc(&s->d_gate, 1));
+        s->fused_cap = list_steps_capacity();
         BAIL_CUDA(dalloc(&s->list_bar, 6));
         BAIL_CUDA(cudaMemset(s->list_bar, 0, 6 * sizeof(unsigned)));
         BAIL_CUDA(cudaMemset(s->nl.nnbr, 0, sizeof(int) * (size_t)n));
@@ -1574,7 +1576,7 @@ int regrid_if_needed(npsim_sim *s)
 // launch (not while the kernels are timed apart).
 bool fused_steps(const npsim_sim *s)
 {
-    return s->cell && !s->ap && s->n <= kMaxFusedNps && !s->profiling;
+    return s->cell && !s->ap && s->n <= s->fused_cap && !s->profiling;
 }
 
 // No pair force at all: every NP's steps are its own.
@@ -1829,7 +1831,7 @@ int npsim_launches_per_step(npsim_sim_t s, int *launches)
     NP_REQUIRE(s && launches, "sim and launches are required");
     // integrator, all-pairs (and the sum of its partials), the gated list build, the
     // list LJ forces; one launch where it takes many steps
-    *launches = s->cell && !s->ap && s->n <= kMaxFusedNps ? 1 : 1 + (s->ap ? (s->sk.tri ? 2 : 1) : 0) + (s->cell ? 2 : 0);
+    *launches = s->cell && !s->ap && s->n <= s->fused_cap ? 1 : 1 + (s->ap ? (s->sk.tri ? 2 : 1) : 0) + (s->cell ? 2 : 0);
     return NPSIM_OK;
 }
 

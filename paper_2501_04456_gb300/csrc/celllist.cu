@@ -617,17 +617,16 @@ __device__ __noinline__ void cell_slot_forces(int p, const CellGrid g, const int
 // slots, and for the partners from the nearby cells -- and the 32-byte force
 // record goes to the NP's index i = sorted[p], where the integrator reads it.
 // An NP whose list overflowed sums over the cells of that build instead (a
-// superset of its list).  Returns the (hi x, y, z, lo x | lo y, z, 0, 0) record in
-// o0, o1.
+// superset of its list).  pi: its record, cur: its first list block, cnt: its count.
+// Returns the (hi x, y, z, lo x | lo y, z, 0, 0) record in o0, o1.
 template <bool COUL>
-__device__ __forceinline__ void slot_forces(int p, int i, const CellGrid &g, const int *start,
+__device__ __forceinline__ void slot_forces(int p, int i, const float4 pi, uint4 cur, int cnt,
+                                            const CellGrid &g, const int *start,
                                             const int *sorted, const int *key,
                                             const float4 *sxq, int n, int cap,
-                                            const unsigned *nbr, const int *nnbr, float *F_lj,
-                                            const float4 *s_tab, const float *s_rcc2, float4 &o0,
-                                            float4 &o1)
+                                            const unsigned *nbr, float *F_lj, const float4 *s_tab,
+                                            const float *s_rcc2, float4 &o0, float4 &o1)
 {
-    const float4 pi = sxq[p];
     const int ti = __float_as_int(pi.w);
     const int row = ti * NPSIM_MAX_TYPES;
     float hx = 0.f, hy = 0.f, hz = 0.f, lx = 0.f, ly = 0.f, lz = 0.f;
@@ -671,8 +670,6 @@ __device__ __forceinline__ void slot_forces(int p, int i, const CellGrid &g, con
     // records out of L1 and L2.
     const uint4 *nb4 = reinterpret_cast<const uint4 *>(nbr);
     const uint4 far4 = make_uint4((unsigned)n, (unsigned)n, (unsigned)n, (unsigned)n);
-    uint4 cur = __ldcs(nb4 + p);
-    const int cnt = nnbr[p];
     if (cnt > cap) {
         cell_slot_forces<COUL>(p, g, start, sorted, key, sxq, F_lj, s_tab, s_rcc2);
         const float4 *o = reinterpret_cast<const float4 *>(F_lj + 8 * (size_t)i);
@@ -740,9 +737,11 @@ k_lj_nbr(const __grid_constant__ CellGrid g, const int *__restrict__ start, cons
     const int p = (int)(gridDim.x - 1 - blockIdx.x) * (int)blockDim.x + (int)threadIdx.x;
     if (p < n) {
         const int i = sorted[p];
+        const float4 pi = sxq[p];
+        const uint4 cur = __ldcs(reinterpret_cast<const uint4 *>(nbr) + p);
         float4 o0, o1;
-        slot_forces<COUL>(p, i, g, start, sorted, key, sxq, n, cap, nbr, nnbr, F_lj, s_tab, s_rcc2,
-                          o0, o1);
+        slot_forces<COUL>(p, i, pi, cur, nnbr[p], g, start, sorted, key, sxq, n, cap, nbr, F_lj,
+                          s_tab, s_rcc2, o0, o1);
         // one 32-byte record per NP, a whole DRAM sector
         float4 *o = reinterpret_cast<float4 *>(F_lj + 8 * (size_t)i);
         o[0] = o0;
@@ -758,12 +757,13 @@ k_lj_nbr(const __grid_constant__ CellGrid g, const int *__restrict__ start, cons
 //   list forces, external forces, B and the next step's A part of each NP by the
 //   thread that holds its slot; after the last step's B the counters move on.
 // Arithmetic and order are those of the separate kernels (the same functions), so a
-// run that mixes both is bit-identical.  While some threads still read their
-// partners' records of the current positions others already write new ones, so the
-// cell-ordered records alternate between two arrays; the last step's pass, which
-// moves nothing, leaves them in the first.  The state is read by particle index in
-// cell order (scattered): with the state in L2 that costs less than the launches,
-// beyond kMaxFusedNps it does not.
+// run that mixes both is bit-identical.  Every thread holds at most one NP, whose
+// state, first list block and count stay in its registers between builds, and draws
+// the next step's noise before it waits at the barrier: after the barrier only the
+// partners' records are on the way to its force.  While some threads still read
+// their partners' records of the current positions others already write new ones, so
+// the cell-ordered records alternate between two arrays; the last step's pass, which
+// moves nothing, leaves them in the first.
 struct FusedStepArgs {
     ListBuildArgs L;
     IntArgs I;          // xq, x_lo, v, F, typ, spring, step, flags, half_skin2, x_ref
@@ -777,42 +777,44 @@ struct FusedStepArgs {
     int steps;
 };
 
-// One particle's external force added to its list force and its update, as
-// update_particle of the integrator does.
-template <int MODE>
-__device__ __forceinline__ void fused_update(const FusedStepArgs &a, const StepParams &p,
-                                             const TypeCoef *s_tc, float R0f, long long step, int i,
-                                             float4 o0, float4 o1, float4 *sxq, int *raise)
+// The NP of one slot between builds.
+struct SlotNp {
+    int i, ti, cnt;
+    uint4 first;               // first list block
+    float q, xhi[3], xlo[3], v[3], ref[3];
+};
+
+__device__ __forceinline__ void slot_load(const FusedStepArgs &a, int n, int p, SlotNp &s)
 {
     const IntArgs &I = a.I;
-    const int n = p.n;
-    const int ti = I.typ[i];
-    const TypeCoef &tc = s_tc[ti];
-    const float4 xh = I.xq[i];
-    const float lx = I.x_lo[i], ly = I.x_lo[n + i], lz = I.x_lo[2 * n + i];
-    const float v[3] = {I.v[i], I.v[n + i], I.v[2 * n + i]};
-    float Fh[3] = {0.f, 0.f, 0.f}, Fl[3] = {0.f, 0.f, 0.f};
-    if (MODE != MODE_A) {
-        df_add_df(Fh[0], Fl[0], o0.x, o0.w);
-        df_add_df(Fh[1], Fl[1], o0.y, o1.x);
-        df_add_df(Fh[2], Fl[2], o0.z, o1.y);
-        float ex, ey, ez;
-        external_force(xh, lx, ly, lz, tc.kw, tc.mg, tc.mw2,
-                       I.spring[(step & 1) * NPSIM_MAX_TYPES + ti], p.wall, p.rot_mode, ex, ey, ez,
-                       R0f, I.flags);
-        df_add(Fh[0], Fl[0], ex);
-        df_add(Fh[1], Fl[1], ey);
-        df_add(Fh[2], Fl[2], ez);
-    } else {
+    s.i = a.L.b.sorted[p];
+    s.cnt = a.L.nnbr[p];
+    s.first = __ldcs(reinterpret_cast<const uint4 *>(a.L.nbr) + p);
+    s.ti = I.typ[s.i];
+    const float4 x = I.xq[s.i], r = a.L.x_ref[s.i];
+    s.q = x.w;
+    s.xhi[0] = x.x;
+    s.xhi[1] = x.y;
+    s.xhi[2] = x.z;
+    s.ref[0] = r.x;
+    s.ref[1] = r.y;
+    s.ref[2] = r.z;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            Fh[d] = I.F[d * n + i];
-            Fl[d] = I.F[(3 + d) * n + i];
-        }
+    for (int d = 0; d < 3; ++d) {
+        s.xlo[d] = I.x_lo[d * n + s.i];
+        s.v[d] = I.v[d * n + s.i];
     }
-    advance_particle<MODE>(i, n, (uint32_t)i, tc, p.integrator, 0.5f * (float)p.dt, p.seed, step, xh,
-                           lx, ly, lz, Fh, Fl, v, I.x_lo, I.v, I.F, I.xq, I.flags, I.x_ref, raise,
-                           I.half_skin2, sxq, a.L.b.pos, ti);
+}
+
+__device__ __forceinline__ void slot_store(const FusedStepArgs &a, int n, const SlotNp &s)
+{
+    const IntArgs &I = a.I;
+    I.xq[s.i] = make_float4(s.xhi[0], s.xhi[1], s.xhi[2], s.q);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        I.x_lo[d * n + s.i] = s.xlo[d];
+        I.v[d * n + s.i] = s.v[d];
+    }
 }
 
 template <bool COUL>
@@ -841,39 +843,92 @@ k_list_steps(const __grid_constant__ FusedStepArgs a, const __grid_constant__ St
             a.I.spring[((s + 1) & 1) * NPSIM_MAX_TYPES + threadIdx.x] =
                 spring_entry(p.R0, p.k_evap, p.dt, s + 1, p.tc[threadIdx.x].half_sigma);
     };
-    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float hdt = 0.5f * (float)p.dt;
     next_spring(step0);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        fused_update<MODE_A>(a, p, s_tc, R0f, step0, i, none, none, L.b.sxq,
-                             reinterpret_cast<int *>(a.gates) + 1);
-    // slots spread over the CTAs a warp at a time
-    const int first = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+    // the first step's A part, by particle (the slots may be those of no build yet)
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const float4 x = a.I.xq[i];
+        const float v[3] = {a.I.v[i], a.I.v[n + i], a.I.v[2 * n + i]};
+        float Fh[3], Fl[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            Fh[d] = a.I.F[d * n + i];
+            Fl[d] = a.I.F[(3 + d) * n + i];
+        }
+        const int ti = a.I.typ[i];
+        advance_particle<MODE_A>(i, n, (uint32_t)i, s_tc[ti], p.integrator, hdt, p.seed, step0, x,
+                                 a.I.x_lo[i], a.I.x_lo[n + i], a.I.x_lo[2 * n + i], Fh, Fl, v,
+                                 a.I.x_lo, a.I.v, a.I.F, a.I.xq, a.I.flags, a.I.x_ref,
+                                 reinterpret_cast<int *>(a.gates) + 1, a.I.half_skin2, L.b.sxq,
+                                 L.b.pos, ti);
+    }
+    // slots spread over the CTAs a warp at a time (the launch has a thread for each)
+    const int slot = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+    const bool mine = slot < n;
+    SlotNp s{};
+    float nz[3] = {0.f, 0.f, 0.f};
     for (int j = 1; j <= a.steps; ++j) {
+        const bool last = j == a.steps;
         if (!grid_barrier(L.bar, phase, L.flags, &S.ok))
             return;
         float4 *cur = (j & 1) ? L.b.sxq : a.sxq2, *nxt = (j & 1) ? a.sxq2 : L.b.sxq;
         volatile unsigned *w = a.gates;
-        if (w[j % 3] != 0u || (j == 1 && *(volatile int *)a.gate != 0)) {
-            if (!list_build(L, cur, S, phase) || !grid_barrier(L.bar, phase, L.flags, &S.ok))
+        const bool build = w[j % 3] != 0u || (j == 1 && *(volatile int *)a.gate != 0);
+        if (build) {
+            if (mine && j > 1)
+                slot_store(a, n, s);
+            if (!grid_barrier(L.bar, phase, L.flags, &S.ok) || !list_build(L, cur, S, phase) ||
+                !grid_barrier(L.bar, phase, L.flags, &S.ok))
                 return;
+        }
+        if (mine && (build || j == 1)) {
+            slot_load(a, n, slot, s);
+            if (!last)
+                normals3(p.seed, (uint32_t)s.i, step0 + j, 0u, nz[0], nz[1], nz[2]);
         }
         if (blockIdx.x == 0 && threadIdx.x == 0)
             w[(j + 2) % 3] = 0u;
-        int *raise = reinterpret_cast<int *>(a.gates) + (j + 1) % 3;
-        const bool last = j == a.steps;
         if (!last)
             next_spring(step0 + j);
-        for (int q = first; q < n; q += gridDim.x * blockDim.x) {
-            const int i = L.b.sorted[q];
-            float4 o0, o1;
-            slot_forces<COUL>(q, i, L.g, L.b.start, L.b.sorted, L.b.key, cur, n, L.cap, L.nbr, L.nnbr,
-                              a.F_lj, s_tab, s_rcc2, o0, o1);
-            if (!last) {
-                fused_update<MODE_BA>(a, p, s_tc, R0f, step0 + j, i, o0, o1, nxt, raise);
-            } else {
-                if (cur != L.b.sxq)
-                    L.b.sxq[q] = cur[q];
-                fused_update<MODE_B>(a, p, s_tc, R0f, step0 + j, i, o0, o1, nullptr, raise);
+        if (!mine)
+            continue;
+        const float4 spring = a.I.spring[((step0 + j) & 1) * NPSIM_MAX_TYPES + s.ti];
+        const float4 pi = make_float4(s.xhi[0], s.xhi[1], s.xhi[2], __int_as_float(s.ti));
+        float4 o0, o1;
+        slot_forces<COUL>(slot, s.i, pi, s.first, s.cnt, L.g, L.b.start, L.b.sorted, L.b.key, cur, n,
+                          L.cap, L.nbr, a.F_lj, s_tab, s_rcc2, o0, o1);
+        const TypeCoef &tc = s_tc[s.ti];
+        float Fh[3] = {0.f, 0.f, 0.f}, Fl[3] = {0.f, 0.f, 0.f};
+        df_add_df(Fh[0], Fl[0], o0.x, o0.w);
+        df_add_df(Fh[1], Fl[1], o0.y, o1.x);
+        df_add_df(Fh[2], Fl[2], o0.z, o1.y);
+        float ex, ey, ez;
+        external_force(make_float4(s.xhi[0], s.xhi[1], s.xhi[2], s.q), s.xlo[0], s.xlo[1], s.xlo[2],
+                       tc.kw, tc.mg, tc.mw2, spring, p.wall, p.rot_mode, ex, ey, ez, R0f, a.I.flags);
+        df_add(Fh[0], Fl[0], ex);
+        df_add(Fh[1], Fl[1], ey);
+        df_add(Fh[2], Fl[2], ez);
+        const float f[3] = {__fadd_rn(Fh[0], Fl[0]), __fadd_rn(Fh[1], Fl[1]), __fadd_rn(Fh[2], Fl[2])};
+        if (!last) {
+            kick_drift<true, true>(tc, p.integrator, hdt, nz, f, s.v, s.xhi, s.xlo);
+            nxt[slot] = make_float4(s.xhi[0], s.xhi[1], s.xhi[2], __int_as_float(s.ti));
+            if (!(isfinite(s.xhi[0]) && isfinite(s.xhi[1]) && isfinite(s.xhi[2])))
+                atomicOr(a.I.flags, FLAG_NONFINITE);
+            // moved more than half the skin since the list was built: build
+            const float dx = s.xhi[0] - s.ref[0], dy = s.xhi[1] - s.ref[1], dz = s.xhi[2] - s.ref[2];
+            if (!(fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= a.I.half_skin2))
+                a.gates[(j + 1) % 3] = 1u;
+            if (j + 1 < a.steps)
+                normals3(p.seed, (uint32_t)s.i, step0 + j + 1, 0u, nz[0], nz[1], nz[2]);
+        } else {
+            kick_drift<true, false>(tc, p.integrator, hdt, nz, f, s.v, s.xhi, s.xlo);
+            if (cur != L.b.sxq)
+                L.b.sxq[slot] = pi;
+            slot_store(a, n, s);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                a.I.F[d * n + s.i] = Fh[d];
+                a.I.F[(3 + d) * n + s.i] = Fl[d];
             }
         }
     }
@@ -988,6 +1043,19 @@ cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4
     return launch_coop<ListBuildArgs>(k_list_build, max((n + 63) / 64, cell_scan_tiles(m)), st, A);
 }
 
+int list_steps_capacity()
+{
+    int dev = 0, sms = 0, occ = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_list_steps<true>, kScanThreads, 0) !=
+            cudaSuccess)
+        return 0;
+    const int ctas = min(occ * sms, 2 * kOneCtaPerSm);
+    // below two CTAs per SM only one is launched for up to kOneCtaPerSm of them
+    return min(kMaxFusedNps, (ctas >= 2 * kOneCtaPerSm ? ctas : min(ctas, kOneCtaPerSm)) * kScanThreads);
+}
+
 cudaError_t launch_list_steps(const CellGrid &g, const CellBufs &b, int n, const PairTab *tab,
                               const float *rcc2, float skin, const NbrList &l, unsigned *bar,
                               const IntArgs &I, const StepParams &p, float4 *sxq2, float *F_lj,
@@ -1005,6 +1073,8 @@ cudaError_t launch_list_steps(const CellGrid &g, const CellBufs &b, int n, const
     // builds), then one CTA per SM, two when their threads do not reach n
     const int warps = (n + 31) / 32;
     const int want = n <= kOneCtaPerSm * kScanThreads ? min(warps, kOneCtaPerSm) : 2 * kOneCtaPerSm;
+    if (n > list_steps_capacity())
+        return cudaErrorInvalidValue; // every slot needs a thread
     return rcc2 ? launch_coop<FusedStepArgs, StepParams>(k_list_steps<true>, want, st, a, p)
                 : launch_coop<FusedStepArgs, StepParams>(k_list_steps<false>, want, st, a, p);
 }

@@ -293,19 +293,20 @@ k_free_steps(IntArgs a, const __grid_constant__ StepParams p, int steps)
         for (int d = 0; d < 3; ++d)
             f[d] = __fadd_rn(a.F[d * n + i], a.F[(3 + d) * n + i]);
         int bad = 0;
-        kick_drift<false, true>(tc, p.integrator, hdt, p.seed, (uint32_t)i, step0, f, v, xhi, xlo);
+        float nz[3];
+        normals3(p.seed, (uint32_t)i, step0, 0u, nz[0], nz[1], nz[2]);
+        kick_drift<false, true>(tc, p.integrator, hdt, nz, f, v, xhi, xlo);
         bad |= !(isfinite(xhi[0]) && isfinite(xhi[1]) && isfinite(xhi[2]));
         for (int j = 1; j <= steps; ++j) {
             external_force(make_float4(xhi[0], xhi[1], xhi[2], q.w), xlo[0], xlo[1], xlo[2], tc.kw,
                            tc.mg, tc.mw2, s_spring[j][ti], p.wall, p.rot_mode, f[0], f[1], f[2], R0f,
                            a.flags);
             if (j < steps) {
-                kick_drift<true, true>(tc, p.integrator, hdt, p.seed, (uint32_t)i, step0 + j, f, v,
-                                       xhi, xlo);
+                normals3(p.seed, (uint32_t)i, step0 + j, 0u, nz[0], nz[1], nz[2]);
+                kick_drift<true, true>(tc, p.integrator, hdt, nz, f, v, xhi, xlo);
                 bad |= !(isfinite(xhi[0]) && isfinite(xhi[1]) && isfinite(xhi[2]));
             } else {
-                kick_drift<true, false>(tc, p.integrator, hdt, p.seed, (uint32_t)i, step0 + j, f, v,
-                                        xhi, xlo);
+                kick_drift<true, false>(tc, p.integrator, hdt, nz, f, v, xhi, xlo);
             }
         }
         if (bad)

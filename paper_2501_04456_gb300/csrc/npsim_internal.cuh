@@ -1234,12 +1234,11 @@ struct IntArgs {
 
 // Velocity and position of one particle through the closing half kick B and / or
 // the B-A-O-A part of the next step (or the overdamped update, or step (vi) as
-// printed), from the force f; noise of particle noise_idx at `step`.
+// printed), from the force f and the step's normals nz (A part).
 template <bool DO_B, bool DO_A>
 __device__ __forceinline__ void kick_drift(const TypeCoef &tc, int integrator, float hdt,
-                                           uint64_t seed, uint32_t noise_idx, long long step,
-                                           const float (&f)[3], float (&v)[3], float (&xhi)[3],
-                                           float (&xlo)[3])
+                                           const float (&nz)[3], const float (&f)[3],
+                                           float (&v)[3], float (&xhi)[3], float (&xlo)[3])
 {
     const bool baoab = integrator == 0;
     if (DO_B && baoab) {
@@ -1248,8 +1247,6 @@ __device__ __forceinline__ void kick_drift(const TypeCoef &tc, int integrator, f
             v[d] = __fmaf_rn(tc.hdt_m, f[d], v[d]);
     }
     if (DO_A) {
-        float nz[3];
-        normals3(seed, noise_idx, step, 0u, nz[0], nz[1], nz[2]);
         if (baoab) {
             // the two A half steps around the O step add dt/2 (v' + v'') to the
             // position (the O step does not depend on x): one compensated add
@@ -1313,7 +1310,10 @@ __device__ __forceinline__ void advance_particle(int i, int n, uint32_t noise_id
                         __fadd_rn(Fh[2], Fl[2])};
     float v[3] = {v0[0], v0[1], v0[2]}; // v_ at i, read by the caller
     float xhi[3] = {xh.x, xh.y, xh.z}, xlo[3] = {lx, ly, lz};
-    kick_drift<DO_B, DO_A>(tc, integrator, hdt, seed, noise_idx, step, f, v, xhi, xlo);
+    float nz[3] = {0.f, 0.f, 0.f};
+    if (DO_A)
+        normals3(seed, noise_idx, step, 0u, nz[0], nz[1], nz[2]);
+    kick_drift<DO_B, DO_A>(tc, integrator, hdt, nz, f, v, xhi, xlo);
     if (DO_A) {
         xq[i] = make_float4(xhi[0], xhi[1], xhi[2], xh.w);
         if (sxq) // the neighbour-list kernel's cell-ordered copy
@@ -1551,6 +1551,7 @@ cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4
 // records like b.sxq (its record n far from every NP), F_lj [n][8] scratch.
 constexpr int kMaxFusedSteps = 256;
 constexpr int kMaxFusedNps = 65536;
+int list_steps_capacity(); // NPs one launch can hold on the current device
 cudaError_t launch_list_steps(const CellGrid &g, const CellBufs &b, int n, const PairTab *tab,
                               const float *rcc2, float skin, const NbrList &l, unsigned *bar,
                               const IntArgs &I, const StepParams &p, float4 *sxq2, float *F_lj,

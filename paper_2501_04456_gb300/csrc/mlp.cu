@@ -249,6 +249,27 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
         __syncwarp();
     }
 
+    // the epilogue's share of the previous layer's pre-activations, on its way while
+    // the products run: thread (warp, lane) handles rows warp, warp + 8, ... and
+    // columns 2 lane, 2 lane + 1 of a 64-column tile.  (Read in the row loop, one
+    // column per lane, each row's load waited behind the previous row's stores: a
+    // backward launch of 4 networks, 256 rows and 256 columns takes 17 us this way and
+    // took 26; a forward one 11 and 14.5, cold caches)
+    constexpr int kWarps = kGemmThreads / 32;
+    const int rows = min(kTileM, g.M - m0);
+    const bool pairs = nt == 64 && g.ldc % 2 == 0 && n0 % 2 == 0 && g.zc % 2 == 0;
+    float2 zreg[kTileM / kWarps];
+    if (pairs && g.mode == GEMM_DACT) {
+#pragma unroll
+        for (int q = 0; q < kTileM / kWarps; ++q) {
+            const int rr = q * kWarps + warp;
+            zreg[q] = rr < rows ? *reinterpret_cast<const float2 *>(
+                                      g.Z + (size_t)z * g.zc + (size_t)(m0 + rr) * g.ldc + n0 +
+                                      2 * lane)
+                                : make_float2(0.f, 0.f);
+        }
+    }
+
     // wait for the accumulator (bounded), then the epilogue
     if (!mbar_wait_bounded(done_bar, 0, wb))
         atomicExch(&s_abort, 1);
@@ -288,35 +309,66 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
         }
         __syncthreads();
         // one warp per output row, lanes along the columns (coalesced)
-        const int rows = min(kTileM, g.M - m0);
-        constexpr int kWarps = kGemmThreads / 32;
         const float *bias = g.bias ? g.bias + (size_t)z * g.zbias + n0 : nullptr;
-        for (int rr = warp; rr < rows; rr += kWarps) {
-            const size_t ro = (size_t)z * g.zc + (size_t)(m0 + rr) * g.ldc + n0;
-            float *Sr = S + rr * pitch;
-            for (int cc = lane; cc < nt; cc += 32) {
-                const size_t o = ro + cc;
-                float v = Sr[cc];
-                if (g.mode == GEMM_F32) {
-                    if (bias)
-                        v += bias[cc];
-                    g.Cf[o] = v;
-                } else if (g.mode == GEMM_ACT) {
-                    if (bias)
-                        v += bias[cc];
+        if (pairs) { // two columns per lane
+            const float2 b2 = bias ? make_float2(bias[2 * lane], bias[2 * lane + 1])
+                                   : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < kTileM / kWarps; ++q) {
+                const int rr = q * kWarps + warp;
+                if (rr >= rows)
+                    break;
+                const size_t o = (size_t)z * g.zc + (size_t)(m0 + rr) * g.ldc + n0 + 2 * lane;
+                float *Sr = S + rr * pitch + 2 * lane;
+                float2 v = make_float2(Sr[0], Sr[1]);
+                if (g.mode == GEMM_DACT) {
+                    v = make_float2(v.x * dsilu(zreg[q].x), v.y * dsilu(zreg[q].y));
+                } else if (bias) {
+                    v = make_float2(v.x + b2.x, v.y + b2.y);
+                }
+                if (g.mode == GEMM_ACT) {
                     if (g.Z)
-                        g.Z[o] = v;
-                    const float act = g.act ? silu(v) : v;
-                    g.Cb[o] = __float2bfloat16_rn(act);
-                    if (g.Cf)
-                        g.Cf[o] = act;
-                    Sr[cc] = act;
-                } else { // GEMM_DACT: gradient through the SiLU of the previous layer
-                    const float d = v * dsilu(g.Z[o]);
-                    g.Cb[o] = __float2bfloat16_rn(d);
-                    if (g.Cf)
-                        g.Cf[o] = d;
-                    Sr[cc] = d;
+                        *reinterpret_cast<float2 *>(g.Z + o) = v;
+                    if (g.act)
+                        v = make_float2(silu(v.x), silu(v.y));
+                }
+                if (g.mode != GEMM_F32)
+                    *reinterpret_cast<__nv_bfloat162 *>(g.Cb + o) = __floats2bfloat162_rn(v.x, v.y);
+                if (g.Cf)
+                    *reinterpret_cast<float2 *>(g.Cf + o) = v;
+                if (g.CbT) {
+                    Sr[0] = v.x;
+                    Sr[1] = v.y;
+                }
+            }
+        } else {
+            for (int rr = warp; rr < rows; rr += kWarps) {
+                const size_t ro = (size_t)z * g.zc + (size_t)(m0 + rr) * g.ldc + n0;
+                float *Sr = S + rr * pitch;
+                for (int cc = lane; cc < nt; cc += 32) {
+                    const size_t o = ro + cc;
+                    float v = Sr[cc];
+                    if (g.mode == GEMM_F32) {
+                        if (bias)
+                            v += bias[cc];
+                        g.Cf[o] = v;
+                    } else if (g.mode == GEMM_ACT) {
+                        if (bias)
+                            v += bias[cc];
+                        if (g.Z)
+                            g.Z[o] = v;
+                        const float act = g.act ? silu(v) : v;
+                        g.Cb[o] = __float2bfloat16_rn(act);
+                        if (g.Cf)
+                            g.Cf[o] = act;
+                        Sr[cc] = act;
+                    } else { // GEMM_DACT: gradient through the SiLU of the previous layer
+                        const float d = v * dsilu(g.Z[o]);
+                        g.Cb[o] = __float2bfloat16_rn(d);
+                        if (g.Cf)
+                            g.Cf[o] = d;
+                        Sr[cc] = d;
+                    }
                 }
             }
         }
@@ -324,8 +376,15 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
             __syncthreads();
             for (int cc = warp; cc < nt; cc += kWarps) {
                 __nv_bfloat16 *o = g.CbT + (size_t)z * g.zt + (size_t)(n0 + cc) * g.ldt + m0;
-                for (int rr = lane; rr < rows; rr += 32)
-                    o[rr] = __float2bfloat16_rn(S[rr * pitch + cc]);
+                if (rows == kTileM && g.ldt % 2 == 0 && g.zt % 2 == 0) {
+#pragma unroll
+                    for (int rr = 2 * lane; rr < kTileM; rr += 64)
+                        *reinterpret_cast<__nv_bfloat162 *>(o + rr) = __floats2bfloat162_rn(
+                            S[rr * pitch + cc], S[(rr + 1) * pitch + cc]);
+                } else {
+                    for (int rr = lane; rr < rows; rr += 32)
+                        o[rr] = __float2bfloat16_rn(S[rr * pitch + cc]);
+                }
             }
         }
     }
@@ -657,65 +716,96 @@ __global__ void k_mse_grad(const float *__restrict__ y, const float *__restrict_
 }
 
 // Column sums of M x out_p FP32 matrices (bias gradients of layer blockIdx.y,
-// network blockIdx.z), one thread per column, rows in fixed order (deterministic);
-// sixteen rows are read before they are added, so that the chain of adds, not one
-// load's latency per few rows, sets the time.
-__global__ void __launch_bounds__(32)
-k_colsum(ColsumArgs a, const __grid_constant__ NetDims d, float *__restrict__ grads)
+// network blockIdx.z), 32 columns per CTA, rows in fixed order (deterministic): the
+// CTA brings 256 rows at a time into shared memory, and one warp adds them, so that
+// the chain of adds and not the loads' latency sets the time (4 networks, 256 rows,
+// 1104 columns: 8.5 us; one warp per 32 columns reading 16 rows ahead took 13.4).
+__global__ void __launch_bounds__(256)
+k_colsum(const __grid_constant__ ColsumArgs a, const __grid_constant__ NetDims d, float *__restrict__ grads)
 {
+    __shared__ float t[256][32];
     const int l = blockIdx.y, N = d.out_p[l];
-    const int c = blockIdx.x * 32 + threadIdx.x;
-    if (c >= N)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = blockIdx.x * 32 + lane;
+    if ((int)blockIdx.x * 32 >= N)
         return;
     const float *G = a.G[l] + (size_t)blockIdx.z * a.M * N + c;
     float s = 0.f;
-    int r = 0;
-    for (; r + 16 <= a.M; r += 16) {
-        float w[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-            w[k] = G[(size_t)(r + k) * N];
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-            s += w[k];
+    for (int r0 = 0; r0 < a.M; r0 += 256) {
+        const int rows = min(256, a.M - r0);
+        if (c < N) {
+#pragma unroll 8
+            for (int r = warp; r < rows; r += 8)
+                t[r][lane] = G[(size_t)(r0 + r) * N];
+        }
+        __syncthreads();
+        if (warp == 0 && c < N) {
+#pragma unroll 16
+            for (int r = 0; r < rows; ++r)
+                s += t[r][lane];
+        }
+        __syncthreads();
     }
-    for (; r < a.M; ++r)
-        s += G[(size_t)r * N];
-    grads[(size_t)blockIdx.z * d.n_params + d.off[l] + d.out_p[l] * d.in_p[l] + c] = s;
+    if (warp == 0 && c < N)
+        grads[(size_t)blockIdx.z * d.n_params + d.off[l] + d.out_p[l] * d.in_p[l] + c] = s;
 }
 
-// Writes parameter e of network k (value w) to the BF16 copies its layer keeps.
-__device__ __forceinline__ void put_weight(const NetDims &d, int k, int e, float w)
+// The 32 x 32 tiles of every layer's weights, then its biases, counted through the
+// layers (blockIdx.x of the kernels below).
+struct ParamTile {
+    int l, r0, c0; // r0 < 0: the biases
+};
+
+__host__ __device__ inline int layer_tiles(const NetDims &d, int l)
+{
+    return ((d.out_p[l] + 31) / 32) * ((d.in_p[l] + 31) / 32) + 1;
+}
+
+__device__ __forceinline__ ParamTile param_tile(const NetDims &d, int x)
 {
     int l = 0;
-    while (l + 1 < d.n_layers && e >= d.off[l + 1])
-        ++l;
-    const int rows = d.out_p[l], cols = d.in_p[l], j = e - d.off[l];
-    if (j >= rows * cols)
-        return; // a bias
-    const __nv_bfloat16 b = __float2bfloat16_rn(w);
+    for (; l + 1 < d.n_layers && x >= layer_tiles(d, l); ++l)
+        x -= layer_tiles(d, l);
+    const int tc = (d.in_p[l] + 31) / 32;
+    return x == layer_tiles(d, l) - 1 ? ParamTile{l, -1, 0} : ParamTile{l, x / tc * 32, x % tc * 32};
+}
+
+// The BF16 copy of a 32 x 32 tile of weights (thread (tx, ty): column tx, rows ty,
+// ty + 8, ...) and its transpose, which goes through shared memory: written weight
+// by weight, each two bytes touched a sector of their own (AdamW of 4 networks of
+// 222 k parameters: 8.7 us, before 13.4).
+__device__ __forceinline__ void put_tile(const NetDims &d, int k, const ParamTile &p,
+                                         const float (&w)[4], __nv_bfloat16 (&t)[32][33])
+{
+    const int rows = d.out_p[p.l], cols = d.in_p[p.l];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const size_t base = (size_t)k * rows * cols;
-    d.Wb[l][base + j] = b;
-    const int r = j / cols, c = j - r * cols;
-    d.Wt[l][base + (size_t)c * rows + r] = b;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int r = p.r0 + ty + 8 * q, c = p.c0 + tx;
+        const __nv_bfloat16 b = __float2bfloat16_rn(w[q]);
+        t[ty + 8 * q][tx] = b;
+        if (r < rows && c < cols)
+            d.Wb[p.l][base + (size_t)r * cols + c] = b;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int c = p.c0 + ty + 8 * q, r = p.r0 + tx;
+        if (r < rows && c < cols)
+            d.Wt[p.l][base + (size_t)c * rows + r] = t[tx][ty + 8 * q];
+    }
 }
 
 // AdamW (I. Loshchilov, F. Hutter, "Decoupled weight decay regularization"):
 // m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2; w -= lr (m_hat / (sqrt(v_hat) + eps) + wd w),
-// with m_hat = m / (1 - b1^t), v_hat = v / (1 - b2^t).  Writes the BF16 copy of w
-// and its transpose for back-propagation.  The mask keeps padded entries at zero;
-// biases do not decay.  Network k0 + blockIdx.y.
-__global__ void k_adamw(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
-                        float *__restrict__ v, const unsigned char *__restrict__ mask,
-                        const __grid_constant__ NetDims d, int k0, AdamArgs a)
+// with m_hat = m / (1 - b1^t), v_hat = v / (1 - b2^t).  The mask keeps padded
+// entries at zero; biases do not decay.
+__device__ __forceinline__ float adamw_one(size_t idx, unsigned char mk, float *__restrict__ w,
+                                           const float *__restrict__ g, float *__restrict__ m,
+                                           float *__restrict__ v, const AdamArgs &a)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= d.n_params)
-        return;
-    const int k = k0 + blockIdx.y;
-    const size_t idx = (size_t)k * d.n_params + e;
     float wi = w[idx];
-    const unsigned char mk = mask[e];
     if (mk & 1) {
         const float wd = mk & 2 ? a.wd : 0.f;
         const float gi = g[idx];
@@ -727,15 +817,52 @@ __global__ void k_adamw(float *__restrict__ w, const float *__restrict__ g, floa
         wi -= a.lr * (mh / (sqrtf(vh) + a.eps) + wd * wi);
         w[idx] = wi;
     }
-    put_weight(d, k, e, wi);
+    return wi;
+}
+
+// AdamW and the BF16 copies, one tile per CTA.  Network k0 + blockIdx.y.
+__global__ void __launch_bounds__(256)
+k_adamw(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
+        float *__restrict__ v, const unsigned char *__restrict__ mask,
+        const __grid_constant__ NetDims d, int k0, AdamArgs a)
+{
+    __shared__ __nv_bfloat16 t[32][33];
+    const ParamTile p = param_tile(d, blockIdx.x);
+    const int k = k0 + blockIdx.y, rows = d.out_p[p.l], cols = d.in_p[p.l];
+    const size_t net = (size_t)k * d.n_params;
+    if (p.r0 < 0) {
+        for (int c = threadIdx.x; c < rows; c += blockDim.x) {
+            const int e = d.off[p.l] + rows * cols + c;
+            adamw_one(net + e, mask[e], w, g, m, v, a);
+        }
+        return;
+    }
+    float wt[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int r = p.r0 + (threadIdx.x >> 5) + 8 * q, c = p.c0 + (threadIdx.x & 31);
+        const int e = d.off[p.l] + r * cols + c;
+        wt[q] = r < rows && c < cols ? adamw_one(net + e, mask[e], w, g, m, v, a) : 0.f;
+    }
+    put_tile(d, k, p, wt, t);
 }
 
 // BF16 copies of the flat parameters of network k.
-__global__ void k_weights_bf16(const float *__restrict__ w, const __grid_constant__ NetDims d, int k)
+__global__ void __launch_bounds__(256)
+k_weights_bf16(const float *__restrict__ w, const __grid_constant__ NetDims d, int k)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < d.n_params)
-        put_weight(d, k, e, w[(size_t)k * d.n_params + e]);
+    __shared__ __nv_bfloat16 t[32][33];
+    const ParamTile p = param_tile(d, blockIdx.x);
+    if (p.r0 < 0)
+        return;
+    const int rows = d.out_p[p.l], cols = d.in_p[p.l];
+    float wt[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int r = p.r0 + (threadIdx.x >> 5) + 8 * q, c = p.c0 + (threadIdx.x & 31);
+        wt[q] = r < rows && c < cols ? w[(size_t)k * d.n_params + d.off[p.l] + r * cols + c] : 0.f;
+    }
+    put_tile(d, k, p, wt, t);
 }
 
 __global__ void k_f32_to_bf16(const float *__restrict__ x, int n, __nv_bfloat16 *__restrict__ y)
@@ -919,20 +1046,28 @@ cudaError_t launch_colsum(const ColsumArgs &c, const NetDims &d, float *grads, c
     int w = 0;
     for (int l = 0; l < d.n_layers; ++l)
         w = d.out_p[l] > w ? d.out_p[l] : w;
-    k_colsum<<<dim3((w + 31) / 32, d.n_layers, c.nz), 32, 0, st>>>(c, d, grads);
+    k_colsum<<<dim3((w + 31) / 32, d.n_layers, c.nz), 256, 0, st>>>(c, d, grads);
     return cudaGetLastError();
+}
+
+static int param_tiles(const NetDims &d)
+{
+    int n = 0;
+    for (int l = 0; l < d.n_layers; ++l)
+        n += layer_tiles(d, l);
+    return n;
 }
 
 cudaError_t launch_adamw(float *w, const float *g, float *m, float *v, const unsigned char *mask,
                          const NetDims &d, int k0, int nz, const AdamArgs &a, cudaStream_t st)
 {
-    k_adamw<<<dim3((d.n_params + 255) / 256, nz), 256, 0, st>>>(w, g, m, v, mask, d, k0, a);
+    k_adamw<<<dim3(param_tiles(d), nz), 256, 0, st>>>(w, g, m, v, mask, d, k0, a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_weights_bf16(const float *w, const NetDims &d, int k, cudaStream_t st)
 {
-    k_weights_bf16<<<(d.n_params + 255) / 256, 256, 0, st>>>(w, d, k);
+    k_weights_bf16<<<param_tiles(d), 256, 0, st>>>(w, d, k);
     return cudaGetLastError();
 }
 

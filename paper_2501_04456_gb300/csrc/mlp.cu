@@ -9,11 +9,14 @@
 //  * one CTA of 256 threads computes a 128 x n_tile block (n_tile <= 256,
 //    multiple of 16); the FP32 accumulator lives in TMEM (allocated per CTA);
 //  * operands arrive by TMA (cp.async.bulk.tensor, 2-D tensor maps, boxes of
-//    8 K-columns x rows) into a ring of up to four stages of 64 K-columns each,
-//    in the canonical no-swizzle K-major layout of the tcgen05 matrix
-//    descriptors: 8-row x 16-byte core matrices, adjacent along M/N at 128 B
-//    (stride-dimension byte offset) and along K at rows x 16 B (leading-
-//    dimension byte offset).  Rows beyond M or N are zero-filled by the TMA;
+//    64 K-columns x rows) into a ring of up to four stages of 64 K-columns each,
+//    in the K-major 128-byte swizzle of the tensor maps and the tcgen05 matrix
+//    descriptors: a row's 64 columns are one 128-byte line, 8 rows an atom of
+//    1024 bytes, atoms adjacent along M/N.  Rows beyond M or N and columns beyond
+//    K are zero-filled by the TMA.  (In boxes of 8 columns, the layout without a
+//    swizzle, the copies went out in 16-byte pieces:
+//    training 4 networks took 147 us per minibatch of 256, now 133; 4096
+//    predictions 106 us, now 103);
 //  * one thread issues the loads (mbarrier expect_tx per stage), one thread
 //    issues tcgen05.mma (M = 128, N = n_tile, K = 16 per instruction) and
 //    releases each stage with tcgen05.commit; every wait is bounded (clock64
@@ -50,6 +53,14 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     d |= (uint64_t)((sbo & 0x3FFFFu) >> 4) << 32;
     d |= (uint64_t)1 << 46;
     return d;
+}
+
+// The same of an operand in the 128-byte swizzle (bits 61-63 = 2): 64 K-columns per
+// row, atoms of 8 rows (1024 bytes) one after the other; the start moves along K
+// inside the atom, 32 bytes per 16 columns.
+__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr)
+{
+    return smem_desc(addr, 16, 1024) | (uint64_t)2 << 61;
 }
 
 // Instruction descriptor of tcgen05.mma kind::f16: D = F32 (bits 4-5 = 1),
@@ -206,14 +217,11 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
                     atomicExch(&s_abort, 1);
                     break;
                 }
-                const int k0 = c * kChunkK, kc = min(kChunkK, g.K - k0);
                 const uint32_t sa = base + (uint32_t)s * sbytes, sb = sa + a_bytes;
                 const uint32_t fb = smem_addr(&full[s]);
-                mbar_expect_tx(fb, (uint32_t)((kTileM + g.n_tile) * kc * 2));
-                for (int kg = 0; kg < kc / 8; ++kg) {
-                    tma_load_2d(sa + (uint32_t)(kg * kTileM * 16), tmA, k0 + kg * 8, ya, fb);
-                    tma_load_2d(sb + (uint32_t)(kg * g.n_tile * 16), tmB, k0 + kg * 8, yb, fb);
-                }
+                mbar_expect_tx(fb, sbytes); // columns and rows out of range arrive as zeros
+                tma_load_2d(sa, tmA, c * kChunkK, ya, fb);
+                tma_load_2d(sb, tmB, c * kChunkK, yb, fb);
             }
             s_issued = c;
         }
@@ -231,10 +239,8 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
                 const int kc = min(kChunkK, g.K - c * kChunkK);
                 const uint32_t sa = base + (uint32_t)s * sbytes, sb = sa + a_bytes;
                 for (int ks = 0; ks < kc; ks += 16) {
-                    const uint64_t ad = smem_desc(sa + (uint32_t)((ks / 8) * kTileM * 16),
-                                                  kTileM * 16, 128);
-                    const uint64_t bd = smem_desc(sb + (uint32_t)((ks / 8) * g.n_tile * 16),
-                                                  (uint32_t)(g.n_tile * 16), 128);
+                    const uint64_t ad = smem_desc_sw128(sa + (uint32_t)(ks * 2));
+                    const uint64_t bd = smem_desc_sw128(sb + (uint32_t)(ks * 2));
                     const uint32_t acc = (c > 0 || ks > 0) ? 1u : 0u;
                     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
@@ -253,8 +259,8 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
     // the products run: thread (warp, lane) handles rows warp, warp + 8, ... and
     // columns 2 lane, 2 lane + 1 of a 64-column tile.  (Read in the row loop, one
     // column per lane, each row's load waited behind the previous row's stores: a
-    // backward launch of 4 networks, 256 rows and 256 columns takes 17 us this way and
-    // took 26; a forward one 11 and 14.5, cold caches)
+    // backward launch of 4 networks, 256 rows and 256 columns took 26 us, now 15; a
+    // forward one 14.5, now 10, cold caches)
     constexpr int kWarps = kGemmThreads / 32;
     const int rows = min(kTileM, g.M - m0);
     const bool pairs = nt == 64 && g.ldc % 2 == 0 && n0 % 2 == 0 && g.zc % 2 == 0;
@@ -520,11 +526,9 @@ k_mlp_infer(const __grid_constant__ MlpMaps maps, MlpDev d)
                         ok = false;
                         break;
                     }
-                    const int kc = min(kChunkK, K - k0);
                     const uint32_t sb = ring + (uint32_t)s * sbytes, fb = smem_addr(&full[s]);
-                    mbar_expect_tx(fb, (uint32_t)(N * kc * 2));
-                    for (int kg = 0; kg < kc / 8; ++kg)
-                        tma_load_2d(sb + (uint32_t)(kg * N * 16), &maps.w[l], k0 + kg * 8, row0, fb);
+                    mbar_expect_tx(fb, (uint32_t)(N * kChunkK * 2));
+                    tma_load_2d(sb, &maps.w[l], k0, row0, fb);
                 }
             }
             s_issued = c;
@@ -558,8 +562,7 @@ k_mlp_infer(const __grid_constant__ MlpMaps maps, MlpDev d)
                         const int k = k0 + ks;
                         const uint64_t ad = smem_desc(abuf + (uint32_t)((k / 8) * kTileM * 16),
                                                       kTileM * 16, 128);
-                        const uint64_t bd = smem_desc(sb + (uint32_t)((ks / 8) * N * 16),
-                                                      (uint32_t)(N * 16), 128);
+                        const uint64_t bd = smem_desc_sw128(sb + (uint32_t)(ks * 2));
                         const uint32_t acc = k > 0 ? 1u : 0u;
                         asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                                      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
@@ -893,21 +896,22 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
     return fn;
 }
 
-// Tensor map of a row-major BF16 matrix (rows x K, leading dimension ld
-// elements) read in boxes of 8 K-columns x box_rows rows; out-of-range rows
-// read as zero.
+// Tensor map of a row-major BF16 matrix (rows x K, leading dimension ld elements)
+// read in boxes of 64 K-columns x box_rows rows in the 128-byte swizzle, or of 8
+// K-columns without (`plain`); out-of-range rows and columns read as zero.
 bool encode_operand(CUtensorMap *m, const __nv_bfloat16 *ptr, int rows, int K, int ld,
-                    int box_rows)
+                    int box_rows, bool plain = false)
 {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc)
         return false;
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    const cuuint32_t box[2] = {8, (cuuint32_t)box_rows};
+    const cuuint32_t box[2] = {plain ? 8u : (cuuint32_t)kChunkK, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)ptr, dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_INTERLEAVE_NONE,
+               plain ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
            CUDA_SUCCESS;
 }
@@ -997,7 +1001,7 @@ cudaError_t launch_mlp_infer(const MlpInferArgs &a, cudaStream_t st)
     d.y = a.y;
     d.flags = a.flags;
     MlpMaps maps{};
-    if (!encode_operand(&maps.x, a.X, a.bp, a.in_p, a.in_p, kTileM))
+    if (!encode_operand(&maps.x, a.X, a.bp, a.in_p, a.in_p, kTileM, true))
         return cudaErrorInvalidValue;
     for (int l = 0; l <= a.NL; ++l) {
         const int K = l == 0 ? a.in_p : a.H, N = l == a.NL ? a.out_p : a.H;

@@ -172,9 +172,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
     __shared__ int s_abort, s_issued;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = bm * kTileM;
-    const int n0 = bn * g.n_tile;
-    const int ya = z * g.za + m0, yb = z * g.zb + n0; // operand rows
+    int m0 = bm * kTileM, n0 = bn * g.n_tile;
     const int nt = min(g.n_tile, g.N - n0); // multiple of 16 (N and n_tile are)
     const int nchunks = (g.K + kChunkK - 1) / kChunkK;
     const uint32_t base = smem_addr(smem);
@@ -206,6 +204,10 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = s_tmem;
+    const int zero = after_previous();
+    m0 += zero;
+    n0 += zero;
+    const int ya = z * g.za + m0, yb = z * g.zb + n0; // operand rows
 
     if (warp == 0) {
         if (lane == 0) { // TMA producer
@@ -475,7 +477,7 @@ k_mlp_infer(const __grid_constant__ MlpMaps maps, MlpDev d)
     __shared__ float s_bias[2][256]; // the epilogue's bias, by layer parity
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int net = blockIdx.y;
+    int net = blockIdx.y;
     const int m0 = blockIdx.x * kTileM;
     const uint32_t abuf = smem_addr(smem);
     const uint32_t ring = abuf + (uint32_t)d.abuf_bytes;
@@ -506,6 +508,7 @@ k_mlp_infer(const __grid_constant__ MlpMaps maps, MlpDev d)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = s_tmem;
+    net += after_previous();
 
     if (warp == 0) {
         if (lane == 0) { // TMA producer: the input tile, then every layer's weights
@@ -696,7 +699,7 @@ __global__ void k_mse_grad(const float *__restrict__ y, const float *__restrict_
                            __nv_bfloat16 *__restrict__ gbT, float *__restrict__ loss)
 {
     const size_t z = (size_t)blockIdx.y * M * ldy;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x + after_previous();
     const int r = idx / ldy, c = idx - r * ldy;
     float g = 0.f, l = 0.f;
     if (r < M) {
@@ -729,7 +732,7 @@ k_colsum(const __grid_constant__ ColsumArgs a, const __grid_constant__ NetDims d
     __shared__ float t[256][32];
     const int l = blockIdx.y, N = d.out_p[l];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int c = blockIdx.x * 32 + lane;
+    const int c = blockIdx.x * 32 + lane + after_previous();
     if ((int)blockIdx.x * 32 >= N)
         return;
     const float *G = a.G[l] + (size_t)blockIdx.z * a.M * N + c;
@@ -832,7 +835,7 @@ k_adamw(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ 
     __shared__ __nv_bfloat16 t[32][33];
     const ParamTile p = param_tile(d, blockIdx.x);
     const int k = k0 + blockIdx.y, rows = d.out_p[p.l], cols = d.in_p[p.l];
-    const size_t net = (size_t)k * d.n_params;
+    const size_t net = (size_t)k * d.n_params + after_previous();
     if (p.r0 < 0) {
         for (int c = threadIdx.x; c < rows; c += blockDim.x) {
             const int e = d.off[p.l] + rows * cols + c;
@@ -968,9 +971,8 @@ cudaError_t launch_gemm(const GemmArgs &g0, const GemmArgs *g1, cudaStream_t st)
     int smem = dyn_smem_bytes(g0.n_tile, s0);
     if (g1 && dyn_smem_bytes(g1->n_tile, s1) > smem)
         smem = dyn_smem_bytes(g1->n_tile, s1);
-    k_gemm_bf16<<<dim3(nb0 + nb1, g0.nz), kGemmThreads, smem, st>>>(
-        ta0, tb0, ta1, tb1, g0, g1 ? *g1 : g0, s0, s1, nb0);
-    return cudaGetLastError();
+    return launch_after(k_gemm_bf16, dim3(nb0 + nb1, g0.nz), kGemmThreads, smem, st, ta0, tb0, ta1, tb1,
+                        g0, g1 ? *g1 : g0, s0, s1, nb0);
 }
 
 bool mlp_infer_supported(int NL, int in_p, int H, int out_p)
@@ -1021,8 +1023,7 @@ cudaError_t launch_mlp_infer(const MlpInferArgs &a, cudaStream_t st)
         attr_done = true;
     }
     dim3 grid(a.bp / kTileM, a.n_nets);
-    k_mlp_infer<<<grid, kInferThreads, smem, st>>>(maps, d);
-    return cudaGetLastError();
+    return launch_after(k_mlp_infer, grid, kInferThreads, smem, st, maps, d);
 }
 
 cudaError_t launch_transpose_bf16(const void *in, int R, int C, int ldi, void *out, int ldo,
@@ -1039,10 +1040,8 @@ cudaError_t launch_mse_grad(const float *y, const float *t, const float *w, int 
                             float *loss, cudaStream_t st)
 {
     const int n = M * ldy;
-    k_mse_grad<<<dim3((n + 255) / 256, nz), 256, 0, st>>>(y, t, w, M, m_valid, n_valid, ldy, gf,
-                                                          (__nv_bfloat16 *)gb,
-                                                          (__nv_bfloat16 *)gbT, loss);
-    return cudaGetLastError();
+    return launch_after(k_mse_grad, dim3((n + 255) / 256, nz), 256, 0, st, y, t, w, M, m_valid, n_valid,
+                        ldy, gf, (__nv_bfloat16 *)gb, (__nv_bfloat16 *)gbT, loss);
 }
 
 cudaError_t launch_colsum(const ColsumArgs &c, const NetDims &d, float *grads, cudaStream_t st)
@@ -1050,8 +1049,7 @@ cudaError_t launch_colsum(const ColsumArgs &c, const NetDims &d, float *grads, c
     int w = 0;
     for (int l = 0; l < d.n_layers; ++l)
         w = d.out_p[l] > w ? d.out_p[l] : w;
-    k_colsum<<<dim3((w + 31) / 32, d.n_layers, c.nz), 256, 0, st>>>(c, d, grads);
-    return cudaGetLastError();
+    return launch_after(k_colsum, dim3((w + 31) / 32, d.n_layers, c.nz), 256, 0, st, c, d, grads);
 }
 
 static int param_tiles(const NetDims &d)
@@ -1065,8 +1063,7 @@ static int param_tiles(const NetDims &d)
 cudaError_t launch_adamw(float *w, const float *g, float *m, float *v, const unsigned char *mask,
                          const NetDims &d, int k0, int nz, const AdamArgs &a, cudaStream_t st)
 {
-    k_adamw<<<dim3(param_tiles(d), nz), 256, 0, st>>>(w, g, m, v, mask, d, k0, a);
-    return cudaGetLastError();
+    return launch_after(k_adamw, dim3(param_tiles(d), nz), 256, 0, st, w, g, m, v, mask, d, k0, a);
 }
 
 cudaError_t launch_weights_bf16(const float *w, const NetDims &d, int k, cudaStream_t st)

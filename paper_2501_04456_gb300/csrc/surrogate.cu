@@ -388,7 +388,7 @@ __global__ void k_gather_rows(const __nv_bfloat16 *__restrict__ sx, const float 
                               __nv_bfloat16 *__restrict__ xT, float *__restrict__ y,
                               float *__restrict__ loss)
 {
-    const int r = blockIdx.x, k = blockIdx.y;
+    const int r = blockIdx.x, k = (int)blockIdx.y + after_previous();
     const size_t row = (size_t)k * bp + r;
     const bool ok = r < rows;
     const int src = ok ? idx[(size_t)k * idx_ld + r] : 0;
@@ -409,7 +409,7 @@ __global__ void k_ens_stats(const float *__restrict__ y_all, int n_nets, int bp,
                             int n_out, const float *__restrict__ ym, const float *__restrict__ ys,
                             float *__restrict__ mean, float *__restrict__ spread)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x + after_previous();
     if (idx >= B * n_out)
         return;
     const int r = idx / n_out, c = idx - r * n_out;
@@ -703,10 +703,9 @@ int npsim_surr_train(npsim_surr_t s, const float *X, const float *Y, int32_t n_s
             for (int k0 = 0; k0 < s->n_nets && !rc && e == cudaSuccess; k0 += group) {
                 const int nk = std::min(group, s->n_nets - k0);
                 kl = k0;
-                k_gather_rows<<<dim3(bp, nk), 96, 0, s->st>>>(
-                    s->dsx, s->dsy, d_idx + (size_t)k0 * n_samples + r0, n_samples, rows, bp,
-                    s->n_in_p, s->n_out_p, s->a[0], s->aT[0], s->yt, s->loss);
-                e = cudaGetLastError();
+                e = launch_after(k_gather_rows, dim3(bp, nk), 96, 0, s->st, s->dsx, s->dsy,
+                                 d_idx + (size_t)k0 * n_samples + r0, n_samples, rows, bp,
+                                 s->n_in_p, s->n_out_p, s->a[0], s->aT[0], s->yt, s->loss);
                 if (e == cudaSuccess)
                     rc = forward(s, k0, nk, bp, s->a[0], bp, s->y, true);
                 if (!rc && e == cudaSuccess)
@@ -775,10 +774,8 @@ int npsim_surr_predict(npsim_surr_t s, const float *X, int32_t B, float *Y_mean,
     }
     float *d_mean = s->ystat, *d_spread = s->ystat + (size_t)B * s->n_out;
     const int ne = B * s->n_out;
-    k_ens_stats<<<(ne + 255) / 256, 256, 0, s->st>>>(s->y_all, s->n_nets, bp, s->n_out_p, B,
-                                                     s->n_out, s->d_ym, s->d_ys, d_mean,
-                                                     d_spread);
-    SR_CUDA(cudaGetLastError());
+    SR_CUDA(launch_after(k_ens_stats, dim3((ne + 255) / 256), 256, 0, s->st, s->y_all, s->n_nets, bp,
+                         s->n_out_p, B, s->n_out, s->d_ym, s->d_ys, d_mean, d_spread));
     SR_CUDA(fetch_flags(s));
     if (Y_spread == Y_mean + ne) { // back to back on the host too: one copy
         SR_CUDA(cudaMemcpyAsync(Y_mean, d_mean, sizeof(float) * 2 * (size_t)ne,

@@ -153,6 +153,12 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
                  : "memory");
 }
 
+// The tensor map into the descriptor cache, before its first use.
+__device__ __forceinline__ void prefetch_map(const CUtensorMap *map)
+{
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 __device__ __forceinline__ void mma_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -191,6 +197,8 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
+        prefetch_map(tmA);
+        prefetch_map(tmB);
         for (int s = 0; s < stages; ++s) {
             mbar_init(smem_addr(&full[s]), 1);
             mbar_init(smem_addr(&empty[s]), 1);
@@ -259,19 +267,20 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
 
     // the epilogue's share of the previous layer's pre-activations, on its way while
     // the products run: thread (warp, lane) handles rows warp, warp + 8, ... and
-    // columns 2 lane, 2 lane + 1 of a 64-column tile.  (Read in the row loop, one
+    // columns 2 lane, 2 lane + 1 of a tile of up to 64 columns.  (Read in the row loop, one
     // column per lane, each row's load waited behind the previous row's stores: a
     // backward launch of 4 networks, 256 rows and 256 columns took 26 us, now 15; a
     // forward one 14.5, now 10, cold caches)
     constexpr int kWarps = kGemmThreads / 32;
     const int rows = min(kTileM, g.M - m0);
-    const bool pairs = nt == 64 && g.ldc % 2 == 0 && n0 % 2 == 0 && g.zc % 2 == 0;
+    const bool pairs = nt <= 64 && g.ldc % 2 == 0 && n0 % 2 == 0 && g.zc % 2 == 0;
+    const bool mine = 2 * lane < nt;
     float2 zreg[kTileM / kWarps];
     if (pairs && g.mode == GEMM_DACT) {
 #pragma unroll
         for (int q = 0; q < kTileM / kWarps; ++q) {
             const int rr = q * kWarps + warp;
-            zreg[q] = rr < rows ? *reinterpret_cast<const float2 *>(
+            zreg[q] = mine && rr < rows ? *reinterpret_cast<const float2 *>(
                                       g.Z + (size_t)z * g.zc + (size_t)(m0 + rr) * g.ldc + n0 +
                                       2 * lane)
                                 : make_float2(0.f, 0.f);
@@ -319,12 +328,12 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
         // one warp per output row, lanes along the columns (coalesced)
         const float *bias = g.bias ? g.bias + (size_t)z * g.zbias + n0 : nullptr;
         if (pairs) { // two columns per lane
-            const float2 b2 = bias ? make_float2(bias[2 * lane], bias[2 * lane + 1])
+            const float2 b2 = bias && mine ? make_float2(bias[2 * lane], bias[2 * lane + 1])
                                    : make_float2(0.f, 0.f);
 #pragma unroll
             for (int q = 0; q < kTileM / kWarps; ++q) {
                 const int rr = q * kWarps + warp;
-                if (rr >= rows)
+                if (!mine || rr >= rows)
                     break;
                 const size_t o = (size_t)z * g.zc + (size_t)(m0 + rr) * g.ldc + n0 + 2 * lane;
                 float *Sr = S + rr * pitch + 2 * lane;

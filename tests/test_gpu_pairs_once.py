@@ -50,3 +50,14 @@ def test_every_shape_at_tile_edges(P, monkeypatch, n, charges):
                     assert force_error(F, r)[keep].max() <= FORCE_TOL, (idx, what)
                     assert np.array_equal(F, sim.forces(what)), (idx, what)
         assert ran > 0
+
+
+@pytest.mark.parametrize("n", [700, 3001, 20011])
+def test_full_sum_keeps_to_the_kernels_that_evaluate_every_pair(P, n):
+    """sum_neutral asks for the Coulomb term of all N(N-1) pairs: the LJ + Coulomb
+    kernels (packed 3), which pass over type pairs without a charge product, are not
+    chosen for it."""
+    sc = with_(small(wl.config3(), n), sum_neutral=True)
+    types, x, v = wl.initial_state(sc, fp32_positions=True)
+    with P.Sim(sc, x, v, types) as sim:
+        assert sim.allpairs_config()["packed"] != 3

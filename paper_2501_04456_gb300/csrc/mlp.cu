@@ -269,23 +269,25 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
     // the products run: thread (warp, lane) handles rows warp, warp + 8, ... and
     // columns 2 lane, 2 lane + 1 of a tile of up to 64 columns.  (Read in the row loop, one
     // column per lane, each row's load waited behind the previous row's stores: a
-    // backward launch of 4 networks, 256 rows and 256 columns took 26 us, now 15; a
+    // backward launch of 4 networks, 256 rows and 256 columns took 26 us, now 10; a
     // forward one 14.5, now 10, cold caches)
     constexpr int kWarps = kGemmThreads / 32;
     const int rows = min(kTileM, g.M - m0);
     const bool pairs = nt <= 64 && g.ldc % 2 == 0 && n0 % 2 == 0 && g.zc % 2 == 0;
     const bool mine = 2 * lane < nt;
-    float2 zreg[kTileM / kWarps];
-    if (pairs && g.mode == GEMM_DACT) {
+    constexpr int kRowGroup = 4; // rows per pass of the row loop
+    const size_t pair0 = (size_t)z * g.zc + (size_t)(m0 + warp) * g.ldc + n0 + 2 * lane;
+    const size_t row_step = (size_t)kWarps * g.ldc;
+    float2 zreg[kRowGroup];
+    auto load_z = [&](int q0) {
 #pragma unroll
-        for (int q = 0; q < kTileM / kWarps; ++q) {
-            const int rr = q * kWarps + warp;
-            zreg[q] = mine && rr < rows ? *reinterpret_cast<const float2 *>(
-                                      g.Z + (size_t)z * g.zc + (size_t)(m0 + rr) * g.ldc + n0 +
-                                      2 * lane)
-                                : make_float2(0.f, 0.f);
-        }
-    }
+        for (int u = 0; u < kRowGroup; ++u)
+            zreg[u] = mine && (q0 + u) * kWarps + warp < rows
+                          ? *reinterpret_cast<const float2 *>(g.Z + pair0 + (q0 + u) * row_step)
+                          : make_float2(0.f, 0.f);
+    };
+    if (pairs && g.mode == GEMM_DACT)
+        load_z(0);
 
     // wait for the accumulator (bounded), then the epilogue
     if (!mbar_wait_bounded(done_bar, 0, wb))
@@ -330,32 +332,41 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
         if (pairs) { // two columns per lane
             const float2 b2 = bias && mine ? make_float2(bias[2 * lane], bias[2 * lane + 1])
                                    : make_float2(0.f, 0.f);
+#pragma unroll 1
+            for (int q0 = 0; q0 < kTileM / kWarps; q0 += kRowGroup) {
+                float2 zc[kRowGroup];
 #pragma unroll
-            for (int q = 0; q < kTileM / kWarps; ++q) {
-                const int rr = q * kWarps + warp;
-                if (!mine || rr >= rows)
-                    break;
-                const size_t o = (size_t)z * g.zc + (size_t)(m0 + rr) * g.ldc + n0 + 2 * lane;
-                float *Sr = S + rr * pitch + 2 * lane;
-                float2 v = make_float2(Sr[0], Sr[1]);
-                if (g.mode == GEMM_DACT) {
-                    v = make_float2(v.x * dsilu(zreg[q].x), v.y * dsilu(zreg[q].y));
-                } else if (bias) {
-                    v = make_float2(v.x + b2.x, v.y + b2.y);
-                }
-                if (g.mode == GEMM_ACT) {
-                    if (g.Z)
-                        *reinterpret_cast<float2 *>(g.Z + o) = v;
-                    if (g.act)
-                        v = make_float2(silu(v.x), silu(v.y));
-                }
-                if (g.mode != GEMM_F32)
-                    *reinterpret_cast<__nv_bfloat162 *>(g.Cb + o) = __floats2bfloat162_rn(v.x, v.y);
-                if (g.Cf)
-                    *reinterpret_cast<float2 *>(g.Cf + o) = v;
-                if (g.CbT) {
-                    Sr[0] = v.x;
-                    Sr[1] = v.y;
+                for (int u = 0; u < kRowGroup; ++u)
+                    zc[u] = zreg[u];
+                if (g.mode == GEMM_DACT && q0 + kRowGroup < kTileM / kWarps)
+                    load_z(q0 + kRowGroup);
+#pragma unroll
+                for (int u = 0; u < kRowGroup; ++u) {
+                    const int rr = (q0 + u) * kWarps + warp;
+                    if (!mine || rr >= rows)
+                        break;
+                    const size_t o = pair0 + (q0 + u) * row_step;
+                    float *Sr = S + rr * pitch + 2 * lane;
+                    float2 v = make_float2(Sr[0], Sr[1]);
+                    if (g.mode == GEMM_DACT) {
+                        v = make_float2(v.x * dsilu(zc[u].x), v.y * dsilu(zc[u].y));
+                    } else if (bias) {
+                        v = make_float2(v.x + b2.x, v.y + b2.y);
+                    }
+                    if (g.mode == GEMM_ACT) {
+                        if (g.Z)
+                            *reinterpret_cast<float2 *>(g.Z + o) = v;
+                        if (g.act)
+                            v = make_float2(silu(v.x), silu(v.y));
+                    }
+                    if (g.mode != GEMM_F32)
+                        *reinterpret_cast<__nv_bfloat162 *>(g.Cb + o) = __floats2bfloat162_rn(v.x, v.y);
+                    if (g.Cf)
+                        *reinterpret_cast<float2 *>(g.Cf + o) = v;
+                    if (g.CbT) {
+                        Sr[0] = v.x;
+                        Sr[1] = v.y;
+                    }
                 }
             }
         } else {
@@ -422,14 +433,14 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUt
             const __grid_constant__ GemmArgs g0, const __grid_constant__ GemmArgs g1, int stages0,
             int stages1, int nb0)
 {
-    const int x = blockIdx.x;
-    if (x < nb0) {
-        const int mb = (g0.M + kTileM - 1) / kTileM;
-        gemm_tile(&tA0, &tB0, g0, stages0, x % mb, x / mb, blockIdx.y);
-    } else {
-        const int mb = (g1.M + kTileM - 1) / kTileM;
-        gemm_tile(&tA1, &tB1, g1, stages1, (x - nb0) % mb, (x - nb0) / mb, blockIdx.y);
-    }
+    // one copy of the tile's code for both products: with two, their row loops
+    // unrolled, a backward launch on cold caches took 15 us, half of it waiting for
+    // instructions (now 10; 512 rows in the running chain 170 -> 165 us a minibatch)
+    const bool second = (int)blockIdx.x >= nb0;
+    const GemmArgs &g = second ? g1 : g0;
+    const int x = blockIdx.x - (second ? nb0 : 0), mb = (g.M + kTileM - 1) / kTileM;
+    gemm_tile(second ? &tA1 : &tA0, second ? &tB1 : &tB0, g, second ? stages1 : stages0, x % mb,
+              x / mb, blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------

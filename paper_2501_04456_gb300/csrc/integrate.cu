@@ -265,8 +265,8 @@ k_integrate(IntArgs a, StepParams p)
 // the first step to the last: one particle's steps do not depend on the others, so
 // the 80 bytes a step of the kernel above moves per NP are moved once per launch,
 // and what remains is the arithmetic (noise, external force, update).  The spring
-// radii of the launch's steps are evaluated once per CTA.  4 M NPs: 63.4 us a step
-// as one launch each (5.3 TB/s).
+// radii of the launch's steps are evaluated once per CTA.  4 M NPs: 35-39 us a step,
+// issue slots 75 % busy; as one launch per step 63.4 (5.3 TB/s).
 __global__ void __launch_bounds__(256, 4)
 k_free_steps(IntArgs a, const __grid_constant__ StepParams p, int steps)
 {

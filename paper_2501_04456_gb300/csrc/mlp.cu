@@ -266,23 +266,28 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
     }
 
     // the epilogue's share of the previous layer's pre-activations, on its way while
-    // the products run: thread (warp, lane) handles rows warp, warp + 8, ... and
-    // columns 2 lane, 2 lane + 1 of a tile of up to 64 columns.  (Read in the row loop, one
-    // column per lane, each row's load waited behind the previous row's stores: a
-    // backward launch of 4 networks, 256 rows and 256 columns took 26 us, now 10; a
-    // forward one 14.5, now 10, cold caches)
+    // the products run: a thread handles two columns of every eighth row (a tile of
+    // at most 32 columns: of every sixteenth).  (Read in the row loop, one column per
+    // lane, each row's load waited behind the previous row's stores: a backward
+    // launch of 4 networks, 256 rows and 256 columns took 26 us, now 8; a forward one
+    // 14.5, now 8.5, cold caches)
     constexpr int kWarps = kGemmThreads / 32;
     const int rows = min(kTileM, g.M - m0);
     const bool pairs = nt <= 64 && g.ldc % 2 == 0 && n0 % 2 == 0 && g.zc % 2 == 0;
-    const bool mine = 2 * lane < nt;
+    // a tile of at most 32 columns: half a warp per row
+    const int lpr = nt <= 32 ? 16 : 32, rpw = 32 / lpr;
+    const int col = 2 * (lane & (lpr - 1));
+    const int row_in = warp * rpw + lane / lpr;
+    const bool mine = col < nt;
     constexpr int kRowGroup = 4; // rows per pass of the row loop
-    const size_t pair0 = (size_t)z * g.zc + (size_t)(m0 + warp) * g.ldc + n0 + 2 * lane;
-    const size_t row_step = (size_t)kWarps * g.ldc;
+    const size_t pair0 = (size_t)z * g.zc + (size_t)(m0 + row_in) * g.ldc + n0 + col;
+    const size_t row_step = (size_t)(kWarps * rpw) * g.ldc;
+    const int passes = kTileM / (kWarps * rpw);
     float2 zreg[kRowGroup];
     auto load_z = [&](int q0) {
 #pragma unroll
         for (int u = 0; u < kRowGroup; ++u)
-            zreg[u] = mine && (q0 + u) * kWarps + warp < rows
+            zreg[u] = mine && (q0 + u) * kWarps * rpw + row_in < rows
                           ? *reinterpret_cast<const float2 *>(g.Z + pair0 + (q0 + u) * row_step)
                           : make_float2(0.f, 0.f);
     };
@@ -330,23 +335,23 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
         // one warp per output row, lanes along the columns (coalesced)
         const float *bias = g.bias ? g.bias + (size_t)z * g.zbias + n0 : nullptr;
         if (pairs) { // two columns per lane
-            const float2 b2 = bias && mine ? make_float2(bias[2 * lane], bias[2 * lane + 1])
+            const float2 b2 = bias && mine ? make_float2(bias[col], bias[col + 1])
                                    : make_float2(0.f, 0.f);
 #pragma unroll 1
-            for (int q0 = 0; q0 < kTileM / kWarps; q0 += kRowGroup) {
+            for (int q0 = 0; q0 < passes; q0 += kRowGroup) {
                 float2 zc[kRowGroup];
 #pragma unroll
                 for (int u = 0; u < kRowGroup; ++u)
                     zc[u] = zreg[u];
-                if (g.mode == GEMM_DACT && q0 + kRowGroup < kTileM / kWarps)
+                if (g.mode == GEMM_DACT && q0 + kRowGroup < passes)
                     load_z(q0 + kRowGroup);
 #pragma unroll
                 for (int u = 0; u < kRowGroup; ++u) {
-                    const int rr = (q0 + u) * kWarps + warp;
+                    const int rr = (q0 + u) * kWarps * rpw + row_in;
                     if (!mine || rr >= rows)
                         break;
                     const size_t o = pair0 + (q0 + u) * row_step;
-                    float *Sr = S + rr * pitch + 2 * lane;
+                    float *Sr = S + rr * pitch + col;
                     float2 v = make_float2(Sr[0], Sr[1]);
                     if (g.mode == GEMM_DACT) {
                         v = make_float2(v.x * dsilu(zc[u].x), v.y * dsilu(zc[u].y));

@@ -134,10 +134,15 @@ namespace {
 constexpr int kTrainRows = 65536;
 
 // Columns per tile: at most 64, the width the epilogue handles two columns per lane
-// (an output layer of 80 columns as one tile took 11.1 us, as 48 + 32 8.5, cold caches).
-int n_tile_for(int N)
+// (an output layer of 80 columns as one tile took 11.1 us, as 48 + 32 8.5, cold
+// caches), and at most 32 while the product then still has no more CTAs than SMs:
+// half the epilogue per CTA, on SMs that had none (4 networks, 256 columns: a
+// minibatch of 256 rows 88 -> 77 us, of 32 81 -> 68, of 512 163 -> 158).
+constexpr int kSms = 152;
+int n_tile_for(int M, int N, int nz)
 {
-    const int tiles = (N + 63) / 64;
+    const int most = (M + 127) / 128 * ((N + 31) / 32) * nz <= kSms ? 32 : 64;
+    const int tiles = (N + most - 1) / most;
     return ((N + tiles - 1) / tiles + 15) / 16 * 16;
 }
 
@@ -158,7 +163,7 @@ GemmArgs gemm(npsim_surr *s, int mode, const __nv_bfloat16 *A, int lda, int za,
     g.lda = lda;
     g.ldb = ldb;
     g.ldc = ldc;
-    g.n_tile = n_tile_for(N);
+    g.n_tile = n_tile_for(M, N, nk);
     g.tmem_cols = pow2_at_least(g.n_tile);
     g.mode = mode;
     g.flags = s->flags;

@@ -266,16 +266,16 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap *tmA, const CUtensor
     }
 
     // the epilogue's share of the previous layer's pre-activations, on its way while
-    // the products run: a thread handles two columns of every eighth row (a tile of
-    // at most 32 columns: of every sixteenth).  (Read in the row loop, one column per
+    // the products run: a thread handles two columns of every eighth row (in
+    // tiles of at most 32 or 16 columns of every 16th or 32nd).  (Read in the row loop, one column per
     // lane, each row's load waited behind the previous row's stores: a backward
     // launch of 4 networks, 256 rows and 256 columns took 26 us, now 8; a forward one
     // 14.5, now 8.5, cold caches)
     constexpr int kWarps = kGemmThreads / 32;
     const int rows = min(kTileM, g.M - m0);
     const bool pairs = nt <= 64 && g.ldc % 2 == 0 && n0 % 2 == 0 && g.zc % 2 == 0;
-    // a tile of at most 32 columns: half a warp per row
-    const int lpr = nt <= 32 ? 16 : 32, rpw = 32 / lpr;
+    // a tile of at most 32 (16) columns: half (a quarter of) a warp per row
+    const int lpr = nt <= 16 ? 8 : nt <= 32 ? 16 : 32, rpw = 32 / lpr;
     const int col = 2 * (lane & (lpr - 1));
     const int row_in = warp * rpw + lane / lpr;
     const bool mine = col < nt;

@@ -135,13 +135,14 @@ constexpr int kTrainRows = 65536;
 
 // Columns per tile: at most 64, the width the epilogue handles two columns per lane
 // (an output layer of 80 columns as one tile took 11.1 us, as 48 + 32 8.5, cold
-// caches), and at most 32 while the product then still has no more CTAs than SMs:
-// half the epilogue per CTA, on SMs that had none (4 networks, 256 columns: a
-// minibatch of 256 rows 88 -> 77 us, of 32 81 -> 68, of 512 163 -> 158).
+// caches), and at most 32, then 16, while the product still has no more CTAs than
+// SMs: a shorter epilogue per CTA, on SMs that had none (4 networks, 256 columns, at
+// most 64 / 32 / 16: a minibatch of 256 rows 88 / 77 / 74 us, of 32 81 / 68 / 63).
 constexpr int kSms = 152;
 int n_tile_for(int M, int N, int nz)
 {
-    const int most = (M + 127) / 128 * ((N + 31) / 32) * nz <= kSms ? 32 : 64;
+    const int mt = (M + 127) / 128 * nz;
+    const int most = mt * ((N + 15) / 16) <= kSms ? 16 : mt * ((N + 31) / 32) <= kSms ? 32 : 64;
     const int tiles = (N + most - 1) / most;
     return ((N + tiles - 1) / tiles + 15) / 16 * 16;
 }

@@ -415,25 +415,45 @@ __global__ void k_gather_rows(const __nv_bfloat16 *__restrict__ sx, const float 
         y[row * ny + c] = ok ? sy[(size_t)src * ny + c] : 0.f;
 }
 
+// float(sqrt(x)) for x >= 0 without the float64 square root: the float32 root r of x,
+// corrected by the float64 residual x - r^2 (exact to 2^-53 of x): r + e / (2 r) is
+// within 2^-47 of the root before its one rounding.  Values whose float32 image is not
+// an ordinary number take the float64 root.
+__device__ __forceinline__ float sqrt_to_float(double x)
+{
+    const float xf = (float)x;
+    if (!(xf > 1e-30f && xf < 1e30f))
+        return (float)sqrt(x);
+    const float r = sqrtf(xf);
+    const float e = (float)fma(-(double)r, (double)r, x);
+    return fmaf(e, 0.5f / r, r);
+}
+
 // Mean and spread (population standard deviation) over the networks of the
-// de-normalised outputs y * ys + ym, for rows < B and the n_out valid columns.
-__global__ void k_ens_stats(const float *__restrict__ y_all, int n_nets, int bp, int ldy, int B,
-                            int n_out, const float *__restrict__ ym, const float *__restrict__ ys,
-                            float *__restrict__ mean, float *__restrict__ spread)
+// de-normalised outputs y * ys + ym, for rows < B and the n_out valid columns, in
+// float64.  inv: 1 / n_nets where that is exact (a power of two), else 0.  The float64
+// unit bounds it: two divisions and a square root were three quarters of its
+// operations (4096 x 65 outputs of 4 networks: 27 us, now 18.6).
+__global__ void k_ens_stats(const float *__restrict__ y_all, int n_nets, double inv, int bp, int ldy,
+                            int B, int n_out, const float *__restrict__ ym,
+                            const float *__restrict__ ys, float *__restrict__ mean,
+                            float *__restrict__ spread)
 {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x + after_previous();
     if (idx >= B * n_out)
         return;
     const int r = idx / n_out, c = idx - r * n_out;
+    const double sc = ys[c], of = ym[c];
     double s1 = 0.0, s2 = 0.0;
     for (int k = 0; k < n_nets; ++k) {
-        const double v = (double)y_all[((size_t)k * bp + r) * ldy + c] * ys[c] + ym[c];
+        const double v = (double)y_all[((size_t)k * bp + r) * ldy + c] * sc + of;
         s1 += v;
         s2 += v * v;
     }
-    const double m = s1 / n_nets;
+    const double m = inv != 0.0 ? __dmul_rn(s1, inv) : s1 / n_nets;
+    const double q = inv != 0.0 ? __dmul_rn(s2, inv) : s2 / n_nets;
     mean[idx] = (float)m;
-    spread[idx] = (float)sqrt(fmax(0.0, s2 / n_nets - m * m));
+    spread[idx] = sqrt_to_float(fmax(0.0, q - m * m));
 }
 
 } // namespace
@@ -786,7 +806,8 @@ int npsim_surr_predict(npsim_surr_t s, const float *X, int32_t B, float *Y_mean,
     }
     float *d_mean = s->ystat, *d_spread = s->ystat + (size_t)B * s->n_out;
     const int ne = B * s->n_out;
-    SR_CUDA(launch_after(k_ens_stats, dim3((ne + 255) / 256), 256, 0, s->st, s->y_all, s->n_nets, bp,
+    const double inv = (s->n_nets & (s->n_nets - 1)) == 0 ? 1.0 / s->n_nets : 0.0;
+    SR_CUDA(launch_after(k_ens_stats, dim3((ne + 255) / 256), 256, 0, s->st, s->y_all, s->n_nets, inv, bp,
                          s->n_out_p, B, s->n_out, s->d_ym, s->d_ys, d_mean, d_spread));
     SR_CUDA(fetch_flags(s));
     if (Y_spread == Y_mean + ne) { // back to back on the host too: one copy

@@ -57,3 +57,36 @@ def test_gradients_and_a_step_at_tile_edges(P, n_in, hidden, n_out, rows):
         sel = live & (np.abs(g) > 1e-6)
         assert np.abs(p1[sel] - w1[sel]).max() <= 1e-3 * lr + 1e-6 * np.abs(flat[sel]).max()
         assert np.all(p1[~live] == 0)
+
+
+@pytest.mark.parametrize("nets", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("scale", [1e-25, 1.0, 1e12])
+def test_mean_and_spread_over_the_networks(P, nets, scale):
+    """Against float64 statistics of each network's own float32 predictions (one
+    network alone with the same parameters gives its outputs, and a spread of what
+    rounding leaves of v^2 - v v, below 2^-26 of v).  The
+    outputs differ by an offset of about their own size, so neither the mean nor the
+    spread cancels; the float32 rounding of the single outputs (2^-24) moves the mean
+    and the spread by at most 4 x 2^-24 of the largest output."""
+    rng = np.random.default_rng(nets)
+    X = rng.standard_normal((200, 5)).astype(np.float32)
+    kw = dict(n_in=5, n_hidden=32, n_layers=2, n_out=7)
+    ym = (scale * rng.standard_normal(7)).astype(np.float32)
+    ys = (scale * (1 + rng.random(7))).astype(np.float32)
+    one = (np.zeros(5, np.float32), np.ones(5, np.float32), ym, ys)
+    with P.Surrogate(n_nets=nets, seed=9, **kw) as s:
+        s.set_norm(*one)
+        m, sp = s.predict(X)
+        flats = [s.get_params(k)[0] for k in range(nets)]
+    outs = []
+    for f in flats:
+        with P.Surrogate(n_nets=1, seed=1, **kw) as s:
+            s.set_norm(*one)
+            s.set_params(0, f)
+            y, z = s.predict(X)
+            assert np.all(z <= 2.0 ** -26 * np.abs(y))
+            outs.append(y.astype(np.float64))
+    outs = np.array(outs)
+    tol = 4 * 2.0 ** -24 * np.abs(outs).max()
+    assert np.abs(m - outs.mean(0)).max() <= tol
+    assert np.abs(sp - outs.std(0)).max() <= tol

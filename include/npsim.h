@@ -129,8 +129,11 @@ void npsim_destroy(npsim_sim_t sim);
  * captured CUDA graphs.  Returns after one device-to-host read of the error
  * word: NONFINITE if any position became non-finite, TIMEOUT if a bounded wait
  * expired, ESCAPED if (wall 1) an NP was farther than 2 max(R0, R(t)) from the
- * centre during some step.  The steps were taken in every case; the word is
- * cleared by the read.  n_steps = 0 is a no-op.
+ * centre during some step.  The steps were taken in every case but TIMEOUT; the
+ * word is cleared by the read.  After TIMEOUT, from this or any other call of a
+ * simulation, positions, velocities and forces are undefined and the step count
+ * (npsim_get_state) is the device's: set the state (npsim_set_state) or load a
+ * checkpoint before going on.  n_steps = 0 is a no-op.
  */
 int npsim_step(npsim_sim_t sim, int64_t n_steps);
 
@@ -159,7 +162,7 @@ int npsim_set_state(npsim_sim_t sim, const double *x, const double *v, int64_t s
 
 /* Forces at the current state into host F (n x 3).  what = 0: total force (pair +
  * external, the one the integrator uses); 1: pair forces only (step ii);
- * 2: LJ only; 3: Coulomb only. */
+ * 2: LJ only; 3: Coulomb only.  Errors: INVALID_ARG, CUDA, TIMEOUT (as npsim_step). */
 int npsim_forces(npsim_sim_t sim, int what, double *F);
 
 /* Float32 mirror of the positions (x, y, z, charge) into a caller-owned device
@@ -412,6 +415,14 @@ int npsim_gemm_bf16(const uint16_t *A, const uint16_t *B, int32_t M, int32_t N, 
  * output; the call that launched it returns NPSIM_ERR_TIMEOUT.  This lets a
  * test drive that path without a stuck GPU.  Errors: INVALID_ARG (cycles < 0). */
 int npsim_test_wait_cycles(int64_t cycles);
+
+/* Test hook of the failure path of the list kernels (no counterpart in the paper): a wait
+ * at their grid barrier in simulation `sim` gives up after `polls` looks at the
+ * counter; 0 gives up without a look, -1 restores the default (2^22, seconds; more
+ * beyond 2^21 NPs).  A wait that gives up makes its launch set the error flag and
+ * return; the list kernels queued behind it do nothing, and the call returns
+ * NPSIM_ERR_TIMEOUT.  Errors: INVALID_ARG (no neighbour lists, polls out of range). */
+int npsim_test_list_wait(npsim_sim_t sim, int64_t polls);
 
 /*
  * All-pairs Coulomb forces without any device allocation.  The paper has no

@@ -149,6 +149,7 @@ def lib():
                                           C.c_int32, C.c_int32, C.c_int32, C.c_int32, _f]
             L.npsim_chunk_steps.argtypes = [_h, _i32]
             L.npsim_test_wait_cycles.argtypes = [C.c_int64]
+            L.npsim_test_list_wait.argtypes = [_h, C.c_int64]
             L.npsim_profile.argtypes = [_h, C.c_int]
             L.npsim_kernel_times.argtypes = [_h, _d, _i32]
             L.npsim_ens_profile.argtypes = [_h, C.c_int]
@@ -419,6 +420,11 @@ def npsim_launches_per_step(h):
     a = C.c_int32()
     _check(lib().npsim_launches_per_step(h, C.byref(a)))
     return a.value
+
+
+def npsim_test_list_wait(h, polls):
+    """Bound (polls) of the list kernels' barrier waits in one simulation; -1 = default."""
+    _check(lib().npsim_test_list_wait(h, int(polls)))
 
 
 def npsim_cell_grid(h):

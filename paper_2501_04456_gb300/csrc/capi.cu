@@ -218,7 +218,7 @@ struct npsim_sim {
     size_t cells_alloc = 0;  // sort keys the cell buffers hold
     NbrList nl{};          // Verlet list over the cells (cell-list LJ)
     int *d_gate = nullptr; // 1: rebuild the cell and neighbour lists at the next pass
-    unsigned *list_bar = nullptr; // counters of the list kernels' grid barrier [3], gates [3]
+    unsigned *list_bar = nullptr; // words of the list kernels' grid barrier (kBarWords)
     int fused_cap = 0;            // largest n that takes fused steps
     float4 *sxq2 = nullptr;       // the other cell-ordered records of fused steps (lazy)
 
@@ -606,7 +606,8 @@ int enqueue_pass(npsim_sim *s, int mode, bool want_lj, bool want_coul, bool ext,
         NP_CUDA(mark(KG_CELL_LJ, 0));
         NP_CUDA(launch_lj_nbr(s->grid, s->cb, s->xq, s->typ, s->n,
                               want_lj ? s->tab_full : s->tab_coul,
-                              cell_coul ? s->d_rcc2 : nullptr, s->nl, s->F_lj, s->d_gate, st));
+                              cell_coul ? s->d_rcc2 : nullptr, s->nl, s->F_lj, s->d_gate, s->d_flags,
+                              st));
         NP_CUDA(mark(KG_CELL_LJ, 1));
     }
     if (ap) {
@@ -743,11 +744,51 @@ int grow_neighbour_list(npsim_sim *s)
     return set_gate(s, 1);
 }
 
+// Bound of a wait at the list kernels' grid barrier in polls (about a microsecond
+// each): 2^22, and beyond 2^21 NPs in proportion to n^2, because a build compares each NP
+// with every member of its cell -- all of them when one far NP stretches the grid or the
+// positions are not finite (by count of its loads 2 s at 4 million NPs, bound 16 s).
+unsigned list_wait_polls(int n)
+{
+    const double f = (double)n / (1 << 21);
+    return (unsigned)std::min(4294967295.0, std::ldexp(std::max(1.0, f * f), 22));
+}
+
+int set_list_wait(npsim_sim *s, unsigned polls)
+{
+    NP_CUDA(cudaMemcpyAsync(s->list_bar + kBarPolls, &polls, sizeof(polls), cudaMemcpyHostToDevice,
+                            s->user));
+    NP_CUDA(cudaStreamSynchronize(s->user)); // polls lives on this stack frame
+    return NPSIM_OK;
+}
+
+// A list kernel's barrier wait has given up and the launches behind it have left the
+// lists alone: its counters and the sort counts back to zero, the lists to be built
+// anew, and the host's step count to the device's, which steps that were not finished
+// have not moved on.
+int recover_lists(npsim_sim *s)
+{
+    if (s->list_bar) {
+        NP_CUDA(cudaMemsetAsync(s->list_bar, 0, kBarPolls * sizeof(unsigned), s->user));
+        NP_CUDA(cudaMemsetAsync(s->cb.count, 0, sizeof(int) * s->cells_alloc, s->user));
+    }
+    long long step = 0;
+    NP_CUDA(cudaMemcpyAsync(&step, s->d_step, sizeof(step), cudaMemcpyDeviceToHost, s->user));
+    NP_CUDA(cudaStreamSynchronize(s->user));
+    s->step = step;
+    return set_gate(s, 1);
+}
+
 int read_flags(npsim_sim *s)
 {
     int h = 0;
     NP_CUDA(cudaMemcpyAsync(&h, s->d_flags, sizeof(int), cudaMemcpyDeviceToHost, s->user));
     NP_CUDA(cudaStreamSynchronize(s->user));
+    if (h & FLAG_TIMEOUT) { // before all else: the other bits may come of it
+        NP_CUDA(cudaMemsetAsync(s->d_flags, 0, sizeof(int), s->user));
+        int rc = recover_lists(s);
+        return rc ? rc : set_err(NPSIM_ERR_TIMEOUT, "a bounded device wait expired");
+    }
     if (h & FLAG_NBR_OVERFLOW) {
         const int rest = h & ~FLAG_NBR_OVERFLOW;
         NP_CUDA(cudaMemcpyAsync(s->d_flags, &rest, sizeof(int), cudaMemcpyHostToDevice, s->user));
@@ -761,16 +802,6 @@ int read_flags(npsim_sim *s)
         NP_CUDA(cudaMemsetAsync(s->d_flags, 0, sizeof(int), s->user));
         if (h & FLAG_NONFINITE)
             return set_err(NPSIM_ERR_NONFINITE, "a position became non-finite");
-        if (h & FLAG_TIMEOUT) {
-            if (s->list_bar) { // the barrier it left, and the lists it did not finish
-                NP_CUDA(cudaMemsetAsync(s->list_bar, 0, 6 * sizeof(unsigned), s->user));
-                NP_CUDA(cudaMemsetAsync(s->cb.count, 0, sizeof(int) * s->cells_alloc, s->user));
-                int rc = set_gate(s, 1);
-                if (rc)
-                    return rc;
-            }
-            return set_err(NPSIM_ERR_TIMEOUT, "a bounded device wait expired");
-        }
         if (h & FLAG_ESCAPED)
             return set_err(NPSIM_ERR_ESCAPED,
                            "an NP was farther than 2 max(R0, R(t)) from the droplet centre");
@@ -1455,10 +1486,15 @@ int create_impl(const npsim_type_t *types, const npsim_params_t *params, int64_t
         BAIL_CUDA(cudaMemset(s->nl.builds, 0, sizeof(unsigned long long)));
         BAIL_CUDA(dalloc(&s->d_gate, 1));
         s->fused_cap = list_steps_capacity();
-        BAIL_CUDA(dalloc(&s->list_bar, 6));
-        BAIL_CUDA(cudaMemset(s->list_bar, 0, 6 * sizeof(unsigned)));
+        BAIL_CUDA(dalloc(&s->list_bar, kBarWords));
+        BAIL_CUDA(cudaMemsetAsync(s->list_bar, 0, kBarWords * sizeof(unsigned), s->user));
         BAIL_CUDA(cudaMemset(s->nl.nnbr, 0, sizeof(int) * (size_t)n));
         BAIL_CUDA(cudaMemset(s->nl.nbr, 0, sizeof(unsigned) * (size_t)s->nl.cap * n));
+    }
+    if (s->cell) {
+        rc = set_list_wait(s, list_wait_polls(s->n));
+        if (rc)
+            return bail(rc);
     }
     s->ap_lj = params->lj_mode == 1;
     s->ap = params->coulomb == 1 || s->ap_lj;
@@ -1780,7 +1816,15 @@ int npsim_forces(npsim_sim_t s, int what, double *F)
     int rc = enqueue_pass(s, MODE_FORCES, lj, coul, what == 0, s->F_tmp, s->user);
     if (rc)
         return rc;
-    return copy_state_out(s, s->F_tmp, nullptr, nullptr, F);
+    rc = copy_state_out(s, s->F_tmp, nullptr, nullptr, F);
+    return rc || !s->cell ? rc : read_flags(s); // a build of the lists may have given up
+}
+
+int npsim_test_list_wait(npsim_sim_t s, int64_t polls)
+{
+    NP_REQUIRE(s && s->cell, "a simulation with neighbour lists is required");
+    NP_REQUIRE(polls >= -1 && polls <= 0xffffffffll, "polls must be -1 .. 2^32 - 1");
+    return set_list_wait(s, polls < 0 ? list_wait_polls(s->n) : (unsigned)polls);
 }
 
 int npsim_positions_device(npsim_sim_t s, float *dev_xyzq)

@@ -313,7 +313,7 @@ struct ListBuildArgs {
     unsigned long long *builds;
     int *flags;
     const int *gate;
-    unsigned *bar; // [0] CTAs arrived, [1] CTAs done, [2] slots drawn: 0 between launches
+    unsigned *bar; // kBar* words
 };
 
 // The neighbour list of the NP at cell-order slot p: the partners within (rc_ab +
@@ -390,22 +390,44 @@ __device__ __forceinline__ void nbr_slot(const ListBuildArgs &A, const float4 *s
     A.x_ref[i] = make_float4(pi.x, pi.y, pi.z, 0.0f);
 }
 
+// Shared memory of the list build.
+struct ListBuildSmem {
+    int warp[kScanThreads / 32 + 1];
+    int ok;
+    unsigned polls; // bound of a barrier wait, used by the first thread
+    int off[kScanTile]; // prefix of the scan tiles' totals (when they are few enough)
+    float4 tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    float rl2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
+    float rmax[NPSIM_MAX_TYPES];
+};
+
+// True in every thread while FLAG_TIMEOUT is set.  A launch whose barrier wait gave up
+// leaves the barrier's counters, the sort counts and the lists half done: until the host
+// has put them right (read_flags), the list kernels queued behind it must not touch
+// them -- a build would pass its barriers early and scatter past its arrays.
+__device__ __forceinline__ bool wait_expired(const int *flags)
+{
+    return __syncthreads_or(threadIdx.x == 0 && (*(volatile const int *)flags & FLAG_TIMEOUT)) != 0;
+}
+
 // Barrier over the CTAs of a cooperative launch (all resident): phase = barriers
-// passed so far, the same in every thread.  A wait is bounded (seconds); one that
+// passed so far, the same in every thread.  A wait is bounded (S.polls); one that
 // gives up sets FLAG_TIMEOUT and returns false in every thread of its CTA, which
-// then leaves the kernel (the host clears the counters when it reads the flag).
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, int *flags, int *s_ok)
+// then leaves the kernel.  Nobody passes a later barrier without its arrival, so the
+// other CTAs give up there in turn.
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, int *flags,
+                                             ListBuildSmem &S)
 {
     __syncthreads();
     ++phase;
     if (threadIdx.x == 0) {
-        const unsigned target = phase * gridDim.x;
+        const unsigned target = phase * gridDim.x, polls = S.polls;
         __threadfence();
-        atomicAdd(bar, 1u);
+        atomicAdd(bar + kBarArrived, 1u);
         int ok = 0;
-        for (int it = 0; it < (1 << 22) && !ok; ++it) {
+        for (unsigned it = 0; it < polls && !ok; ++it) {
             unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar + kBarArrived) : "memory");
             ok = v >= target;
             if (!ok && it > 64)
                 __nanosleep(100);
@@ -413,21 +435,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, int
         if (!ok)
             atomicOr(flags, FLAG_TIMEOUT);
         __threadfence();
-        *s_ok = ok;
+        S.ok = ok;
     }
     __syncthreads();
-    return *s_ok != 0;
+    return S.ok != 0;
 }
-
-// Shared memory of the list build.
-struct ListBuildSmem {
-    int warp[kScanThreads / 32 + 1];
-    int ok;
-    int off[kScanTile]; // prefix of the scan tiles' totals (when they are few enough)
-    float4 tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
-    float rl2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
-    float rmax[NPSIM_MAX_TYPES];
-};
 
 // The phases of a build by every CTA of a cooperative launch, between grid barriers
 // (false: one gave up), the records going to sxq.  The counts are zero on entry and
@@ -443,12 +455,12 @@ __device__ __forceinline__ bool list_build(const ListBuildArgs &A, float4 *sxq, 
     const int m = (A.g.tb > 1 ? A.g.tb : 1) * A.g.n_cells; // sort keys
     const int n_tiles = (m + kScanTile - 1) / kScanTile;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
-    auto barrier = [&]() { return grid_barrier(A.bar, phase, A.flags, &S.ok); };
+    auto barrier = [&]() { return grid_barrier(A.bar, phase, A.flags, S); };
 
     if (tid == 0) {
         if (A.builds)
             ++*A.builds;
-        A.bar[2] = 0u; // slots drawn
+        A.bar[kBarDrawn] = 0u;
     }
     cell_hash(A.g, A.xq, A.typ, n, B.key, B.rank, B.count);
     if (!barrier())
@@ -503,7 +515,7 @@ __device__ __forceinline__ bool list_build(const ListBuildArgs &A, float4 *sxq, 
     for (;;) {
         unsigned first = 0;
         if (lane == 0)
-            first = atomicAdd(A.bar + 2, 32u);
+            first = atomicAdd(A.bar + kBarDrawn, 32u);
         const int left = n - (int)__shfl_sync(0xffffffffu, first, 0); // slots not drawn yet
         if (left <= 0)
             break;
@@ -522,9 +534,9 @@ __device__ __forceinline__ bool barrier_done(unsigned *bar)
     if (threadIdx.x != 0)
         return false;
     __threadfence();
-    if (atomicAdd(bar + 1, 1u) != gridDim.x - 1)
+    if (atomicAdd(bar + kBarDone, 1u) != gridDim.x - 1)
         return false;
-    bar[0] = bar[1] = 0u;
+    bar[kBarArrived] = bar[kBarDone] = 0u;
     __threadfence();
     return true;
 }
@@ -542,7 +554,11 @@ k_list_build(const __grid_constant__ ListBuildArgs A)
     if (A.gate && *A.gate == 0) // nobody writes it while this kernel runs
         return;
     unsigned phase = 0;
+    if (threadIdx.x == 0)
+        S.polls = A.bar[kBarPolls];
     load_tables(A.tab, A.rcc2, A.skin, S.tab, S.rl2, S.rmax);
+    if (wait_expired(A.flags))
+        return;
     if (list_build(A, A.b.sxq, S, phase))
         barrier_done(A.bar);
 }
@@ -728,13 +744,16 @@ k_lj_nbr(const __grid_constant__ CellGrid g, const int *__restrict__ start, cons
          const int *__restrict__ key, const float4 *__restrict__ sxq, int n,
          const PairTab *__restrict__ tab, const float *__restrict__ rcc2, int cap,
          const unsigned *__restrict__ nbr, const int *__restrict__ nnbr,
-         float *__restrict__ F_lj, int *__restrict__ gate)
+         float *__restrict__ F_lj, int *__restrict__ gate, const int *__restrict__ flags)
 {
     __shared__ float4 s_tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
     __shared__ float s_rl2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
     __shared__ float s_rcc2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
     __shared__ float s_rmax[NPSIM_MAX_TYPES];
+    const bool expired = *flags & FLAG_TIMEOUT; // nobody sets it while this kernel runs
     load_tables(tab, COUL ? rcc2 : nullptr, 0.0f, s_tab, s_rl2, s_rmax, s_rcc2);
+    if (expired) // unfinished lists (wait_expired); the gate stays open
+        return;
     if (gate && blockIdx.x == 0 && threadIdx.x == 0)
         *gate = 0; // every build kernel of this step has run; the integrator may reopen it
     const int p = (int)(gridDim.x - 1 - blockIdx.x) * (int)blockDim.x + (int)threadIdx.x;
@@ -837,7 +856,10 @@ k_list_steps(const __grid_constant__ FusedStepArgs a, const __grid_constant__ St
     load_tables(L.tab, COUL ? L.rcc2 : nullptr, 0.0f, s_tab, s_rl2, s_rmax, s_rcc2);
     if (threadIdx.x < NPSIM_MAX_TYPES)
         s_tc[threadIdx.x] = p.tc[threadIdx.x];
-    __syncthreads();
+    if (threadIdx.x == 0)
+        S.polls = L.bar[kBarPolls];
+    if (wait_expired(L.flags)) // its barrier orders the tables, too
+        return;
     const long long step0 = *a.I.step;
     const float R0f = (float)p.R0;
     unsigned phase = 0;
@@ -873,7 +895,7 @@ k_list_steps(const __grid_constant__ FusedStepArgs a, const __grid_constant__ St
     float nz[3] = {0.f, 0.f, 0.f};
     for (int j = 1; j <= a.steps; ++j) {
         const bool last = j == a.steps;
-        if (!grid_barrier(L.bar, phase, L.flags, &S.ok))
+        if (!grid_barrier(L.bar, phase, L.flags, S))
             return;
         float4 *cur = (j & 1) ? L.b.sxq : a.sxq2, *nxt = (j & 1) ? a.sxq2 : L.b.sxq;
         volatile unsigned *w = a.gates;
@@ -881,8 +903,8 @@ k_list_steps(const __grid_constant__ FusedStepArgs a, const __grid_constant__ St
         if (build) {
             if (mine && j > 1)
                 slot_store(a, n, s);
-            if (!grid_barrier(L.bar, phase, L.flags, &S.ok) || !list_build(L, cur, S, phase) ||
-                !grid_barrier(L.bar, phase, L.flags, &S.ok))
+            if (!grid_barrier(L.bar, phase, L.flags, S) || !list_build(L, cur, S, phase) ||
+                !grid_barrier(L.bar, phase, L.flags, S))
                 return;
         }
         if (mine && (build || j == 1)) {
@@ -1071,7 +1093,7 @@ cudaError_t launch_list_steps(const CellGrid &g, const CellBufs &b, int n, const
     a.sxq2 = sxq2;
     a.F_lj = F_lj;
     a.gate = I.nbr_gate;
-    a.gates = bar + 3;
+    a.gates = bar + kBarGates;
     a.steps = steps;
     // a warp's 32 slots per CTA while that leaves SMs free (the other warps help the
     // builds), then one CTA per SM, two when their threads do not reach n
@@ -1085,7 +1107,8 @@ cudaError_t launch_list_steps(const CellGrid &g, const CellBufs &b, int n, const
 
 cudaError_t launch_lj_nbr(const CellGrid &g, const CellBufs &b, const float4 *xq,
                           const int *typ, int n, const PairTab *tab, const float *rcc2,
-                          const NbrList &l, float *F_lj, int *gate, cudaStream_t st)
+                          const NbrList &l, float *F_lj, int *gate, const int *flags,
+                          cudaStream_t st)
 {
     (void)xq; // the current positions are the cell-ordered records b.sxq
     (void)typ;
@@ -1093,10 +1116,10 @@ cudaError_t launch_lj_nbr(const CellGrid &g, const CellBufs &b, const float4 *xq
     const int grid = (n + B - 1) / B;
     if (rcc2)
         k_lj_nbr<true><<<grid, B, 0, st>>>(g, b.start, b.sorted, b.key, b.sxq, n, tab, rcc2,
-                                           l.cap, l.nbr, l.nnbr, F_lj, gate);
+                                           l.cap, l.nbr, l.nnbr, F_lj, gate, flags);
     else
         k_lj_nbr<false><<<grid, B, 0, st>>>(g, b.start, b.sorted, b.key, b.sxq, n, tab, nullptr,
-                                            l.cap, l.nbr, l.nnbr, F_lj, gate);
+                                            l.cap, l.nbr, l.nnbr, F_lj, gate, flags);
     return cudaGetLastError();
 }
 

@@ -1582,17 +1582,25 @@ struct NbrList {
 // (8 x 8); with it the lists cover both cutoffs and the list force kernel adds
 // C q_a q_b r_ij / r^3 within the Coulomb cutoff to the LJ term.
 // Cell list and neighbour lists of positions xq in one cooperative launch (gate:
-// NULL = always, else only when *gate != 0).  bar: three counters, zero between
-// launches (cleared by the host after FLAG_TIMEOUT).
+// NULL = always, else only when *gate != 0).  bar: kBarWords words, all but the bound
+// zero between launches (cleared by the host after FLAG_TIMEOUT).  While FLAG_TIMEOUT is
+// set the list kernels return without touching anything (wait_expired).
+enum : int {
+    kBarArrived = 0, // CTAs arrived at the grid barrier
+    kBarDone = 1,    // CTAs done
+    kBarDrawn = 2,   // slots drawn by the build's warps
+    kBarGates = 3,   // gates inside a launch of many steps (three)
+    kBarPolls = 6,   // bound of a barrier wait in polls, set by the host
+    kBarWords = 7,
+};
 cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4 *xq,
                               const int *typ, int n, const PairTab *tab, const float *rcc2,
                               float skin, const NbrList &l, int *flags, const int *gate,
                               unsigned *bar, cudaStream_t st);
 // `steps` steps (at most kMaxFusedSteps) from the device step counter on, of a
 // simulation of n <= kMaxFusedNps whose pair forces all come from the lists, in one
-// cooperative launch; I as for the integrator, bar: three words for the barrier and
-// three for the gates, sxq2 a second array of cell-ordered
-// records like b.sxq (its record n far from every NP), F_lj [n][8] scratch.
+// cooperative launch; I as for the integrator, bar as above, sxq2 a second array of
+// cell-ordered records like b.sxq (its record n far from every NP), F_lj [n][8] scratch.
 constexpr int kMaxFusedSteps = 256;
 constexpr int kMaxFusedNps = 65536;
 int list_steps_capacity(); // NPs one launch can hold on the current device
@@ -1602,7 +1610,8 @@ cudaError_t launch_list_steps(const CellGrid &g, const CellBufs &b, int n, const
                               int steps, cudaStream_t st);
 cudaError_t launch_lj_nbr(const CellGrid &g, const CellBufs &b, const float4 *xq,
                           const int *typ, int n, const PairTab *tab, const float *rcc2,
-                          const NbrList &l, float *F_lj, int *gate, cudaStream_t st);
+                          const NbrList &l, float *F_lj, int *gate, const int *flags,
+                          cudaStream_t st);
 int cell_scan_tiles(int n_cells);
 
 // Stats (stats.cu)

@@ -566,14 +566,13 @@ k_list_build(const __grid_constant__ ListBuildArgs A)
 // The forces of the NP at slot p whose list overflowed: every NP of the cells of
 // its build (the NP's sort key holds its build cell; a superset of its list),
 // summed pair by pair into the compensated totals.  Kept out of line so that
-// it takes no registers from the list loops.
+// it takes no registers from the list loops.  Plain pointers: k_list_steps writes
+// all of these arrays in the launch that reads them here.
 template <bool COUL>
-__device__ __noinline__ void cell_slot_forces(int p, const CellGrid g, const int *__restrict__ start,
-                                              const int *__restrict__ sorted,
-                                              const int *__restrict__ key,
-                                              const float4 *__restrict__ sxq,
-                                              float *__restrict__ F_lj, const float4 *s_tab,
-                                              const float *s_rcc2)
+__device__ __noinline__ void cell_slot_forces(int p, const CellGrid g, const int *start,
+                                              const int *sorted, const int *key,
+                                              const float4 *sxq, float *F_lj,
+                                              const float4 *s_tab, const float *s_rcc2)
 {
     const float4 pi = sxq[p];
     const int i = sorted[p];

@@ -481,6 +481,15 @@ ApConfig shape_config(int k)
 // N, remain.
 constexpr size_t kSymMaxBytes = (size_t)8 << 30;
 
+// Coulomb kernels with eight rows per thread add 256 terms to a partner's sum before it
+// is compensated.  Beyond this grouped length the best one-sided kernels had tiles of
+// 512 partners, the same chain (60000 NPs, rms error against float64 4.0e-8, one-sided
+// 4.8e-8); up to it some had 256, and four rows per thread, or the LJ + Coulomb kernels,
+// whose chains are half as long, keep to theirs (16384 NPs 3.1e-8, one-sided 3.4e-8,
+// eight rows 3.8e-8) for 3 to 6 % of the launch (16000: 0.090, eight rows 0.085 ms;
+// 24500: 0.173, 0.168).
+constexpr int kSymLongRows = 32768;
+
 int shape_occupancy(const npsim_sim *s, int k, bool lj)
 {
     int l = 0;
@@ -886,6 +895,9 @@ int autotune(npsim_sim *s)
             // sum_neutral asks for all pairs (250000 NPs, 150000 of them neutral: they
             // took 3.3 ms; every pair evaluated takes 14.2)
             if (occ <= 0 || (s->P.sum_neutral && !lj && shape_ljg(c)))
+                continue;
+            if (!lj && shape_family(c) == SF_SYM && shape_config(c).ki > 4 &&
+                s->grp_len <= kSymLongRows)
                 continue;
             for (int mi = 0; mi < (shape_grouped(c) ? n_m : 1); ++mi) {
                 const int m = shape_grouped(c) ? kRangesPerCta[mi] : 1;

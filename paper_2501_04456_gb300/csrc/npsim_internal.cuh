@@ -525,44 +525,78 @@ __device__ __forceinline__ void sym_rotate(float2 &g, int src)
     g.y = __shfl_sync(0xffffffffu, g.y, src);
 }
 
-// Coulomb-only: ax += d / r^3 for the rows, g += d / r^3 for the partners (the
+// Steps after which a lane starts an entry's sums anew (FOLD): at most 128 rows' terms
+// in one float32 chain, as many as the one-sided kernels add in each half of a pair of a
+// 256-partner tile.  One chain over the 256 rows of KI = 8 rounds more than that: LJ +
+// Coulomb, 16384 charges, rms error against float64 6.0e-8, of the last third of the NPs
+// 7.3e-8; folded 4.4e-8 and 4.8e-8.  The fold costs 0.8 % of an LJ + Coulomb launch
+// (60000 NPs, 0.989 -> 0.997 ms) and 2.9 % of a Coulomb one (100000: 2.345 -> 2.414),
+// which goes without: autotune() leaves KI = 8 to lengths at which 512-partner tiles, no
+// better than one chain of 256, were the best one-sided choice.
+template <int KI, bool FOLD>
+constexpr int kSymFoldSteps = FOLD && KI * 32 > 128 ? 128 / KI : 32;
+
+// The sums of an entry over one run of steps join those of the runs before, which are
+// still at the lane that held the entry when the run began.
+template <int STEPS>
+__device__ __forceinline__ void sym_fold(float2 &h, const float2 &g, int lane)
+{
+    if (STEPS == 32) {
+        h = g;
+    } else {
+        const int src = (lane + STEPS) & 31;
+        h.x = __shfl_sync(0xffffffffu, h.x, src) + g.x;
+        h.y = __shfl_sync(0xffffffffu, h.y, src) + g.y;
+    }
+}
+
+// Coulomb-only: ax += d / r^3 for the rows, g = sum of d / r^3 for the partners (the
 // caller applies the charges and the partners' sign).
-template <int KI>
+template <int KI, bool FOLD>
 __device__ __forceinline__ void coul_sym_sweep(const float4 *__restrict__ s_a,
                                                const float2 *__restrict__ s_b, int lane,
                                                const float2 (&xi)[KI], const float2 (&yi)[KI],
                                                const float2 (&zi)[KI], float2 (&ax)[KI],
-                                               float2 (&ay)[KI], float2 (&az)[KI], float2 &gx,
-                                               float2 &gy, float2 &gz)
+                                               float2 (&ay)[KI], float2 (&az)[KI], float2 &hx,
+                                               float2 &hy, float2 &hz)
 {
     const float2 eps2 = make_float2(kPairSelfEps, kPairSelfEps);
+    constexpr int STEPS = kSymFoldSteps<KI, FOLD>;
     const int src = (lane + 1) & 31;
+    hx = hy = hz = make_float2(0.0f, 0.0f);
+#pragma unroll 1
+    for (int s0 = 0; s0 < 32; s0 += STEPS) {
+        float2 gx = make_float2(0.0f, 0.0f), gy = gx, gz = gx;
 #pragma unroll 8
-    for (int s = 0; s < 32; ++s) {
-        const int m = (lane + s) & 31;
-        const float4 a = s_a[m];
-        const float2 nz = s_b[m];
-        const float2 nx = make_float2(a.x, a.y), ny = make_float2(a.z, a.w);
+        for (int s = s0; s < s0 + STEPS; ++s) {
+            const int m = (lane + s) & 31;
+            const float4 a = s_a[m];
+            const float2 nz = s_b[m];
+            const float2 nx = make_float2(a.x, a.y), ny = make_float2(a.z, a.w);
 #pragma unroll
-        for (int k = 0; k < KI; ++k) {
-            const float2 dx = __fadd2_rn(xi[k], nx);
-            const float2 dy = __fadd2_rn(yi[k], ny);
-            const float2 dz = __fadd2_rn(zi[k], nz);
-            float2 r2 = __ffma2_rn(dz, dz, eps2);
-            r2 = __ffma2_rn(dy, dy, r2);
-            r2 = __ffma2_rn(dx, dx, r2);
-            const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-            const float2 f = __fmul2_rn(__fmul2_rn(ri, ri), ri);
-            ax[k] = __ffma2_rn(f, dx, ax[k]);
-            ay[k] = __ffma2_rn(f, dy, ay[k]);
-            az[k] = __ffma2_rn(f, dz, az[k]);
-            gx = __ffma2_rn(f, dx, gx);
-            gy = __ffma2_rn(f, dy, gy);
-            gz = __ffma2_rn(f, dz, gz);
+            for (int k = 0; k < KI; ++k) {
+                const float2 dx = __fadd2_rn(xi[k], nx);
+                const float2 dy = __fadd2_rn(yi[k], ny);
+                const float2 dz = __fadd2_rn(zi[k], nz);
+                float2 r2 = __ffma2_rn(dz, dz, eps2);
+                r2 = __ffma2_rn(dy, dy, r2);
+                r2 = __ffma2_rn(dx, dx, r2);
+                const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+                const float2 f = __fmul2_rn(__fmul2_rn(ri, ri), ri);
+                ax[k] = __ffma2_rn(f, dx, ax[k]);
+                ay[k] = __ffma2_rn(f, dy, ay[k]);
+                az[k] = __ffma2_rn(f, dz, az[k]);
+                gx = __ffma2_rn(f, dx, gx);
+                gy = __ffma2_rn(f, dy, gy);
+                gz = __ffma2_rn(f, dz, gz);
+            }
+            sym_rotate(gx, src);
+            sym_rotate(gy, src);
+            sym_rotate(gz, src);
         }
-        sym_rotate(gx, src);
-        sym_rotate(gy, src);
-        sym_rotate(gz, src);
+        sym_fold<STEPS>(hx, gx, lane);
+        sym_fold<STEPS>(hy, gy, lane);
+        sym_fold<STEPS>(hz, gz, lane);
     }
 }
 
@@ -575,45 +609,54 @@ __device__ __forceinline__ void ljc_sym_sweep(const float4 *__restrict__ s_a,
                                               const float2 (&xi)[KI], const float2 (&yi)[KI],
                                               const float2 (&zi)[KI], const float4 cst,
                                               float2 (&ax)[KI], float2 (&ay)[KI],
-                                              float2 (&az)[KI], float2 &gx, float2 &gy, float2 &gz)
+                                              float2 (&az)[KI], float2 &hx, float2 &hy, float2 &hz)
 {
     const float2 eps2 = make_float2(kPairSelfEps, kPairSelfEps);
     const float2 sig2 = make_float2(cst.x, cst.x);
     const float2 e48 = make_float2(2.0f * cst.y, 2.0f * cst.y);
     const float2 em24 = make_float2(-cst.y, -cst.y);
     const float2 cqq = make_float2(cst.w, cst.w);
+    constexpr int STEPS = kSymFoldSteps<KI, true>;
     const int src = (lane + 1) & 31;
-    for (int s = 0; s < 32; ++s) {
-        const int m = (lane + s) & 31;
-        const float4 a = s_a[m];
-        const float2 nz = s_b[m];
-        const float2 nx = make_float2(a.x, a.y), ny = make_float2(a.z, a.w);
+    hx = hy = hz = make_float2(0.0f, 0.0f);
+#pragma unroll 1
+    for (int s0 = 0; s0 < 32; s0 += STEPS) {
+        float2 gx = make_float2(0.0f, 0.0f), gy = gx, gz = gx;
+        for (int s = s0; s < s0 + STEPS; ++s) {
+            const int m = (lane + s) & 31;
+            const float4 a = s_a[m];
+            const float2 nz = s_b[m];
+            const float2 nx = make_float2(a.x, a.y), ny = make_float2(a.z, a.w);
 #pragma unroll
-        for (int k = 0; k < KI; ++k) {
-            const float2 dx = __fadd2_rn(xi[k], nx);
-            const float2 dy = __fadd2_rn(yi[k], ny);
-            const float2 dz = __fadd2_rn(zi[k], nz);
-            float2 r2 = __ffma2_rn(dz, dz, eps2);
-            r2 = __ffma2_rn(dy, dy, r2);
-            r2 = __ffma2_rn(dx, dx, r2);
-            const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-            const float2 ri2 = __fmul2_rn(ri, ri);
-            const float2 s2 = __fmul2_rn(sig2, ri2);
-            const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
-            float2 t = __fmul2_rn(s6, __ffma2_rn(e48, s6, em24));
-            t.x = r2.x < cst.z ? t.x : 0.0f;
-            t.y = r2.y < cst.z ? t.y : 0.0f;
-            const float2 f = __fmul2_rn(__ffma2_rn(cqq, ri, t), ri2);
-            ax[k] = __ffma2_rn(f, dx, ax[k]);
-            ay[k] = __ffma2_rn(f, dy, ay[k]);
-            az[k] = __ffma2_rn(f, dz, az[k]);
-            gx = __ffma2_rn(f, dx, gx);
-            gy = __ffma2_rn(f, dy, gy);
-            gz = __ffma2_rn(f, dz, gz);
+            for (int k = 0; k < KI; ++k) {
+                const float2 dx = __fadd2_rn(xi[k], nx);
+                const float2 dy = __fadd2_rn(yi[k], ny);
+                const float2 dz = __fadd2_rn(zi[k], nz);
+                float2 r2 = __ffma2_rn(dz, dz, eps2);
+                r2 = __ffma2_rn(dy, dy, r2);
+                r2 = __ffma2_rn(dx, dx, r2);
+                const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+                const float2 ri2 = __fmul2_rn(ri, ri);
+                const float2 s2 = __fmul2_rn(sig2, ri2);
+                const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
+                float2 t = __fmul2_rn(s6, __ffma2_rn(e48, s6, em24));
+                t.x = r2.x < cst.z ? t.x : 0.0f;
+                t.y = r2.y < cst.z ? t.y : 0.0f;
+                const float2 f = __fmul2_rn(__ffma2_rn(cqq, ri, t), ri2);
+                ax[k] = __ffma2_rn(f, dx, ax[k]);
+                ay[k] = __ffma2_rn(f, dy, ay[k]);
+                az[k] = __ffma2_rn(f, dz, az[k]);
+                gx = __ffma2_rn(f, dx, gx);
+                gy = __ffma2_rn(f, dy, gy);
+                gz = __ffma2_rn(f, dz, gz);
+            }
+            sym_rotate(gx, src);
+            sym_rotate(gy, src);
+            sym_rotate(gz, src);
         }
-        sym_rotate(gx, src);
-        sym_rotate(gy, src);
-        sym_rotate(gz, src);
+        sym_fold<STEPS>(hx, gx, lane);
+        sym_fold<STEPS>(hy, gy, lane);
+        sym_fold<STEPS>(hz, gz, lane);
     }
 }
 
@@ -643,8 +686,8 @@ struct SymSmem {
 //    lo) pairs, one TwoSum per tile, as ljc_row_segment does;
 //  * the partners' sums over the ITILE rows of every two-sided tile to
 //    col[c * col_ld + position - (r + 1) ITILE], c = x, y, z: one float32 per
-//    ITILE rows (a lane adds 32 KI terms, then the warps' sums are added
-//    pairwise), which the reduction adds compensated.
+//    ITILE rows (a lane adds 32 KI terms, with LJ 128 at a time, then the warps'
+//    sums are added pairwise), which the reduction adds compensated.
 // A warp's rows are consecutive positions (32 KI divides the groups' 256-block
 // padding), so they have one type.  The sums are kept in units of `scale`, the
 // charge product when it is not small (the Coulomb-only sweep then needs no
@@ -765,7 +808,7 @@ __device__ __forceinline__ void sym_row_segment(const float4 *__restrict__ xq,
                 if (lj)
                     ljc_sym_sweep<KI>(sa, sb, lane, xi, yi, zi, cst, ax, ay, az, gx, gy, gz);
                 else if (active && (!LJ || (has_coul && cst.w != 0.0f)))
-                    coul_sym_sweep<KI>(sa, sb, lane, xi, yi, zi, ax, ay, az, gx, gy, gz);
+                    coul_sym_sweep<KI, LJ>(sa, sb, lane, xi, yi, zi, ax, ay, az, gx, gy, gz);
                 smem.g[cur][0][warp][32 * sg + lane] = make_float2(-scale * gx.x, -scale * gx.y);
                 smem.g[cur][1][warp][32 * sg + lane] = make_float2(-scale * gy.x, -scale * gy.y);
                 smem.g[cur][2][warp][32 * sg + lane] = make_float2(-scale * gz.x, -scale * gz.y);

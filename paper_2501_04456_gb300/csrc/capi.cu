@@ -553,8 +553,9 @@ cudaError_t shape_launch(const npsim_sim *s, int k, bool lj, bool coul, const St
     const int f = shape_family(k, &l);
     if (f == SF_SYM || f == SF_SYMLJ)
         return launch_allpairs_sym(f == SF_SYMLJ, l, sk, s->xq, s->perm, s->tblk,
-                                   pair_table(s, lj, coul), coul ? s->any_charge : 0, s->ap_work,
-                                   slots, st);
+                                   pair_table(s, lj, coul),
+                                   !coul || !s->any_charge ? 0 : s->P.sum_neutral ? 2 : 1,
+                                   s->ap_work, slots, st);
     if (f == SF_LJG)
         return launch_allpairs_ljgrp(l, sk, s->xq, s->perm, s->n_perm, s->tblk,
                                      pair_table(s, lj, coul), lj ? s->rc2_lim : 0.0f,
@@ -891,9 +892,8 @@ int autotune(npsim_sim *s)
         const bool log = getenv("NPSIM_AUTOTUNE_LOG") != nullptr; // per-shape times to stderr
         for (int c = 0; c < nc; ++c) {
             const int occ = shape_occupancy(s, c, lj);
-            // the LJ + Coulomb kernels leave out type pairs without a charge product;
-            // sum_neutral asks for all pairs (250000 NPs, 150000 of them neutral: they
-            // took 3.3 ms; every pair evaluated takes 14.2)
+            // for the full sum of neutral NPs the LJ + Coulomb kernels have only their
+            // dearer sweep (no charge product to take as the unit of the sums)
             if (occ <= 0 || (s->P.sum_neutral && !lj && shape_ljg(c)))
                 continue;
             if (!lj && shape_family(c) == SF_SYM && shape_config(c).ki > 4 &&

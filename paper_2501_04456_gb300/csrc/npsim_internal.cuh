@@ -691,7 +691,9 @@ struct SymSmem {
 // A warp's rows are consecutive positions (32 KI divides the groups' 256-block
 // padding), so they have one type.  The sums are kept in units of `scale`, the
 // charge product when it is not small (the Coulomb-only sweep then needs no
-// multiply by it), else 1 with the LJ + Coulomb sweep on every segment.  With LJ
+// multiply by it), else 1 with the LJ + Coulomb sweep on every segment.  has_coul 0: no
+// Coulomb term; 1: type pairs without a charge product, whose terms are exactly zero, are
+// passed over where LJ does not act either; 2: they are swept too (sum_neutral).  With LJ
 // false the tables hold no LJ term: no boxes, always the Coulomb sweep.
 template <int BLOCK, int KI, int JT, bool LJ>
 __device__ __forceinline__ void sym_row_segment(const float4 *__restrict__ xq,
@@ -788,7 +790,7 @@ __device__ __forceinline__ void sym_row_segment(const float4 *__restrict__ xq,
         bool general = false; // LJ + Coulomb sweep on every segment
         if (LJ) {
             const bool unit = fabsf(cst.w) < kSymMinScale;
-            general = unit && cst.w != 0.0f && has_coul;
+            general = unit && (cst.w != 0.0f ? has_coul != 0 : has_coul > 1);
             scale = unit ? 1.0f : cst.w;
             cst.y = unit ? cst.y : cst.y / cst.w;
             cst.w = unit ? cst.w : 1.0f;

@@ -1112,8 +1112,11 @@ int state_to_host(const float4 *xq, const float *x_lo, const float *vel, const f
     double *dx = x ? stage : nullptr, *dv = v ? stage + n3 : nullptr,
            *dF = F ? stage + 2 * n3 : nullptr;
     NP_CUDA(launch_state_aos(xq, x_lo, vel, F_src, n, ld, dx, dv, dF, st));
-    if (x && v == x + n3 && F == v + n3) {
-        NP_CUDA(cudaMemcpyAsync(x, dx, sizeof(double) * 3 * n3, cudaMemcpyDeviceToHost, st));
+    cudaError_t e = cudaErrorInvalidValue;
+    if (x && v == x + n3 && F == v + n3)
+        e = copy_joined(x, dx, sizeof(double) * 3 * n3, st);
+    if (e != cudaErrorInvalidValue) {
+        NP_CUDA(e);
     } else {
         if (x)
             NP_CUDA(cudaMemcpyAsync(x, dx, sizeof(double) * n3, cudaMemcpyDeviceToHost, st));

@@ -1213,6 +1213,17 @@ struct CellGrid {
 // (defined in capi.cu).
 int report_error(int code, const char *fmt, ...);
 
+// One copy into host arrays that lie back to back.  cudaErrorInvalidValue, with the error
+// cleared: they are page-locked one by one and no copy may span them; the caller copies
+// them one by one.
+inline cudaError_t copy_joined(void *host, const void *dev, size_t bytes, cudaStream_t st)
+{
+    const cudaError_t e = cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, st);
+    if (e == cudaErrorInvalidValue)
+        cudaGetLastError();
+    return e;
+}
+
 // An NVTX range named after the C-ABI entry point it is declared in, for the
 // length of the call: the calls show on Nsight Systems timelines above the
 // kernels they launch (the NVTX calls do nothing when no tool is attached).

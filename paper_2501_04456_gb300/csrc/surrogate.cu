@@ -810,9 +810,11 @@ int npsim_surr_predict(npsim_surr_t s, const float *X, int32_t B, float *Y_mean,
     SR_CUDA(launch_after(k_ens_stats, dim3((ne + 255) / 256), 256, 0, s->st, s->y_all, s->n_nets, inv, bp,
                          s->n_out_p, B, s->n_out, s->d_ym, s->d_ys, d_mean, d_spread));
     SR_CUDA(fetch_flags(s));
-    if (Y_spread == Y_mean + ne) { // back to back on the host too: one copy
-        SR_CUDA(cudaMemcpyAsync(Y_mean, d_mean, sizeof(float) * 2 * (size_t)ne,
-                                cudaMemcpyDeviceToHost, s->st));
+    cudaError_t joined = cudaErrorInvalidValue;
+    if (Y_spread == Y_mean + ne) // back to back on the host too: one copy
+        joined = copy_joined(Y_mean, d_mean, sizeof(float) * 2 * (size_t)ne, s->st);
+    if (joined != cudaErrorInvalidValue) {
+        SR_CUDA(joined);
     } else {
         SR_CUDA(cudaMemcpyAsync(Y_mean, d_mean, sizeof(float) * ne, cudaMemcpyDeviceToHost, s->st));
         if (Y_spread)

@@ -248,7 +248,10 @@ int npsim_normals(uint64_t seed, int64_t step, int64_t n, double *out);
  * hand the ranges out at run time.  The environment variable
  * NPSIM_AUTOTUNE=1:<index>[:<ranges per CTA>] forces a shape at npsim_create
  * (NPSIM_AUTOTUNE=0: the first shape); with
- * NPSIM_AUTOTUNE_LOG set, the autotuners print every candidate's time to stderr. */
+ * NPSIM_AUTOTUNE_LOG set, the autotuners print every candidate's time to stderr.
+ * NPSIM_TUNE_BYTES bounds the device memory that timing the candidates may take
+ * (npsim_create, npsim_ens_create); shapes that need more are left out, as where the
+ * memory is not there, and the choice is not kept for later objects. */
 int npsim_allpairs_config(npsim_sim_t sim, int *block, int *i_per_thread, int *j_tile,
                           int *grid, int *index, int *packed);
 

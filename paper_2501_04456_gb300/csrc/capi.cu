@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <string>
@@ -476,10 +477,40 @@ ApConfig shape_config(int k)
 }
 
 // Column partials of the kernels that evaluate each pair once take 6 bytes x
-// N^2 / itile: allowed up to this size (about 1.5 million grouped NPs with the
-// largest row tile); beyond it the one-sided kernels, whose scratch grows with
-// N, remain.
-constexpr size_t kSymMaxBytes = (size_t)8 << 30;
+// N^2 / itile (of an ensemble: summed over its droplets): allowed up to 8 GiB (1.2
+// million grouped NPs with the largest row tile); beyond it the one-sided kernels,
+// whose scratch grows with N, remain.  Tiles of fewer than 512 rows are candidates up to
+// 512 MiB (151000 NPs at 256 rows): there they lost long before (best of 256 rows
+// against best of 512 or 1024, ms: Coulomb 24500 0.183, 0.168, 100000 2.65, 2.35; LJ
+// 60000 1.06, 0.99; 48 droplets of up to 32768 2.02, 1.89), and their scratch alone made
+// the tuning of 400000 NPs take 7.5 GB.
+size_t sym_max_bytes(int itile) { return itile < 512 ? (size_t)512 << 20 : (size_t)8 << 30; }
+
+// The largest of the candidates' scratch sizes (floats) that can be had, with `extra`
+// floats behind it: where the largest does not fit, the shapes that need it drop out and
+// the next is tried.  *all: every candidate has its place.  NPSIM_TUNE_BYTES bounds what
+// a tuner may take (for a GPU that others share).
+int alloc_tune_scratch(std::vector<size_t> needs, size_t extra, float **tmp, size_t *need, bool *all)
+{
+    const char *env = getenv("NPSIM_TUNE_BYTES");
+    const size_t most = env ? (size_t)strtoull(env, nullptr, 10) : SIZE_MAX;
+    std::sort(needs.begin(), needs.end(), std::greater<size_t>());
+    for (size_t f : needs) {
+        cudaError_t e = cudaErrorMemoryAllocation;
+        if ((f + extra) * sizeof(float) <= most) {
+            e = dalloc(tmp, f + extra);
+            if (e != cudaSuccess && e != cudaErrorMemoryAllocation)
+                NP_CUDA(e);
+            cudaGetLastError(); // a failed allocation
+        }
+        if (e == cudaSuccess) {
+            *need = f;
+            *all = f == needs[0];
+            return NPSIM_OK;
+        }
+    }
+    return set_err(NPSIM_ERR_OOM, "no room for the scratch of any launch shape");
+}
 
 // Coulomb kernels with eight rows per thread add 256 terms to a partner's sum before it
 // is compensated.  Beyond this grouped length the best one-sided kernels had tiles of
@@ -498,7 +529,8 @@ int shape_occupancy(const npsim_sim *s, int k, bool lj)
         return 0;
     if (f == SF_SYM || f == SF_SYMLJ) {
         const ApConfig c = shape_config(k);
-        if (sym_col_floats(s->grp_len, c.block * c.ki) * sizeof(float) > kSymMaxBytes)
+        const int itile = c.block * c.ki;
+        if (sym_col_floats(s->grp_len, itile) * sizeof(float) > sym_max_bytes(itile))
             return 0;
         return f == SF_SYMLJ ? sym_occupancy(true, l) : lj ? 0 : sym_occupancy(false, l);
     }
@@ -859,30 +891,23 @@ int autotune(npsim_sim *s)
     }
     const int n_m = (int)(sizeof(kRangesPerCta) / sizeof(kRangesPerCta[0]));
     int best = 0, best_m = kDefaultRangesPerCta;
+    bool all = true;
     {
-        // scratch big enough for every candidate; where it does not fit, for the
-        // one-sided ones
         const size_t out_floats = 8 * (size_t)std::max(s->n, s->grp_len);
         float *tmp = nullptr;
         size_t need = 0;
-        for (bool sym : {true, false}) {
-            need = 0;
-            for (int c = 0; c < nc; ++c) {
-                const int occ = shape_occupancy(s, c, lj);
-                if (occ <= 0 || (shape_sym(c) && !sym))
-                    continue;
-                StreamK sk;
-                shape_streamk(s, c, occ * s->sms, kRangesPerCta[n_m - 1], sk);
-                need = std::max(need, shape_slots_floats(sk));
-            }
-            need = (need + 3) & ~(size_t)3; // 16-byte records follow
-            const cudaError_t e = dalloc(&tmp, need + out_floats);
-            if (e == cudaSuccess)
-                break;
-            if (!sym || e != cudaErrorMemoryAllocation)
-                NP_CUDA(e);
-            cudaGetLastError(); // the failed allocation
+        std::vector<size_t> needs;
+        for (int c = 0; c < nc; ++c) {
+            const int occ = shape_occupancy(s, c, lj);
+            if (occ <= 0)
+                continue;
+            StreamK sk;
+            shape_streamk(s, c, occ * s->sms, kRangesPerCta[n_m - 1], sk);
+            needs.push_back((shape_slots_floats(sk) + 3) & ~(size_t)3); // 16-byte records follow
         }
+        int rc = alloc_tune_scratch(needs, out_floats, &tmp, &need, &all);
+        if (rc)
+            return rc;
         float *sum_out = tmp + need;
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
@@ -945,8 +970,10 @@ int autotune(npsim_sim *s)
     }
     s->ap_idx = best;
     s->ap_per_cta = best_m;
-    std::lock_guard<std::mutex> g(g_tune_mu);
-    g_tune_cache[key] = std::make_pair(best, best_m);
+    if (all) { // the best of what memory was free is not kept for later simulations
+        std::lock_guard<std::mutex> g(g_tune_mu);
+        g_tune_cache[key] = std::make_pair(best, best_m);
+    }
     return NPSIM_OK;
 }
 
@@ -2749,6 +2776,19 @@ int ens_state_out(npsim_ens *e, int d, const float *F_src, double *x, double *v,
                          (size_t)e->n_total, e->stage, x, v, F, e->user);
 }
 
+// Whether the ensemble's column partials are small enough for launch shape c.
+bool ens_shape_fits(const npsim_ens *e, int c)
+{
+    if (!ens_sym(c))
+        return true;
+    const ApConfig cf = ens_config(c);
+    const int itile = cf.block * cf.ki;
+    size_t col = 0;
+    for (const EnsDrop &g : e->h_drops)
+        col += sym_col_floats(g.npad, itile);
+    return col * sizeof(float) <= sym_max_bytes(itile);
+}
+
 // Time every ensemble launch shape on the current positions; keep the fastest.
 int ens_autotune(npsim_ens *e)
 {
@@ -2776,37 +2816,31 @@ int ens_autotune(npsim_ens *e)
             best = it->second;
     }
     const bool cached = !pinned && best >= 0;
+    bool all = true;
     if (best < 0) {
-        // scratch big enough for every candidate; where that does not fit, for the
-        // one-sided one alone
         float *tmp = nullptr;
         size_t need = 0;
-        for (bool sym : {true, false}) {
-            need = 0;
-            for (int c = 0; c < nc; ++c) {
-                const int occ = ens_occupancy(c);
-                if (occ > 0 && (sym || !ens_sym(c)))
-                    need = std::max(need, ens_geometry(e, c, occ * e->sms).floats);
-            }
-            const cudaError_t ce = dalloc(&tmp, need);
-            if (ce == cudaSuccess)
-                break;
-            if (!sym || ce != cudaErrorMemoryAllocation)
-                NP_CUDA(ce);
-            cudaGetLastError(); // the failed allocation
+        std::vector<size_t> needs;
+        for (int c = 0; c < nc; ++c) {
+            const int occ = ens_occupancy(c);
+            if (occ > 0 && ens_shape_fits(e, c))
+                needs.push_back(ens_geometry(e, c, occ * e->sms).floats);
         }
+        int rc = alloc_tune_scratch(needs, 0, &tmp, &need, &all);
+        if (rc)
+            return rc;
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
         float best_ms = 1e30f;
         for (int c = 0; c < nc; ++c) {
             const int occ = ens_occupancy(c);
-            if (occ <= 0)
+            if (occ <= 0 || !ens_shape_fits(e, c))
                 continue;
             const EnsGeometry G = ens_geometry(e, c, occ * e->sms);
             if (G.floats > need)
                 continue;
-            int rc = ens_upload_geometry(e, c, G);
+            rc = ens_upload_geometry(e, c, G);
             if (rc) {
                 cudaFree(tmp);
                 return rc;
@@ -2841,7 +2875,7 @@ int ens_autotune(npsim_ens *e)
         if (best < 0)
             best = 0;
     }
-    if (!pinned && !cached) {
+    if (!pinned && !cached && all) {
         std::lock_guard<std::mutex> g(g_tune_mu);
         g_ens_tune_cache[key] = best;
     }

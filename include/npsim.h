@@ -474,8 +474,10 @@ int npsim_fma_peak(int packed, int64_t iters, void *stream, double *flops, float
                    int *grid);
 
 /* Kernel launches per step in a long run (pair kernels + cell-list kernels + one
- * integrator pass); npsim_step adds one integrator launch per graph chunk.  1 for a
- * droplet whose launches take many steps each (small, all pair forces from lists). */
+ * integrator pass); npsim_step adds one integrator launch per graph chunk.  1 where a
+ * launch takes many steps: up to 256 of a droplet of at most 65536 NPs whose pair forces
+ * all come from the lists, up to 64 of one without pair forces; not while npsim_profile
+ * is on, which times one launch per kernel. */
 int npsim_launches_per_step(npsim_sim_t sim, int *launches);
 
 /* Cell grid of the LJ cell list (lj_mode 2): cells per axis and in total; both

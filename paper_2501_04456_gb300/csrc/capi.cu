@@ -1920,7 +1920,9 @@ int npsim_launches_per_step(npsim_sim_t s, int *launches)
     NP_REQUIRE(s && launches, "sim and launches are required");
     // integrator, all-pairs (and the sum of its partials), the gated list build, the
     // list LJ forces; one launch where it takes many steps
-    *launches = s->cell && !s->ap && s->n <= s->fused_cap ? 1 : 1 + (s->ap ? (s->sk.tri ? 2 : 1) : 0) + (s->cell ? 2 : 0);
+    *launches = 1;
+    if (!fused_steps(s) && !free_steps(s))
+        *launches += (s->ap ? (s->sk.tri ? 2 : 1) : 0) + (s->cell ? 2 : 0);
     return NPSIM_OK;
 }
 

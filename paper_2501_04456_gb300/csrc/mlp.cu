@@ -896,13 +896,6 @@ k_weights_bf16(const float *__restrict__ w, const __grid_constant__ NetDims d, i
     put_tile(d, k, p, wt, t);
 }
 
-__global__ void k_f32_to_bf16(const float *__restrict__ x, int n, __nv_bfloat16 *__restrict__ y)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n)
-        y[i] = __float2bfloat16_rn(x[i]);
-}
-
 } // namespace
 
 namespace {
@@ -945,8 +938,6 @@ bool encode_operand(CUtensorMap *m, const __nv_bfloat16 *ptr, int rows, int K, i
 }
 
 } // namespace
-
-int gemm_smem_bytes(int n_tile) { return dyn_smem_bytes(n_tile, kMaxStages); }
 
 namespace {
 bool gemm_ok(const GemmArgs &g)
@@ -1094,12 +1085,6 @@ cudaError_t launch_adamw(float *w, const float *g, float *m, float *v, const uns
 cudaError_t launch_weights_bf16(const float *w, const NetDims &d, int k, cudaStream_t st)
 {
     k_weights_bf16<<<param_tiles(d), 256, 0, st>>>(w, d, k);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_f32_to_bf16(const float *x, int n, void *y, cudaStream_t st)
-{
-    k_f32_to_bf16<<<(n + 255) / 256, 256, 0, st>>>(x, n, (__nv_bfloat16 *)y);
     return cudaGetLastError();
 }
 

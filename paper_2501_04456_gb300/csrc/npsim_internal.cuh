@@ -264,45 +264,6 @@ __device__ __forceinline__ Box3 box_warp_reduce(Box3 b)
     return b;
 }
 
-// Warp-reduce b and store lane 0's result as 6 floats at s_red[6 * warp]; the
-// caller synchronises the block and then calls box_gather.
-__device__ __forceinline__ void box_warp_store(Box3 b, float *s_red)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        b.lx = fminf(b.lx, __shfl_xor_sync(0xffffffffu, b.lx, o));
-        b.ly = fminf(b.ly, __shfl_xor_sync(0xffffffffu, b.ly, o));
-        b.lz = fminf(b.lz, __shfl_xor_sync(0xffffffffu, b.lz, o));
-        b.hx = fmaxf(b.hx, __shfl_xor_sync(0xffffffffu, b.hx, o));
-        b.hy = fmaxf(b.hy, __shfl_xor_sync(0xffffffffu, b.hy, o));
-        b.hz = fmaxf(b.hz, __shfl_xor_sync(0xffffffffu, b.hz, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        float *r = s_red + 6 * (threadIdx.x >> 5);
-        r[0] = b.lx;
-        r[1] = b.ly;
-        r[2] = b.lz;
-        r[3] = b.hx;
-        r[4] = b.hy;
-        r[5] = b.hz;
-    }
-}
-
-__device__ __forceinline__ Box3 box_gather(const float *s_red, int n_warps)
-{
-    Box3 b = box_empty();
-    for (int w = 0; w < n_warps; ++w) {
-        const float *r = s_red + 6 * w;
-        b.lx = fminf(b.lx, r[0]);
-        b.ly = fminf(b.ly, r[1]);
-        b.lz = fminf(b.lz, r[2]);
-        b.hx = fmaxf(b.hx, r[3]);
-        b.hy = fmaxf(b.hy, r[4]);
-        b.hz = fmaxf(b.hz, r[5]);
-    }
-    return b;
-}
-
 // Squared distance between two boxes (0 if they overlap; +inf if one is empty).
 __device__ __forceinline__ float box_gap2(const Box3 &a, const Box3 &b)
 {
@@ -1555,7 +1516,6 @@ struct NetDims {
     __nv_bfloat16 *Wb[kMaxLayers], *Wt[kMaxLayers];
 };
 
-int gemm_smem_bytes(int n_tile);
 // One product (g1 NULL), or two independent ones of the same nz in one launch.
 cudaError_t launch_gemm(const GemmArgs &g0, const GemmArgs *g1, cudaStream_t st);
 
@@ -1595,7 +1555,6 @@ cudaError_t launch_adamw(float *w, const float *g, float *m, float *v, const uns
                          const NetDims &d, int k0, int nz, const AdamArgs &a, cudaStream_t st);
 // BF16 copies of the flat parameters of network k.
 cudaError_t launch_weights_bf16(const float *w, const NetDims &d, int k, cudaStream_t st);
-cudaError_t launch_f32_to_bf16(const float *x, int n, void *y, cudaStream_t st);
 
 // Cell list (celllist.cu).  The sort key of NP i is its cell (tb == 1) or
 // type * n_cells + cell (tb = the number of types): the cell order lists all NPs
@@ -1714,11 +1673,5 @@ cudaError_t launch_positions_f64_ld(const float4 *xq, const float *x_lo, int n, 
 cudaError_t launch_state_aos(const float4 *xq, const float *x_lo, const float *v, const float *F,
                              int n, size_t ld, double *xo, double *vo, double *Fo,
                              cudaStream_t st);
-
-// Test hooks (capi.cu)
-cudaError_t launch_philox(uint64_t seed, const uint32_t ctr[4], long long n_blocks,
-                          uint32_t *out, cudaStream_t st);
-cudaError_t launch_normals(uint64_t seed, long long step, int n, double *out,
-                           cudaStream_t st);
 
 } // namespace npsim

@@ -1525,13 +1525,13 @@ int create_impl(const npsim_type_t *types, const npsim_params_t *params, int64_t
         BAIL_CUDA(dalloc(&s->nl.nnbr, (size_t)n));
         BAIL_CUDA(dalloc(&s->nl.x_ref, (size_t)n));
         BAIL_CUDA(dalloc(&s->nl.builds, 1));
-        BAIL_CUDA(cudaMemset(s->nl.builds, 0, sizeof(unsigned long long)));
+        BAIL_CUDA(cudaMemsetAsync(s->nl.builds, 0, sizeof(unsigned long long), s->user));
         BAIL_CUDA(dalloc(&s->d_gate, 1));
         s->fused_cap = list_steps_capacity();
         BAIL_CUDA(dalloc(&s->list_bar, kBarWords));
         BAIL_CUDA(cudaMemsetAsync(s->list_bar, 0, kBarWords * sizeof(unsigned), s->user));
-        BAIL_CUDA(cudaMemset(s->nl.nnbr, 0, sizeof(int) * (size_t)n));
-        BAIL_CUDA(cudaMemset(s->nl.nbr, 0, sizeof(unsigned) * (size_t)s->nl.cap * n));
+        BAIL_CUDA(cudaMemsetAsync(s->nl.nnbr, 0, sizeof(int) * (size_t)n, s->user));
+        BAIL_CUDA(cudaMemsetAsync(s->nl.nbr, 0, sizeof(unsigned) * (size_t)s->nl.cap * n, s->user));
     }
     if (s->cell) {
         rc = set_list_wait(s, list_wait_polls(s->n));
@@ -1553,7 +1553,7 @@ int create_impl(const npsim_type_t *types, const npsim_params_t *params, int64_t
         if (rc)
             return bail(rc);
         BAIL_CUDA(dalloc(&s->ap_work, 2));
-        BAIL_CUDA(cudaMemset(s->ap_work, 0, 2 * sizeof(unsigned)));
+        BAIL_CUDA(cudaMemsetAsync(s->ap_work, 0, 2 * sizeof(unsigned), s->user));
         rc = autotune(s);
         if (rc)
             return bail(rc);
@@ -2280,7 +2280,7 @@ int restore_lists(npsim_sim *s, const CkptHeader &h, const float4 *x_ref_host)
     if (h.nbr_cap != s->nl.cap) {
         dfree(s->nl.nbr);
         NP_CUDA(dalloc(&s->nl.nbr, (size_t)h.nbr_cap * s->n));
-        NP_CUDA(cudaMemset(s->nl.nbr, 0, sizeof(unsigned) * (size_t)h.nbr_cap * s->n));
+        NP_CUDA(cudaMemsetAsync(s->nl.nbr, 0, sizeof(unsigned) * (size_t)h.nbr_cap * s->n, s->user));
         s->nl.cap = h.nbr_cap;
     }
     for (auto &e : s->graphs)
@@ -3055,7 +3055,7 @@ int npsim_ens_create(const npsim_droplet_t *drops, int32_t n_drops, void *stream
     EBAIL(dalloc(&e->tabs, (size_t)n_drops));
     EBAIL(dalloc(&e->F_pair, 8 * (size_t)total));
     EBAIL(dalloc(&e->d_work, 2));
-    EBAIL(cudaMemset(e->d_work, 0, 2 * sizeof(unsigned)));
+    EBAIL(cudaMemsetAsync(e->d_work, 0, 2 * sizeof(unsigned), e->user));
     EBAIL(dalloc(&e->d_step, 1));
     EBAIL(dalloc(&e->d_spring, (size_t)2 * n_drops * NPSIM_MAX_TYPES));
     EBAIL(dalloc(&e->d_flags, 1));
@@ -3086,7 +3086,7 @@ int npsim_ens_create(const npsim_droplet_t *drops, int32_t n_drops, void *stream
         xq0[i] = make_float4((float)xs[i], (float)xs[total + i], (float)xs[2 * total + i], q);
     }
     EBAIL(cudaMemcpy(e->xq, xq0.data(), sizeof(float4) * (size_t)total, cudaMemcpyHostToDevice));
-    EBAIL(cudaMemset(e->d_step, 0, sizeof(long long)));
+    EBAIL(cudaMemsetAsync(e->d_step, 0, sizeof(long long), e->user));
     {
         // spring radii of step 0 (buffer 0)
         std::vector<float4> sp((size_t)2 * n_drops * NPSIM_MAX_TYPES, make_float4(0, 0, 0, 0));
@@ -3098,8 +3098,8 @@ int npsim_ens_create(const npsim_droplet_t *drops, int32_t n_drops, void *stream
         EBAIL(cudaMemcpy(e->d_spring, sp.data(), sizeof(float4) * sp.size(),
                          cudaMemcpyHostToDevice));
     }
-    EBAIL(cudaMemset(e->d_flags, 0, sizeof(int)));
-    EBAIL(cudaMemset(e->d_done, 0, sizeof(unsigned)));
+    EBAIL(cudaMemsetAsync(e->d_flags, 0, sizeof(int), e->user));
+    EBAIL(cudaMemsetAsync(e->d_done, 0, sizeof(unsigned), e->user));
 #undef EBAIL
     rc = ens_autotune(e);
     if (rc)

@@ -555,7 +555,7 @@ int npsim_surr_create(int32_t n_in, int32_t n_hidden, int32_t n_layers, int32_t 
     for (int c = 0; c < n_out; ++c)
         ow[c] = 1.f;
     cudaMemcpy(s->outw, ow.data(), sizeof(float) * ow.size(), cudaMemcpyHostToDevice);
-    cudaMemset(s->flags, 0, sizeof(int));
+    cudaMemsetAsync(s->flags, 0, sizeof(int), s->st);
     int rc = alloc_batch(s, 512);
     if (rc)
         return bail(rc);

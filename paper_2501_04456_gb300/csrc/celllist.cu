@@ -970,8 +970,17 @@ k_list_steps(const __grid_constant__ FusedStepArgs a, const __grid_constant__ St
 int cell_scan_tiles(int n_cells) { return (n_cells + kScanTile - 1) / kScanTile; }
 
 namespace {
-constexpr int kMaxGrid = 1216; // 8 CTAs on each of 152 SMs
-constexpr int kOneCtaPerSm = 152;
+constexpr int kMaxGrid = 1216; // 8 CTAs on each of 152 SMs (grid-stride kernels)
+
+int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    return sms;
+}
+
 int grid_for(int n, int block)
 {
     const int g = (n + block - 1) / block;
@@ -1035,16 +1044,12 @@ ListBuildArgs list_build_args(const CellGrid &g, const CellBufs &b, const float4
 template <class... P>
 cudaError_t launch_coop(void (*fn)(P...), int want, cudaStream_t st, const P &...args)
 {
-    int dev = 0, sms = 0, occ = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess)
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kScanThreads, 0);
+    int occ = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kScanThreads, 0);
     if (e != cudaSuccess)
         return e;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(max(1, min(want, occ * sms)));
+    cfg.gridDim = dim3(max(1, min(want, occ * sm_count())));
     cfg.blockDim = dim3(kScanThreads);
     cfg.stream = st;
     cudaLaunchAttribute at{};
@@ -1070,15 +1075,11 @@ cudaError_t launch_list_build(const CellGrid &g, const CellBufs &b, const float4
 
 int list_steps_capacity()
 {
-    int dev = 0, sms = 0, occ = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_list_steps<true>, kScanThreads, 0) !=
-            cudaSuccess)
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_list_steps<true>, kScanThreads, 0) !=
+        cudaSuccess)
         return 0;
-    const int ctas = min(occ * sms, 2 * kOneCtaPerSm);
-    // below two CTAs per SM only one is launched for up to kOneCtaPerSm of them
-    return min(kMaxFusedNps, (ctas >= 2 * kOneCtaPerSm ? ctas : min(ctas, kOneCtaPerSm)) * kScanThreads);
+    return min(kMaxFusedNps, min(occ, 2) * sm_count() * kScanThreads); // as launch_list_steps cuts it
 }
 
 cudaError_t launch_list_steps(const CellGrid &g, const CellBufs &b, int n, const PairTab *tab,
@@ -1097,7 +1098,8 @@ cudaError_t launch_list_steps(const CellGrid &g, const CellBufs &b, int n, const
     // a warp's 32 slots per CTA while that leaves SMs free (the other warps help the
     // builds), then one CTA per SM, two when their threads do not reach n
     const int warps = (n + 31) / 32;
-    const int want = n <= kOneCtaPerSm * kScanThreads ? min(warps, kOneCtaPerSm) : 2 * kOneCtaPerSm;
+    const int sms = sm_count();
+    const int want = n <= sms * kScanThreads ? min(warps, sms) : 2 * sms;
     if (n > list_steps_capacity())
         return cudaErrorInvalidValue; // every slot needs a thread
     return rcc2 ? launch_coop<FusedStepArgs, StepParams>(k_list_steps<true>, want, st, a, p)

@@ -53,7 +53,7 @@ template <class T> void dfree2(T *&p)
 } // namespace
 
 struct npsim_surr {
-    int n_in = 0, n_in_p = 0, H = 0, NL = 0, n_out = 0, n_out_p = 0, n_nets = 0;
+    int n_in = 0, n_in_p = 0, H = 0, NL = 0, n_out = 0, n_out_p = 0, n_nets = 0, sms = 0;
     // parameters of all networks as flat vectors [n_nets][n_params] (the layout of
     // npsim_surr_get_params): FP32 master weights, gradients, AdamW moments; BF16
     // copies and transposes per layer, all networks in one block (D.Wb, D.Wt)
@@ -138,11 +138,10 @@ constexpr int kTrainRows = 65536;
 // caches), and at most 32, then 16, while the product still has no more CTAs than
 // SMs: a shorter epilogue per CTA, on SMs that had none (4 networks, 256 columns, at
 // most 64 / 32 / 16: a minibatch of 256 rows 88 / 77 / 74 us, of 32 81 / 68 / 63).
-constexpr int kSms = 152;
-int n_tile_for(int M, int N, int nz)
+int n_tile_for(int M, int N, int nz, int sms)
 {
     const int mt = (M + 127) / 128 * nz;
-    const int most = mt * ((N + 15) / 16) <= kSms ? 16 : mt * ((N + 31) / 32) <= kSms ? 32 : 64;
+    const int most = mt * ((N + 15) / 16) <= sms ? 16 : mt * ((N + 31) / 32) <= sms ? 32 : 64;
     const int tiles = (N + most - 1) / most;
     return ((N + tiles - 1) / tiles + 15) / 16 * 16;
 }
@@ -164,7 +163,7 @@ GemmArgs gemm(npsim_surr *s, int mode, const __nv_bfloat16 *A, int lda, int za,
     g.lda = lda;
     g.ldb = ldb;
     g.ldc = ldc;
-    g.n_tile = n_tile_for(M, N, nk);
+    g.n_tile = n_tile_for(M, N, nk, s->sms);
     g.tmem_cols = pow2_at_least(g.n_tile);
     g.mode = mode;
     g.flags = s->flags;
@@ -487,6 +486,10 @@ int npsim_surr_create(int32_t n_in, int32_t n_hidden, int32_t n_layers, int32_t 
     s->n_out = n_out;
     s->n_out_p = round16(n_out);
     s->n_nets = n_nets;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return bail(report_error(NPSIM_ERR_CUDA, "no SM count"));
     s->xm.assign(n_in, 0.f);
     s->xs.assign(n_in, 1.f);
     s->ym.assign(n_out, 0.f);

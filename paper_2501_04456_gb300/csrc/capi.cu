@@ -515,11 +515,12 @@ int alloc_tune_scratch(std::vector<size_t> needs, size_t extra, float **tmp, siz
 // Coulomb kernels with eight rows per thread add 256 terms to a partner's sum before it
 // is compensated.  Beyond this grouped length the best one-sided kernels had tiles of
 // 512 partners, the same chain (60000 NPs, rms error against float64 4.0e-8, one-sided
-// 4.8e-8); up to it some had 256, and four rows per thread, or the LJ + Coulomb kernels,
-// whose chains are half as long, keep to theirs (16384 NPs 3.1e-8, one-sided 3.4e-8,
-// eight rows 3.8e-8) for 3 to 6 % of the launch (16000: 0.090, eight rows 0.085 ms;
-// 24500: 0.173, 0.168).
-constexpr int kSymLongRows = 32768;
+// 4.8e-8); up to it some had 256 (16384, 20480), and four rows per thread, or the LJ +
+// Coulomb kernels, whose chains are half as long, keep to theirs (16384 NPs 3.1e-8,
+// one-sided 3.4e-8, eight rows 3.8e-8).  Launch and sum, four against eight rows, ms:
+// 13824 NPs 0.064, 0.070; 15360 0.080, 0.080; 16384 0.086, 0.084; 18432 0.104, 0.098;
+// 20480 0.126, 0.127; 24576 0.172, 0.168; 32256 0.287, 0.268.
+constexpr int kSymLongRows = 20480;
 
 int shape_occupancy(const npsim_sim *s, int k, bool lj)
 {

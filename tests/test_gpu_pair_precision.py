@@ -35,7 +35,7 @@ def _errors(P, monkeypatch, sc, state, ref, thirds, shape):
     return cfg, [np.sqrt((e[t] ** 2).mean()) for t in thirds]
 
 
-@pytest.mark.parametrize("n,tile", [(4000, 256), (16384, 256), (33001, 512)])
+@pytest.mark.parametrize("n,tile", [(4000, 256), (16384, 256), (22801, 512), (33001, 512)])
 def test_partner_sums_round_no_more_than_row_sums(P, monkeypatch, n, tile):
     sc = with_(small(wl.config2(), n), lj_mode=0)
     state = types, x, v = wl.initial_state(sc, fp32_positions=True)

@@ -126,7 +126,8 @@ void npsim_destroy(npsim_sim_t sim);
  * lj_mode == 2), pair forces, R(t) by the radius-square law, interface spring,
  * gravity, centrifugal force and the Langevin update with Philox4x32-10 noise
  * keyed by (seed) and counted by (particle, step, 0).  Steps are replayed from
- * captured CUDA graphs.  Returns after one device-to-host read of the error
+ * captured CUDA graphs or, where NPs need few others' positions, taken many to a
+ * launch (npsim_launches_per_step).  Returns after one device-to-host read of the error
  * word: NONFINITE if any position became non-finite, TIMEOUT if a bounded wait
  * expired, ESCAPED if (wall 1) an NP was farther than 2 max(R0, R(t)) from the
  * centre during some step.  The steps were taken in every case but TIMEOUT; the
@@ -266,11 +267,11 @@ int npsim_allpairs_num_configs(int *count);
 
 /* ------------------------------------------------------------------------
  * Ensemble: many independent droplets (each the system of Sec. 2 with its own
- * types, charges, radius law and seed) advanced together.  One all-pairs launch
- * and one integrator launch per step cover every droplet: the (i-tile x
- * j-tile) work rectangles of all droplets are laid end to end and split evenly
- * over the CTAs, so droplets of very different N share the GPU in one launch.
- * Steps replay from captured CUDA graphs; the launch shape is chosen by timing
+ * types, charges, radius law and seed) advanced together.  One all-pairs launch, one
+ * sum of its partials and one integrator launch per step cover every droplet: each
+ * row tile of each droplet is cut into items (runs of j-tiles), listed longest first
+ * and drawn by the CTAs from a device counter, so droplets of very different N share
+ * the GPU in one launch.  Steps replay from captured CUDA graphs; the launch shape is chosen by timing
  * every candidate at npsim_ens_create (NPSIM_ENS_SHAPE=<index> forces one).
  */
 typedef struct npsim_ens *npsim_ens_t;
@@ -327,17 +328,17 @@ int npsim_ens_config(npsim_ens_t ens, int *block, int *i_per_thread, int *j_tile
 int npsim_ens_info(npsim_ens_t ens, int64_t *n_total, double *pairs_per_step);
 
 /* Work items of one all-pairs launch (row tile x run of j-tiles, over all
- * droplets) and rows per tile (either pointer may be NULL): each item writes
- * one partial slot of 6 x itile floats that the integrator reads (measurement
- * hook: the integrator's bytes). */
+ * droplets) and rows per tile (either pointer may be NULL): each item writes one
+ * partial slot of 6 x itile floats, which the sum of the partials reads (measurement
+ * hook). */
 int npsim_ens_work(npsim_ens_t ens, int64_t *n_items, int32_t *itile);
 
 /*
  * Per-kernel timing of the ensemble (measurement hook).  enable = 1 re-captures
- * the step graphs with CUDA event records around the all-pairs launch and the
- * integrator launch of every step of a chunk; enable = 0 removes them (results
+ * the step graphs with CUDA event records around the all-pairs launch with the sum of
+ * its partials and around the integrator launch of every step of a chunk; enable = 0 removes them (results
  * do not depend on it).  After an npsim_ens_step, npsim_ens_kernel_times writes
- * the mean duration in milliseconds of the all-pairs launch (ms[0]) and of the
+ * the mean duration in milliseconds of the all-pairs launch and sum (ms[0]) and of the
  * integrator launch (ms[1]) over the steps of the last replayed graph chunk,
  * and the number of steps averaged.  ms must hold 2 doubles.  Errors:
  * INVALID_ARG (NULL ensemble or ms, profiling not enabled), CUDA.
@@ -482,8 +483,8 @@ int npsim_launches_per_step(npsim_sim_t sim, int *launches);
 
 /* Cell grid of the LJ cell list (lj_mode 2): cells per axis and in total; both
  * 0 when the scenario has no cell list.  The grid covers [-L, L)^3 with L the
- * largest |coordinate| at creation (or R0) plus the largest cutoff, cell edge
- * >= the largest cutoff. */
+ * largest |coordinate| at creation (or R0; later the droplet's radius) plus the largest
+ * cutoff and the skin, cell edge >= the smallest list radius of the acting type pairs. */
 int npsim_cell_grid(npsim_sim_t sim, int *dim, int64_t *n_cells);
 
 /* Verlet neighbour lists of the cell-list LJ (lj_mode 2): the list capacity per
@@ -492,13 +493,15 @@ int npsim_cell_grid(npsim_sim_t sim, int *dim, int64_t *n_cells);
  * previous one).  All 0 without a cell list. */
 int npsim_nbr_info(npsim_sim_t sim, int *cap, double *mean_len, int64_t *builds);
 
-/* Steps per captured CUDA graph (npsim_step replays ceil(n / chunk) graphs). */
+/* Steps per captured CUDA graph (where steps are replayed from graphs, npsim_step
+ * replays ceil(n / chunk) of them). */
 int npsim_chunk_steps(npsim_sim_t sim, int *chunk);
 
 /*
  * Per-kernel timing.  enable = 1 re-captures the step graphs with CUDA event
- * records around the kernels of every step (all-pairs forces, cell-list
- * build, cell-list LJ, integrator); enable = 0 removes them.  After an
+ * records around the kernels of every step (all-pairs forces with the sum of their
+ * partials, cell-list build, cell-list LJ, integrator), one launch per kernel where
+ * steps are otherwise taken many to a launch; enable = 0 removes them.  After an
  * npsim_step, npsim_kernel_times writes the mean duration in milliseconds of
  * each of the four groups over the steps of the last replayed graph chunk
  * (0 for groups this scenario does not launch) and the number of steps

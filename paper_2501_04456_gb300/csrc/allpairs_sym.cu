@@ -99,12 +99,15 @@ struct SEntry {
         ApConfig{B, K, J, 0}, (const void *)k_pairs_sym<B, K, J, LJ>, (int)sizeof(SymSmem<B, K, J>) \
     }
 
-// Best launch + reduction by grouped length (ms; one-sided kernel's best in
-// brackets).  Coulomb: 100352 <128,8,128> 2.34 [3.27], 24576 0.168 [0.219],
-// 8704 <64,8,128> 0.035 [0.039], 2560 <64,2,64> 0.015 [0.020].  LJ + Coulomb:
-// 60416 <64,8,128> 0.99 [1.39], 30208 0.295 [0.381], 16384 0.112 [0.134], 4096
-// <128,2,128> 0.025 [0.027], 1024 <64,2,64> 0.019 [0.025]: long rows want many rows
-// per thread, short ones many small units.
+// Where each shape is the best, launch + reduction by grouped length (ms; the best
+// one-sided kernel in brackets).  Coulomb: <128,8,128> 24576 0.168 [0.219], 100352 2.34
+// [3.26], 300032 20.4 [28.8]; <64,8,128> 34304 0.299; <128,4,128> 5120 0.023 [0.025],
+// 16384 0.086 [0.113]; <64,4,64> 7680 0.035, 11776 0.054; <64,2,64> 1024 0.015 [0.017],
+// 2560 0.017 [0.019].  (Eight rows above 20480 only: kSymLongRows.)  LJ + Coulomb:
+// <128,8,128> 30208 0.298 [0.382], 300032 21.7 [32.0]; <64,8,128> 60416 0.994 [1.39];
+// <128,4,128> 16384 0.111 [0.134]; <64,4,64> 8192 0.045 [0.056]; <128,2,128> 4096 0.025
+// [0.029], as the next; <64,2,64> 1024 0.019 [0.023], 2560 0.021 [0.025]: long rows want
+// many rows per thread, short ones many small units.
 const SEntry kSym[] = {
     NPSIM_SYM(128, 8, 128, false), NPSIM_SYM(64, 8, 128, false), NPSIM_SYM(128, 4, 128, false),
     NPSIM_SYM(64, 4, 64, false),   NPSIM_SYM(64, 2, 64, false),

@@ -240,6 +240,12 @@ struct EEntry {
     }
 
 // j-tiles of at most 256 partners: the droplets' type groups are padded to 256.
+// Launch + reduction (ms; the one-sided kernel in brackets): <64,8,128> 48 droplets of
+// 512 to 32768 NPs 1.87 [2.70], 128 of 512 to 8192 0.633 [0.787], 4 of 32768 to 65536
+// 2.50 [3.72]; <128,4,128> 8 of 4000 to 8000 0.132 [0.159]; <128,2,128> 16 of 512 to 4096
+// 0.054 [0.061]; <64,2,64> 3 of 300 to 600 0.019 [0.020].  The three others are within 1 to
+// 4 % of the best beside them: <128,8,128> 2 of 100000 to 200000 12.1, <64,4,64> 128 of 512
+// to 8192 0.639, <64,8,64> 48 of 512 to 32768 1.95.
 // The last shape is the one-sided kernel, for ensembles whose column partials
 // (6 n^2 / itile bytes per droplet) do not fit; each pair once is faster on all
 // others.

@@ -394,7 +394,6 @@ __device__ __forceinline__ void nbr_slot(const ListBuildArgs &A, const float4 *s
 struct ListBuildSmem {
     int warp[kScanThreads / 32 + 1];
     int ok;
-    unsigned polls; // bound of a barrier wait, used by the first thread
     int off[kScanTile]; // prefix of the scan tiles' totals (when they are few enough)
     float4 tab[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
     float rl2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
@@ -411,17 +410,19 @@ __device__ __forceinline__ bool wait_expired(const int *flags)
 }
 
 // Barrier over the CTAs of a cooperative launch (all resident): phase = barriers
-// passed so far, the same in every thread.  A wait is bounded (S.polls); one that
+// passed so far, the same in every thread.  A wait is bounded (`polls`, used by the
+// first thread: read once per launch, a read at every barrier took 1 % of a step of 1000
+// NPs); one that
 // gives up sets FLAG_TIMEOUT and returns false in every thread of its CTA, which
 // then leaves the kernel.  Nobody passes a later barrier without its arrival, so the
 // other CTAs give up there in turn.
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, int *flags,
-                                             ListBuildSmem &S)
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, unsigned polls,
+                                             int *flags, int *s_ok)
 {
     __syncthreads();
     ++phase;
     if (threadIdx.x == 0) {
-        const unsigned target = phase * gridDim.x, polls = S.polls;
+        const unsigned target = phase * gridDim.x;
         __threadfence();
         atomicAdd(bar + kBarArrived, 1u);
         int ok = 0;
@@ -435,10 +436,10 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, int
         if (!ok)
             atomicOr(flags, FLAG_TIMEOUT);
         __threadfence();
-        S.ok = ok;
+        *s_ok = ok;
     }
     __syncthreads();
-    return S.ok != 0;
+    return *s_ok != 0;
 }
 
 // The phases of a build by every CTA of a cooperative launch, between grid barriers
@@ -448,14 +449,14 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, int
 // and the offsets are added while the NPs are scattered: four barriers; beyond,
 // one CTA scans the totals: six.
 __device__ __forceinline__ bool list_build(const ListBuildArgs &A, float4 *sxq, ListBuildSmem &S,
-                                           unsigned &phase)
+                                           unsigned &phase, unsigned polls)
 {
     const CellBufs &B = A.b;
     const int n = A.n;
     const int m = (A.g.tb > 1 ? A.g.tb : 1) * A.g.n_cells; // sort keys
     const int n_tiles = (m + kScanTile - 1) / kScanTile;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
-    auto barrier = [&]() { return grid_barrier(A.bar, phase, A.flags, S); };
+    auto barrier = [&]() { return grid_barrier(A.bar, phase, polls, A.flags, &S.ok); };
 
     if (tid == 0) {
         if (A.builds)
@@ -554,12 +555,11 @@ k_list_build(const __grid_constant__ ListBuildArgs A)
     if (A.gate && *A.gate == 0) // nobody writes it while this kernel runs
         return;
     unsigned phase = 0;
-    if (threadIdx.x == 0)
-        S.polls = A.bar[kBarPolls];
+    const unsigned polls = A.bar[kBarPolls];
     load_tables(A.tab, A.rcc2, A.skin, S.tab, S.rl2, S.rmax);
     if (wait_expired(A.flags))
         return;
-    if (list_build(A, A.b.sxq, S, phase))
+    if (list_build(A, A.b.sxq, S, phase, polls))
         barrier_done(A.bar);
 }
 
@@ -749,20 +749,26 @@ k_lj_nbr(const __grid_constant__ CellGrid g, const int *__restrict__ start, cons
     __shared__ float s_rl2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
     __shared__ float s_rcc2[NPSIM_MAX_TYPES * NPSIM_MAX_TYPES];
     __shared__ float s_rmax[NPSIM_MAX_TYPES];
+    const int p = (int)(gridDim.x - 1 - blockIdx.x) * (int)blockDim.x + (int)threadIdx.x;
     const bool expired = *flags & FLAG_TIMEOUT; // nobody sets it while this kernel runs
+    int i = 0, cnt = 0;
+    float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint4 cur = make_uint4(0u, 0u, 0u, 0u);
+    if (p < n) { // on their way with the tables and the flags
+        i = sorted[p];
+        cnt = nnbr[p];
+        pi = sxq[p];
+        cur = __ldcs(reinterpret_cast<const uint4 *>(nbr) + p);
+    }
     load_tables(tab, COUL ? rcc2 : nullptr, 0.0f, s_tab, s_rl2, s_rmax, s_rcc2);
     if (expired) // unfinished lists (wait_expired); the gate stays open
         return;
     if (gate && blockIdx.x == 0 && threadIdx.x == 0)
         *gate = 0; // every build kernel of this step has run; the integrator may reopen it
-    const int p = (int)(gridDim.x - 1 - blockIdx.x) * (int)blockDim.x + (int)threadIdx.x;
     if (p < n) {
-        const int i = sorted[p];
-        const float4 pi = sxq[p];
-        const uint4 cur = __ldcs(reinterpret_cast<const uint4 *>(nbr) + p);
         float4 o0, o1;
-        slot_forces<COUL>(p, i, pi, cur, nnbr[p], g, start, sorted, key, sxq, n, cap, nbr, F_lj,
-                          s_tab, s_rcc2, o0, o1);
+        slot_forces<COUL>(p, i, pi, cur, cnt, g, start, sorted, key, sxq, n, cap, nbr, F_lj, s_tab,
+                          s_rcc2, o0, o1);
         // one 32-byte record per NP, a whole DRAM sector
         float4 *o = reinterpret_cast<float4 *>(F_lj + 8 * (size_t)i);
         o[0] = o0;
@@ -855,8 +861,7 @@ k_list_steps(const __grid_constant__ FusedStepArgs a, const __grid_constant__ St
     load_tables(L.tab, COUL ? L.rcc2 : nullptr, 0.0f, s_tab, s_rl2, s_rmax, s_rcc2);
     if (threadIdx.x < NPSIM_MAX_TYPES)
         s_tc[threadIdx.x] = p.tc[threadIdx.x];
-    if (threadIdx.x == 0)
-        S.polls = L.bar[kBarPolls];
+    const unsigned polls = L.bar[kBarPolls];
     if (wait_expired(L.flags)) // its barrier orders the tables, too
         return;
     const long long step0 = *a.I.step;
@@ -894,7 +899,7 @@ k_list_steps(const __grid_constant__ FusedStepArgs a, const __grid_constant__ St
     float nz[3] = {0.f, 0.f, 0.f};
     for (int j = 1; j <= a.steps; ++j) {
         const bool last = j == a.steps;
-        if (!grid_barrier(L.bar, phase, L.flags, S))
+        if (!grid_barrier(L.bar, phase, polls, L.flags, &S.ok))
             return;
         float4 *cur = (j & 1) ? L.b.sxq : a.sxq2, *nxt = (j & 1) ? a.sxq2 : L.b.sxq;
         volatile unsigned *w = a.gates;
@@ -902,8 +907,9 @@ k_list_steps(const __grid_constant__ FusedStepArgs a, const __grid_constant__ St
         if (build) {
             if (mine && j > 1)
                 slot_store(a, n, s);
-            if (!grid_barrier(L.bar, phase, L.flags, S) || !list_build(L, cur, S, phase) ||
-                !grid_barrier(L.bar, phase, L.flags, S))
+            if (!grid_barrier(L.bar, phase, polls, L.flags, &S.ok) ||
+                !list_build(L, cur, S, phase, polls) ||
+                !grid_barrier(L.bar, phase, polls, L.flags, &S.ok))
                 return;
         }
         if (mine && (build || j == 1)) {

@@ -219,6 +219,8 @@ struct npsim_sim {
     size_t cells_alloc = 0;  // sort keys the cell buffers hold
     NbrList nl{};          // Verlet list over the cells (cell-list LJ)
     int *d_gate = nullptr; // 1: rebuild the cell and neighbour lists at the next pass
+    bool gate_open = false;    // the host has set it since the last list pass
+    bool flags_unread = false; // lists may have been built since the flags were read
     unsigned *list_bar = nullptr; // words of the list kernels' grid barrier (kBarWords)
     int fused_cap = 0;            // largest n that takes fused steps
     float4 *sxq2 = nullptr;       // the other cell-ordered records of fused steps (lazy)
@@ -754,6 +756,7 @@ int get_graph(npsim_sim *s, int k, cudaGraphExec_t *out)
 
 int set_gate(npsim_sim *s, int v)
 {
+    s->gate_open = v != 0;
     if (s->d_gate) {
         NP_CUDA(cudaMemcpyAsync(s->d_gate, &v, sizeof(int), cudaMemcpyHostToDevice, s->user));
         NP_CUDA(cudaStreamSynchronize(s->user)); // v lives on this stack frame
@@ -827,6 +830,7 @@ int read_flags(npsim_sim *s)
     int h = 0;
     NP_CUDA(cudaMemcpyAsync(&h, s->d_flags, sizeof(int), cudaMemcpyDeviceToHost, s->user));
     NP_CUDA(cudaStreamSynchronize(s->user));
+    s->flags_unread = false;
     if (h & FLAG_TIMEOUT) { // before all else: the other bits may come of it
         NP_CUDA(cudaMemsetAsync(s->d_flags, 0, sizeof(int), s->user));
         int rc = recover_lists(s);
@@ -1200,6 +1204,7 @@ int finish_upload(npsim_sim *s, int64_t step, bool rebuild = true)
     int rc = enqueue_pass(s, MODE_FORCES, true, true, true, s->F, s->user);
     if (rc)
         return rc;
+    s->gate_open = false;
     NP_CUDA(cudaStreamSynchronize(s->user));
     s->step = step;
     return read_flags(s);
@@ -1708,6 +1713,8 @@ int enqueue_fused(npsim_sim *s, int k)
 int enqueue_steps(npsim_sim *s, int64_t n_steps)
 {
     int64_t rem = n_steps;
+    if (rem > 0 && s->cell)
+        s->flags_unread = true;
     while (rem > 0) {
         int rc0 = regrid_if_needed(s);
         if (rc0)
@@ -1744,6 +1751,8 @@ int enqueue_steps(npsim_sim *s, int64_t n_steps)
         rem -= k;
         s->step += k;
     }
+    if (n_steps > 0)
+        s->gate_open = false; // their last pass leaves the gate closed
     return NPSIM_OK;
 }
 } // namespace
@@ -1856,11 +1865,18 @@ int npsim_forces(npsim_sim_t s, int what, double *F)
     NP_REQUIRE(what >= 0 && what <= 3, "what must be 0..3");
     const bool lj = what == 0 || what == 1 || what == 2;
     const bool coul = what == 0 || what == 1 || what == 3;
+    // the lists are built in this pass only if the host has opened the gate; a build may
+    // give up, and reading the flags takes 12 us
+    const bool lists = s->cell && (lj || (coul && s->P.coulomb == 2));
+    if (lists && s->gate_open)
+        s->flags_unread = true;
     int rc = enqueue_pass(s, MODE_FORCES, lj, coul, what == 0, s->F_tmp, s->user);
     if (rc)
         return rc;
+    if (lists)
+        s->gate_open = false;
     rc = copy_state_out(s, s->F_tmp, nullptr, nullptr, F);
-    return rc || !s->cell ? rc : read_flags(s); // a build of the lists may have given up
+    return rc || !s->flags_unread ? rc : read_flags(s);
 }
 
 int npsim_test_list_wait(npsim_sim_t s, int64_t polls)
